@@ -83,10 +83,13 @@ struct stp_handle {
   bool host_solve = false;     // STP_HOST_SOLVE=1: drive the solve from the host
   int cycle_blocks = 0;        // >0: FP32 cycles run as one persistent cooperative kernel
   int line_rb = 0;             // >0: FP32 z-line cycles run as one persistent kernel (tile rows)
+  bool colour = false;         // FP32 inner solves by two-colour sweeps (see use_colour)
+  std::vector<float> col_omega;  // their schedule
   int line_variant = 0;        // FP32 z-line sweep kernel: 1 register-chunked columns, 0 shared-memory lock step
   int* line_flags = nullptr;   // its per-tile sweep counters
   int sweep_variant = -1;      // FP32 sweep kernel variant chosen by the autotuner (-1: not yet)
   float sweep_us = 0.f;        // its measured time per sweep
+  bool tuned_colour = false;   // sweep_variant is a two-colour variant
   float* d_omega32 = nullptr;  // the schedule on the device (FP32)
   GridBar bar{};
   // learned guess and training-pair harvest
@@ -320,6 +323,19 @@ std::vector<double> chebyshev(double mn, double mx, int M) {
   return om;
 }
 
+// the factors of M two-colour sweeps (kernels_colour.cu): Chebyshev
+// acceleration for a Jacobi spectrum within [mn, 2 - mn]
+std::vector<float> colour_schedule(double mn, int M) {
+  const double s2 = (1.0 - mn) * (1.0 - mn);
+  std::vector<float> om;
+  double w = 1.0;
+  for (int m = 0; m < M; m++) {
+    om.push_back((float)w);
+    w = m == 0 ? 1.0 / (1.0 - 0.5 * s2) : 1.0 / (1.0 - 0.25 * s2 * w);
+  }
+  return om;
+}
+
 bool pow2(int m) { return m >= 1 && (m & (m - 1)) == 0; }
 
 int auto_cycle(double mn, double mx) {
@@ -550,6 +566,40 @@ bool uses_pairs(const stp_handle* h) {
          h->omega.size() % 4 == 0;
 }
 
+// the inner solve runs two-colour sweeps (a learned guess hands residuals and
+// corrections to the network in the natural layout, so it keeps Jacobi sweeps)
+bool use_colour(const stp_handle* h) { return h->colour && !h->net; }
+
+// refinement residual into r32, in the layout of the inner solve
+cudaError_t launch_inner_residual(stp_handle* h, int after_pass, int graph, cudaGraphConditionalHandle h_loop,
+                                  cudaStream_t s) {
+  return use_colour(h) ? launch_colour_outer(h->g64, h->p, h->b, h->r32, h->cfg.zline, h->ctl, h->red, after_pass, graph,
+                                             h_loop, s)
+                       : launch_outer(h->g64, h->p, h->b, h->r32, h->ctl, h->red, after_pass, graph, h_loop, s);
+}
+// p += the inner solve's correction
+cudaError_t launch_inner_correction(stp_handle* h, cudaStream_t s) {
+  return use_colour(h) ? launch_colour_addcorr(h->g64, h->p, h->d1, h->cfg.zline, s)
+                       : launch_addcorr(h->p, h->d1, h->nc, s);
+}
+// one cycle of the inner solve, in place in d1
+int launch_colour_cycle(stp_handle* h, cudaStream_t s) {
+  const int M = (int)h->col_omega.size();
+  for (int m = 0; m < M; m++)
+    CUDA_TRY(h, launch_colour_sweep(h->g32, h->d1, h->r32, h->col_omega[m], m & 1, h->cfg.zline, h->sweep_variant, s));
+  return STP_OK;
+}
+cudaError_t launch_cycle_check(stp_handle* h, const Geom<double>& g, const double* A, const double* rhs, int mode, int graph,
+                               cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_body, cudaStream_t s) {
+  return launch_check<double>(g, A, rhs, mode, h->ctl, h->red, graph, h_loop, h_body, s);
+}
+cudaError_t launch_cycle_check(stp_handle* h, const Geom<float>& g, const float* A, const float* rhs, int mode, int graph,
+                               cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_body, cudaStream_t s) {
+  if (use_colour(h))
+    return launch_colour_check(g, A, rhs, h->cfg.zline, h->ctl, h->red, graph, h_loop, h_body, s);
+  return launch_check<float>(g, A, rhs, mode, h->ctl, h->red, graph, h_loop, h_body, s);
+}
+
 // the cycle: check -> IF { M sweeps }, inside the WHILE body `wb`
 template <typename T>
 int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphConditionalHandle h_loop, T* A, T* B,
@@ -558,7 +608,7 @@ int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphCondit
   CUDA_TRY(h, cudaGraphConditionalHandleCreate(&h_body, wb, 0, cudaGraphCondAssignDefault));
   int rc;
   if ((rc = begin_capture(h, wb, nullptr))) return rc;
-  CUDA_TRY(h, launch_check<T>(g, A, rhs, mode, h->ctl, h->red, 1, h_loop, h_body, h->cap));
+  CUDA_TRY(h, launch_cycle_check(h, g, A, rhs, mode, 1, h_loop, h_body, h->cap));
   if ((rc = end_capture(h, wb))) return rc;
   cudaGraph_t ib;
   cudaGraphNode_t ifn;
@@ -572,6 +622,10 @@ int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphCondit
     if ((rc = unet_guess(h->net, h->r32, h->red.sc + SC_INNER_REF, h->d1, h->cap, &h->guess_kernels)))
       return fail(h, rc, "learned preconditioner: " + std::string(stp_unet_last_error(h->net)));
     CUDA_TRY(h, launch_addcorr(h->p, h->d1, h->nc, h->cap));
+  }
+  if (sizeof(T) == sizeof(float) && use_colour(h)) {
+    if ((rc = launch_colour_cycle(h, h->cap))) return rc;
+    return end_capture(h, ib);
   }
   if (sizeof(T) == sizeof(float) && h->cycle_blocks > 0) {
     // the whole cycle in one persistent kernel
@@ -612,12 +666,15 @@ int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphCondit
 // as the solve runs it: 20 sweeps (10 launches of a pair variant) captured
 // into a graph (programmatic dependent launches between them), best of
 // three launches after a warm-up launch, CUDA events on the handle's stream.
-int time_sweeps(stp_handle* h, bool pair, float* us) {
+int time_sweeps(stp_handle* h, bool pair, float* us, bool colour = false) {
   cudaGraph_t g = nullptr;
   cudaGraphExec_t x = nullptr;
   cudaError_t e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeRelaxed);
   const bool capturing = e == cudaSuccess;
-  if (pair) {
+  if (colour) {
+    for (int w = 0; w < 20 && e == cudaSuccess; w++)
+      e = launch_colour_sweep(h->g32, h->d1, h->r32, 1.0f, w & 1, h->cfg.zline, h->sweep_variant, h->cap);
+  } else if (pair) {
     for (int w = 0; w < 10 && e == cudaSuccess; w++)
       e = launch_sweep_pair(h->g32, (w & 1) ? h->d2 : h->d1, h->r32, 1.0f, 1.0f, (w & 1) ? h->d1 : h->d2, h->cap);
   } else {
@@ -661,13 +718,56 @@ int pick_variant(const std::vector<std::pair<int, float>>& timed, float* us) {
   return 0;
 }
 
+// Autotuner of the two-colour sweep: the levels a thread relaxes, timed as
+// tune_sweep times its tiles; cached per device, grid and kind.
+int tune_colour(stp_handle* h) {
+  const bool line = h->cfg.zline != 0;
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int, int, bool>, std::pair<int, float>> cache;
+  const auto key = std::make_tuple(h->dev, h->nx, h->ny, h->nz, line);
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find(key);
+    if (it != cache.end()) {
+      h->sweep_variant = it->second.first;
+      h->sweep_us = it->second.second;
+      return STP_OK;
+    }
+  }
+  CUDA_TRY(h, cudaMemsetAsync(h->d1, 0, sizeof(float) * h->nc, h->st));
+  CUDA_TRY(h, cudaMemsetAsync(h->r32, 0, sizeof(float) * h->nc, h->st));
+  std::vector<std::pair<int, float>> timed;
+  for (int v = 0; v < colour_variants(line); v++) {
+    if (!colour_variant_ok(v, h->nx, h->nz, line)) continue;
+    h->sweep_variant = v;
+    float us = 0.f;
+    if (int rc = time_sweeps(h, false, &us, true)) return rc;
+    timed.emplace_back(v, us);
+  }
+  const int bv = pick_variant(timed, &h->sweep_us);
+  h->sweep_variant = bv;
+  if (const char* lg = std::getenv("STP_TUNE_LOG")) {
+    if (std::atoi(lg)) {
+      std::fprintf(stderr, "stp: two-colour sweeps at %dx%dx%d (us per sweep):", h->nx, h->ny, h->nz);
+      for (const auto& t : timed) std::fprintf(stderr, " %d=%.3f", t.first, t.second);
+      std::fprintf(stderr, " -> %d\n", bv);
+    }
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  cache[key] = std::make_pair(bv, h->sweep_us);
+  return STP_OK;
+}
+
 // Autotuner of the FP32 sweep kernel: times every variant valid for this
 // grid (time_sweeps, on the handle's own scratch buffers) and keeps the
 // choice of pick_variant; cached per (device, nx, ny, nz).
 // STP_SWEEP_VARIANT=<v> forces a variant.  All variants compute the same values.
 int tune_sweep(stp_handle* h) {
-  if (h->sweep_variant >= 0) return STP_OK;
+  const bool colour = use_colour(h);
+  if (h->sweep_variant >= 0 && h->tuned_colour == colour) return STP_OK;
   h->sweep_variant = 0;
+  h->tuned_colour = colour;
+  if (colour) return tune_colour(h);
   if (h->prec != STP_FP32_REFINE || h->nx % 4 || h->cfg.zline) return STP_OK;
   if (const char* env = std::getenv("STP_SWEEP_VARIANT")) {
     const int v = std::atoi(env);
@@ -758,7 +858,7 @@ int append_solve(stp_handle* h, cudaGraph_t G, cudaGraphNode_t dep, cudaGraphNod
     CUDA_TRY(h, cudaGraphConditionalHandleCreate(&h_pass, G, 0, cudaGraphCondAssignDefault));
     if ((rc = begin_capture(h, G, dep))) return rc;
     CUDA_TRY(h, launch_begin(h->ctl, 0, 0, h->cap));
-    CUDA_TRY(h, launch_outer(h->g64, h->p, h->b, h->r32, h->ctl, h->red, 0, 1, h_pass, h->cap));
+    CUDA_TRY(h, launch_inner_residual(h, 0, 1, h_pass, h->cap));
     if (h->net && h->learned_mode == 0) {
       // learned guess at the start of the solve: p += s U(r / s), then the
       // residual of the new p decides the first pass
@@ -785,8 +885,8 @@ int append_solve(stp_handle* h, cudaGraph_t G, cudaGraphNode_t dep, cudaGraphNod
     if ((rc = add_conditional(h, pb, leaf_node(pb), h_loop, cudaGraphCondTypeWhile, &wb, &wn))) return rc;
     if ((rc = build_cycle<float>(h, h->g32, wb, h_loop, h->d1, h->d2, h->r32, 1))) return rc;
     if ((rc = begin_capture(h, pb, wn))) return rc;
-    CUDA_TRY(h, launch_addcorr(h->p, h->d1, h->nc, h->cap));
-    CUDA_TRY(h, launch_outer(h->g64, h->p, h->b, h->r32, h->ctl, h->red, 1, 1, h_pass, h->cap));
+    CUDA_TRY(h, launch_inner_correction(h, h->cap));
+    CUDA_TRY(h, launch_inner_residual(h, 1, 1, h_pass, h->cap));
     if ((rc = end_capture(h, pb))) return rc;
     *last = pn;
   }
@@ -813,7 +913,7 @@ int arm_solves(stp_handle* h, double tol, int maxit) {
   c.max_sweeps = maxit;
   c.max_passes = 64;
   c.M = (int)h->omega.size();
-  c.kpc = (h->cycle_blocks > 0 || h->line_rb > 0) ? 1 : uses_pairs(h) ? c.M / 2 : c.M;
+  c.kpc = use_colour(h) ? c.M : (h->cycle_blocks > 0 || h->line_rb > 0) ? 1 : uses_pairs(h) ? c.M / 2 : c.M;
   c.bar_wait = 2000000000LL;
   if (const char* e = std::getenv("STP_BARRIER_WAIT")) {
     const long long w = std::atoll(e);
@@ -845,7 +945,7 @@ template <typename T>
 int host_cycles(stp_handle* h, const Geom<T>& g, T* A, T* B, const T* rhs, int mode) {
   const int M = (int)h->omega.size();
   for (;;) {
-    CUDA_TRY(h, launch_check<T>(g, A, rhs, mode, h->ctl, h->red, 0, 0, 0, h->st));
+    CUDA_TRY(h, launch_cycle_check(h, g, A, rhs, mode, 0, 0, 0, h->st));
     int go = 0, rc = read_go(h, &go);
     if (rc) return rc;
     if (!go) return STP_OK;
@@ -854,6 +954,10 @@ int host_cycles(stp_handle* h, const Geom<T>& g, T* A, T* B, const T* rhs, int m
       rc = unet_guess(h->net, h->r32, h->red.sc + SC_INNER_REF, h->d1, h->st, &h->guess_kernels);
       if (rc) return fail(h, rc, "learned preconditioner failed");
       CUDA_TRY(h, launch_addcorr(h->p, h->d1, h->nc, h->st));
+    }
+    if (sizeof(T) == sizeof(float) && use_colour(h)) {
+      if ((rc = launch_colour_cycle(h, h->st))) return rc;
+      continue;
     }
     if (sizeof(T) == sizeof(float) && h->cycle_blocks > 0) {
       CUDA_TRY(h, launch_cycle_f32(h->g32, (float*)A, (float*)B, (const float*)rhs, h->d_omega32, M, h->bar, h->ctl,
@@ -896,7 +1000,7 @@ int host_solve(stp_handle* h) {
     }
     return host_cycles<double>(h, h->g64, h->p, h->p2, h->b, 0);
   }
-  CUDA_TRY(h, launch_outer(h->g64, h->p, h->b, h->r32, h->ctl, h->red, 0, 0, 0, h->st));
+  CUDA_TRY(h, launch_inner_residual(h, 0, 0, 0, h->st));
   if (h->net && h->learned_mode == 0) {
     int rc = unet_guess(h->net, h->r32, h->red.sc + SC_INNER_REF, h->d1, h->st, &h->guess_kernels);
     if (rc) return fail(h, rc, "learned guess failed");
@@ -913,8 +1017,8 @@ int host_solve(stp_handle* h) {
       if (rc) return fail(h, rc, "learned preconditioner failed");
     }
     if ((rc = host_cycles<float>(h, h->g32, h->d1, h->d2, h->r32, 1))) return rc;
-    CUDA_TRY(h, launch_addcorr(h->p, h->d1, h->nc, h->st));
-    CUDA_TRY(h, launch_outer(h->g64, h->p, h->b, h->r32, h->ctl, h->red, 1, 0, 0, h->st));
+    CUDA_TRY(h, launch_inner_correction(h, h->st));
+    CUDA_TRY(h, launch_inner_residual(h, 1, 0, 0, h->st));
   }
 }
 
@@ -1233,11 +1337,13 @@ int stp_init(const stp_config* cfg, stp_handle** out) {
       cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess)
     return bail(fail(h, STP_ECUDA, "event or stream creation failed"));
   // schedule
+  double mu_min = 0.0;
   if (cfg->srj_omega) {
     h->omega.assign(cfg->srj_omega, cfg->srj_omega + cfg->srj_m);
   } else {
     double mn, mx;
     solve_bounds(*cfg, &mn, &mx);
+    mu_min = mn;
     const int M = cfg->srj_m > 0 ? cfg->srj_m : auto_cycle(mn, mx);
     h->omega = chebyshev(mn, mx, M);
   }
@@ -1328,6 +1434,13 @@ int stp_init(const stp_config* cfg, stp_handle** out) {
       if (rb > 0 && dalloc(h, (void**)&h->line_flags, sizeof(int) * line_cycle_tiles(gtmp, rb)) == STP_OK)
         h->line_rb = rb;
     }
+  }
+  if (h->prec == STP_FP32_REFINE && !cfg->srj_omega && h->cycle_blocks == 0 && h->line_rb == 0 &&
+      (!cfg->zline || h->line_variant == 1 || !line_chunk_ok(h->nx, h->nz)) &&
+      colour_ok(h->nx, h->ny, h->nz, cfg->zline != 0)) {
+    const char* env = std::getenv("STP_SRJ_COLOURS");
+    h->colour = !(env && env[0] == '0') && !std::getenv("STP_SWEEP_VARIANT");
+    if (h->colour) h->col_omega = colour_schedule(mu_min, (int)h->omega.size());
   }
   if (cudaMallocHost((void**)&h->h_sc, sizeof(double) * SC_COUNT) != cudaSuccess ||
       cudaMallocHost((void**)&h->h_flag, sizeof(int) * FL_COUNT) != cudaSuccess ||
@@ -1799,6 +1912,7 @@ void plan_groups(stp_batch* b) {
   std::map<int, std::vector<int>> byM;
   for (size_t i = 0; i < b->hs.size(); i++) {
     stp_handle* h = b->hs[i];
+    if (use_colour(h)) continue;
     if (h->prec != STP_FP32_REFINE || h->nx % 4 || h->net || h->cycle_blocks > 0 || h->cfg.zline) continue;
     if (max_ch >= 0 && (long long)h->nc > max_ch) continue;
     byM[(int)h->omega.size()].push_back((int)i);

@@ -242,6 +242,23 @@ cudaError_t launch_difference(const double* a, const double* b, float* out, size
 // (in a graph it also arms the WHILE handle h_loop of an FP64 solve)
 cudaError_t launch_begin(SolveCtl* ctl, int graph, cudaGraphConditionalHandle h_loop, cudaStream_t s);
 
+// Two-colour FP32 sweeps (kernels_colour.cu): inner solves on the library's own
+// schedule with nx, ny even.  d and r hold the two colours one after the
+// other, each [nz][ny][nx/2]; sweep m relaxes colour m & 1 in place.  line:
+// z-line sweeps (columns of up to 192 levels).
+bool colour_ok(int nx, int ny, int nz, bool line);
+int colour_variants(bool line);
+bool colour_variant_ok(int v, int nx, int nz, bool line);
+cudaError_t launch_colour_sweep(const Geom<float>& g, float* d, const float* r, float om, int c, int line, int variant,
+                                cudaStream_t s);
+cudaError_t launch_colour_check(const Geom<float>& g, const float* d, const float* r, int line, SolveCtl* ctl, Red red,
+                                int graph, cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_body,
+                                cudaStream_t s);
+cudaError_t launch_colour_outer(const Geom<double>& g, const double* p, const double* b, float* r32, int line,
+                                SolveCtl* ctl, Red red, int after_pass, int graph, cudaGraphConditionalHandle h_loop,
+                                cudaStream_t s);
+cudaError_t launch_colour_addcorr(const Geom<double>& g, double* p, const float* d, int line, cudaStream_t s);
+
 // ---------------------------------------------------------------------------
 // Grouped FP32 pressure solves (kernels_group.cu).  In the batched step the
 // channels that share an SRJ cycle length M are solved in lock step: each
