@@ -90,6 +90,7 @@ struct stp_handle {
   int sweep_variant = -1;      // FP32 sweep kernel variant chosen by the autotuner (-1: not yet)
   float sweep_us = 0.f;        // its measured time per sweep
   bool tuned_colour = false;   // sweep_variant is a two-colour variant
+  double* sweep_tab = nullptr; // FP64 point sweeps: level coefficients of every sweep of a cycle (launch_sweep_table)
   float* d_omega32 = nullptr;  // the schedule on the device (FP32)
   GridBar bar{};
   // learned guess and training-pair harvest
@@ -420,8 +421,10 @@ Geom<T> geom_from(const stp_handle* h, T* pack) {
   g.tli = pack + 13 * L;
   g.tlf = pack + 14 * L;
   g.tlb = pack + 15 * L;
+  g.pf = pack + 16 * L;
+  g.pe = pack + 17 * L;
   // the packed level coefficients follow the kMetricArrays arrays (offset
-  // 64 L bytes: 16-byte aligned)
+  // 80 L bytes: 16-byte aligned)
   if constexpr (sizeof(T) == sizeof(float)) g.lz4 = reinterpret_cast<const float4*>(pack + kMetricArrays * L);
   else g.lz4 = nullptr;
   return g;
@@ -489,6 +492,18 @@ std::vector<double> metric_pack(const stp_config& c) {
         m[14 * L + k] = cdn[k] / gam;
         m[15 * L + k] = cup[k] / gam;
       }
+    }
+  }
+  // products of the elimination's and the substitution's coefficients inside
+  // the FP64 z-line chunks
+  if (const int nch = line_f64_chunks(c.nx, c.ny, nz)) {
+    for (int ch = 0; ch < nch; ch++) {
+      const int k0 = line_chunk_start(ch, nch, nz), k1 = line_chunk_start(ch + 1, nch, nz);
+      const bool lower = ch < nch / 2;
+      const int f0 = ch == nch / 2 ? k0 + 1 : k0;  // the twist level stays out
+      double up = 1.0, dn = 1.0;
+      for (int k = f0; k < k1; k++) m[(lower ? 16 : 17) * L + k] = up *= m[(lower ? 14 : 15) * L + k];
+      for (int k = k1 - 1; k >= f0; k--) m[(lower ? 17 : 16) * L + k] = dn *= m[(lower ? 15 : 14) * L + k];
     }
   }
   for (int k = 0; k <= nz; k++) {
@@ -570,6 +585,23 @@ bool uses_pairs(const stp_handle* h) {
 // corrections to the network in the natural layout, so it keeps Jacobi sweeps)
 bool use_colour(const stp_handle* h) { return h->colour && !h->net; }
 
+// cycles run as one launch on a thread-block cluster
+bool uses_cluster(const stp_handle* h) {
+  return h->prec == STP_FP32_REFINE && !use_colour(h) && h->cycle_blocks == 0 && !h->cfg.zline &&
+         h->sweep_variant >= kClusterVariant0;
+}
+cudaError_t launch_cluster(stp_handle* h, float* d, const float* r, int M, cudaStream_t s) {
+  return launch_cluster_cycle(h->g32, d, r, h->d_omega32, M, h->sweep_variant - kClusterVariant0, s);
+}
+
+// sweep m of a cycle of point Jacobi-SOR sweeps
+cudaError_t launch_jacobi(stp_handle* h, const double* p, const double* b, int m, double* out, cudaStream_t s) {
+  return launch_sweep_f64(h->g64, p, b, h->omega[m], h->sweep_tab ? h->sweep_tab + (size_t)5 * h->nz * m : nullptr, out, s);
+}
+cudaError_t launch_jacobi(stp_handle* h, const float* p, const float* b, int m, float* out, cudaStream_t s) {
+  return launch_sweep_f32(h->g32, p, b, (float)h->omega[m], out, s);
+}
+
 // refinement residual into r32, in the layout of the inner solve
 cudaError_t launch_inner_residual(stp_handle* h, int after_pass, int graph, cudaGraphConditionalHandle h_loop,
                                   cudaStream_t s) {
@@ -644,6 +676,10 @@ int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphCondit
                                        h->line_variant));
     return end_capture(h, ib);
   }
+  if (sizeof(T) == sizeof(float) && uses_cluster(h)) {
+    CUDA_TRY(h, launch_cluster(h, (float*)A, (const float*)rhs, M, h->cap));
+    return end_capture(h, ib);
+  }
   if (sizeof(T) == sizeof(float) && uses_pairs(h)) {
     // two sweeps per launch: A -> B, B -> A, ... (M / 2 even: ends in A)
     for (int m = 0; m < M; m += 2) {
@@ -657,7 +693,7 @@ int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphCondit
   for (int m = 0; m < M; m++) {
     const T* src = (m % 2 == 0) ? A : B;
     T* dst = (m % 2 == 0) ? B : A;
-    CUDA_TRY(h, launch_sweep<T>(g, src, rhs, (T)h->omega[m], dst, h->cap));
+    CUDA_TRY(h, launch_jacobi(h, src, rhs, m, dst, h->cap));
   }
   return end_capture(h, ib);
 }
@@ -666,12 +702,15 @@ int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphCondit
 // as the solve runs it: 20 sweeps (10 launches of a pair variant) captured
 // into a graph (programmatic dependent launches between them), best of
 // three launches after a warm-up launch, CUDA events on the handle's stream.
-int time_sweeps(stp_handle* h, bool pair, float* us, bool colour = false) {
+int time_sweeps(stp_handle* h, bool pair, float* us, bool colour = false, bool cluster = false) {
   cudaGraph_t g = nullptr;
   cudaGraphExec_t x = nullptr;
   cudaError_t e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeRelaxed);
   const bool capturing = e == cudaSuccess;
-  if (colour) {
+  const int cycle = std::min(256, (int)h->omega.size());
+  if (cluster) {
+    e = launch_cluster(h, h->d1, h->r32, cycle, h->cap);
+  } else if (colour) {
     for (int w = 0; w < 20 && e == cudaSuccess; w++)
       e = launch_colour_sweep(h->g32, h->d1, h->r32, 1.0f, w & 1, h->cfg.zline, h->sweep_variant, h->cap);
   } else if (pair) {
@@ -679,7 +718,7 @@ int time_sweeps(stp_handle* h, bool pair, float* us, bool colour = false) {
       e = launch_sweep_pair(h->g32, (w & 1) ? h->d2 : h->d1, h->r32, 1.0f, 1.0f, (w & 1) ? h->d1 : h->d2, h->cap);
   } else {
     for (int w = 0; w < 20 && e == cudaSuccess; w++)
-      e = launch_sweep<float>(h->g32, (w & 1) ? h->d2 : h->d1, h->r32, 1.0f, (w & 1) ? h->d1 : h->d2, h->cap);
+      e = launch_sweep_f32(h->g32, (w & 1) ? h->d2 : h->d1, h->r32, 1.0f, (w & 1) ? h->d1 : h->d2, h->cap);
   }
   if (capturing) {
     const cudaError_t e2 = cudaStreamEndCapture(h->cap, &g);
@@ -699,7 +738,7 @@ int time_sweeps(stp_handle* h, bool pair, float* us, bool colour = false) {
   if (x) cudaGraphExecDestroy(x);
   if (g) cudaGraphDestroy(g);
   if (e != cudaSuccess) return fail(h, STP_ECUDA, std::string("sweep autotuner: ") + cudaGetErrorString(e));
-  *us = best * 1e3f / 20.f;
+  *us = best * 1e3f / (cluster ? (float)cycle : 20.f);
   return STP_OK;
 }
 
@@ -768,10 +807,13 @@ int tune_sweep(stp_handle* h) {
   h->sweep_variant = 0;
   h->tuned_colour = colour;
   if (colour) return tune_colour(h);
-  if (h->prec != STP_FP32_REFINE || h->nx % 4 || h->cfg.zline) return STP_OK;
+  if (h->prec != STP_FP32_REFINE || h->cfg.zline) return STP_OK;
+  const bool can_cluster = h->cycle_blocks == 0;
   if (const char* env = std::getenv("STP_SWEEP_VARIANT")) {
     const int v = std::atoi(env);
-    if (sweep_variant_ok(v, h->nx, h->ny, h->nz)) h->sweep_variant = v;
+    if (sweep_variant_ok(v, h->nx, h->ny, h->nz) ||
+        (can_cluster && cluster_ok(v - kClusterVariant0, h->nx, h->ny, h->nz)))
+      h->sweep_variant = v;
     return STP_OK;
   }
   static std::mutex mu;
@@ -790,7 +832,8 @@ int tune_sweep(stp_handle* h) {
   CUDA_TRY(h, cudaMemsetAsync(h->r32, 0, sizeof(float) * h->nc, h->st));
   std::vector<std::pair<int, float>> timed;
   for (int v = 0; v < sweep_variant_count(); v++) {
-    if (!sweep_variant_ok(v, h->nx, h->ny, h->nz)) continue;
+    // (rows that are no multiple of 4 cells have one launched kernel, 0)
+    if (h->nx % 4 ? v != 0 : !sweep_variant_ok(v, h->nx, h->ny, h->nz)) continue;
     const bool pair = sweep_variant_is_pair(v);
     if (pair && (h->omega.size() % 4 != 0 || h->cycle_blocks > 0)) continue;
     set_sweep_variant(v);
@@ -803,7 +846,27 @@ int tune_sweep(stp_handle* h) {
     }
     timed.emplace_back(v, us);
   }
-  const int bv = pick_variant(timed, &h->sweep_us);
+  const size_t n_launched = timed.size();
+  for (int v = 0; can_cluster && v < cluster_variants(); v++) {
+    if (!cluster_ok(v, h->nx, h->ny, h->nz)) continue;
+    h->sweep_variant = kClusterVariant0 + v;
+    float us = 0.f;
+    if (time_sweeps(h, false, &us, false, true)) {
+      cudaGetLastError();  // no such cluster on this device: not a candidate
+      h->err.clear();
+      continue;
+    }
+    timed.emplace_back(kClusterVariant0 + v, us);
+  }
+  // a cluster loads its channel once a cycle, which the timing spreads over
+  // 256 sweeps at best: it has to be clearly faster
+  std::vector<std::pair<int, float>> launched(timed.begin(), timed.begin() + n_launched);
+  int bv = pick_variant(launched, &h->sweep_us);
+  for (size_t q = n_launched; q < timed.size(); q++)
+    if (timed[q].second < (bv >= kClusterVariant0 ? 1.0f : 0.85f) * h->sweep_us) {
+      bv = timed[q].first;
+      h->sweep_us = timed[q].second;
+    }
   h->sweep_variant = bv;
   if (const char* lg = std::getenv("STP_TUNE_LOG")) {
     if (std::atoi(lg)) {
@@ -913,7 +976,7 @@ int arm_solves(stp_handle* h, double tol, int maxit) {
   c.max_sweeps = maxit;
   c.max_passes = 64;
   c.M = (int)h->omega.size();
-  c.kpc = use_colour(h) ? c.M : (h->cycle_blocks > 0 || h->line_rb > 0) ? 1 : uses_pairs(h) ? c.M / 2 : c.M;
+  c.kpc = use_colour(h) ? c.M : (uses_cluster(h) || h->cycle_blocks > 0 || h->line_rb > 0) ? 1 : uses_pairs(h) ? c.M / 2 : c.M;
   c.bar_wait = 2000000000LL;
   if (const char* e = std::getenv("STP_BARRIER_WAIT")) {
     const long long w = std::atoll(e);
@@ -975,6 +1038,10 @@ int host_cycles(stp_handle* h, const Geom<T>& g, T* A, T* B, const T* rhs, int m
                                          h->st, h->line_variant));
       continue;
     }
+    if (sizeof(T) == sizeof(float) && uses_cluster(h)) {
+      CUDA_TRY(h, launch_cluster(h, (float*)A, (const float*)rhs, M, h->st));
+      continue;
+    }
     if (sizeof(T) == sizeof(float) && uses_pairs(h)) {
       for (int m = 0; m < M; m += 2)
         CUDA_TRY(h, launch_sweep_pair(h->g32, (const float*)((m % 4 == 0) ? A : B), (const float*)rhs,
@@ -983,7 +1050,7 @@ int host_cycles(stp_handle* h, const Geom<T>& g, T* A, T* B, const T* rhs, int m
       continue;
     }
     for (int m = 0; m < M; m++)
-      CUDA_TRY(h, launch_sweep<T>(g, (m % 2 == 0) ? A : B, rhs, (T)h->omega[m], (m % 2 == 0) ? B : A, h->st));
+      CUDA_TRY(h, launch_jacobi(h, (m % 2 == 0) ? A : B, rhs, m, (m % 2 == 0) ? B : A, h->st));
   }
 }
 
@@ -1361,7 +1428,12 @@ int stp_init(const stp_config* cfg, stp_handle** out) {
     if (rc == STP_OK) rc = dalloc(h, p, bytes);
   };
   const int L = h->nz + 1;
-  A((void**)&h->m64, sizeof(double) * kMetricArrays * L);
+  // the metrics and, behind them, the level coefficients of the FP64 point
+  // sweeps (up to 64 MB; beyond it the sweeps form them) and the schedule
+  size_t tab_words = (size_t)5 * h->nz * h->omega.size();
+  if (h->prec != STP_FP64 || cfg->zline || tab_words > (size_t)8 << 20) tab_words = 0;
+  A((void**)&h->m64, sizeof(double) * ((size_t)kMetricArrays * L + tab_words + (tab_words ? h->omega.size() : 0)));
+  if (tab_words && h->m64) h->sweep_tab = h->m64 + (size_t)kMetricArrays * L;
   A((void**)&h->m32, sizeof(float) * (kMetricArrays + 4) * L);
   A(&h->u, es * nc);
   A(&h->v, es * nc);
@@ -1484,6 +1556,11 @@ int stp_init(const stp_config* cfg, stp_handle** out) {
   if (e == cudaSuccess) e = cudaMemsetAsync(h->ctl, 0, sizeof(SolveCtl), h->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->bar.count, 0, sizeof(unsigned) * 4, h->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_step, 0, sizeof(int) * 4, h->st);
+  if (e == cudaSuccess && h->sweep_tab) {
+    double* om = h->sweep_tab + tab_words;
+    e = cudaMemcpyAsync(om, h->omega.data(), sizeof(double) * h->omega.size(), cudaMemcpyHostToDevice, h->st);
+    if (e == cudaSuccess) e = launch_sweep_table(h->g64, om, (int)h->omega.size(), h->sweep_tab, h->st);
+  }
   if (e == cudaSuccess) {
     std::vector<float> om32(h->omega.begin(), h->omega.end());
     e = cudaMemcpyAsync(h->d_omega32, om32.data(), sizeof(float) * om32.size(), cudaMemcpyHostToDevice, h->st);

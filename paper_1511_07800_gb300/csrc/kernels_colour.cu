@@ -470,11 +470,20 @@ cudaError_t line_w(const Geom<float>& g, float* own, const float* oth, const flo
   return launch_dep(k_col_line<W, NCH, kLineLevels, MINB>, blocks, 8 * NCH, s, g, own, oth, r, om, c);
 }
 
+// Channels of at least this many cells.  Below it a sweep is bound by its launch
+// rather than by its cells (us a Jacobi / colour sweep: 32^3 1.68 / 1.62,
+// 64 x 48 x 40 1.73 / 1.58, 128 x 64 x 128 2.83 / 2.33; 240 x 140 x 120 6.7 /
+// 5.2, 256 x 128 x 192 z lines 17.7 / 11.5), and such channels have other ways
+// to save launches (kernels_cluster.cu).
+constexpr long long kColourCells = 1 << 21;
+
 int col_width(int nx) { return nx % 8 == 0 ? 4 : nx % 4 == 0 ? 2 : 1; }
 
 }  // namespace
 
-bool colour_ok(int nx, int ny, int nz, bool line) { return nx % 2 == 0 && ny % 2 == 0 && (!line || nz <= 192); }
+bool colour_ok(int nx, int ny, int nz, bool line) {
+  return nx % 2 == 0 && ny % 2 == 0 && (!line || nz <= 192) && (long long)nx * ny * nz >= kColourCells;
+}
 
 int colour_variants(bool line) { return line ? (int)(sizeof(kLineVariants) / sizeof(LineVariant)) : 3; }
 

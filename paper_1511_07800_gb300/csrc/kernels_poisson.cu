@@ -24,43 +24,36 @@
 namespace stp {
 
 namespace {
-// FP32: difference form (no cancellation against S p).
+// FP32 sweep of rows that are no multiple of 4 cells: W (2 or 1) cells a
+// thread, the row's units, then the rows, in one sequence (full warps on any
+// row length).  Difference form (no cancellation against S p).
+template <int W>
 __global__ void __launch_bounds__(kBX* kBY) k_sweep_f32(Geom<float> g, const float* __restrict__ p,
                                                          const float* __restrict__ b, float omega,
                                                          float* __restrict__ out) {
-  const int i = blockIdx.x * kBX + threadIdx.x, j = blockIdx.y * kBY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.nx || j >= g.ny) return;
-  const int nx = g.nx, plane = g.nx * g.ny;
-  const int ip = i == nx - 1 ? 0 : i + 1, im = i == 0 ? nx - 1 : i - 1;
-  const int jp = j == g.ny - 1 ? 0 : j + 1, jm = j == 0 ? g.ny - 1 : j - 1;
-  const int row = k * plane, q = row + j * nx + i;
-  const float pc = __ldg(p + q);
-  const float uu = k < g.nz - 1 ? __ldg(p + q + plane) : pc, dd = k > 0 ? __ldg(p + q - plane) : pc;
-  out[q] = srj_cell_f32(pc, __ldg(p + row + j * nx + im), __ldg(p + row + j * nx + ip), __ldg(p + row + jp * nx + i),
-                        __ldg(p + row + jm * nx + i), uu, dd, __ldg(b + q), g.idx2, g.idy2, __ldg(g.cup + k),
-                        __ldg(g.cdn + k), __ldg(g.iS + k), omega);
-}
-
-// FP64: the neighbour-sum form p + omega (p^J - p), p^J = (sum_nb c p_nb - b)/S,
-// which needs fewest FP64 operations (the FP64 sweep is bound by FP64
-// arithmetic on this part, not by memory).
-__global__ void __launch_bounds__(kBX* kBY) k_sweep_f64(Geom<double> g, const double* __restrict__ p,
-                                                         const double* __restrict__ b, double omega,
-                                                         double* __restrict__ out) {
-  const int i = blockIdx.x * kBX + threadIdx.x, j = blockIdx.y * kBY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.nx || j >= g.ny) return;
-  const int nx = g.nx, plane = g.nx * g.ny;
-  const int ip = i == nx - 1 ? 0 : i + 1, im = i == 0 ? nx - 1 : i - 1;
-  const int jp = j == g.ny - 1 ? 0 : j + 1, jm = j == 0 ? g.ny - 1 : j - 1;
-  const int row = k * plane;
-  const int q = row + j * nx + i;
-  const double pc = __ldg(p + q);
-  double nb = g.idx2 * (__ldg(p + row + j * nx + ip) + __ldg(p + row + j * nx + im)) +
-              g.idy2 * (__ldg(p + row + jp * nx + i) + __ldg(p + row + jm * nx + i));
-  if (k < g.nz - 1) nb += __ldg(g.cup + k) * __ldg(p + q + plane);
-  if (k > 0) nb += __ldg(g.cdn + k) * __ldg(p + q - plane);
-  const double pj = (nb - __ldg(b + q)) * __ldg(g.iS + k);
-  out[q] = pc + omega * (pj - pc);
+  const unsigned nx = g.nx, ny = g.ny, nz = g.nz, plane = nx * ny, uw = nx / W;
+  const unsigned f = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned row = f / uw, i = (f - row * uw) * W, k = row / ny, j = row - k * ny;
+  cudaGridDependencySynchronize();
+  if (k >= nz) return;
+  const unsigned q = row * nx + i;
+  const unsigned qn = j + 1 == ny ? q + nx - plane : q + nx, qs = j == 0 ? q + plane - nx : q - nx;
+  const float left = __ldg(p + (i == 0 ? q + nx - 1 : q - 1)), right = __ldg(p + (i + W == nx ? q + W - nx : q + W));
+  const float cup = __ldg(g.cup + k), cdn = __ldg(g.cdn + k), iS = __ldg(g.iS + k);
+  const bool up = k + 1 < nz, dn = k > 0;
+  if constexpr (W == 2) {
+    auto l2 = [](const float* a) { return __ldg(reinterpret_cast<const float2*>(a)); };
+    const float2 c = l2(p + q), n = l2(p + qn), s = l2(p + qs), bb = l2(b + q);
+    const float2 u = up ? l2(p + q + plane) : c, d = dn ? l2(p + q - plane) : c;
+    float2 o;
+    o.x = srj_cell_f32(c.x, left, c.y, n.x, s.x, u.x, d.x, bb.x, g.idx2, g.idy2, cup, cdn, iS, omega);
+    o.y = srj_cell_f32(c.y, c.x, right, n.y, s.y, u.y, d.y, bb.y, g.idx2, g.idy2, cup, cdn, iS, omega);
+    *reinterpret_cast<float2*>(out + q) = o;
+  } else {
+    const float c = __ldg(p + q), u = up ? __ldg(p + q + plane) : c, d = dn ? __ldg(p + q - plane) : c;
+    out[q] = srj_cell_f32(c, left, right, __ldg(p + qn), __ldg(p + qs), u, d, __ldg(b + q), g.idx2, g.idy2, cup, cdn, iS,
+                          omega);
+  }
 }
 
 // Vectorised sweeps: each thread owns 4 consecutive cells of a row (float4
@@ -188,47 +181,6 @@ __global__ void __launch_bounds__(256) k_sweep_f32_pair(Geom<float> g, const flo
     o.w = srj_cell_f32(c.w, c.z, right, yn.w, ys.w, zu.w, zd.w, bq.w, idx2, idy2, cup, cdn, iS, om_b);
     reinterpret_cast<float4*>(out)[((size_t)k * ny + j0 + yt) * nx4 + x4] = o;
   }
-}
-
-template <bool PDL>
-__global__ void __launch_bounds__(kBX* kBY) k_sweep_f64_v2(Geom<double> g, const double* __restrict__ p,
-                                                            const double* __restrict__ b, double omega,
-                                                            double* __restrict__ out) {
-  const int lane = threadIdx.x;
-  const int nx = g.nx, ny = g.ny, nx2 = nx >> 1;
-  const int x2 = blockIdx.x * kBX + lane;
-  const int j = blockIdx.y * kBY + threadIdx.y, k = blockIdx.z;
-  const bool active = x2 < nx2 && j < ny;
-  const int xx = x2 < nx2 ? x2 : nx2 - 1;
-  const int jj = j < ny ? j : ny - 1;
-  const int jp = jj == ny - 1 ? 0 : jj + 1, jm = jj == 0 ? ny - 1 : jj - 1;
-  const size_t plane2 = (size_t)nx2 * ny;
-  const size_t rc = ((size_t)k * ny + jj) * nx2;
-  const double cup = __ldg(g.cup + k), cdn = __ldg(g.cdn + k), iS = __ldg(g.iS + k);
-  const double idx2 = g.idx2, idy2 = g.idy2;
-  const bool has_up = k < g.nz - 1, has_dn = k > 0;
-  if (PDL) cudaGridDependencySynchronize();
-  const double2* P = reinterpret_cast<const double2*>(p);
-  const double2 c = __ldg(P + rc + xx);
-  double left = __shfl_up_sync(0xffffffffu, c.y, 1);
-  double right = __shfl_down_sync(0xffffffffu, c.x, 1);
-  const double* prow = p + rc * 2;
-  if (lane == 0 || xx == 0) left = __ldg(prow + (2 * xx - 1 + nx) % nx);
-  if (lane == kBX - 1 || xx == nx2 - 1) right = __ldg(prow + (2 * xx + 2) % nx);
-  const double2 yn = __ldg(P + ((size_t)k * ny + jp) * nx2 + xx);
-  const double2 ys = __ldg(P + ((size_t)k * ny + jm) * nx2 + xx);
-  const double2 zu = has_up ? __ldg(P + rc + plane2 + xx) : c;
-  const double2 zd = has_dn ? __ldg(P + rc - plane2 + xx) : c;
-  const double2 bq = __ldg(reinterpret_cast<const double2*>(b) + rc + xx);
-  auto cell = [&](double pc, double xl, double xr, double nn, double ss, double uu, double dd, double bb) {
-    const double nbs = idx2 * (xr + xl) + idy2 * (nn + ss) + cup * uu + cdn * dd;
-    const double pj = (nbs - bb) * iS;
-    return pc + omega * (pj - pc);
-  };
-  double2 o;
-  o.x = cell(c.x, left, c.y, yn.x, ys.x, zu.x, zd.x, bq.x);
-  o.y = cell(c.y, c.x, right, yn.y, ys.y, zu.y, zd.y, bq.y);
-  if (active) reinterpret_cast<double2*>(out)[rc + x2] = o;
 }
 
 // ---------------------------------------------------------------------------
@@ -1071,25 +1023,6 @@ __global__ void k_sub_vmean(size_t n, double* __restrict__ a, double inv_lz_plan
 
 }  // namespace
 
-// Vector kernels when the row length allows aligned vectors (nx a multiple
-// of 4 in FP32, of 2 in FP64), launched as programmatic dependents; the
-// one-cell-per-thread kernels otherwise.
-template <typename K, typename T>
-static cudaError_t launch_pdl(K kern, dim3 grid, dim3 block, cudaStream_t s, const Geom<T>& g, const T* p,
-                              const T* b, T omega, T* out) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, g, p, b, omega, out);
-}
-
 // FP32 sweep variant per host thread (poisson_common.cuh numbers them)
 static thread_local int t_sweep_variant = 0;
 void set_sweep_variant(int v) { t_sweep_variant = v; }
@@ -1184,9 +1117,8 @@ static cudaError_t launch_z(const Geom<float>& g, const float* p, const float* b
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <>
-cudaError_t launch_sweep<float>(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
-                                cudaStream_t s) {
+cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
+                             cudaStream_t s) {
   if (g.nx % 4 == 0) {
     const int v = sweep_variant_ok(t_sweep_variant, g.nx, g.ny, g.nz) ? t_sweep_variant : 0;
     switch (v) {
@@ -1201,21 +1133,11 @@ cudaError_t launch_sweep<float>(const Geom<float>& g, const float* p, const floa
       default: return launch_z<1, 8>(g, p, b, omega, out, s);
     }
   }
-  Launch l = plane_launch(g.nx, g.ny, g.nz);
-  k_sweep_f32<<<l.grid, l.block, 0, s>>>(g, p, b, omega, out);
-  return cudaGetLastError();
-}
-template <>
-cudaError_t launch_sweep<double>(const Geom<double>& g, const double* p, const double* b, double omega, double* out,
-                                 cudaStream_t s) {
-  if (g.nx % 2 == 0) {
-    const dim3 grid((g.nx / 2 + kBX - 1) / kBX, (g.ny + kBY - 1) / kBY, g.nz), block(kBX, kBY, 1);
-    cudaError_t e = launch_pdl(k_sweep_f64_v2<true>, grid, block, s, g, p, b, omega, out);
-    return e != cudaSuccess ? e : cudaGetLastError();
-  }
-  Launch l = plane_launch(g.nx, g.ny, g.nz);
-  k_sweep_f64<<<l.grid, l.block, 0, s>>>(g, p, b, omega, out);
-  return cudaGetLastError();
+  const int w = g.nx % 2 == 0 ? 2 : 1;
+  const dim3 grid((unsigned)(((long long)(g.nx / w) * g.ny * g.nz + kBX * kBY - 1) / (kBX * kBY))), block(kBX * kBY);
+  Geom<float> gg = g;
+  void* args[] = {&gg, &p, &b, &omega, &out};
+  return launch_sweep_cfg(w == 2 ? (const void*)k_sweep_f32<2> : (const void*)k_sweep_f32<1>, grid, block, s, args);
 }
 
 // rows per block of the shared-memory line sweep: 4, 2 or 1 (so that the
@@ -1278,6 +1200,9 @@ cudaError_t launch_line_sweep(const Geom<T>& g, const T* p, const T* b, T omega,
       return e != cudaSuccess ? e : cudaGetLastError();
     }
   }
+  if constexpr (sizeof(T) == 8) {
+    if (line_f64_chunks(g.nx, g.ny, g.nz) > 0) return launch_line_f64(g, p, b, omega, out, s);
+  } else
   switch (line_rows(g.nz, sizeof(T))) {
     case 4: return launch_line_rows<T, 4>(g, p, b, omega, out, s, attr);
     case 2: return launch_line_rows<T, 2>(g, p, b, omega, out, s, attr);

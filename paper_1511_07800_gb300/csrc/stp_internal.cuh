@@ -48,13 +48,45 @@ struct Geom {
   const T* tli;    // [nz]    1/m_k (k < t), 1/gamma_t (k = t), 1/m'_k (k > t)
   const T* tlf;    // [nz]    elimination: cdn_k/m_k (k < t), cdn_t/gamma_t, cup_k/m'_k (k > t)
   const T* tlb;    // [nz]    substitution: cup_k/m_k (k < t), cup_t/gamma_t, cdn_k/m'_k (k > t)
+  // FP64 z-line chunks (line_chunk_start): products of the elimination's
+  // (pf) and the substitution's (pe) coefficients from the level where the
+  // recurrence enters the chunk through level k (the twist level left out)
+  const T* pf;     // [nz]
+  const T* pe;     // [nz]
   // FP32 only (null in FP64): {cup_k, cdn_k, tli_k, tlf_k} packed per level,
   // one 16-byte load for the z-line sweep's level coefficients
   const float4* lz4;
 };
 
 // Number of metric arrays packed into one device allocation per precision.
-constexpr int kMetricArrays = 16;
+constexpr int kMetricArrays = 20;  // a multiple of 4: lz4 after them stays 16-byte aligned
+
+// Level chunks of a z column: nch/2 cut [0, t), nch/2 cut [t, nz), t = nz/2, the
+// first of those never empty; start of chunk c (c = nch: nz).
+__host__ __device__ constexpr int line_chunk_start(int c, int nch, int nz) {
+  const int t = nz >> 1, h = nch / 2;
+  return c < h ? c * t / h : c >= nch ? nz : t + ((c - h) * (nz - t) + h - 1) / h;
+}
+// most levels a chunk holds
+constexpr int line_f64_levels(int nz, int nch) {
+  int m = 0;
+  for (int c = 0; c < nch; c++) {
+    const int l = line_chunk_start(c + 1, nch, nz) - line_chunk_start(c, nch, nz);
+    m = l > m ? l : m;
+  }
+  return m;
+}
+// chunks of the FP64 z-line kernel: the fewest (4, 8, 16, 32) of at most 12
+// levels, then more while the channel has under two warps a scheduler and a
+// chunk over two levels (0: the column is too tall)
+constexpr int line_f64_chunks(int nx, int ny, int nz) {
+  int nch = 4;
+  while (nch <= 32 && line_f64_levels(nz, nch) > 12) nch *= 2;
+  if (nch > 32) return 0;
+  const long long rows = (long long)((nx + 31) / 32) * ny;
+  while (nch < 32 && rows * nch < 2 * 4 * 152 && line_f64_levels(nz, nch) > 2) nch *= 2;
+  return nch;
+}
 
 // Reduction workspace (device).  Every reducing kernel writes one partial per
 // block, then the last block to finish sums the partials in block order, so
@@ -191,20 +223,24 @@ cudaError_t launch_line_sweep(const Geom<T>& g, const T* p, const T* b, T omega,
 bool line_chunk_ok(int nx, int nz);
 
 // One Jacobi-SOR sweep of L p = b with factor omega: out = p - omega (b - Lp)/S.
-template <typename T>
-cudaError_t launch_sweep(const Geom<T>& g, const T* p, const T* b, T omega, T* out, cudaStream_t s);
-template <>
-cudaError_t launch_sweep<float>(const Geom<float>&, const float*, const float*, float, float*, cudaStream_t);
-template <>
-cudaError_t launch_sweep<double>(const Geom<double>&, const double*, const double*, double, double*, cudaStream_t);
+cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
+                             cudaStream_t s);
 
-// FP32 sweep variant used by launch_sweep<float> on this host thread
+// FP64 sweeps (kernels_f64.cu).  tab: the level coefficients of this sweep's
+// factor (5 nz doubles of launch_sweep_table's M), null: formed in the kernel.
+cudaError_t launch_sweep_table(const Geom<double>& g, const double* omega, int M, double* tab, cudaStream_t s);
+cudaError_t launch_sweep_f64(const Geom<double>& g, const double* p, const double* b, double omega, const double* tab,
+                             double* out, cudaStream_t s);
+cudaError_t launch_line_f64(const Geom<double>& g, const double* p, const double* b, double omega, double* out,
+                            cudaStream_t s);
+
+// FP32 sweep variant used by launch_sweep_f32 on this host thread
 // (chosen by the autotuner in api.cu).
 void set_sweep_variant(int v);
 int sweep_variant_count();
 bool sweep_variant_ok(int v, int nx, int ny, int nz);
 // variants 9..11 run two sweeps per launch (launch_sweep_pair, cycles of a
-// multiple of 4 sweeps only); launch_sweep falls back to variant 0 for them
+// multiple of 4 sweeps only); launch_sweep_f32 falls back to variant 0 for them
 bool sweep_variant_is_pair(int v);
 cudaError_t launch_sweep_pair(const Geom<float>& g, const float* p, const float* b, float om_a, float om_b,
                               float* out, cudaStream_t s);
@@ -241,6 +277,14 @@ cudaError_t launch_difference(const double* a, const double* b, float* out, size
 // start of a solve: fold the previous solve into the totals, reset the state
 // (in a graph it also arms the WHILE handle h_loop of an FP64 solve)
 cudaError_t launch_begin(SolveCtl* ctl, int graph, cudaGraphConditionalHandle h_loop, cudaStream_t s);
+
+// Whole FP32 SRJ cycles on one thread-block cluster (kernels_cluster.cu), for
+// channels that fit its shared memory: sweep variants kClusterVariant0 + v.
+constexpr int kClusterVariant0 = 12;
+int cluster_variants();
+bool cluster_ok(int v, int nx, int ny, int nz);
+cudaError_t launch_cluster_cycle(const Geom<float>& g, float* d, const float* r, const float* omega, int M, int v,
+                                 cudaStream_t s);
 
 // Two-colour FP32 sweeps (kernels_colour.cu): inner solves on the library's own
 // schedule with nx, ny even.  d and r hold the two colours one after the
