@@ -42,8 +42,6 @@ __device__ __forceinline__ void mma16816(float* c, const unsigned* a, const unsi
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__device__ __forceinline__ unsigned ld_u32(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
-
 __device__ __forceinline__ unsigned pack2(bf16 lo, bf16 hi) {
   return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
 }
@@ -81,92 +79,145 @@ __device__ __forceinline__ long long tap_from(const Dims& dm, const Coord& c, in
 }
 
 // ---------------------------------------------------------------------------
-// 3x3x3 convolution as an implicit GEMM on the tensor cores:
+// 3x3x3 convolution as an implicit GEMM on the tensor cores (mma.sync):
 //   y[v][o] = b[o] + sum_{t, c} wt[t][o][c] x[v + off(t)][c]
-// M = voxels, N = output channels, K = 27 taps x input channels.  A warp
-// computes 32 voxels x 8*NT channels; a block has 4 warps (128 voxels).
+// M = voxels, N = output channels, K = 27 taps x input channels, for the levels
+// k_conv3_tc does not take.  A block computes 8 x 4 x 2 voxels (a warp two x
+// rows of them) x 8 NT channels.  These levels are small, so what they cost
+// is latency: the block stages its halo and all 27 taps' weights of its
+// channels in shared memory up front (three cp.async groups, the later taps'
+// weights landing while the first are multiplied), and a K step is then two
+// ldmatrix and NT multiplies.  Each output sees the same sequence of MMAs (taps,
+// then channels) at every NT.  Loading operands step by step from global
+// memory instead took 85 us for 128 -> 128 at 16 x 8 x 16 voxels; the figures
+// now stand at conv3.
 // Options: ReLU; multiply by (mask > 0) (the derivative of the ReLU that
 // produced this layer's input, used when the kernel runs the backward data
 // pass with transposed weights); no bias when bias is NULL.
 // ---------------------------------------------------------------------------
+constexpr int CS_TX = 8, CS_TY = 4, CS_TZ = 2, CS_HX = CS_TX + 2, CS_HY = CS_TY + 2, CS_HZ = CS_TZ + 2;
+constexpr int CS_HVOX = CS_HX * CS_HY * CS_HZ;
+
+__device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool fill) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(fill ? 16 : 0)
+               : "memory");
+}
+// a coordinate at most one tile outside [0, n), wrapped
+__device__ __forceinline__ int wrap1(int a, int n) { return a < 0 ? a + n : a >= n ? (a - n) % n : a; }
+
+// shared memory: the halo, then 27 taps' weights, both in chunks of 8 input
+// channels (16 bytes a voxel or output channel)
+constexpr size_t conv3_smem(int cin, int nt) { return (size_t)(cin / 8) * 16 * (CS_HVOX + 27 * 8 * nt); }
+
 template <int NT>
 __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__ x, int ldx, int cin,
                                                const bf16* __restrict__ wt, const float* __restrict__ bias, int cout,
                                                bf16* __restrict__ y, int ldy, int relu, const bf16* __restrict__ mask,
                                                int ldm) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-  const long long V = dm.vox();
-  const long long vb = ((long long)blockIdx.x * 4 + warp) * 32;
+  extern __shared__ __align__(128) uint8_t csm[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
+  const int nch = cin / 8;
+  const uint32_t sx = su32(csm), sw = sx + 16 * CS_HVOX * nch;
+  const int tx = (dm.w + CS_TX - 1) / CS_TX, ty = (dm.h + CS_TY - 1) / CS_TY, tz = (dm.d + CS_TZ - 1) / CS_TZ;
+  int r = blockIdx.x;
+  const int x0 = (r % tx) * CS_TX;
+  r /= tx;
+  const int y0 = (r % ty) * CS_TY;
+  r /= ty;
+  const int z0 = (r % tz) * CS_TZ, nn = r / tz;
   const int cob = blockIdx.y * NT * 8;
-  float acc[2][NT][4];
-#pragma unroll
-  for (int m = 0; m < 2; m++)
-#pragma unroll
-    for (int n = 0; n < NT; n++) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
-  long long vrow[4];
-  Coord crow[4];
-#pragma unroll
-  for (int r = 0; r < 4; r++) {
-    vrow[r] = vb + (r >> 1) * 16 + g + (r & 1) * 8;
-    crow[r] = coord_of(dm, (unsigned)(vrow[r] < V ? vrow[r] : 0));
+  for (int i = tid; i < CS_HVOX; i += 128) {
+    const int hx = i % CS_HX, hy = (i / CS_HX) % CS_HY, hz = i / (CS_HX * CS_HY);
+    const int vz = z0 - 1 + hz;
+    const bool in = vz >= 0 && vz < dm.d;
+    const bf16* src = x + voxel_at(dm, nn, in ? vz : 0, wrap1(y0 - 1 + hy, dm.h), wrap1(x0 - 1 + hx, dm.w)) * ldx;
+    for (int c = 0; c < nch; c++) cp16(sx + 16 * (c * CS_HVOX + i), src + 8 * c, in);
   }
-  const int kc = cin >> 4;
+  for (int part = 0; part < 3; part++) {
+    for (int i = tid; i < 9 * 8 * NT * nch; i += 128) {
+      const int c = i % nch, o = (i / nch) % (8 * NT), t = part * 9 + i / (nch * 8 * NT);
+      cp16(sw + 16 * ((t * nch + c) * 8 * NT + o), wt + ((long long)t * cout + cob + o) * cin + 8 * c, true);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float acc[NT][4];
+#pragma unroll
+  for (int n = 0; n < NT; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+  // the warp's voxel rows: y = y0 + 2 (warp & 1) + {0, 1}, z = z0 + warp / 2
+  const int wy = 2 * (warp & 1), wz = warp >> 1;
+  // A matrices: (rows 0-7, 8-15) x (channels 0-7, 8-15); B: (outputs 0-7 of
+  // an 8-channel tile pair) x (channels 0-7, 8-15)
+  const int mi = lane >> 3, mr = lane & 7;
+  const uint32_t a_lane = sx + 16 * ((mi >> 1) * CS_HVOX + (wz * CS_HY + wy + (mi & 1)) * CS_HX + mr);
+  const uint32_t b_lane = sw + 16 * ((mi & 1) * 8 * NT + (mi >> 1) * 8 + mr);
   for (int t = 0; t < 27; t++) {
-    long long src[4];
+    if (t % 9 == 0) {
+      if (t == 0)
+        asm volatile("cp.async.wait_group 2;" ::: "memory");
+      else if (t == 9)
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+    }
+    const uint32_t at = a_lane + 16 * ((t / 9 * CS_HY + t / 3 % 3) * CS_HX + t % 3);
+    const uint32_t bt = b_lane + 16 * t * nch * 8 * NT;
+#pragma unroll 2
+    for (int c = 0; c < nch; c += 2) {
+      unsigned a[4];
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                   : "r"(at + 16 * c * CS_HVOX)
+                   : "memory");
+      const uint32_t bc = bt + 16 * c * 8 * NT;
+      if constexpr (NT == 1) {
+        unsigned b[2];
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+                     : "=r"(b[0]), "=r"(b[1])
+                     : "r"(bc)
+                     : "memory");
+        mma16816(acc[0], a, b);
+      } else {
 #pragma unroll
-    for (int r = 0; r < 4; r++) src[r] = vrow[r] < V ? tap_from(dm, crow[r], t) : -1;
-    for (int c = 0; c < kc; c++) {
-      unsigned a[2][4];
-#pragma unroll
-      for (int m = 0; m < 2; m++) {
-        const long long s0 = src[2 * m], s1 = src[2 * m + 1];
-        const int col = c * 16 + 2 * q;
-        a[m][0] = s0 >= 0 ? ld_u32(x + s0 * ldx + col) : 0u;
-        a[m][1] = s1 >= 0 ? ld_u32(x + s1 * ldx + col) : 0u;
-        a[m][2] = s0 >= 0 ? ld_u32(x + s0 * ldx + col + 8) : 0u;
-        a[m][3] = s1 >= 0 ? ld_u32(x + s1 * ldx + col + 8) : 0u;
-      }
-#pragma unroll
-      for (int n = 0; n < NT; n++) {
-        const int co = cob + n * 8 + g;
-        unsigned b[2] = {0u, 0u};
-        if (co < cout) {
-          const bf16* wp = wt + ((long long)t * cout + co) * cin + c * 16 + 2 * q;
-          b[0] = ld_u32(wp);
-          b[1] = ld_u32(wp + 8);
+        for (int n = 0; n < NT; n += 2) {
+          unsigned b[4];
+          asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                       : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                       : "r"(bc + 16 * 8 * n)
+                       : "memory");
+          mma16816(acc[n], a, b);
+          mma16816(acc[n + 1], a, b + 2);
         }
-        mma16816(acc[0][n], a[0], b);
-        mma16816(acc[1][n], a[1], b);
       }
     }
   }
+  const int vx = x0 + g, vz = z0 + wz;
 #pragma unroll
-  for (int m = 0; m < 2; m++)
+  for (int n = 0; n < NT; n++) {
+    const int co = cob + n * 8 + 2 * q;
 #pragma unroll
-    for (int n = 0; n < NT; n++) {
-      const int co = cob + n * 8 + 2 * q;
-      if (co >= cout) continue;
-#pragma unroll
-      for (int h = 0; h < 2; h++) {
-        const long long v = vrow[2 * m + h];
-        if (v >= V) continue;
-        float v0 = acc[m][n][2 * h], v1 = acc[m][n][2 * h + 1];
-        if (bias) {
-          v0 += bias[co];
-          v1 += bias[co + 1];
-        }
-        if (relu) {
-          v0 = fmaxf(v0, 0.f);
-          v1 = fmaxf(v1, 0.f);
-        }
-        if (mask) {
-          const bf16* mp = mask + v * ldm + co;
-          if (!(__bfloat162float(mp[0]) > 0.f)) v0 = 0.f;
-          if (!(__bfloat162float(mp[1]) > 0.f)) v1 = 0.f;
-        }
-        *reinterpret_cast<unsigned*>(y + v * ldy + co) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+    for (int h = 0; h < 2; h++) {
+      const int vy = y0 + wy + h;
+      if (vx >= dm.w || vy >= dm.h || vz >= dm.d) continue;
+      const long long v = voxel_at(dm, nn, vz, vy, vx);
+      float v0 = acc[n][2 * h], v1 = acc[n][2 * h + 1];
+      if (bias) {
+        v0 += bias[co];
+        v1 += bias[co + 1];
       }
+      if (relu) {
+        v0 = fmaxf(v0, 0.f);
+        v1 = fmaxf(v1, 0.f);
+      }
+      if (mask) {
+        const bf16* mp = mask + v * ldm + co;
+        if (!(__bfloat162float(mp[0]) > 0.f)) v0 = 0.f;
+        if (!(__bfloat162float(mp[1]) > 0.f)) v1 = 0.f;
+      }
+      *reinterpret_cast<unsigned*>(y + v * ldy + co) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
     }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -200,13 +251,6 @@ constexpr int TC_TX = 8, TC_TY = 16, TC_HX = 10, TC_HY = 18;
 constexpr int TC_PLANE = TC_HX * TC_HY * 16;  // bytes of one halo plane of one 8-channel chunk
 constexpr int TC_CG = 64;                     // channels per halo group
 constexpr int TC_STAGES = 3;
-
-__device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool fill) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(fill ? 16 : 0)
-               : "memory");
-}
 
 // shared-memory matrix descriptor: no swizzle, K-major core matrices
 __device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
@@ -566,111 +610,259 @@ __global__ void k_conv_out_bwd(long long V, const float* __restrict__ gy, const 
 
 // ---------------------------------------------------------------------------
 // Weight gradient of a 3x3x3 layer on the tensor cores:
-//   gw[o][c][t] += sum_v gz[v][o] x[v + off(t)][c],   gb[o] += sum_v gz[v][o]
-// GEMM with M = output channels (16 per warp), N = input channels (32 per
-// warp, 4 n-tiles), K = voxels.  Block = 4 warps over consecutive voxel
-// chunks of one (tap, o-tile, c-tile); partial sums are reduced in shared
-// memory and added to the FP32 gradient with atomics.
+//   gw[o][c][t] = sum_v gz[v][o] x[v + off(t)][c],   gb[o] = sum_v gz[v][o]
+// GEMMs with M = output channels, N = input channels, K = voxels, one a tap.
+// A block takes OT output and CT input channels and all 27 taps over a range
+// of spatial tiles of 8 x 8 x 4 voxels: it stages the tile of gz and the tile
+// of x with its halo in shared memory once, and the 27 taps read the same
+// halo, a tap's operand being the halo rows moved by its offset (ldmatrix
+// takes a row address a lane, so no data moves).  Both operands are stored
+// voxel by voxel and needed along the voxels: ldmatrix.trans.  Warp w of nine
+// keeps the accumulators of the three x taps of row offset (kz, ky) = (w/3,
+// w%3) in registers over all its tiles.  Partial sums go to scratch in one
+// slice a block range and are added in a fixed order by k_wgrad_sum (no
+// atomics: results repeat bitwise); the bias gradient is the product with a
+// column of ones, taken by the centre warp of the first input tile.
+// Shared memory holds 8-channel chunks, 16 bytes a voxel: eight consecutive x
+// are one conflict-free ldmatrix row set.
+// A tap at a time from global memory (the kernel this replaces) read both
+// operands 27 times in 2-byte loads: 3.8 ms of a 6.2 ms gradient of 4 x 64 x
+// 32 x 64; the figures now stand at wgrad3.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_wgrad3(Dims dm, const bf16* __restrict__ x, int ldx, int cin,
+constexpr int WG_TX = 8, WG_TY = 8, WG_TZ = 4, WG_VOX = WG_TX * WG_TY * WG_TZ;
+constexpr int WG_HX = WG_TX + 2, WG_HY = WG_TY + 2, WG_HZ = WG_TZ + 2, WG_HVOX = WG_HX * WG_HY * WG_HZ;
+constexpr int WG_SLOTS = 28;  // taps, then the bias
+
+// smem of a block: gz tile and x halo, in chunks
+constexpr int wg_smem(int OT, int CT) { return 16 * (WG_VOX * OT / 8 + WG_HVOX * CT / 8); }
+
+__device__ __forceinline__ void ldsm4t(unsigned* r, uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+
+struct WgTiles {
+  int nx, ny, nz;  // tiles along x, y, z (z within a sample)
+  __host__ __device__ int count(int n) const { return nx * ny * nz * n; }
+};
+__host__ __device__ inline WgTiles wg_tiles(const Dims& dm) {
+  return WgTiles{(dm.w + WG_TX - 1) / WG_TX, (dm.h + WG_TY - 1) / WG_TY, (dm.d + WG_TZ - 1) / WG_TZ};
+}
+template <int OT, int CT>
+__global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict__ x, int ldx, int cin,
                                                 const bf16* __restrict__ gz, int ldg, int cout,
-                                                float* __restrict__ gw, float* __restrict__ gb, long long vchunk) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-  const int ct = (cin + 31) / 32;
-  int idx = blockIdx.x;
-  const int t = idx % 27;
-  idx /= 27;
-  const int cti = idx % ct;
-  const int oti = idx / ct;
-  const int ob = oti * 16, cb = cti * 32;
-  const long long V = dm.vox();
-  const long long v0 = (long long)blockIdx.y * vchunk;
-  const long long v1 = V < v0 + vchunk ? V : v0 + vchunk;
-  float acc[4][4];
+                                                float* __restrict__ part) {
+  extern __shared__ __align__(128) uint8_t wsm[];
+  const uint32_t sg = (uint32_t)__cvta_generic_to_shared(wsm), sx = sg + 16 * WG_VOX * (OT / 8);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
+  const int cts = cin / CT;
+  const int ob = (int)(blockIdx.x / cts) * OT, cb = (int)(blockIdx.x % cts) * CT;
+  const WgTiles tl = wg_tiles(dm);
+  const int ntiles = tl.count(dm.n);
+  const int t0 = (int)((long long)blockIdx.y * ntiles / gridDim.y), t1 = (int)((long long)(blockIdx.y + 1) * ntiles / gridDim.y);
+  const bool bias = warp == 4 && cb == 0;
+  float acc[3][OT / 16][CT / 8][4], accb[OT / 16][4];
 #pragma unroll
-  for (int n = 0; n < 4; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
-  const bf16 zero = __float2bfloat16(0.f);
-  for (long long vs = v0 + warp * 16; vs < v1; vs += 64) {
-    // the four voxels of this thread in the chunk: k = 2q, 2q+1, 2q+8, 2q+9
-    long long vk[4] = {vs + 2 * q, vs + 2 * q + 1, vs + 2 * q + 8, vs + 2 * q + 9};
-    long long sk[4];
-    bf16 gzv[2][4];
+  for (int m = 0; m < OT / 16; m++) {
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-      const bool ok = vk[i] < v1;
-      sk[i] = ok ? tap_from(dm, coord_of(dm, (unsigned)vk[i]), t) : -1;
-      gzv[0][i] = ok ? gz[vk[i] * ldg + ob + g] : zero;
-      gzv[1][i] = ok ? gz[vk[i] * ldg + ob + g + 8] : zero;
+    for (int i = 0; i < 4; i++) accb[m][i] = 0.f;
+#pragma unroll
+    for (int t = 0; t < 3; t++)
+#pragma unroll
+      for (int n = 0; n < CT / 8; n++) acc[t][m][n][0] = acc[t][m][n][1] = acc[t][m][n][2] = acc[t][m][n][3] = 0.f;
+  }
+  const unsigned ones[2] = {0x3F803F80u, 0x3F803F80u};  // BF16 1, 1
+  // ldmatrix rows: lanes 8 i .. 8 i + 7 address matrix i.  A (gz): matrices
+  // (voxels 0-7, 8-15) x (channels 0-7, 8-15) in the order a0 (v0, o0), a1 (v0,
+  // o1), a2 (v1, o0), a3 (v1, o1); B (x): b0, b1 of channels 0-7, then of 8-15.
+  const int mi = lane >> 3, mr = lane & 7;
+  const uint32_t a_lane = sg + 16 * ((mi & 1) * WG_VOX + (mi >> 1) * 8 + mr);
+  const uint32_t b_lane = sx + 16 * ((mi >> 1) * WG_HVOX + (mi & 1) * WG_HX + mr);
+  const int kz = warp / 3, ky = warp % 3;
+  for (int tile = t0; tile < t1; tile++) {
+    int r = tile;
+    const int x0 = (r % tl.nx) * WG_TX;
+    r /= tl.nx;
+    const int y0 = (r % tl.ny) * WG_TY;
+    r /= tl.ny;
+    const int z0 = (r % tl.nz) * WG_TZ, nn = r / tl.nz;
+    __syncthreads();  // the previous tile has been read
+    for (int i = tid; i < WG_VOX * (OT / 8); i += 288) {
+      const int v = i % WG_VOX, ch = i / WG_VOX;
+      const int vx = x0 + v % WG_TX, vy = y0 + (v / WG_TX) % WG_TY, vz = z0 + v / (WG_TX * WG_TY);
+      const bool in = vx < dm.w && vy < dm.h && vz < dm.d;
+      const long long w = in ? voxel_at(dm, nn, vz, vy, vx) : 0;
+      cp16(sg + 16 * i, gz + w * ldg + ob + 8 * ch, in);
     }
-    unsigned a[4];
-    a[0] = pack2(gzv[0][0], gzv[0][1]);
-    a[1] = pack2(gzv[1][0], gzv[1][1]);
-    a[2] = pack2(gzv[0][2], gzv[0][3]);
-    a[3] = pack2(gzv[1][2], gzv[1][3]);
+    for (int i = tid; i < WG_HVOX * (CT / 8); i += 288) {
+      const int v = i % WG_HVOX, ch = i / WG_HVOX;
+      const int hx = v % WG_HX, hy = (v / WG_HX) % WG_HY, hz = v / (WG_HX * WG_HY);
+      const int vx = wrap1(x0 - 1 + hx, dm.w), vy = wrap1(y0 - 1 + hy, dm.h), vz = z0 - 1 + hz;
+      const bool in = vz >= 0 && vz < dm.d;
+      const long long w = voxel_at(dm, nn, in ? vz : 0, vy, vx);
+      cp16(sx + 16 * i, x + w * ldx + cb + 8 * ch, in);
+    }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    // K steps of 16 voxels: two x rows of the tile
+#pragma unroll 2
+    for (int s = 0; s < WG_VOX / 16; s++) {
+      const int vy = (2 * s) % WG_TY, vz = (2 * s) / WG_TY;
+      unsigned a[OT / 16][4];
 #pragma unroll
-    for (int n = 0; n < 4; n++) {
-      const int c = cb + n * 8 + g;
-      bf16 xv[4];
+      for (int m = 0; m < OT / 16; m++) ldsm4t(a[m], a_lane + 16 * (2 * m * WG_VOX + 16 * s));
+      const uint32_t br = b_lane + 16 * (((vz + kz) * WG_HY + vy + ky) * WG_HX);
 #pragma unroll
-      for (int i = 0; i < 4; i++) xv[i] = (c < cin && sk[i] >= 0) ? x[sk[i] * ldx + c] : zero;
-      unsigned b[2] = {pack2(xv[0], xv[1]), pack2(xv[2], xv[3])};
-      mma16816(acc[n], a, b);
+      for (int t = 0; t < 3; t++)
+#pragma unroll
+        for (int n = 0; n < CT / 16; n++) {
+          unsigned b[4];
+          ldsm4t(b, br + 16 * (t + 2 * n * WG_HVOX));
+#pragma unroll
+          for (int m = 0; m < OT / 16; m++) {
+            mma16816(acc[t][m][2 * n], a[m], b);
+            mma16816(acc[t][m][2 * n + 1], a[m], b + 2);
+          }
+        }
+      if (bias)
+#pragma unroll
+        for (int m = 0; m < OT / 16; m++) mma16816(accb[m], a[m], ones);
     }
   }
-  __shared__ float red[4][16][33];
+  // slice blockIdx.y of the scratch: [slot][cout][cin]
+  float* out = part + (size_t)blockIdx.y * WG_SLOTS * cout * cin;
+#pragma unroll
+  for (int t = 0; t < 3; t++)
+#pragma unroll
+    for (int m = 0; m < OT / 16; m++)
+#pragma unroll
+      for (int n = 0; n < CT / 8; n++) {
+        float* o = out + ((size_t)(warp * 3 + t) * cout + ob + 16 * m + g) * cin + cb + 8 * n + 2 * q;
+        *reinterpret_cast<float2*>(o) = make_float2(acc[t][m][n][0], acc[t][m][n][1]);
+        *reinterpret_cast<float2*>(o + 8 * cin) = make_float2(acc[t][m][n][2], acc[t][m][n][3]);
+      }
+  if (bias && q == 0)
+#pragma unroll
+    for (int m = 0; m < OT / 16; m++) {
+      out[((size_t)27 * cout + ob + 16 * m + g) * cin] = accb[m][0];
+      out[((size_t)27 * cout + ob + 16 * m + g + 8) * cin] = accb[m][2];
+    }
+}
+
+// gw[o][c][t], gb[o] = sum over the slices in order
+__global__ void k_wgrad_sum(const float* __restrict__ part, int slices, int cin, int cout, float* __restrict__ gw,
+                            float* __restrict__ gb) {
+  const int n = 27 * cout * cin, e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n + cout) return;
+  const size_t off = e < n ? e : (size_t)27 * cout * cin + (size_t)(e - n) * cin;
+  const size_t stride = (size_t)WG_SLOTS * cout * cin;
+  float s = 0.f;
+#pragma unroll 8
+  for (int i = 0; i < slices; i++) s += part[off + i * stride];
+  if (e < n) {
+    const int oc = e % (cout * cin), t = e / (cout * cin);
+    gw[(size_t)oc * 27 + t] = s;
+  } else {
+    gb[e - n] = s;
+  }
+}
+
+// The same for the input layer (one input channel): M = 16 output channels,
+// N = 32 columns, the 27 taps' shifted inputs and, as column 27, ones (the
+// bias), K = voxels.  The block's eight warps share a tile's K steps; slices
+// [32][16] in scratch, one a block.
+__global__ void __launch_bounds__(256) k_wgrad_in(Dims dm, const float* __restrict__ x, const bf16* __restrict__ gz,
+                                                  int ldg, float* __restrict__ part) {
+  __shared__ __align__(128) uint4 sgz[2 * WG_VOX];
+  __shared__ unsigned short sxv[WG_HVOX];
+  __shared__ float red[8][16][33];
+  const uint32_t sg = (uint32_t)__cvta_generic_to_shared(sgz);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
+  const WgTiles tl = wg_tiles(dm);
+  const int ntiles = tl.count(dm.n);
+  const int t0 = (int)((long long)blockIdx.x * ntiles / gridDim.x), t1 = (int)((long long)(blockIdx.x + 1) * ntiles / gridDim.x);
+  const int mi = lane >> 3, mr = lane & 7;
+  const uint32_t a_lane = sg + 16 * ((mi & 1) * WG_VOX + (mi >> 1) * 8 + mr);
+  float acc[4][4];
+  int toff[4];  // halo offset of column 8 n + g
 #pragma unroll
   for (int n = 0; n < 4; n++) {
-    red[warp][g][n * 8 + 2 * q] = acc[n][0];
-    red[warp][g][n * 8 + 2 * q + 1] = acc[n][1];
-    red[warp][g + 8][n * 8 + 2 * q] = acc[n][2];
-    red[warp][g + 8][n * 8 + 2 * q + 1] = acc[n][3];
+    acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+    const int t = 8 * n + g;
+    toff[n] = t < 27 ? (t / 9 * WG_HY + t / 3 % 3) * WG_HX + t % 3 : 0;
+  }
+  for (int tile = t0; tile < t1; tile++) {
+    int r = tile;
+    const int x0 = (r % tl.nx) * WG_TX;
+    r /= tl.nx;
+    const int y0 = (r % tl.ny) * WG_TY;
+    r /= tl.ny;
+    const int z0 = (r % tl.nz) * WG_TZ, nn = r / tl.nz;
+    __syncthreads();
+    for (int i = tid; i < 2 * WG_VOX; i += 256) {
+      const int v = i % WG_VOX, ch = i / WG_VOX;
+      const int vx = x0 + v % WG_TX, vy = y0 + (v / WG_TX) % WG_TY, vz = z0 + v / (WG_TX * WG_TY);
+      const bool in = vx < dm.w && vy < dm.h && vz < dm.d;
+      const long long w = in ? voxel_at(dm, nn, vz, vy, vx) : 0;
+      cp16(sg + 16 * i, gz + w * ldg + 8 * ch, in);
+    }
+    for (int v = tid; v < WG_HVOX; v += 256) {
+      const int hx = v % WG_HX, hy = (v / WG_HX) % WG_HY, hz = v / (WG_HX * WG_HY);
+      const int vx = wrap1(x0 - 1 + hx, dm.w), vy = wrap1(y0 - 1 + hy, dm.h), vz = z0 - 1 + hz;
+      const bool in = vz >= 0 && vz < dm.d;
+      sxv[v] = in ? __bfloat16_as_ushort(__float2bfloat16(x[voxel_at(dm, nn, vz, vy, vx)])) : (unsigned short)0;
+    }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < WG_VOX / 16 / 8; e++) {
+      const int s = warp + 8 * e;
+      const int vy = (2 * s) % WG_TY, vz = (2 * s) / WG_TY;
+      unsigned a[4];
+      ldsm4t(a, a_lane + 16 * 16 * s);
+      const int base = (vz * WG_HY + vy) * WG_HX + 2 * q;
+#pragma unroll
+      for (int n = 0; n < 4; n++) {
+        unsigned b[2];
+        if (n < 3 || g < 3) {
+          const unsigned short* c = sxv + base + toff[n];
+          b[0] = c[0] | ((unsigned)c[1] << 16);
+          b[1] = c[WG_HX] | ((unsigned)c[WG_HX + 1] << 16);
+        } else {
+          b[0] = b[1] = g == 3 ? 0x3F803F80u : 0u;
+        }
+        mma16816(acc[n], a, b);
+      }
+    }
+  }
+#pragma unroll
+  for (int n = 0; n < 4; n++) {
+    red[warp][g][8 * n + 2 * q] = acc[n][0];
+    red[warp][g][8 * n + 2 * q + 1] = acc[n][1];
+    red[warp][g + 8][8 * n + 2 * q] = acc[n][2];
+    red[warp][g + 8][8 * n + 2 * q + 1] = acc[n][3];
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < 16 * 32; e += 128) {
-    const int o = e / 32, c = e % 32;
-    if (cb + c >= cin) continue;
-    const float s = red[0][o][c] + red[1][o][c] + red[2][o][c] + red[3][o][c];
-    atomicAdd(gw + ((long long)(ob + o) * cin + cb + c) * 27 + t, s);
+  for (int e = tid; e < 16 * 32; e += 256) {
+    const int o = e / 32, t = e % 32;
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; w++) s += red[w][o][t];
+    part[(size_t)blockIdx.x * 512 + t * 16 + o] = s;
   }
-  (void)gb;
 }
-
-// bias gradient: gb[o] += sum_v gz[v][o]
-__global__ void k_bias_grad(long long V, const bf16* __restrict__ gz, int ldg, int cout, float* __restrict__ gb) {
-  const int o = blockIdx.y * blockDim.x + threadIdx.x;
-  if (o >= cout) return;
+__global__ void k_wgrad_in_sum(const float* __restrict__ part, int slices, float* __restrict__ gw,
+                               float* __restrict__ gb) {
+  // a warp an output (28 x 16 of them): lanes stride the slices
+  const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (e >= 28 * 16) return;
+  const int t = e / 16, o = e % 16;
   float s = 0.f;
-  for (long long v = blockIdx.x; v < V; v += gridDim.x) s += __bfloat162float(gz[v * ldg + o]);
-  atomicAdd(gb + o, s);
-}
-
-// first-layer weight gradient: gw[o][0][t] += sum_v gz[v][o] x[v + off(t)];
-// one tap per blockIdx.y
-__global__ void k_wgrad_in(Dims dm, const float* __restrict__ x, const bf16* __restrict__ gz, int ldg,
-                           float* __restrict__ gw) {
-  __shared__ float red[16];
-  if (threadIdx.x < 16) red[threadIdx.x] = 0.f;
-  __syncthreads();
-  const int t = blockIdx.y;
-  float acc[16];
-#pragma unroll
-  for (int o = 0; o < 16; o++) acc[o] = 0.f;
-  const long long V = dm.vox();
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
-    const long long s = tap_from(dm, coord_of(dm, (unsigned)v), t);
-    if (s < 0) continue;
-    const float xv = __bfloat162float(__float2bfloat16(x[s]));
-#pragma unroll
-    for (int o = 0; o < 16; o++) acc[o] = fmaf(__bfloat162float(gz[v * ldg + o]), xv, acc[o]);
-  }
-#pragma unroll
-  for (int o = 0; o < 16; o++) {
-    float s = acc[o];
-    for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&red[o], s);
-  }
-  __syncthreads();
-  if (threadIdx.x < 16) atomicAdd(gw + threadIdx.x * 27 + t, red[threadIdx.x]);
+  for (int i = lane; i < slices; i += 32) s += part[(size_t)i * 512 + t * 16 + o];
+  for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
+  if (lane == 0) (t < 27 ? gw[o * 27 + t] : gb[o]) = s;
 }
 
 // ---------------------------------------------------------------------------
@@ -944,6 +1136,7 @@ struct stp_unet {
   // gradients of activations
   bf16 *ga[4] = {}, *gb[4] = {}, *gu[3] = {};
   float *y = nullptr, *gy = nullptr, *loss = nullptr, *h_loss = nullptr;
+  float* wpart = nullptr;                                  // slices of the weight gradients (kWgradScratch)
   float *xin = nullptr, *tin = nullptr, *snorm = nullptr;  // normalised pairs, per-sample norms
   int guess_kernels = 0;                                   // kernels launched by one guess
   float out_scale = 1.f;                                   // the network predicts out_scale * dp / s
@@ -1040,56 +1233,69 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
     UTRY(n, cudaGetLastError());
     return STP_OK;
   }
-  // output channels a block: 64, 32, 16 or 8, the widest that still gives two
-  // blocks an SM (small levels have few 128-voxel rows); each output sees the
-  // same sequence of MMAs whichever width computes it (STP_UNET_MMA_NT =
-  // 8, 4, 2 or 1 forces a width where the channel count allows it)
-  const unsigned gx = (unsigned)((V + 127) / 128);
-  const long long enough = 2LL * 152;
-  int nt = n->mma_nt;
-  if (nt != 8 && nt != 4 && nt != 2 && nt != 1) {
-    nt = 1;
-    for (int c = 8; c > 1; c /= 2)
-      if (cout % (8 * c) == 0 && (long long)gx * (cout / (8 * c)) >= enough) {
-        nt = c;
-        break;
-      }
-    if (nt == 1 && (long long)gx * ((cout + 15) / 16) >= enough) nt = 2;
-  }
-  if (nt == 8 && cout % 64) nt = 4;
-  if (nt == 4 && cout % 32) nt = 2;
-  switch (nt) {
-    case 8:
-      k_conv3<8><<<dim3(gx, cout / 64), 128, 0, n->st>>>(dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask, ldm);
-      break;
-    case 4:
-      k_conv3<4><<<dim3(gx, cout / 32), 128, 0, n->st>>>(dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask, ldm);
-      break;
-    case 2:
-      k_conv3<2><<<dim3(gx, (cout + 15) / 16), 128, 0, n->st>>>(dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask,
-                                                                 ldm);
-      break;
-    default:
-      k_conv3<1><<<dim3(gx, (cout + 7) / 8), 128, 0, n->st>>>(dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask,
-                                                               ldm);
-  }
-  UTRY(n, cudaGetLastError());
+  // output channels a block: 32, 16 or 8, the widest that its shared memory
+  // takes and that still gives 100 blocks; each output sees the same
+  // sequence of MMAs whichever width computes it (STP_UNET_MMA_NT = 8, 4, 2 or
+  // 1 asks for a width, taken where channels and shared memory allow)
+  const long long tiles = (long long)dm.n * ((dm.w + CS_TX - 1) / CS_TX) * ((dm.h + CS_TY - 1) / CS_TY) *
+                          ((dm.d + CS_TZ - 1) / CS_TZ);
+  const bool forced = n->mma_nt == 8 || n->mma_nt == 4 || n->mma_nt == 2 || n->mma_nt == 1;
+  int nt = forced ? std::min(n->mma_nt, 4) : 4;
+  while (nt > 1 && (cout % (8 * nt) || conv3_smem(cin, nt) > kTcSmemMax ||
+                    (!forced && tiles * (cout / (8 * nt)) < 100)))
+    nt /= 2;
+  auto go = [&](auto kern, std::atomic<unsigned>& done) -> cudaError_t {
+    if (cudaError_t e = smem_limit_once(kern, (int)kTcSmemMax, done)) return e;
+    kern<<<dim3((unsigned)tiles, (unsigned)(cout / (8 * nt))), 128, conv3_smem(cin, nt), n->st>>>(
+        dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask, ldm);
+    return cudaGetLastError();
+  };
+  static std::atomic<unsigned> done4{0u}, done2{0u}, done1{0u};
+  UTRY(n, nt == 4 ? go(k_conv3<4>, done4) : nt == 2 ? go(k_conv3<2>, done2) : go(k_conv3<1>, done1));
   return STP_OK;
 }
 
+// slices of a layer's weight gradient: enough blocks for two a SM, at most one
+// tile each, and at most the scratch
+int wgrad_tile(int c) { return c % 32 == 0 ? 32 : 16; }
+constexpr size_t kWgradScratch = (size_t)6 << 20;  // floats
+int wgrad_slices(const Dims& dm, int cin, int cout) {
+  const long long pairs = (long long)(cin / wgrad_tile(cin)) * (cout / wgrad_tile(cout));
+  const long long tiles = wg_tiles(dm).count(dm.n);
+  long long s = std::max<long long>(1, (2 * 152 + pairs - 1) / pairs);
+  s = std::min(s, (long long)(kWgradScratch / ((size_t)WG_SLOTS * cin * cout)));
+  return (int)std::max<long long>(1, std::min(s, tiles));
+}
+
+template <int OT, int CT>
+cudaError_t wgrad_launch(const Dims& dm, const bf16* x, int ldx, int cin, const bf16* gz, int ldg, int cout, float* part,
+                         int slices, cudaStream_t st) {
+  static std::atomic<unsigned> done{0u};
+  if (cudaError_t e = smem_limit_once(k_wgrad3<OT, CT>, wg_smem(OT, CT), done)) return e;
+  k_wgrad3<OT, CT><<<dim3((unsigned)((cin / CT) * (cout / OT)), (unsigned)slices), 288, wg_smem(OT, CT), st>>>(
+      dm, x, ldx, cin, gz, ldg, cout, part);
+  return cudaGetLastError();
+}
+
+// weight and bias gradient of a 3x3x3 layer, stored (not added) into n->grad
 int wgrad3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf16* gz, int ldg, int cout,
            const Layer& ly) {
-  const long long V = dm.vox();
-  const int tiles = 27 * ((cin + 31) / 32) * (cout / 16);
-  long long splits = std::max<long long>(1, std::min<long long>((152LL * 16) / tiles + 1, (V + 63) / 64));
-  long long chunk = (V + splits - 1) / splits;
-  chunk = ((chunk + 63) / 64) * 64;
-  splits = (V + chunk - 1) / chunk;
-  k_wgrad3<<<dim3(tiles, (unsigned)splits), 128, 0, n->st>>>(dm, x, ldx, cin, gz, ldg, cout, n->grad + ly.woff,
-                                                             nullptr, chunk);
+  const int slices = wgrad_slices(dm, cin, cout);
+  const int ot = wgrad_tile(cout), ct = wgrad_tile(cin);
+  if (ot == 32)
+    UTRY(n, (ct == 32 ? wgrad_launch<32, 32> : wgrad_launch<32, 16>)(dm, x, ldx, cin, gz, ldg, cout, n->wpart, slices, n->st));
+  else
+    UTRY(n, (ct == 32 ? wgrad_launch<16, 32> : wgrad_launch<16, 16>)(dm, x, ldx, cin, gz, ldg, cout, n->wpart, slices, n->st));
+  const int total = 27 * cin * cout + cout;
+  k_wgrad_sum<<<(total + 127) / 128, 128, 0, n->st>>>(n->wpart, slices, cin, cout, n->grad + ly.woff, n->grad + ly.boff);
   UTRY(n, cudaGetLastError());
-  const int bx = (int)std::min<long long>(V, 1024);
-  k_bias_grad<<<dim3(bx, (cout + 127) / 128), 128, 0, n->st>>>(V, gz, ldg, cout, n->grad + ly.boff);
+  return STP_OK;
+}
+int wgrad_in(stp_unet* n, const Dims& dm, const float* x, const bf16* gz, int ldg, const Layer& ly) {
+  const int slices = std::min(wg_tiles(dm).count(dm.n), 4 * 152);
+  k_wgrad_in<<<slices, 256, 0, n->st>>>(dm, x, gz, ldg, n->wpart);
+  UTRY(n, cudaGetLastError());
+  k_wgrad_in_sum<<<(28 * 16 * 32 + 127) / 128, 128, 0, n->st>>>(n->wpart, slices, n->grad + ly.woff, n->grad + ly.boff);
   UTRY(n, cudaGetLastError());
   return STP_OK;
 }
@@ -1221,12 +1427,7 @@ int backward(stp_unet* n, const float* x, int nb) {
       gq_in = gq;
     } else {
       // conv a of level 1: the network input (1 channel)
-      k_wgrad_in<<<dim3((unsigned)std::min<long long>(152 * 2, (dm[0].vox() + 255) / 256), 27), 256, 0, n->st>>>(
-          dm[0], x, gha, c, n->grad + la.woff);
-      UTRY(n, cudaGetLastError());
-      const int bx = (int)std::min<long long>(dm[0].vox(), 1024);
-      k_bias_grad<<<dim3(bx, 1), 128, 0, n->st>>>(dm[0].vox(), gha, c, c, n->grad + la.boff);
-      UTRY(n, cudaGetLastError());
+      if ((rc = wgrad_in(n, dm[0], x, gha, c, la))) return rc;
     }
   }
   return STP_OK;
@@ -1366,6 +1567,7 @@ int stp_unet_create(int nmax, int nz, int ny, int nx, void* stream, stp_unet** o
   A(&n->snorm, (size_t)nmax);
   A(&n->gy, (size_t)V[0]);
   A(&n->loss, 1);
+  A(&n->wpart, kWgradScratch);
   A(&n->d_err, 1);
   if (const char* e = std::getenv("STP_UNET_TC")) n->use_tc = std::atoi(e) != 0;
   if (const char* e = std::getenv("STP_UNET_TC_PLANES")) n->tc_planes = std::atoi(e);
@@ -1507,10 +1709,7 @@ int stp_unet_layer(stp_unet* n, int layer, int mode, const float* a, const float
     if ((rc = talloc(&xb, V * co))) return done(ufail(n, rc, "cudaMalloc failed"));
     k_to_bf16<<<blocks_for(V * co), 256, 0, n->st>>>(V * co, b, xb);
     if (layer == 0) {
-      k_wgrad_in<<<dim3((unsigned)std::min<long long>(152 * 2, (V + 255) / 256), 27), 256, 0, n->st>>>(
-          dm, a, xb, co, n->grad + ly.woff);
-      const int bx = (int)std::min<long long>(V, 1024);
-      k_bias_grad<<<dim3(bx, 1), 128, 0, n->st>>>(V, xb, co, co, n->grad + ly.boff);
+      if ((rc = wgrad_in(n, dm, a, xb, co, ly))) return done(rc);
     } else {
       if ((rc = talloc(&xa, V * ci))) return done(ufail(n, rc, "cudaMalloc failed"));
       k_to_bf16<<<blocks_for(V * ci), 256, 0, n->st>>>(V * ci, a, xa);
