@@ -46,7 +46,24 @@ __device__ __forceinline__ unsigned pack2(bf16 lo, bf16 hi) {
   return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
 }
 
-// source voxel of v shifted by tap t (periodic y, x; -1 outside the walls)
+// eight BF16 of a 16-byte vector, as floats and back
+__device__ __forceinline__ void unpack8(const uint4& u, float* f) {
+  const unsigned w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    f[2 * i] = __bfloat162float(__ushort_as_bfloat16((unsigned short)(w[i] & 0xFFFFu)));
+    f[2 * i + 1] = __bfloat162float(__ushort_as_bfloat16((unsigned short)(w[i] >> 16)));
+  }
+}
+__device__ __forceinline__ uint4 pack8(const float* f) {
+  return make_uint4(pack2(__float2bfloat16(f[0]), __float2bfloat16(f[1])),
+                    pack2(__float2bfloat16(f[2]), __float2bfloat16(f[3])),
+                    pack2(__float2bfloat16(f[4]), __float2bfloat16(f[5])),
+                    pack2(__float2bfloat16(f[6]), __float2bfloat16(f[7])));
+}
+__device__ __forceinline__ uint4 ld16(const bf16* p) { return *reinterpret_cast<const uint4*>(p); }
+__device__ __forceinline__ void st16(bf16* p, const uint4& u) { *reinterpret_cast<uint4*>(p) = u; }
+
 // voxel index (below 2^31, checked at creation) as sample and coordinates,
 // in 32-bit arithmetic
 struct Coord {
@@ -64,18 +81,6 @@ __device__ __forceinline__ Coord coord_of(const Dims& dm, unsigned v) {
 }
 __device__ __forceinline__ long long voxel_at(const Dims& dm, int n, int z, int y, int x) {
   return ((long long)(n * dm.d + z) * dm.h + y) * dm.w + x;
-}
-
-// source voxel of tap t = (kz*3 + ky)*3 + kx at c: periodic in x and y,
-// -1 outside the walls in z
-__device__ __forceinline__ long long tap_from(const Dims& dm, const Coord& c, int t) {
-  const int z2 = c.z + t / 9 - 1;
-  if (z2 < 0 || z2 >= dm.d) return -1;
-  int y2 = c.y + (t / 3) % 3 - 1;
-  int x2 = c.x + t % 3 - 1;
-  y2 = y2 < 0 ? y2 + dm.h : (y2 >= dm.h ? y2 - dm.h : y2);
-  x2 = x2 < 0 ? x2 + dm.w : (x2 >= dm.w ? x2 - dm.w : x2);
-  return voxel_at(dm, c.n, z2, y2, x2);
 }
 
 // ---------------------------------------------------------------------------
@@ -106,11 +111,16 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool fill) {
 // a coordinate at most one tile outside [0, n), wrapped
 __device__ __forceinline__ int wrap1(int a, int n) { return a < 0 ? a + n : a >= n ? (a - n) % n : a; }
 
-// shared memory: the halo, then 27 taps' weights, both in chunks of 8 input
-// channels (16 bytes a voxel or output channel)
-constexpr size_t conv3_smem(int cin, int nt) { return (size_t)(cin / 8) * 16 * (CS_HVOX + 27 * 8 * nt); }
+// shared memory: the halo, then the weights of `taps` taps, both in chunks of
+// 8 input channels (16 bytes a voxel or output channel).  RING: the weights
+// stream through a ring of CS_RING taps (several blocks an SM, or channel
+// counts whose 27 taps do not fit); else all are resident.
+constexpr int CS_RING = 6;
+constexpr size_t conv3_smem(int cin, int nt, bool ring) {
+  return (size_t)(cin / 8) * 16 * (CS_HVOX + (ring ? CS_RING : 27) * 8 * nt);
+}
 
-template <int NT>
+template <int NT, bool RING>
 __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__ x, int ldx, int cin,
                                                const bf16* __restrict__ wt, const float* __restrict__ bias, int cout,
                                                bf16* __restrict__ y, int ldy, int relu, const bf16* __restrict__ mask,
@@ -134,12 +144,19 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
     const bf16* src = x + voxel_at(dm, nn, in ? vz : 0, wrap1(y0 - 1 + hy, dm.h), wrap1(x0 - 1 + hx, dm.w)) * ldx;
     for (int c = 0; c < nch; c++) cp16(sx + 16 * (c * CS_HVOX + i), src + 8 * c, in);
   }
-  for (int part = 0; part < 3; part++) {
-    for (int i = tid; i < 9 * 8 * NT * nch; i += 128) {
-      const int c = i % nch, o = (i / nch) % (8 * NT), t = part * 9 + i / (nch * 8 * NT);
-      cp16(sw + 16 * ((t * nch + c) * 8 * NT + o), wt + ((long long)t * cout + cob + o) * cin + 8 * c, true);
+  // weights of taps [ta, tb), one group
+  auto load_w = [&](int ta, int tb) {
+    for (int i = tid; i < (tb - ta) * 8 * NT * nch; i += 128) {
+      const int c = i % nch, o = (i / nch) % (8 * NT), t = ta + i / (nch * 8 * NT);
+      cp16(sw + 16 * (((RING ? t % CS_RING : t) * nch + c) * 8 * NT + o),
+           wt + ((long long)t * cout + cob + o) * cin + 8 * c, true);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if constexpr (RING) {
+    for (int t = 0; t < CS_RING - 1; t++) load_w(t, t + 1);
+  } else {
+    for (int part = 0; part < 3; part++) load_w(9 * part, 9 * part + 9);
   }
   float acc[NT][4];
 #pragma unroll
@@ -152,7 +169,17 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
   const uint32_t a_lane = sx + 16 * ((mi >> 1) * CS_HVOX + (wz * CS_HY + wy + (mi & 1)) * CS_HX + mr);
   const uint32_t b_lane = sw + 16 * ((mi & 1) * 8 * NT + (mi >> 1) * 8 + mr);
   for (int t = 0; t < 27; t++) {
-    if (t % 9 == 0) {
+    if constexpr (RING) {
+      // tap t has landed when at most the CS_RING - 2 groups after it are in
+      // flight; past the barrier every warp has left tap t - 1, whose slot
+      // takes tap t + CS_RING - 1
+      asm volatile("cp.async.wait_group %0;" ::"n"(CS_RING - 2) : "memory");
+      __syncthreads();
+      if (t + CS_RING - 1 < 27)
+        load_w(t + CS_RING - 1, t + CS_RING);
+      else
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    } else if (t % 9 == 0) {
       if (t == 0)
         asm volatile("cp.async.wait_group 2;" ::: "memory");
       else if (t == 9)
@@ -162,7 +189,7 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
       __syncthreads();
     }
     const uint32_t at = a_lane + 16 * ((t / 9 * CS_HY + t / 3 % 3) * CS_HX + t % 3);
-    const uint32_t bt = b_lane + 16 * t * nch * 8 * NT;
+    const uint32_t bt = b_lane + 16 * (RING ? t % CS_RING : t) * nch * 8 * NT;
 #pragma unroll 2
     for (int c = 0; c < nch; c += 2) {
       unsigned a[4];
@@ -518,35 +545,64 @@ __global__ void __launch_bounds__(128) k_conv3_tc(Dims dm, const bf16* __restric
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
 }
 
-// First layer: 1 input channel (FP32 input rounded to BF16) -> 16 channels, ReLU.
-__global__ void k_conv_in(Dims dm, const float* __restrict__ x, const float* __restrict__ w /*[16][27]*/,
+// First layer: 1 input channel (FP32 input rounded to BF16) -> 16 channels,
+// ReLU.  A thread takes four voxels of a row (the width is a multiple of 8):
+// a tap's 16 weights are four vector reads of shared memory for 64
+// multiply-adds (one scalar read each when a thread took one voxel: 67 us at
+// 128 x 64 x 128, FP32 multiply-adds alone 12), and a row's six inputs serve
+// its three taps.  The taps are added in order.
+__global__ void __launch_bounds__(128) k_conv_in(Dims dm, const float* __restrict__ x, const float* __restrict__ w /*[16][27]*/,
                           const float* __restrict__ bias, bf16* __restrict__ y, int ldy) {
-  __shared__ float ws[16 * 27 + 16];
-  for (int i = threadIdx.x; i < 16 * 27; i += blockDim.x) ws[i] = __bfloat162float(__float2bfloat16(w[i]));
-  for (int i = threadIdx.x; i < 16; i += blockDim.x) ws[16 * 27 + i] = bias[i];
+  __shared__ __align__(16) float ws[28][16];
+  for (int i = threadIdx.x; i < 16 * 27; i += blockDim.x) ws[i % 27][i / 27] = __bfloat162float(__float2bfloat16(w[i]));
+  for (int i = threadIdx.x; i < 16; i += blockDim.x) ws[27][i] = bias[i];
   __syncthreads();
-  const long long V = dm.vox();
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
-    float acc[16];
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;  // the caller's array
+  const unsigned units = (unsigned)(dm.vox() / 4);
+  for (unsigned f = blockIdx.x * blockDim.x + threadIdx.x; f < units; f += gridDim.x * blockDim.x) {
+    const Coord c = coord_of(dm, 4 * f);
+    float acc[4][16];
 #pragma unroll
-    for (int o = 0; o < 16; o++) acc[o] = ws[16 * 27 + o];
-    // the taps in order, one z plane of 9 at a time: its 9 inputs are loaded
-    // together, then multiplied in; planes outside the walls add nothing
-    const Coord cv = coord_of(dm, (unsigned)v);
-    for (int kz = 0; kz < 3; kz++) {
-      if (tap_from(dm, cv, kz * 9) < 0) continue;
-      float xt[9];
+    for (int o = 0; o < 16; o++)
 #pragma unroll
-      for (int u = 0; u < 9; u++) xt[u] = __bfloat162float(__float2bfloat16(x[tap_from(dm, cv, kz * 9 + u)]));
+      for (int e = 0; e < 4; e++) acc[e][o] = ws[27][o];
+#pragma unroll 1
+    for (int r = 0; r < 9; r++) {
+      const int z = c.z + r / 3 - 1;
+      if (z < 0 || z >= dm.d) continue;  // planes outside the walls add nothing
+      int yy = c.y + r % 3 - 1;
+      yy = yy < 0 ? yy + dm.h : yy >= dm.h ? yy - dm.h : yy;
+      const float* row = x + voxel_at(dm, c.n, z, yy, 0);
+      const float* a = row + c.x;
+      const float4 m = vec ? __ldg(reinterpret_cast<const float4*>(a)) : make_float4(a[0], a[1], a[2], a[3]);
+      float in[6] = {__ldg(row + (c.x == 0 ? dm.w - 1 : c.x - 1)), m.x, m.y, m.z, m.w,
+                     __ldg(row + (c.x + 4 == dm.w ? 0 : c.x + 4))};
 #pragma unroll
-      for (int u = 0; u < 9; u++)
+      for (int i = 0; i < 6; i++) in[i] = __bfloat162float(__float2bfloat16(in[i]));
 #pragma unroll
-        for (int o = 0; o < 16; o++) acc[o] = fmaf(ws[o * 27 + kz * 9 + u], xt[u], acc[o]);
+      for (int kx = 0; kx < 3; kx++)
+#pragma unroll
+        for (int o = 0; o < 16; o += 4) {
+          const float4 wv = *reinterpret_cast<const float4*>(&ws[3 * r + kx][o]);
+#pragma unroll
+          for (int e = 0; e < 4; e++) {
+            acc[e][o] = fmaf(wv.x, in[e + kx], acc[e][o]);
+            acc[e][o + 1] = fmaf(wv.y, in[e + kx], acc[e][o + 1]);
+            acc[e][o + 2] = fmaf(wv.z, in[e + kx], acc[e][o + 2]);
+            acc[e][o + 3] = fmaf(wv.w, in[e + kx], acc[e][o + 3]);
+          }
+        }
     }
 #pragma unroll
-    for (int o = 0; o < 16; o += 2)
-      *reinterpret_cast<unsigned*>(y + v * ldy + o) =
-          pack2(__float2bfloat16(fmaxf(acc[o], 0.f)), __float2bfloat16(fmaxf(acc[o + 1], 0.f)));
+    for (int e = 0; e < 4; e++) {
+      unsigned v[8];
+#pragma unroll
+      for (int o = 0; o < 8; o++)
+        v[o] = pack2(__float2bfloat16(fmaxf(acc[e][2 * o], 0.f)), __float2bfloat16(fmaxf(acc[e][2 * o + 1], 0.f)));
+      uint4* yp = reinterpret_cast<uint4*>(y + (4LL * f + e) * ldy);
+      yp[0] = make_uint4(v[0], v[1], v[2], v[3]);
+      yp[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
   }
 }
 
@@ -558,9 +614,11 @@ __global__ void k_conv_out(long long V, const bf16* __restrict__ x, int ldx, con
   for (int c = 0; c < 16; c++) ws[c] = __bfloat162float(__float2bfloat16(w[c]));
   const float b = bias[0];
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
-    float s = b;
+    float s = b, e[16];
+    unpack8(ld16(x + v * ldx), e);
+    unpack8(ld16(x + v * ldx + 8), e + 8);
 #pragma unroll
-    for (int c = 0; c < 16; c++) s = fmaf(ws[c], __bfloat162float(x[v * ldx + c]), s);
+    for (int c = 0; c < 16; c++) s = fmaf(ws[c], e[c], s);
     y[v] = s;
   }
 }
@@ -581,14 +639,16 @@ __global__ void k_conv_out_bwd(long long V, const float* __restrict__ gy, const 
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
     const float g = gy[v];
     acc[16] += g;
+    float a[16], o[16];
+    unpack8(ld16(d1 + v * ldx), a);
+    unpack8(ld16(d1 + v * ldx + 8), a + 8);
 #pragma unroll
-    for (int c = 0; c < 16; c += 2) {
-      const float a0 = __bfloat162float(d1[v * ldx + c]), a1 = __bfloat162float(d1[v * ldx + c + 1]);
-      acc[c] += g * a0;
-      acc[c + 1] += g * a1;
-      *reinterpret_cast<unsigned*>(gd + v * ldg + c) =
-          pack2(__float2bfloat16(a0 > 0.f ? g * ws[c] : 0.f), __float2bfloat16(a1 > 0.f ? g * ws[c + 1] : 0.f));
+    for (int c = 0; c < 16; c++) {
+      acc[c] += g * a[c];
+      o[c] = a[c] > 0.f ? g * ws[c] : 0.f;
     }
+    st16(gd + v * ldg, pack8(o));
+    st16(gd + v * ldg + 8, pack8(o + 8));
   }
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
 #pragma unroll
@@ -751,16 +811,24 @@ __global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict_
     }
 }
 
-// gw[o][c][t], gb[o] = sum over the slices in order
-__global__ void k_wgrad_sum(const float* __restrict__ part, int slices, int cin, int cout, float* __restrict__ gw,
-                            float* __restrict__ gb) {
-  const int n = 27 * cout * cin, e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n + cout) return;
-  const size_t off = e < n ? e : (size_t)27 * cout * cin + (size_t)(e - n) * cin;
+// gw[o][c][t], gb[o] = sum over the slices: a block takes 32 outputs, its
+// eight warps every eighth slice each, added in a fixed order (one thread an
+// output walking up to 304 slices waited on memory: 15 us a layer)
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, int slices, int cin, int cout,
+                                                   float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ float red[8][32];
+  const int n = 27 * cout * cin, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  const bool in = e < n + cout;
+  const size_t off = e < n ? e : (size_t)27 * cout * cin + (size_t)(in ? e - n : 0) * cin;
   const size_t stride = (size_t)WG_SLOTS * cout * cin;
   float s = 0.f;
-#pragma unroll 8
-  for (int i = 0; i < slices; i++) s += part[off + i * stride];
+#pragma unroll 4
+  for (int i = warp; i < slices; i += 8) s += part[off + i * stride];
+  red[warp][lane] = s;
+  __syncthreads();
+  if (warp || !in) return;
+#pragma unroll
+  for (int w = 1; w < 8; w++) s += red[w][lane];
   if (e < n) {
     const int oc = e % (cout * cin), t = e / (cout * cin);
     gw[(size_t)oc * 27 + t] = s;
@@ -874,23 +942,6 @@ __global__ void k_wgrad_in_sum(const float* __restrict__ part, int slices, float
 // one take one 8-channel vector a thread (blockIdx.y); those that write the
 // fine level take one voxel a thread, all its channels (whole rows of
 // stores).
-__device__ __forceinline__ void unpack8(const uint4& u, float* f) {
-  const unsigned w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    f[2 * i] = __bfloat162float(__ushort_as_bfloat16((unsigned short)(w[i] & 0xFFFFu)));
-    f[2 * i + 1] = __bfloat162float(__ushort_as_bfloat16((unsigned short)(w[i] >> 16)));
-  }
-}
-__device__ __forceinline__ uint4 pack8(const float* f) {
-  return make_uint4(pack2(__float2bfloat16(f[0]), __float2bfloat16(f[1])),
-                    pack2(__float2bfloat16(f[2]), __float2bfloat16(f[3])),
-                    pack2(__float2bfloat16(f[4]), __float2bfloat16(f[5])),
-                    pack2(__float2bfloat16(f[6]), __float2bfloat16(f[7])));
-}
-__device__ __forceinline__ uint4 ld16(const bf16* p) { return *reinterpret_cast<const uint4*>(p); }
-__device__ __forceinline__ void st16(bf16* p, const uint4& u) { *reinterpret_cast<uint4*>(p) = u; }
-
 // out (coarse) = mean of the 2x2x2 fine block (summed in block order); fine dims dm
 __global__ void k_pool(Dims dm, const bf16* __restrict__ x, int ldx, int c, bf16* __restrict__ y, int ldy) {
   const Dims cd{dm.n, dm.d / 2, dm.h / 2, dm.w / 2};
@@ -1019,9 +1070,10 @@ __global__ void k_pack_image(const bf16* __restrict__ wt, int cin, int cout, bf1
   }
 }
 
-// mean((y - t)^2) (per-block partials, summed with atomics) and gy = 2(y - t)/n
-__global__ void k_mse(long long n, const float* __restrict__ y, const float* __restrict__ t, float* __restrict__ gy,
-                      float* __restrict__ loss) {
+// mean((y - t)^2) (block sums, added with one atomic a block) and gy = 2(y - t)/n
+__global__ void __launch_bounds__(256) k_mse(long long n, const float* __restrict__ y, const float* __restrict__ t,
+                                             float* __restrict__ gy, float* __restrict__ loss) {
+  __shared__ float red[8];
   float s = 0.f;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float d = y[i] - t[i];
@@ -1029,7 +1081,12 @@ __global__ void k_mse(long long n, const float* __restrict__ y, const float* __r
     gy[i] = 2.f * d / (float)n;
   }
   for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / (float)n);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) s += red[w];
+    atomicAdd(loss, s / (float)n);
+  }
 }
 
 __global__ void k_adam(long long n, float* __restrict__ th, const float* __restrict__ g, float* __restrict__ m,
@@ -1233,25 +1290,28 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
     UTRY(n, cudaGetLastError());
     return STP_OK;
   }
-  // output channels a block: 32, 16 or 8, the widest that its shared memory
-  // takes and that still gives 100 blocks; each output sees the same
-  // sequence of MMAs whichever width computes it (STP_UNET_MMA_NT = 8, 4, 2 or
-  // 1 asks for a width, taken where channels and shared memory allow)
+  // output channels a block: 32, 16 or 8, the widest that still gives 100
+  // blocks; each output sees the same sequence of MMAs whichever width
+  // computes it (STP_UNET_MMA_NT = 8, 4, 2 or 1 asks for a width, 8 as 4).
+  // Resident weights when they fit and the blocks are one wave of the GPU.
   const long long tiles = (long long)dm.n * ((dm.w + CS_TX - 1) / CS_TX) * ((dm.h + CS_TY - 1) / CS_TY) *
                           ((dm.d + CS_TZ - 1) / CS_TZ);
   const bool forced = n->mma_nt == 8 || n->mma_nt == 4 || n->mma_nt == 2 || n->mma_nt == 1;
   int nt = forced ? std::min(n->mma_nt, 4) : 4;
-  while (nt > 1 && (cout % (8 * nt) || conv3_smem(cin, nt) > kTcSmemMax ||
-                    (!forced && tiles * (cout / (8 * nt)) < 100)))
-    nt /= 2;
+  while (nt > 1 && (cout % (8 * nt) || (!forced && tiles * (cout / (8 * nt)) < 100))) nt /= 2;
+  const long long blocks = tiles * (cout / (8 * nt));
+  const bool ring = !(conv3_smem(cin, nt, false) <= kTcSmemMax && (conv3_smem(cin, nt, false) <= 56 * 1024 || blocks <= 152));
   auto go = [&](auto kern, std::atomic<unsigned>& done) -> cudaError_t {
     if (cudaError_t e = smem_limit_once(kern, (int)kTcSmemMax, done)) return e;
-    kern<<<dim3((unsigned)tiles, (unsigned)(cout / (8 * nt))), 128, conv3_smem(cin, nt), n->st>>>(
+    kern<<<dim3((unsigned)tiles, (unsigned)(cout / (8 * nt))), 128, conv3_smem(cin, nt, ring), n->st>>>(
         dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask, ldm);
     return cudaGetLastError();
   };
-  static std::atomic<unsigned> done4{0u}, done2{0u}, done1{0u};
-  UTRY(n, nt == 4 ? go(k_conv3<4>, done4) : nt == 2 ? go(k_conv3<2>, done2) : go(k_conv3<1>, done1));
+  static std::atomic<unsigned> done[6];
+  if (ring)
+    UTRY(n, nt == 4 ? go(k_conv3<4, true>, done[0]) : nt == 2 ? go(k_conv3<2, true>, done[1]) : go(k_conv3<1, true>, done[2]));
+  else
+    UTRY(n, nt == 4 ? go(k_conv3<4, false>, done[3]) : nt == 2 ? go(k_conv3<2, false>, done[4]) : go(k_conv3<1, false>, done[5]));
   return STP_OK;
 }
 
@@ -1287,7 +1347,7 @@ int wgrad3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const b
   else
     UTRY(n, (ct == 32 ? wgrad_launch<16, 32> : wgrad_launch<16, 16>)(dm, x, ldx, cin, gz, ldg, cout, n->wpart, slices, n->st));
   const int total = 27 * cin * cout + cout;
-  k_wgrad_sum<<<(total + 127) / 128, 128, 0, n->st>>>(n->wpart, slices, cin, cout, n->grad + ly.woff, n->grad + ly.boff);
+  k_wgrad_sum<<<(total + 31) / 32, 256, 0, n->st>>>(n->wpart, slices, cin, cout, n->grad + ly.woff, n->grad + ly.boff);
   UTRY(n, cudaGetLastError());
   return STP_OK;
 }
@@ -1322,7 +1382,7 @@ int forward(stp_unet* n, const float* x, int nb) {
   // encoder
   const Layer* P = n->L.data();
   // level 1: input layer, second conv writes e1 into u[0][:, 32:48]
-  k_conv_in<<<blocks_for(dm[0].vox()), 256, 0, n->st>>>(dm[0], x, n->theta + P[0].woff, n->theta + P[0].boff, n->ha[0],
+  k_conv_in<<<blocks_for(dm[0].vox() / 4, 128), 128, 0, n->st>>>(dm[0], x, n->theta + P[0].woff, n->theta + P[0].boff, n->ha[0],
                                                          16);
   UTRY(n, cudaGetLastError());
   const bf16* in = nullptr;
@@ -1637,7 +1697,7 @@ int stp_unet_gradient(stp_unet* n, const float* x, const float* target, int nb, 
   if (rc) return rc;
   const long long V = n->dm[0].vox() / n->nmax * nb;
   UTRY(n, cudaMemsetAsync(n->loss, 0, sizeof(float), n->st));
-  k_mse<<<blocks_for(V), 256, 0, n->st>>>(V, n->y, target, n->gy, n->loss);
+  k_mse<<<std::min(blocks_for(V), 4 * 152), 256, 0, n->st>>>(V, n->y, target, n->gy, n->loss);
   UTRY(n, cudaGetLastError());
   if ((rc = backward(n, x, nb))) return rc;
   if (grad) UTRY(n, cudaMemcpyAsync(grad, n->grad, sizeof(float) * n->np, cudaMemcpyDeviceToDevice, n->st));
@@ -1688,7 +1748,7 @@ int stp_unet_layer(stp_unet* n, int layer, int mode, const float* a, const float
   if (mode == 0) {
     if (layer == 0) {
       if ((rc = talloc(&y, V * co))) return done(ufail(n, rc, "cudaMalloc failed"));
-      k_conv_in<<<blocks_for(V), 256, 0, n->st>>>(dm, a, n->theta + ly.woff, n->theta + ly.boff, y, co);
+      k_conv_in<<<blocks_for(V / 4, 128), 128, 0, n->st>>>(dm, a, n->theta + ly.woff, n->theta + ly.boff, y, co);
       if (cudaGetLastError() != cudaSuccess) return done(ufail(n, STP_ECUDA, "k_conv_in launch failed"));
     } else {
       if ((rc = talloc(&xa, V * ci)) || (rc = talloc(&y, V * co))) return done(ufail(n, rc, "cudaMalloc failed"));
@@ -1753,7 +1813,7 @@ int stp_unet_eval_pairs(stp_unet* n, const float* r, const float* dp, int nb, fl
   int rc = forward(n, n->xin, nb);
   if (rc) return rc;
   UTRY(n, cudaMemsetAsync(n->loss, 0, sizeof(float), n->st));
-  k_mse<<<blocks_for(Vs * nb), 256, 0, n->st>>>(Vs * nb, n->y, n->tin, n->gy, n->loss);
+  k_mse<<<std::min(blocks_for(Vs * nb), 4 * 152), 256, 0, n->st>>>(Vs * nb, n->y, n->tin, n->gy, n->loss);
   UTRY(n, cudaGetLastError());
   UTRY(n, cudaMemcpyAsync(n->h_loss, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->st));
   UTRY(n, cudaStreamSynchronize(n->st));
