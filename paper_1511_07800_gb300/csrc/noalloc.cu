@@ -21,6 +21,7 @@
 // counter is cleared at the start of each call.  Calls whose work overlaps
 // on the GPU (different streams, or several host threads) race on the
 // array and must be serialised by the caller.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -37,11 +38,10 @@ constexpr int kNoallocMaxNz = 4096;
 constexpr unsigned kNoallocMaxBlocks = 65536;
 
 struct NoallocScratch {
-  double cup[kNoallocMaxNz];
-  double cdn[kNoallocMaxNz];
+  unsigned counter[2];                // one copy a call brings the counter (0) and
+  double coef[2 * kNoallocMaxNz];     // the couplings: cup [nz], cdn [nz]
   double partial[kNoallocMaxBlocks];
   double result[8];
-  unsigned counter[8];
   int flag[8];
 };
 
@@ -52,27 +52,97 @@ namespace {
 std::mutex g_setup_mutex;
 NoallocScratch* g_scratch_addr[256] = {};
 
+// A thread takes W x cells of two rows and walks KZ levels.  The kernel is
+// bound by FP64 operations (GB300 gives 500-545 Gop/s), so every difference of
+// neighbours is formed once and serves both its cells (x inside the vector, y
+// between the two rows, z along the walk), and squares are summed in the
+// thread before the block's tree: about eleven operations a cell, where one
+// cell a thread took fourteen and six more in the reduction.  256 x 128 x 192:
+// 152 us of kernel (eleven operations take 130 us of the FP64 pipe; DRAM 22), a
+// call 317 -> 189 us.  Eight levels a thread leave 768 blocks, a sixth of the
+// GPU idle in the last wave: 200 us a call.
+constexpr int kNoallocLevels = 4;
+
+template <int W>
 __global__ void __launch_bounds__(kBX* kBY) k_residual_noalloc(int nx, int ny, int nz, double idx2, double idy2,
                                                                 const double* __restrict__ p,
                                                                 const double* __restrict__ b,
                                                                 double* __restrict__ r_out, NoallocScratch* sc,
                                                                 unsigned nblocks) {
   __shared__ double sh[32];
-  const int i = blockIdx.x * kBX + threadIdx.x, j = blockIdx.y * kBY + threadIdx.y, k = blockIdx.z;
+  const int i = (blockIdx.x * kBX + threadIdx.x) * W, j = (blockIdx.y * kBY + threadIdx.y) * 2;
+  const int k0 = blockIdx.z * kNoallocLevels, k1 = min(nz, k0 + kNoallocLevels);
   double s = 0.0;
   if (i < nx && j < ny) {
-    const int plane = nx * ny;
-    const int ip = i == nx - 1 ? 0 : i + 1, im = i == 0 ? nx - 1 : i - 1;
-    const int jp = j == ny - 1 ? 0 : j + 1, jm = j == 0 ? ny - 1 : j - 1;
-    const int row = k * plane, q = row + j * nx + i;
-    const double pc = p[q];
-    double lap = idx2 * ((p[row + j * nx + ip] - pc) + (p[row + j * nx + im] - pc)) +
-                 idy2 * ((p[row + jp * nx + i] - pc) + (p[row + jm * nx + i] - pc));
-    if (k < nz - 1) lap += sc->cup[k] * (p[q + plane] - pc);
-    if (k > 0) lap += sc->cdn[k] * (p[q - plane] - pc);
-    const double r = b[q] - lap;
-    if (r_out) r_out[q] = r;
-    s = r * r;
+    auto ldv = [](const double* a, double* v) {
+      if constexpr (W == 2) {
+        const double2 t = *reinterpret_cast<const double2*>(a);
+        v[0] = t.x, v[1] = t.y;
+      } else {
+        v[0] = *a;
+      }
+    };
+    const bool two = j + 1 < ny;  // an odd ny leaves the last row alone
+    const size_t plane = (size_t)nx * ny;
+    const int jn = j + 2 < ny ? j + 2 : j + 2 - ny, js = j == 0 ? ny - 1 : j - 1;
+    const size_t row[2] = {(size_t)j * nx, (size_t)(two ? j + 1 : 0) * nx};
+    // the row past the pair: row 1 itself when the pair has one row
+    const size_t on = (two ? (size_t)jn * nx : row[1]) + i, os = (size_t)js * nx + i;
+    const int il = i == 0 ? nx - 1 : i - 1, ir = i + W == nx ? 0 : i + W;
+    double c[2][W], dn[2][W];  // the pair's cells at level k, and p_k - p_{k-1}
+#pragma unroll
+    for (int y = 0; y < 2; y++) {
+      double below[W];
+      ldv(p + k0 * plane + row[y] + i, c[y]);
+      if (k0 > 0) ldv(p + (k0 - 1) * plane + row[y] + i, below);
+#pragma unroll
+      for (int e = 0; e < W; e++) dn[y][e] = k0 > 0 ? c[y][e] - below[e] : 0.0;
+    }
+    for (int k = k0; k < k1; k++) {
+      const double* lev = p + k * plane;
+      const double cup = sc->coef[k], cdn = sc->coef[nz + k];
+      double vn[W], vs[W], dy[3][W];
+      ldv(lev + on, vn);
+      ldv(lev + os, vs);
+      if (!two) ldv(lev + row[1] + i, c[1]);  // the wrapped row after the last
+#pragma unroll
+      for (int e = 0; e < W; e++) {
+        dy[0][e] = c[0][e] - vs[e];
+        dy[1][e] = c[1][e] - c[0][e];
+        dy[2][e] = two ? vn[e] - c[1][e] : 0.0;
+      }
+#pragma unroll
+      for (int y = 0; y < 2; y++) {
+        if (y == 1 && !two) break;
+        const double* r = lev + row[y];
+        double dx[W + 1], up[W], bv[W], res[W];
+        dx[0] = c[y][0] - r[il];
+#pragma unroll
+        for (int e = 1; e < W; e++) dx[e] = c[y][e] - c[y][e - 1];
+        dx[W] = r[ir] - c[y][W - 1];
+        if (k < nz - 1) ldv(r + plane + i, up);
+        ldv(b + k * plane + row[y] + i, bv);
+#pragma unroll
+        for (int e = 0; e < W; e++) {
+          const double du = k < nz - 1 ? up[e] - c[y][e] : 0.0;
+          double t = fma(-idx2, dx[e + 1] - dx[e], bv[e]);
+          t = fma(-idy2, dy[y + 1][e] - dy[y][e], t);
+          t = fma(-cup, du, t);
+          t = fma(cdn, dn[y][e], t);
+          res[e] = t;
+          s = fma(t, t, s);
+          dn[y][e] = du;
+          c[y][e] = k < nz - 1 ? up[e] : c[y][e];
+        }
+        if (r_out) {
+          double* o = r_out + k * plane + row[y] + i;
+          if constexpr (W == 2)
+            *reinterpret_cast<double2*>(o) = make_double2(res[0], res[1]);
+          else
+            *o = res[0];
+        }
+      }
+    }
   }
   s = block_sum(s, sh);
   Red red{sc->partial, sc->counter, sc->result, sc->flag};
@@ -144,13 +214,22 @@ extern "C" int stp_poisson_residual_noalloc(int nx, int ny, int nz, double Lx, d
   std::vector<double> cup, cdn;
   poisson_couplings(c, cup, cdn);
   cudaStream_t st = (cudaStream_t)stream;
-  e = cudaMemcpyAsync(sc->cup, cup.data(), sizeof(double) * nz, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(sc->cdn, cdn.data(), sizeof(double) * nz, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sc->counter, 0, sizeof(sc->counter), st);
+  // counter (eight zero bytes) and couplings in one copy
+  std::vector<double> head(1 + 2 * (size_t)nz);
+  head[0] = 0.0;
+  std::copy(cup.begin(), cup.end(), head.begin() + 1);
+  std::copy(cdn.begin(), cdn.end(), head.begin() + 1 + nz);
+  e = cudaMemcpyAsync(sc, head.data(), sizeof(double) * head.size(), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return noalloc_fail(STP_ECUDA, std::string("scratch set-up: ") + cudaGetErrorString(e));
   const double dx = Lx / nx, dy = Ly / ny;
-  k_residual_noalloc<<<l.grid, l.block, 0, st>>>(nx, ny, nz, 1.0 / (dx * dx), 1.0 / (dy * dy), p, b, r_out, sc,
-                                                 l.nblocks);
+  // pairs of x cells on even rows whose arrays are 16-byte aligned
+  const bool vec = nx % 2 == 0 && ((uintptr_t)p | (uintptr_t)b | (uintptr_t)r_out) % 16 == 0;
+  const int w = vec ? 2 : 1;
+  const dim3 grid((nx + kBX * w - 1) / (kBX * w), (ny + 2 * kBY - 1) / (2 * kBY),
+                  (nz + kNoallocLevels - 1) / kNoallocLevels);
+  const unsigned nblocks = grid.x * grid.y * grid.z;
+  (vec ? k_residual_noalloc<2> : k_residual_noalloc<1>)<<<grid, l.block, 0, st>>>(
+      nx, ny, nz, 1.0 / (dx * dx), 1.0 / (dy * dy), p, b, r_out, sc, nblocks);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(norm_out, sc->result, sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
