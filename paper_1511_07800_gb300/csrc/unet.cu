@@ -144,12 +144,16 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
     const bf16* src = x + voxel_at(dm, nn, in ? vz : 0, wrap1(y0 - 1 + hy, dm.h), wrap1(x0 - 1 + hx, dm.w)) * ldx;
     for (int c = 0; c < nch; c++) cp16(sx + 16 * (c * CS_HVOX + i), src + 8 * c, in);
   }
-  // weights of taps [ta, tb), one group
+  // weights of taps [ta, tb), one group: a thread keeps its output row and its
+  // chunks from tap to tap
+  constexpr int TPR = 128 / (8 * NT);  // threads a row
+  const int wo = tid / TPR, wc = tid % TPR;
+  const bf16* wrow = wt + (long long)(cob + wo) * cin;
   auto load_w = [&](int ta, int tb) {
-    for (int i = tid; i < (tb - ta) * 8 * NT * nch; i += 128) {
-      const int c = i % nch, o = (i / nch) % (8 * NT), t = ta + i / (nch * 8 * NT);
-      cp16(sw + 16 * (((RING ? t % CS_RING : t) * nch + c) * 8 * NT + o),
-           wt + ((long long)t * cout + cob + o) * cin + 8 * c, true);
+    for (int t = ta; t < tb; t++) {
+      const bf16* src = wrow + (long long)t * cout * cin;
+      const uint32_t dst = sw + 16 * ((RING ? t % CS_RING : t) * nch * 8 * NT + wo);
+      for (int c = wc; c < nch; c += TPR) cp16(dst + 16 * c * 8 * NT, src + 8 * c, true);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -693,8 +697,10 @@ constexpr int WG_TX = 8, WG_TY = 8, WG_TZ = 4, WG_VOX = WG_TX * WG_TY * WG_TZ;
 constexpr int WG_HX = WG_TX + 2, WG_HY = WG_TY + 2, WG_HZ = WG_TZ + 2, WG_HVOX = WG_HX * WG_HY * WG_HZ;
 constexpr int WG_SLOTS = 28;  // taps, then the bias
 
-// smem of a block: gz tile and x halo, in chunks
-constexpr int wg_smem(int OT, int CT) { return 16 * (WG_VOX * OT / 8 + WG_HVOX * CT / 8); }
+// smem of a block: gz tile and x halo, in chunks, twice (the next tile lands
+// while one is multiplied)
+__host__ __device__ constexpr int wg_stage(int OT, int CT) { return 16 * (WG_VOX * OT / 8 + WG_HVOX * CT / 8); }
+constexpr int wg_smem(int OT, int CT) { return 2 * wg_stage(OT, CT); }
 
 __device__ __forceinline__ void ldsm4t(unsigned* r, uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -716,6 +722,7 @@ __global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict_
                                                 float* __restrict__ part) {
   extern __shared__ __align__(128) uint8_t wsm[];
   const uint32_t sg = (uint32_t)__cvta_generic_to_shared(wsm), sx = sg + 16 * WG_VOX * (OT / 8);
+  constexpr uint32_t STAGE = wg_stage(OT, CT);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
   const int cts = cin / CT;
   const int ob = (int)(blockIdx.x / cts) * OT, cb = (int)(blockIdx.x % cts) * CT;
@@ -741,30 +748,35 @@ __global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict_
   const uint32_t a_lane = sg + 16 * ((mi & 1) * WG_VOX + (mi >> 1) * 8 + mr);
   const uint32_t b_lane = sx + 16 * ((mi >> 1) * WG_HVOX + (mi & 1) * WG_HX + mr);
   const int kz = warp / 3, ky = warp % 3;
-  for (int tile = t0; tile < t1; tile++) {
+  auto load = [&](int tile, uint32_t st) {
     int r = tile;
     const int x0 = (r % tl.nx) * WG_TX;
     r /= tl.nx;
     const int y0 = (r % tl.ny) * WG_TY;
     r /= tl.ny;
     const int z0 = (r % tl.nz) * WG_TZ, nn = r / tl.nz;
-    __syncthreads();  // the previous tile has been read
-    for (int i = tid; i < WG_VOX * (OT / 8); i += 288) {
-      const int v = i % WG_VOX, ch = i / WG_VOX;
+    for (int v = tid; v < WG_VOX; v += 288) {
       const int vx = x0 + v % WG_TX, vy = y0 + (v / WG_TX) % WG_TY, vz = z0 + v / (WG_TX * WG_TY);
       const bool in = vx < dm.w && vy < dm.h && vz < dm.d;
-      const long long w = in ? voxel_at(dm, nn, vz, vy, vx) : 0;
-      cp16(sg + 16 * i, gz + w * ldg + ob + 8 * ch, in);
+      const bf16* src = gz + (in ? voxel_at(dm, nn, vz, vy, vx) : 0) * ldg + ob;
+#pragma unroll
+      for (int ch = 0; ch < OT / 8; ch++) cp16(sg + st + 16 * (ch * WG_VOX + v), src + 8 * ch, in);
     }
-    for (int i = tid; i < WG_HVOX * (CT / 8); i += 288) {
-      const int v = i % WG_HVOX, ch = i / WG_HVOX;
+    for (int v = tid; v < WG_HVOX; v += 288) {
       const int hx = v % WG_HX, hy = (v / WG_HX) % WG_HY, hz = v / (WG_HX * WG_HY);
       const int vx = wrap1(x0 - 1 + hx, dm.w), vy = wrap1(y0 - 1 + hy, dm.h), vz = z0 - 1 + hz;
       const bool in = vz >= 0 && vz < dm.d;
-      const long long w = voxel_at(dm, nn, in ? vz : 0, vy, vx);
-      cp16(sx + 16 * i, x + w * ldx + cb + 8 * ch, in);
+      const bf16* src = x + voxel_at(dm, nn, in ? vz : 0, vy, vx) * ldx + cb;
+#pragma unroll
+      for (int ch = 0; ch < CT / 8; ch++) cp16(sx + st + 16 * (ch * WG_HVOX + v), src + 8 * ch, in);
     }
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+  };
+  if (t0 < t1) load(t0, 0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int tile = t0; tile < t1; tile++) {
+    const uint32_t st = ((tile - t0) & 1) * STAGE;
+    if (tile + 1 < t1) load(tile + 1, STAGE - st);
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 1;" ::: "memory");
     __syncthreads();
     // K steps of 16 voxels: two x rows of the tile
 #pragma unroll 2
@@ -772,8 +784,8 @@ __global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict_
       const int vy = (2 * s) % WG_TY, vz = (2 * s) / WG_TY;
       unsigned a[OT / 16][4];
 #pragma unroll
-      for (int m = 0; m < OT / 16; m++) ldsm4t(a[m], a_lane + 16 * (2 * m * WG_VOX + 16 * s));
-      const uint32_t br = b_lane + 16 * (((vz + kz) * WG_HY + vy + ky) * WG_HX);
+      for (int m = 0; m < OT / 16; m++) ldsm4t(a[m], a_lane + st + 16 * (2 * m * WG_VOX + 16 * s));
+      const uint32_t br = b_lane + st + 16 * (((vz + kz) * WG_HY + vy + ky) * WG_HX);
 #pragma unroll
       for (int t = 0; t < 3; t++)
 #pragma unroll
@@ -790,6 +802,7 @@ __global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict_
 #pragma unroll
         for (int m = 0; m < OT / 16; m++) mma16816(accb[m], a[m], ones);
     }
+    __syncthreads();  // every warp has read the tile: its stage takes the one after next
   }
   // slice blockIdx.y of the scratch: [slot][cout][cin]
   float* out = part + (size_t)blockIdx.y * WG_SLOTS * cout * cin;
@@ -1318,9 +1331,11 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
 // slices of a layer's weight gradient: enough blocks for two a SM, at most one
 // tile each, and at most the scratch
 int wgrad_tile(int c) { return c % 32 == 0 ? 32 : 16; }
+// input channels a block: with 16 outputs all of 48 (gz is then read once)
+int wgrad_ctile(int cin, int cout) { return cin == 48 && wgrad_tile(cout) == 16 ? 48 : wgrad_tile(cin); }
 constexpr size_t kWgradScratch = (size_t)6 << 20;  // floats
 int wgrad_slices(const Dims& dm, int cin, int cout) {
-  const long long pairs = (long long)(cin / wgrad_tile(cin)) * (cout / wgrad_tile(cout));
+  const long long pairs = (long long)(cin / wgrad_ctile(cin, cout)) * (cout / wgrad_tile(cout));
   const long long tiles = wg_tiles(dm).count(dm.n);
   long long s = std::max<long long>(1, (2 * 152 + pairs - 1) / pairs);
   s = std::min(s, (long long)(kWgradScratch / ((size_t)WG_SLOTS * cin * cout)));
@@ -1341,11 +1356,11 @@ cudaError_t wgrad_launch(const Dims& dm, const bf16* x, int ldx, int cin, const 
 int wgrad3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf16* gz, int ldg, int cout,
            const Layer& ly) {
   const int slices = wgrad_slices(dm, cin, cout);
-  const int ot = wgrad_tile(cout), ct = wgrad_tile(cin);
+  const int ot = wgrad_tile(cout), ct = wgrad_ctile(cin, cout);
   if (ot == 32)
     UTRY(n, (ct == 32 ? wgrad_launch<32, 32> : wgrad_launch<32, 16>)(dm, x, ldx, cin, gz, ldg, cout, n->wpart, slices, n->st));
   else
-    UTRY(n, (ct == 32 ? wgrad_launch<16, 32> : wgrad_launch<16, 16>)(dm, x, ldx, cin, gz, ldg, cout, n->wpart, slices, n->st));
+    UTRY(n, (ct == 48 ? wgrad_launch<16, 48> : ct == 32 ? wgrad_launch<16, 32> : wgrad_launch<16, 16>)(dm, x, ldx, cin, gz, ldg, cout, n->wpart, slices, n->st));
   const int total = 27 * cin * cout + cout;
   k_wgrad_sum<<<(total + 31) / 32, 256, 0, n->st>>>(n->wpart, slices, cin, cout, n->grad + ly.woff, n->grad + ly.boff);
   UTRY(n, cudaGetLastError());
