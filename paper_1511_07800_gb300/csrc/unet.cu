@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "device_util.cuh"
@@ -93,9 +94,8 @@ __device__ __forceinline__ long long voxel_at(const Dims& dm, int n, int z, int 
 // channels in shared memory up front (three cp.async groups, the later taps'
 // weights landing while the first are multiplied), and a K step is then two
 // ldmatrix and NT multiplies.  Each output sees the same sequence of MMAs (taps,
-// then channels) at every NT.  Loading operands step by step from global
-// memory instead took 85 us for 128 -> 128 at 16 x 8 x 16 voxels; the figures
-// now stand at conv3.
+// then channels) at every NT.  128 -> 128 at 16 x 8 x 16 voxels: 26 us, 85 with
+// operands loaded step by step from global memory.
 // Options: ReLU; multiply by (mask > 0) (the derivative of the ReLU that
 // produced this layer's input, used when the kernel runs the backward data
 // pass with transposed weights); no bias when bias is NULL.
@@ -256,32 +256,45 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
 // accumulator), for layers whose level has w % 8 == 0 and h % 16 == 0 and
 // channel counts that are multiples of 16.
 //
-// A block computes zt planes of 128 voxels, 8 (x) x 16 (y) at zt
-// consecutive z, for all cout channels: per plane M = 128, N = cout,
-// K = 27 taps x cin, the zt accumulators side by side in tensor memory.  The
-// input is staged once per group of up to 64 channels as a halo of
-// 10 x 18 x (zt + 2) voxels (periodic in x and y, zeros outside the walls)
-// in the K-major core-matrix layout without swizzle: 8-channel chunk j of
-// halo voxel (hx, hy, hz) is 16 bytes at j CHUNK + ((hz HY + hy) HX + hx) 16,
-// CHUNK = 16 HX HY (zt + 2).  The A operand of tap (dz, dy, dx) for plane p
-// is then the descriptor whose start is the halo voxel (1+dx, 1+dy, p+dz):
-// its 8-row core matrices are 8 consecutive x (16 bytes apart), the next 8
-// rows are the next y (SBO = 16 HX bytes), the next 8 channels the next
-// chunk (LBO = one chunk of the halo).  So the 27 taps need no data
-// movement.  The weights of a tap (cout x group channels, the same layout
-// with LBO = 128, SBO = 16 x group chunks) are either all resident (every
-// tap of a group loaded at once, then all the group's MMAs back to back,
-// one commit and one wait) or, when they do not fit, stream through a ring
-// of three stages, a stage refilled once the MMAs that read it have
-// completed (tcgen05.commit to that stage's mbarrier).  One thread issues
-// the MMAs and one thread polls each barrier while the others wait at the
-// block barrier.  Every wait is bounded; on a time-out the block sets *err,
-// skips the rest, and still frees its tensor memory.
+// A tile is zt planes of 128 voxels, 8 (x) x 16 (y) at zt consecutive z, for
+// all cout channels: per plane M = 128, N = cout, K = 27 taps x cin, the zt
+// accumulators side by side in tensor memory.  The input is staged by groups
+// of up to 64 channels as a halo of 10 x 18 x (zt + 2) voxels (periodic in x
+// and y, zeros outside the walls) in the K-major core-matrix layout without
+// swizzle: 8-channel chunk j of halo voxel (hx, hy, hz) is 16 bytes at
+// j CHUNK + ((hz HY + hy) HX + hx) 16, CHUNK = 16 HX HY (zt + 2).  The A operand
+// of tap (dz, dy, dx) for plane p is then the descriptor whose start is the
+// halo voxel (1+dx, 1+dy, p+dz): its 8-row core matrices are 8 consecutive x
+// (16 bytes apart), the next 8 rows are the next y (SBO = 16 HX bytes), the
+// next 8 channels the next chunk (LBO = one chunk of the halo).  So the 27
+// taps need no data movement.  The weights come as bulk copies of an image
+// kept in shared-memory order: all groups' taps once a block (resident), or,
+// where they take too much room, a tap at a time through a ring.
+//
+// What bounds it: an MMA of M = 128, K = 16 takes 68 clocks whatever the layout
+// and N up to 128 when one thread issues them in a loop, 48 when an elected
+// thread issues unrolled taps, so a layer cannot take less than
+// 27 cin/16 x 48 clocks a 128 voxels.  To keep the MMAs back to back, blocks
+// stay for many tiles and their warps take roles: four load halos (hs stages),
+// one thread copies weights, two threads issue MMAs, four warps store results
+// (as accumulator stages), each waiting on mbarriers for the others.  128 x 64 x 128 voxels, us, with blocks that load,
+// multiply and store one tile after another, several an SM / this: 16 -> 16 77 /
+// 49, 48 -> 16 190 / 113; 32 -> 32 at half that size 34 / 20, 96 -> 32 125 / 65;
+// all of a forward's layers 755 / 415, of a gradient's (4 x 64 x 32 x 64) 627 /
+// 430.  Without the MMAs 16 -> 16 takes 30 and 48 -> 16 85: the halo copies (16
+// bytes a lane and instruction) bound the widest level, the MMAs the others.
+// Eight loader warps (62, 124) or a pair of lanes a voxel (53, 130) are slower.
+//
+// Each accumulator sees the same MMAs in the same order (groups, taps,
+// 16-channel steps) whatever the plan.  Every wait is bounded; on a time-out
+// the role sets *err and the block's failure flag and leaves, the others
+// follow, and the block still frees its tensor memory.
 // ---------------------------------------------------------------------------
 constexpr int TC_TX = 8, TC_TY = 16, TC_HX = 10, TC_HY = 18;
 constexpr int TC_PLANE = TC_HX * TC_HY * 16;  // bytes of one halo plane of one 8-channel chunk
 constexpr int TC_CG = 64;                     // channels per halo group
-constexpr int TC_STAGES = 3;
+constexpr int TC_RING = 8;                    // most weight stages
+constexpr int TC_THREADS = 352;               // 4 loader warps, 4 store warps, 2 MMA warps, weights
 
 // shared-memory matrix descriptor: no swizzle, K-major core matrices
 __device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
@@ -294,11 +307,10 @@ __host__ __device__ constexpr uint32_t tc_idesc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// bounded wait for phase `parity` of an mbarrier (about one second of
-// clock), polled with a short sleep between tries
+// bounded wait for phase `parity` of an mbarrier (about one second of clock)
 __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity) {
-  const long long t0 = clock64();
-  for (;;) {
+  long long t0 = 0;
+  for (int n = 0;; n++) {
     uint32_t done;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -306,247 +318,303 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity) {
         : "r"(mbar), "r"(parity)
         : "memory");
     if (done) return true;
+    if (n == 0) t0 = clock64();
     if (clock64() - t0 > 2000000000LL) return false;
-    __nanosleep(64);
+    if (n > 16) __nanosleep(40);
   }
 }
+// the same for a whole warp: one lane polls (the others would take its issue slots)
+__device__ __forceinline__ bool tc_wait_warp(uint32_t mbar, uint32_t parity) {
+  int ok = 1;
+  if ((threadIdx.x & 31) == 0) ok = tc_wait(mbar, parity);
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+__device__ __forceinline__ void tc_arrive(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint32_t mbar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
+}
+// bytes (a multiple of 16, at most 1 MB) global -> shared, completing on mbar
+__device__ __forceinline__ void tc_bulk(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+      "r"(bytes), "r"(mbar)
+      : "memory");
+}
 
-__global__ void __launch_bounds__(128) k_conv3_tc(Dims dm, const bf16* __restrict__ x, int ldx, int cin,
-                                                  const bf16* __restrict__ wt, const float* __restrict__ bias,
-                                                  int cout, bf16* __restrict__ y, int ldy, int relu,
-                                                  const bf16* __restrict__ mask, int ldm, int resident, int zt,
-                                                  const bf16* __restrict__ wimg, int* err) {
+// one thread of the (converged) warp, chosen in a form the compiler knows to be
+// warp-uniform: it then keeps descriptors in uniform registers
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred e;\n.reg .b32 t;\nelect.sync t|e, 0xffffffff;\nselp.u32 %0, 1, 0, e;\n}\n" : "=r"(e));
+  return e != 0;
+}
+// descriptors as words: only the low one, which holds the address, changes
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                       uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\n.reg .b64 da, db;\nmov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\nsetp.ne.b32 p, %6, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d),
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc));
+}
+// the MMAs of one tap of a group of 16 NK channels, NP planes (a_lo: the
+// first plane's halo): every offset but the tap's weights is a constant
+// (descriptor addresses count 16 bytes); ZT: planes of the halo
+template <int NK, int NP, int ZT>
+__device__ __forceinline__ void tc_tap(int tap, const uint32_t (&d)[NP], uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                       uint32_t b_hi, uint32_t idesc, bool first) {
+  constexpr int CH = TC_PLANE / 16 * (ZT + 2);
+  const uint32_t a_tap = a_lo + (uint32_t)(((tap / 9) * TC_HY + (tap / 3) % 3) * TC_HX + tap % 3);
+#pragma unroll
+  for (int pl = 0; pl < NP; pl++)
+#pragma unroll
+    for (int kk = 0; kk < NK; kk++)
+      tc_mma(d[pl], a_tap + (uint32_t)(pl * (TC_PLANE / 16) + 2 * kk * CH), a_hi, b_lo + 16u * kk, b_hi, idesc,
+             kk > 0 || !first ? 1u : 0u);
+}
+
+// how k_conv3_tc runs a layer
+struct TcPlan {
+  int zt;      // planes a tile
+  int hs;      // halo stages
+  int ring;    // weight stages, 0: resident
+  int as;      // accumulator stages
+  int cols;    // tensor-memory columns
+  int per_sm;  // blocks an SM
+  size_t smem;
+};
+
+template <int ZT>
+__global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __restrict__ x, int ldx, int cin,
+                                                         const bf16* __restrict__ wimg, const float* __restrict__ bias,
+                                                         int cout, bf16* __restrict__ y, int ldy, int relu,
+                                                         const bf16* __restrict__ mask, int ldm, TcPlan P, int* err) {
   extern __shared__ __align__(1024) uint8_t tsm[];
+  // mbarriers: halo full and empty, weight full and empty (resident: full[0]),
+  // accumulator full and empty
+  __shared__ __align__(8) uint64_t hfull[2], hempty[2], wfull[TC_RING], wempty[TC_RING], afull[2], aempty[2],
+      drain[2];
+  __shared__ uint32_t tslot;
+  __shared__ volatile int sfail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int cgmax = cin < TC_CG ? cin : TC_CG;  // channels of the widest group
-  const int stage_bytes = cout * cgmax * 2;     // one tap's weights of one group
-  const int hz_n = zt + 2;                      // halo planes
-  const int chunk = TC_PLANE * hz_n;            // bytes of one 8-channel chunk of the halo
-  uint8_t* halo = tsm;
-  uint8_t* wst = tsm + (cgmax / 8) * chunk;
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(wst + (resident ? 27 : TC_STAGES) * stage_bytes);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + TC_STAGES + 1);  // mbar[TC_STAGES]: the bulk weight copy
-  volatile int* sfail = reinterpret_cast<volatile int*>(tslot + 1);
-  // block -> tile
-  const int nxt = dm.w / TC_TX, nyt = dm.h / TC_TY;
-  long long b = blockIdx.x;
-  const int xt = (int)(b % nxt);
-  b /= nxt;
-  const int yt = (int)(b % nyt);
-  b /= nyt;
-  const int nzt = dm.d / zt;
-  const int z0 = (int)(b % nzt) * zt;
-  const long long nn = b / nzt;
-  const int x0 = xt * TC_TX, y0 = yt * TC_TY;
+  constexpr int zt = ZT, hz_n = zt + 2;
+  constexpr int NI = ZT > 1 ? 2 : 1, NP = ZT / NI;  // issuing threads, planes each
+  const int cgmax = cin < TC_CG ? cin : TC_CG;            // channels of the widest group
+  const uint32_t stage_bytes = (uint32_t)cout * cgmax * 2;  // one tap's weights of one group
+  constexpr uint32_t chunk = TC_PLANE * hz_n;             // bytes of one 8-channel chunk of the halo
+  const uint32_t halo_bytes = (cgmax / 8) * chunk;
+  const uint32_t halo0 = su32(tsm), w0 = halo0 + P.hs * halo_bytes;
+  const int ngroups = (cin + TC_CG - 1) / TC_CG;
+  const int nxt = dm.w / TC_TX, nyt = dm.h / TC_TY, nzt = dm.d / zt;
+  const int ntiles = nxt * nyt * nzt * dm.n;
   if (tid == 0) {
-    for (int s = 0; s <= TC_STAGES; s++) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(mbar + s)));
+    auto init = [](uint64_t* m, int count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(m)), "r"(count)); };
+    for (int i = 0; i < 2; i++) {
+      init(&hfull[i], 128);
+      init(&hempty[i], NI);
+      init(&afull[i], NI);
+      init(&aempty[i], 128);
+    }
+    for (int i = 0; i < TC_RING; i++) {
+      init(&wfull[i], 1);
+      init(&wempty[i], NI);
+    }
+    for (int i = 0; i < NI; i++) init(&drain[i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    *sfail = 0;
+    sfail = 0;
   }
-  int ncols = 32;
-  while (ncols < zt * cout) ncols <<= 1;
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(ncols));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(P.cols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tslot;
-  const int ngroups = (cin + TC_CG - 1) / TC_CG;
-  const int Q = ngroups * 27;
-  const uint32_t idesc = tc_idesc(128, cout);
-  // streaming: one tap's weights of channel group g into a ring stage
-  auto load_w = [&](int q) {
-    const int g = q / 27, t = q % 27;
-    const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
-    const uint32_t base = su32(wst + (q % TC_STAGES) * stage_bytes);
-    for (int o = tid; o < cout; o += 128) {
-      const bf16* src = wt + ((long long)t * cout + o) * cin + c0;
-      const uint32_t dst = base + (o / 8) * (nch * 128) + (o % 8) * 16;
-      for (int j = 0; j < nch; j++) cp16(dst + j * 128, src + 8 * j, true);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  const uint32_t tmem = tslot;
+  struct Tile {
+    int x0, y0, z0, n;
   };
-  // resident: every tap's weights of group g, (tap, row) pairs spread over the block
-  auto load_w_all = [&](int g) {
-    const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
-    const uint32_t base = su32(wst);
-    for (int i = tid; i < 27 * cout; i += 128) {
-      const int t = i / cout, o = i - t * cout;
-      const bf16* src = wt + ((long long)t * cout + o) * cin + c0;
-      const uint32_t dst = base + t * stage_bytes + (o / 8) * (nch * 128) + (o % 8) * 16;
-      for (int j = 0; j < nch; j++) cp16(dst + j * 128, src + 8 * j, true);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  // halo of group g: one voxel per thread, its chunks inner
-  auto load_halo = [&](int g) {
-    const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
-    const uint32_t base = su32(halo);
-    for (int i = tid; i < TC_HX * TC_HY * hz_n; i += 128) {
-      const int hx = i % TC_HX, hy = (i / TC_HX) % TC_HY, hz = i / (TC_HX * TC_HY);
-      int gx = x0 - 1 + hx, gy = y0 - 1 + hy;
-      const int gz = z0 - 1 + hz;
-      gx = gx < 0 ? gx + dm.w : (gx >= dm.w ? gx - dm.w : gx);
-      gy = gy < 0 ? gy + dm.h : (gy >= dm.h ? gy - dm.h : gy);
-      const bool in = gz >= 0 && gz < dm.d;
-      const long long v = ((nn * dm.d + (in ? gz : 0)) * dm.h + gy) * dm.w + gx;
-      const bf16* src = x + v * ldx + c0;
-      const uint32_t dst = base + i * 16;  // chunk 0 of voxel (hx, hy, hz); chunk j is `chunk` further
-      for (int j = 0; j < nch; j++) cp16(dst + j * chunk, src + 8 * j, in);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  // the MMAs of step q (group q / 27, tap q % 27) for every plane, with that
-  // tap's weights at b0; plane p accumulates in columns [p cout, (p+1) cout)
-  auto issue_tap = [&](int q, uint32_t b0) {
-    const int g = q / 27, t = q % 27;
-    const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
-    const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;  // halo offsets 0..2 (shift + 1)
-    const uint32_t a0 = su32(halo) + ((dz * TC_HY + dy) * TC_HX + dx) * 16;
-    for (int pl = 0; pl < zt; pl++) {
-      for (int kk = 0; kk < nch / 2; kk++) {
-        const uint64_t ad = tc_desc(a0 + pl * TC_PLANE + 2 * kk * chunk, chunk, TC_HX * 16);
-        const uint64_t bd = tc_desc(b0 + 2 * kk * 128, 128, nch * 128);
-        const uint32_t acc = (q > 0 || kk > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(pl * cout)),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-      }
-    }
-  };
-  auto commit = [&](int stage) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     su32(mbar + stage))
-                 : "memory");
-  };
-  // one thread polls the barrier, the others wait at __syncthreads (no issue
-  // slots spent spinning); false on a time-out
-  auto block_wait = [&](int stage, uint32_t parity) {
-    if (tid == 0 && !tc_wait(su32(mbar + stage), parity)) *sfail = 1;
-    __syncthreads();
-    return *sfail == 0;
+  auto tile_at = [&](int t) {
+    Tile r;
+    r.x0 = t % nxt * TC_TX;
+    t /= nxt;
+    r.y0 = t % nyt * TC_TY;
+    t /= nyt;
+    r.z0 = t % nzt * zt;
+    r.n = t / nzt;
+    return r;
   };
   bool ok = true;
-  if (resident) {
-    for (int g = 0; g < ngroups && ok; g++) {
-      if (wimg) {
-        // the group's 27 taps, pre-arranged in this layout, as one bulk copy
-        if (tid == 0) {
-          const uint32_t bytes = 27u * (uint32_t)stage_bytes;
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(mbar + TC_STAGES)),
-                       "r"(bytes)
-                       : "memory");
-          asm volatile(
-              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(su32(wst)),
-              "l"(wimg + (size_t)g * 27 * (stage_bytes / 2)), "r"(bytes), "r"(su32(mbar + TC_STAGES))
-              : "memory");
+  if (warp < 4) {
+    // halos, group by group, tile by tile: a warp takes three rows of ten
+    // voxels at a time, a lane a voxel, its chunks inner
+    const int hx = lane % TC_HX, hr = lane / TC_HX, rows = TC_HY * hz_n;
+    int use = 0;
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      const Tile T = tile_at(t);
+      int gx = T.x0 - 1 + hx;
+      gx = gx < 0 ? gx + dm.w : (gx >= dm.w ? gx - dm.w : gx);
+      for (int g = 0; g < ngroups; g++, use++) {
+        const int st = use % P.hs;
+        if (!(ok = tc_wait_warp(su32(&hempty[st]), ((use / P.hs) & 1) ^ 1))) break;
+        const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
+        const uint32_t base = halo0 + st * halo_bytes + 16 * hx;
+        const bf16* xg = x + (long long)gx * ldx + c0;
+        for (int row = warp * 3 + hr; row < rows; row += 12) {
+          if (hr == 3) break;
+          const int hz = row / TC_HY, hy = row - hz * TC_HY;
+          int gy = T.y0 - 1 + hy;
+          const int gz = T.z0 - 1 + hz;
+          gy = gy < 0 ? gy + dm.h : (gy >= dm.h ? gy - dm.h : gy);
+          const bool in = gz >= 0 && gz < dm.d;
+          const bf16* src = xg + voxel_at(dm, T.n, in ? gz : 0, gy, 0) * ldx;
+          const uint32_t dst = base + row * (16 * TC_HX);  // chunk 0; chunk j is `chunk` further
+          for (int j = 0; j < nch; j++) cp16(dst + j * chunk, src + 8 * j, in);
         }
-        load_halo(g);
-      } else {
-        load_halo(g);
-        load_w_all(g);
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tc_arrive(su32(&hfull[st]));
       }
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncthreads();
-      if (wimg && !block_wait(TC_STAGES, g & 1)) {
-        ok = false;
-        break;
-      }
-      if (tid == 0) {
-        for (int t = 0; t < 27; t++) issue_tap(g * 27 + t, su32(wst + t * stage_bytes));
-        commit(0);
-      }
-      if (g + 1 < ngroups && !block_wait(0, g & 1)) ok = false;  // the next group overwrites halo and weights
     }
-  } else {
-    load_halo(0);
-    load_w(0);
-    if (Q > 1) load_w(1);
-    for (int q = 0; q < Q; q++) {
-      const int g = q / 27, t = q % 27;
-      if (t == 0 && g > 0) {
-        // the previous group's MMAs read the halo: wait for the last of them
-        if (!block_wait((q - 1) % TC_STAGES, ((q - 1) / TC_STAGES) & 1)) {
-          ok = false;
-          break;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  } else if (warp < 8) {
+    // results: TMEM lane = output row (a warp reads the lanes of its quarter)
+    const int r = (warp - 4) * 32 + lane;
+    int it = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
+      const Tile T = tile_at(t);
+      const int st = it % P.as;
+      // (the warp stays together: TMEM loads are warp-wide)
+      if (!(ok = tc_wait_warp(su32(&afull[st]), (it / P.as) & 1))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      for (int pl = 0; pl < zt; pl++) {
+        const long long v = voxel_at(dm, T.n, T.z0 + pl, T.y0 + r / 8, T.x0 + (r % 8));
+        for (int c = 0; c < cout; c += 16) {
+          uint32_t a[16];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+              : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]),
+                "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15])
+              : "r"(tmem + ((uint32_t)((warp - 4) * 32) << 16) + (uint32_t)((st * zt + pl) * cout + c)));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          uint32_t o[8];
+#pragma unroll
+          for (int h = 0; h < 8; h++) {
+            float v0 = __uint_as_float(a[2 * h]), v1 = __uint_as_float(a[2 * h + 1]);
+            const int co = c + 2 * h;
+            if (bias) {
+              v0 += bias[co];
+              v1 += bias[co + 1];
+            }
+            if (relu) {
+              v0 = fmaxf(v0, 0.f);
+              v1 = fmaxf(v1, 0.f);
+            }
+            if (mask) {
+              const bf16* mp = mask + v * ldm + co;
+              if (!(__bfloat162float(mp[0]) > 0.f)) v0 = 0.f;
+              if (!(__bfloat162float(mp[1]) > 0.f)) v1 = 0.f;
+            }
+            o[h] = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+          }
+          // one 32-byte sector (rows and slices are 16 channels)
+          asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(y + v * ldy + c), "r"(o[0]),
+                       "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                       : "memory");
         }
-        load_halo(g);
       }
-      // this step's weights (and a new halo) have landed; the next step's may be in flight
-      if (t == 0 || q + 1 >= Q)
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-      else
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncthreads();
-      if (tid == 0) {
-        issue_tap(q, su32(wst + (q % TC_STAGES) * stage_bytes));
-        commit(q % TC_STAGES);
-      }
-      // refill the stage that step q-1 used with step q+2's weights
-      if (q + 2 < Q) {
-        if (q >= 1 && !block_wait((q - 1) % TC_STAGES, ((q - 1) / TC_STAGES) & 1)) {
-          ok = false;
-          break;
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      tc_arrive(su32(&aempty[st]));
+    }
+  } else if (warp < 8 + NI) {
+    // MMAs.  Issued from a loop with runtime counts by one plain lane they cost
+    // 300-500 clocks each in descriptor arithmetic, against about 50 this way:
+    // an elected thread, every tap unrolled; two threads share a tile's planes
+    // (an accumulator belongs to one of them).
+    if (tc_elect()) {
+      const int mw = warp - 8;
+      const uint32_t idesc = tc_idesc(128, cout);
+      int hst = 0, hph = 0, ws = 0, wph = 0, as = 0, aph = 0;
+      if (P.ring == 0) ok = tc_wait(su32(&wfull[0]), 0);
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        if (!(ok = tc_wait(su32(&aempty[as]), aph ^ 1))) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        uint32_t d[NP];
+#pragma unroll
+        for (int pl = 0; pl < NP; pl++) d[pl] = tmem + (uint32_t)((as * ZT + mw * NP + pl) * cout);
+        for (int g = 0; g < ngroups && ok; g++) {
+          if (!(ok = tc_wait(su32(&hfull[hst]), hph))) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const int nk = min(TC_CG, cin - g * TC_CG) / 16;
+          const uint64_t a_desc = tc_desc(halo0 + hst * halo_bytes + mw * NP * TC_PLANE, chunk, TC_HX * 16);
+          const uint64_t b_desc = tc_desc(w0 + (P.ring ? 0u : g * 27u * stage_bytes), 128, nk * 256);
+          const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32);
+          const uint32_t b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32), stage16 = stage_bytes >> 4;
+          auto group = [&](auto nkc) {
+            constexpr int NK = decltype(nkc)::value;
+            if (P.ring == 0) {
+#pragma unroll
+              for (int tap = 0; tap < 27; tap++)
+                tc_tap<NK, NP, ZT>(tap, d, a_lo, a_hi, b_lo + tap * stage16, b_hi, idesc, g == 0 && tap == 0);
+            } else {
+#pragma unroll 9
+              for (int tap = 0; tap < 27; tap++) {
+                if (!(ok = ok && tc_wait(su32(&wfull[ws]), wph))) continue;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tc_tap<NK, NP, ZT>(tap, d, a_lo, a_hi, b_lo + ws * stage16, b_hi, idesc, g == 0 && tap == 0);
+                tc_commit(su32(&wempty[ws]));
+                if (++ws == P.ring) ws = 0, wph ^= 1;
+              }
+            }
+          };
+          switch (nk) {
+            case 1: group(std::integral_constant<int, 1>{}); break;
+            case 2: group(std::integral_constant<int, 2>{}); break;
+            case 3: group(std::integral_constant<int, 3>{}); break;
+            default: group(std::integral_constant<int, 4>{});
+          }
+          tc_commit(su32(&hempty[hst]));
+          if (++hst == P.hs) hst = 0, hph ^= 1;
         }
-        load_w(q + 2);
+        tc_commit(su32(&afull[as]));
+        if (++as == P.as) as = 0, aph ^= 1;
+      }
+      // the block may not end with MMAs in flight: the store warps have awaited
+      // the last tiles' results; after a time-out they may have left
+      if (!ok || sfail) {
+        tc_commit(su32(&drain[mw]));
+        tc_wait(su32(&drain[mw]), 0);
+      }
+    }
+  } else if (warp == 10 && lane == 0) {
+    // weights
+    if (P.ring == 0) {
+      tc_bulk(w0, wimg, (uint32_t)ngroups * 27u * stage_bytes, su32(&wfull[0]));
+    } else {
+      int wuse = 0;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
+        for (int q = 0; q < ngroups * 27; q++, wuse++) {
+          const int ws = wuse % P.ring;
+          if (!(ok = tc_wait(su32(&wempty[ws]), ((wuse / P.ring) & 1) ^ 1))) break;
+          tc_bulk(w0 + ws * stage_bytes, reinterpret_cast<const uint8_t*>(wimg) + (size_t)q * stage_bytes, stage_bytes,
+                  su32(&wfull[ws]));
+        }
+      // copies still in flight land before the block ends
+      for (int r = 0; r < P.ring && r < wuse; r++) {
+        const int u = wuse - 1 - r;
+        if (!tc_wait(su32(&wfull[u % P.ring]), (u / P.ring) & 1)) ok = false;
       }
     }
   }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  // all MMAs done: the last commit covers every earlier one
-  __syncthreads();
-  const bool done = ok && *sfail == 0 &&
-                    (resident ? block_wait(0, (ngroups - 1) & 1)
-                              : block_wait((Q - 1) % TC_STAGES, ((Q - 1) / TC_STAGES) & 1));
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!done) {
-    if (tid == 0) atomicExch(err, 1);
-  } else {
-    const int r = warp * 32 + lane;  // TMEM lane = output row
-    for (int pl = 0; pl < zt; pl++) {
-      const long long v = ((nn * dm.d + z0 + pl) * dm.h + y0 + r / 8) * dm.w + x0 + (r % 8);
-      for (int c = 0; c < cout; c += 16) {
-        uint32_t a[16];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]),
-              "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15])
-            : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(pl * cout + c)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        uint32_t o[8];
-#pragma unroll
-        for (int h = 0; h < 8; h++) {
-          float v0 = __uint_as_float(a[2 * h]), v1 = __uint_as_float(a[2 * h + 1]);
-          const int co = c + 2 * h;
-          if (bias) {
-            v0 += bias[co];
-            v1 += bias[co + 1];
-          }
-          if (relu) {
-            v0 = fmaxf(v0, 0.f);
-            v1 = fmaxf(v1, 0.f);
-          }
-          if (mask) {
-            const bf16* mp = mask + v * ldm + co;
-            if (!(__bfloat162float(mp[0]) > 0.f)) v0 = 0.f;
-            if (!(__bfloat162float(mp[1]) > 0.f)) v1 = 0.f;
-          }
-          o[h] = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
-        }
-        uint4* yp = reinterpret_cast<uint4*>(y + v * ldy + c);
-        yp[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        yp[1] = make_uint4(o[4], o[5], o[6], o[7]);
-      }
-    }
+  if (!ok) {
+    sfail = 1;
+    atomicExch(err, 1);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(P.cols));
 }
 
 // First layer: 1 input channel (FP32 input rounded to BF16) -> 16 channels,
@@ -691,7 +759,7 @@ __global__ void k_conv_out_bwd(long long V, const float* __restrict__ gy, const 
 // are one conflict-free ldmatrix row set.
 // A tap at a time from global memory (the kernel this replaces) read both
 // operands 27 times in 2-byte loads: 3.8 ms of a 6.2 ms gradient of 4 x 64 x
-// 32 x 64; the figures now stand at wgrad3.
+// 32 x 64, where this takes 0.41 and the sums 0.14.
 // ---------------------------------------------------------------------------
 constexpr int WG_TX = 8, WG_TY = 8, WG_TZ = 4, WG_VOX = WG_TX * WG_TY * WG_TZ;
 constexpr int WG_HX = WG_TX + 2, WG_HY = WG_TY + 2, WG_HZ = WG_TZ + 2, WG_HVOX = WG_HX * WG_HY * WG_HZ;
@@ -1059,9 +1127,9 @@ __global__ void k_pack_weights(const float* __restrict__ w, int cout, int cin, b
   }
 }
 
-// wt [t][cout][cin] (BF16) -> the resident weights of k_conv3_tc exactly as
-// its shared memory holds them, so that a block loads a channel group's 27
-// taps with one bulk copy: for group g (64 channels), tap t, output o and
+// wt [t][cout][cin] (BF16) -> the weights of k_conv3_tc exactly as its shared
+// memory holds them, so that a block loads them, or a tap of them, with one
+// bulk copy: for group g (64 channels), tap t, output o and
 // 8-channel chunk j, 16 bytes at g 27 S + t S + (o/8)(nch 128) + (o%8) 16 +
 // j 128, with S = 2 cout min(cin, 64) bytes a tap and nch the group's chunks
 __global__ void k_pack_image(const bf16* __restrict__ wt, int cin, int cout, bf16* __restrict__ img) {
@@ -1180,8 +1248,7 @@ struct Layer {
   int cin, cout, taps;
   long long woff, boff;  // offsets of W and b in the flat parameter vector
   bf16 *wt = nullptr, *wtt = nullptr;
-  // wt and wtt in the shared-memory order of k_conv3_tc's resident weights
-  // (null where that convolution does not run with resident weights)
+  // wt and wtt in the shared-memory order of k_conv3_tc
   bf16 *img = nullptr, *timg = nullptr;
 };
 
@@ -1250,57 +1317,68 @@ int ualloc(stp_unet* n, T** p, size_t count) {
 // concat widths: decoder level l (0..2) input = kCh[l+1] + kCh[l]
 int cu_width(int l) { return kCh[l + 1] + kCh[l]; }
 
-// shared memory of k_conv3_tc with zt planes a block: the halo of the
-// widest channel group, then the weights (all 27 taps of a group when
-// resident, else three stages)
-size_t conv3_tc_smem(int cin, int cout, bool resident, int zt) {
+constexpr size_t kTcSmemMax = 200 * 1024;  // of the mma.sync convolution
+constexpr size_t kTcSmemSm = 226 * 1024;   // of an SM's blocks of k_conv3_tc
+
+// weights image of k_conv3_tc, elements
+size_t tc_image_elems(int cin, int cout) {
+  return (size_t)((cin + TC_CG - 1) / TC_CG) * 27 * cout * std::min(cin, TC_CG);
+}
+
+// How k_conv3_tc runs a layer; false if it does not take it.  Weights resident
+// up to 64 KB, else a ring of 64 KB.  Two halo stages and two accumulator
+// stages where shared memory (half an SM's, or a whole one's) and 512 columns
+// take them; planes a tile 4, 2 or 1, the most that leave two tiles an SM
+// (planes share halo planes: 6 loaded for 4 computed).  A forced count
+// (STP_UNET_TC_PLANES: 1, 2 or 4) is halved until it fits.
+bool tc_plan(const stp_unet* n, const Dims& dm, int cin, int cout, TcPlan* out) {
   const int cg = std::min(cin, TC_CG);
-  return (size_t)(cg / 8) * TC_PLANE * (zt + 2) + (size_t)(resident ? 27 : TC_STAGES) * cout * cg * 2 + 64;
-}
-constexpr size_t kTcSmemMax = 200 * 1024;
-
-bool conv3_tc_ok(const stp_unet* n, const Dims& dm, int ldx, int cin, int cout, int ldy) {
-  return n->use_tc && dm.w % TC_TX == 0 && dm.h % TC_TY == 0 && cin % 16 == 0 && cout % 16 == 0 && cout <= 256 &&
-         ldx % 8 == 0 && ldy % 8 == 0 && conv3_tc_smem(cin, cout, false, 1) <= kTcSmemMax;
-}
-
-// planes a block of k_conv3_tc computes (measured on GB300 over the
-// network's layer shapes): 4 when the block stays within 64 KB of shared
-// memory (four blocks an SM) and the layer still has 1024 blocks; else 2
-// when it fits and leaves 512 blocks; else 1.  Always a divisor of the depth,
-// accumulators within 128 tensor-memory columns, and resident weights.  A
-// forced count (STP_UNET_TC_PLANES: 1, 2 or 4) is halved until it is valid.
-int conv3_tc_planes(const stp_unet* n, const Dims& dm, int cin, int cout, bool resident) {
-  if (!resident) return 1;
+  const size_t tap = (size_t)2 * cout * cg;
+  const size_t res = (size_t)((cin + TC_CG - 1) / TC_CG) * 27 * tap;
   const long long tiles = dm.vox() / (TC_TX * TC_TY);
-  auto fits = [&](int zt, size_t smem_max, long long min_blocks) {
-    return dm.d % zt == 0 && zt * cout <= 128 && conv3_tc_smem(cin, cout, true, zt) <= smem_max &&
-           tiles / zt >= min_blocks;
-  };
-  if (n->tc_planes == 1 || n->tc_planes == 2 || n->tc_planes == 4) {
-    for (int zt = n->tc_planes; zt > 1; zt /= 2)
-      if (fits(zt, kTcSmemMax, 1)) return zt;
-    return 1;
+  const bool forced = n->tc_planes == 1 || n->tc_planes == 2 || n->tc_planes == 4;
+  for (int q = 0; q < 6; q++) {
+    // two halo stages with the most planes, else one
+    TcPlan p;
+    p.hs = q < 3 ? 2 : 1;
+    const int zt = p.zt = 4 >> (q % 3);
+    if (forced && zt > n->tc_planes) continue;
+    if (dm.d % zt || zt * cout > 256) continue;
+    if (!forced && zt > 1 && tiles / zt < 2 * 152) continue;
+    p.ring = res <= 64 * 1024 ? 0 : (int)std::min<size_t>(TC_RING, std::max<size_t>(2, 64 * 1024 / tap));
+    p.as = 2 * zt * cout <= 256 ? 2 : 1;
+    p.cols = 32;
+    while (p.cols < p.as * zt * cout) p.cols *= 2;
+    const size_t halo = (size_t)(cg / 8) * TC_PLANE * (zt + 2), w = p.ring ? p.ring * tap : res;
+    p.smem = p.hs * halo + w;
+    if (p.smem > kTcSmemSm) continue;
+    p.per_sm = p.smem <= kTcSmemSm / 2 - 2048 && 2 * p.cols <= 512 ? 2 : 1;
+    *out = p;
+    return true;
   }
-  if (fits(4, 64 * 1024, 1024)) return 4;
-  if (fits(2, kTcSmemMax, 512)) return 2;
-  return 1;
+  return false;
+}
+
+bool conv3_tc_ok(const stp_unet* n, const Dims& dm, int ldx, int cin, int cout, int ldy, TcPlan* p) {
+  return n->use_tc && dm.w % TC_TX == 0 && dm.h % TC_TY == 0 && cin % 16 == 0 && cout % 16 == 0 && cout <= 256 &&
+         ldx % 8 == 0 && ldy % 16 == 0 && tc_plan(n, dm, cin, cout, p);
 }
 
 // launch a 3x3x3 convolution (forward form): tcgen05 where the shapes allow, else mma.sync
 int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf16* wt, const bf16* wimg,
           const float* bias, int cout, bf16* y, int ldy, int relu, const bf16* mask, int ldm) {
   const long long V = dm.vox();
-  if (conv3_tc_ok(n, dm, ldx, cin, cout, ldy)) {
-    static std::atomic<unsigned> done{0u};
-    UTRY(n, smem_limit_once(k_conv3_tc, (int)kTcSmemMax, done));
-    const bool resident = conv3_tc_smem(cin, cout, true, 1) <= kTcSmemMax;
-    const int zt = conv3_tc_planes(n, dm, cin, cout, resident);
-    const unsigned blocks = (unsigned)(V / (TC_TX * TC_TY * zt));
-    k_conv3_tc<<<blocks, 128, conv3_tc_smem(cin, cout, resident, zt), n->st>>>(
-        dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask, ldm, resident ? 1 : 0, zt, resident ? wimg : nullptr,
-        n->d_err);
-    UTRY(n, cudaGetLastError());
+  TcPlan p;
+  if (conv3_tc_ok(n, dm, ldx, cin, cout, ldy, &p)) {
+    const unsigned tiles = (unsigned)(V / (TC_TX * TC_TY * p.zt));
+    auto go = [&](auto kern, std::atomic<unsigned>& done) -> cudaError_t {
+      if (cudaError_t e = smem_limit_once(kern, (int)kTcSmemSm, done)) return e;
+      kern<<<std::min(tiles, 152u * p.per_sm), TC_THREADS, p.smem, n->st>>>(dm, x, ldx, cin, wimg, bias, cout, y, ldy, relu,
+                                                                           mask, ldm, p, n->d_err);
+      return cudaGetLastError();
+    };
+    static std::atomic<unsigned> done1{0u}, done2{0u}, done4{0u};
+    UTRY(n, p.zt == 4 ? go(k_conv3_tc<4>, done4) : p.zt == 2 ? go(k_conv3_tc<2>, done2) : go(k_conv3_tc<1>, done1));
     return STP_OK;
   }
   // output channels a block: 32, 16 or 8, the widest that still gives 100
@@ -1382,8 +1460,8 @@ int pack_all(stp_unet* n) {
     const long long tot = (long long)ly.cout * ly.cin * 27;
     k_pack_weights<<<blocks_for(tot), 256, 0, n->st>>>(n->theta + ly.woff, ly.cout, ly.cin, ly.wt, ly.wtt);
     UTRY(n, cudaGetLastError());
-    if (ly.img) k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wt, ly.cin, ly.cout, ly.img);
-    if (ly.timg) k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wtt, ly.cout, ly.cin, ly.timg);
+    k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wt, ly.cin, ly.cout, ly.img);
+    k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wtt, ly.cout, ly.cin, ly.timg);
     UTRY(n, cudaGetLastError());
   }
   return STP_OK;
@@ -1608,18 +1686,12 @@ int stp_unet_create(int nmax, int nz, int ny, int nx, void* stream, stp_unet** o
   A(&n->grad, n->np);
   A(&n->m, n->np);
   A(&n->v, n->np);
-  // elements of the resident-weight image of a convolution cin -> cout, 0
-  // where k_conv3_tc would stream its weights (or not run at all)
-  auto image_elems = [](int ci, int co) -> size_t {
-    if (ci % 16 || co % 16 || co > 256 || conv3_tc_smem(ci, co, true, 1) > kTcSmemMax) return 0;
-    return (size_t)((ci + TC_CG - 1) / TC_CG) * 27 * co * std::min(ci, TC_CG);
-  };
   for (Layer& ly : n->L) {
     if (ly.taps == 27 && ly.cin > 1) {
       A(&ly.wt, (size_t)ly.cout * ly.cin * 27);
       A(&ly.wtt, (size_t)ly.cout * ly.cin * 27);
-      if (const size_t e = image_elems(ly.cin, ly.cout)) A(&ly.img, e);
-      if (const size_t e = image_elems(ly.cout, ly.cin)) A(&ly.timg, e);
+      A(&ly.img, tc_image_elems(ly.cin, ly.cout));
+      A(&ly.timg, tc_image_elems(ly.cout, ly.cin));
     }
   }
   const long long V[4] = {n->dm[0].vox(), n->dm[1].vox(), n->dm[2].vox(), n->dm[3].vox()};
