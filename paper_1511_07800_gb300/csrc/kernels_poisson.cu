@@ -56,9 +56,8 @@ __global__ void __launch_bounds__(kBX* kBY) k_sweep_f32(Geom<float> g, const flo
   }
 }
 
-// Vectorised sweeps: each thread owns 4 consecutive cells of a row (float4
-// in FP32, double2 pairs in FP64); the x-neighbours across lanes come by
-// warp shuffle, so a cell costs one vector load per stencil direction
+// Vectorised FP32 sweeps: each thread owns 4 consecutive cells of a row (a
+// float4); the x-neighbours across lanes come by warp shuffle, so a cell costs one vector load per stencil direction
 // instead of eight scalar loads and their index arithmetic.  Lanes past the
 // end of a row (or rows past ny) read a clamped, in-bounds element, take
 // part in the shuffles and store nothing.  Launched as programmatic
@@ -471,8 +470,8 @@ __global__ void __launch_bounds__(512) k_line_sweep_smem(Geom<T> g, const T* __r
   }
 }
 
-// The shared-memory line sweep with phases 1 and 3 on vector units (float4
-// in FP32, double2 in FP64) of VW consecutive x cells: a thread handles one
+// The shared-memory line sweep with phases 1 and 3 on vector units (float4)
+// of VW consecutive x cells: a thread handles one
 // unit of one row over a chunk of levels, with vector loads of the centre,
 // y and z neighbours and b, and scalar loads of the two x neighbours just
 // outside the unit.  For nx a multiple of the vector width (aligned
@@ -488,15 +487,6 @@ struct VecOf<float> {
   __device__ static float get(const float4& v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
   __device__ static void set(float4& v, int e, float x) {
     if (e == 0) v.x = x; else if (e == 1) v.y = x; else if (e == 2) v.z = x; else v.w = x;
-  }
-};
-template <>
-struct VecOf<double> {
-  using V = double2;
-  static constexpr int W = 2;
-  __device__ static double get(const double2& v, int e) { return e == 0 ? v.x : v.y; }
-  __device__ static void set(double2& v, int e, double x) {
-    if (e == 0) v.x = x; else v.y = x;
   }
 };
 
