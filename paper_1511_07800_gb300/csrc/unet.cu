@@ -268,8 +268,8 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
 // (16 bytes apart), the next 8 rows are the next y (SBO = 16 HX bytes), the
 // next 8 channels the next chunk (LBO = one chunk of the halo).  So the 27
 // taps need no data movement.  The weights come as bulk copies of an image
-// kept in shared-memory order: all groups' taps once a block (resident), or,
-// where they take too much room, a tap at a time through a ring.
+// kept in shared-memory order, a tap at a time through a ring: this kernel takes
+// the layers whose weights do not fit an SM (64 -> 64, 192 -> 64 and back).
 //
 // What bounds it: an MMA of M = 128, K = 16 takes 68 clocks whatever the layout
 // and N up to 128 when one thread issues them in a loop, 48 when an elected
@@ -375,11 +375,78 @@ __device__ __forceinline__ void tc_tap(int tap, const uint32_t (&d)[NP], uint32_
              kk > 0 || !first ? 1u : 0u);
 }
 
+__device__ __forceinline__ void tc_ld16(uint32_t* a, uint32_t col) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]),
+        "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15])
+      : "r"(col));
+}
+// bias (in shared memory, zeros if none), ReLU or mask, BF16 rounding and store
+// of 16 channels of a voxel
+__device__ __forceinline__ void tc_store16(const uint32_t* a, const float* bias, int relu, const bf16* mask, bf16* y) {
+  float v[16];
+#pragma unroll
+  for (int h = 0; h < 4; h++) {
+    const float4 bv = reinterpret_cast<const float4*>(bias)[h];
+    v[4 * h] = __uint_as_float(a[4 * h]) + bv.x;
+    v[4 * h + 1] = __uint_as_float(a[4 * h + 1]) + bv.y;
+    v[4 * h + 2] = __uint_as_float(a[4 * h + 2]) + bv.z;
+    v[4 * h + 3] = __uint_as_float(a[4 * h + 3]) + bv.w;
+  }
+  if (relu)
+#pragma unroll
+    for (int h = 0; h < 16; h++) v[h] = fmaxf(v[h], 0.f);
+  if (mask) {
+    float m[16];
+    unpack8(ld16(mask), m);
+    unpack8(ld16(mask + 8), m + 8);
+#pragma unroll
+    for (int h = 0; h < 16; h++) v[h] = m[h] > 0.f ? v[h] : 0.f;
+  }
+  uint32_t o[8];
+#pragma unroll
+  for (int h = 0; h < 8; h++) o[h] = pack2(__float2bfloat16(v[2 * h]), __float2bfloat16(v[2 * h + 1]));
+  // one 32-byte sector (rows and slices are 16 channels)
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(y), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+               "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+               : "memory");
+}
+// results of a tile: planes of cout columns from tensor-memory column acc, for
+// the voxel v of the first plane, planes vz voxels apart; 32 columns a wait (16
+// a wait with scalar reads of the bias and the mask took 0.4 us each)
+__device__ __forceinline__ void tc_store(uint32_t acc, long long v, long long vz, int planes, const float* bias,
+                                         int cout, bf16* __restrict__ y, int ldy, int relu,
+                                         const bf16* __restrict__ mask, int ldm) {
+  const int n = planes * cout;
+  int c = 0;
+  const bf16* mp = mask ? mask + v * ldm : nullptr;
+  bf16* yp = y + v * ldy;
+  const long long my = vz * ldm, yy = vz * ldy;
+  for (int i = 0; i < n; i += 32) {
+    uint32_t a[32];
+    const bool two = i + 16 < n;
+    tc_ld16(a, acc + i);
+    if (two) tc_ld16(a + 16, acc + i + 16);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      if (h == 1 && !two) break;
+      tc_store16(a + 16 * h, bias + c, relu, mp ? mp + c : nullptr, yp + c);
+      if ((c += 16) == cout) {
+        c = 0;
+        yp += yy;
+        if (mp) mp += my;
+      }
+    }
+  }
+}
+
 // how k_conv3_tc runs a layer
 struct TcPlan {
   int zt;      // planes a tile
   int hs;      // halo stages
-  int ring;    // weight stages, 0: resident
+  int ring;    // weight stages
   int as;      // accumulator stages
   int cols;    // tensor-memory columns
   int per_sm;  // blocks an SM
@@ -392,12 +459,13 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
                                                          int cout, bf16* __restrict__ y, int ldy, int relu,
                                                          const bf16* __restrict__ mask, int ldm, TcPlan P, int* err) {
   extern __shared__ __align__(1024) uint8_t tsm[];
-  // mbarriers: halo full and empty, weight full and empty (resident: full[0]),
-  // accumulator full and empty
+  // mbarriers: halo full and empty, weight full and empty, accumulator full and
+  // empty
   __shared__ __align__(8) uint64_t hfull[2], hempty[2], wfull[TC_RING], wempty[TC_RING], afull[2], aempty[2],
       drain[2];
   __shared__ uint32_t tslot;
   __shared__ volatile int sfail;
+  __shared__ __align__(16) float sbias[256];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int zt = ZT, hz_n = zt + 2;
   constexpr int NI = ZT > 1 ? 2 : 1, NP = ZT / NI;  // issuing threads, planes each
@@ -425,6 +493,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sfail = 0;
   }
+  for (int i = tid; i < cout; i += blockDim.x) sbias[i] = bias ? bias[i] : 0.f;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(P.cols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -489,42 +558,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
       // (the warp stays together: TMEM loads are warp-wide)
       if (!(ok = tc_wait_warp(su32(&afull[st]), (it / P.as) & 1))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int pl = 0; pl < zt; pl++) {
-        const long long v = voxel_at(dm, T.n, T.z0 + pl, T.y0 + r / 8, T.x0 + (r % 8));
-        for (int c = 0; c < cout; c += 16) {
-          uint32_t a[16];
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]),
-                "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15])
-              : "r"(tmem + ((uint32_t)((warp - 4) * 32) << 16) + (uint32_t)((st * zt + pl) * cout + c)));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          uint32_t o[8];
-#pragma unroll
-          for (int h = 0; h < 8; h++) {
-            float v0 = __uint_as_float(a[2 * h]), v1 = __uint_as_float(a[2 * h + 1]);
-            const int co = c + 2 * h;
-            if (bias) {
-              v0 += bias[co];
-              v1 += bias[co + 1];
-            }
-            if (relu) {
-              v0 = fmaxf(v0, 0.f);
-              v1 = fmaxf(v1, 0.f);
-            }
-            if (mask) {
-              const bf16* mp = mask + v * ldm + co;
-              if (!(__bfloat162float(mp[0]) > 0.f)) v0 = 0.f;
-              if (!(__bfloat162float(mp[1]) > 0.f)) v1 = 0.f;
-            }
-            o[h] = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
-          }
-          // one 32-byte sector (rows and slices are 16 channels)
-          asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(y + v * ldy + c), "r"(o[0]),
-                       "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
-                       : "memory");
-        }
-      }
+      tc_store(tmem + ((uint32_t)((warp - 4) * 32) << 16) + (uint32_t)(st * zt * cout),
+               voxel_at(dm, T.n, T.z0, T.y0 + r / 8, T.x0 + (r % 8)), (long long)dm.h * dm.w, zt, sbias, cout, y, ldy,
+               relu, mask, ldm);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       tc_arrive(su32(&aempty[st]));
     }
@@ -537,7 +573,6 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
       const int mw = warp - 8;
       const uint32_t idesc = tc_idesc(128, cout);
       int hst = 0, hph = 0, ws = 0, wph = 0, as = 0, aph = 0;
-      if (P.ring == 0) ok = tc_wait(su32(&wfull[0]), 0);
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         if (!(ok = tc_wait(su32(&aempty[as]), aph ^ 1))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -549,24 +584,18 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const int nk = min(TC_CG, cin - g * TC_CG) / 16;
           const uint64_t a_desc = tc_desc(halo0 + hst * halo_bytes + mw * NP * TC_PLANE, chunk, TC_HX * 16);
-          const uint64_t b_desc = tc_desc(w0 + (P.ring ? 0u : g * 27u * stage_bytes), 128, nk * 256);
+          const uint64_t b_desc = tc_desc(w0, 128, nk * 256);
           const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32);
           const uint32_t b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32), stage16 = stage_bytes >> 4;
           auto group = [&](auto nkc) {
             constexpr int NK = decltype(nkc)::value;
-            if (P.ring == 0) {
-#pragma unroll
-              for (int tap = 0; tap < 27; tap++)
-                tc_tap<NK, NP, ZT>(tap, d, a_lo, a_hi, b_lo + tap * stage16, b_hi, idesc, g == 0 && tap == 0);
-            } else {
 #pragma unroll 9
-              for (int tap = 0; tap < 27; tap++) {
-                if (!(ok = ok && tc_wait(su32(&wfull[ws]), wph))) continue;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                tc_tap<NK, NP, ZT>(tap, d, a_lo, a_hi, b_lo + ws * stage16, b_hi, idesc, g == 0 && tap == 0);
-                tc_commit(su32(&wempty[ws]));
-                if (++ws == P.ring) ws = 0, wph ^= 1;
-              }
+            for (int tap = 0; tap < 27; tap++) {
+              if (!(ok = ok && tc_wait(su32(&wfull[ws]), wph))) continue;
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              tc_tap<NK, NP, ZT>(tap, d, a_lo, a_hi, b_lo + ws * stage16, b_hi, idesc, g == 0 && tap == 0);
+              tc_commit(su32(&wempty[ws]));
+              if (++ws == P.ring) ws = 0, wph ^= 1;
             }
           };
           switch (nk) {
@@ -590,23 +619,266 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
     }
   } else if (warp == 10 && lane == 0) {
     // weights
-    if (P.ring == 0) {
-      tc_bulk(w0, wimg, (uint32_t)ngroups * 27u * stage_bytes, su32(&wfull[0]));
-    } else {
-      int wuse = 0;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
-        for (int q = 0; q < ngroups * 27; q++, wuse++) {
-          const int ws = wuse % P.ring;
-          if (!(ok = tc_wait(su32(&wempty[ws]), ((wuse / P.ring) & 1) ^ 1))) break;
-          tc_bulk(w0 + ws * stage_bytes, reinterpret_cast<const uint8_t*>(wimg) + (size_t)q * stage_bytes, stage_bytes,
-                  su32(&wfull[ws]));
-        }
-      // copies still in flight land before the block ends
-      for (int r = 0; r < P.ring && r < wuse; r++) {
-        const int u = wuse - 1 - r;
-        if (!tc_wait(su32(&wfull[u % P.ring]), (u / P.ring) & 1)) ok = false;
+    int wuse = 0;
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
+      for (int q = 0; q < ngroups * 27; q++, wuse++) {
+        const int ws = wuse % P.ring;
+        if (!(ok = tc_wait(su32(&wempty[ws]), ((wuse / P.ring) & 1) ^ 1))) break;
+        tc_bulk(w0 + ws * stage_bytes, reinterpret_cast<const uint8_t*>(wimg) + (size_t)q * stage_bytes, stage_bytes,
+                su32(&wfull[ws]));
+      }
+    // copies still in flight land before the block ends
+    for (int r = 0; r < P.ring && r < wuse; r++) {
+      const int u = wuse - 1 - r;
+      if (!tc_wait(su32(&wfull[u % P.ring]), (u / P.ring) & 1)) ok = false;
+    }
+  }
+  if (!ok) {
+    sfail = 1;
+    atomicExch(err, 1);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(P.cols));
+}
+
+// The same with resident weights, for layers whose weights fit beside two halo
+// planes.  The A operand of an MMA is read from shared memory at 128 x 32 bytes,
+// about 48 clocks, whatever N up to 128; with N = 16 or 32 output channels the
+// multiply itself would take a quarter of that.  So a plane of the input is read
+// once for the three output planes it contributes to: accumulators of a tile's
+// planes lie side by side in tensor memory, input plane q (from -1) reaches
+// output planes q-1, q, q+1 through z taps 2, 1, 0, and the weights of a (y, x)
+// tap are stacked in that order, so one MMA of N = 3 cout does all three.  An
+// output plane's first product, which must not add, is an MMA of its own.
+// Planes q = -1 and q = zt reach one output plane, their neighbours two.  9
+// (zt + 2) MMAs of 16 channels a tile of zt planes instead of 27 zt.
+//
+// The halo is loaded plane by plane (10 x 18 voxels, up to 64 channels) into a
+// ring, a loader warp a plane, each with one plane landing while it issues the
+// next; no plane is loaded twice in a tile.  Accumulators see the same MMAs in
+// the same order (groups, z, y, x taps, 16-channel steps) as in k_conv3_tc.
+// us at 128 x 64 x 128, a tap at a time (k_conv3_tc with resident weights) /
+// this: 16 -> 16 49 / 38, 48 -> 16 113 / 70; half that size 16 -> 32 20 / 16, 32
+// -> 32 21 / 19, 96 -> 32 65 / 46; a quarter 32 -> 64 17 / 9.5.  16 -> 16 takes
+// 26 without MMAs and stores, 16 with no loads either: what bounds it is what a
+// plane costs its MMA thread (wait, descriptors, commit: some 0.2 us) and the
+// first loads and last stores of a block.  Three blocks an SM (64 registers) 39.
+struct TzPlan {
+  int zt;      // planes a tile
+  int hs;      // halo stages (planes)
+  int as;      // accumulator stages
+  int cols;    // tensor-memory columns
+  int per_sm;  // blocks an SM
+  size_t smem;
+};
+constexpr int TZ_HALO = 8;       // most halo stages
+constexpr int TZ_GROUPS = 4;     // most channel groups
+constexpr int TZ_THREADS = 320;  // 4 loader warps, 4 store warps, MMA, weights
+
+// the MMAs of one input plane and group of 16 NK channels: d, idesc, b_lo are
+// those of all output planes it reaches; with `fresh` the last of them (idesc1,
+// at column offset d1 and weight offset b1; the others are idesc0, none if 0)
+// starts here
+template <int NK>
+__device__ __forceinline__ void tz_plane(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                         uint32_t tap16, uint32_t idesc, bool fresh, uint32_t idesc0, uint32_t idesc1,
+                                         uint32_t d1, uint32_t b1) {
+  constexpr uint32_t CH = TC_PLANE / 16;
+#pragma unroll
+  for (int tap = 0; tap < 9; tap++)
+#pragma unroll
+    for (int kk = 0; kk < NK; kk++) {
+      const uint32_t a = a_lo + (uint32_t)(tap / 3 * TC_HX + tap % 3 + 2 * kk * (int)CH);
+      const uint32_t b = b_lo + tap * tap16 + 16u * kk;
+      if (tap == 0 && kk == 0 && fresh) {
+        if (idesc0) tc_mma(d, a, a_hi, b, b_hi, idesc0, 1u);
+        tc_mma(d + d1, a, a_hi, b + b1, b_hi, idesc1, 0u);
+      } else {
+        tc_mma(d, a, a_hi, b, b_hi, idesc, 1u);
       }
     }
+}
+
+__global__ void __launch_bounds__(TZ_THREADS) k_conv3_tz(Dims dm, const bf16* __restrict__ x, int ldx, int cin,
+                                                         const bf16* __restrict__ wimg, const float* __restrict__ bias,
+                                                         int cout, bf16* __restrict__ y, int ldy, int relu,
+                                                         const bf16* __restrict__ mask, int ldm, TzPlan P, int* err) {
+  extern __shared__ __align__(1024) uint8_t tsm[];
+  __shared__ __align__(8) uint64_t hfull[TZ_HALO], hempty[TZ_HALO], wfull[TZ_GROUPS], afull[2], aempty[2], drain;
+  __shared__ uint32_t tslot;
+  __shared__ volatile int sfail;
+  __shared__ __align__(16) float sbias[256];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, zt = P.zt;
+  const uint32_t plane_bytes = (uint32_t)(min(cin, TC_CG) / 8) * TC_PLANE;
+  const uint32_t halo0 = su32(tsm), w0 = halo0 + P.hs * plane_bytes;
+  const int ngroups = (cin + TC_CG - 1) / TC_CG;
+  const int nxt = dm.w / TC_TX, nyt = dm.h / TC_TY, nzt = dm.d / zt;
+  const int ntiles = nxt * nyt * nzt * dm.n;
+  if (tid == 0) {
+    auto init = [](uint64_t* m, int count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(m)), "r"(count)); };
+    for (int i = 0; i < TZ_HALO; i++) {
+      init(&hfull[i], 32);
+      init(&hempty[i], 1);
+    }
+    for (int i = 0; i < TZ_GROUPS; i++) init(&wfull[i], 1);
+    for (int i = 0; i < 2; i++) {
+      init(&afull[i], 1);
+      init(&aempty[i], 128);
+    }
+    init(&drain, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    sfail = 0;
+  }
+  for (int i = tid; i < cout; i += blockDim.x) sbias[i] = bias ? bias[i] : 0.f;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(P.cols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tslot;
+  struct Tile {
+    int x0, y0, z0, n;
+  };
+  auto tile_at = [&](int t) {
+    Tile r;
+    r.x0 = t % nxt * TC_TX;
+    t /= nxt;
+    r.y0 = t % nyt * TC_TY;
+    t /= nyt;
+    r.z0 = t % nzt * zt;
+    r.n = t / nzt;
+    return r;
+  };
+  bool ok = true;
+  if (warp < 4) {
+    // halo planes: unit u (tile by tile, group by group, plane by plane) belongs
+    // to warp u mod nl; three rows of ten voxels at a time, a lane a voxel, its
+    // chunks inner.  No more warps than stages: a warp that waits for unit u then
+    // knows unit u - 2 hs consumed, so the phase it waits for is unambiguous.  A
+    // plane is handed over once the warp's next one is issued (`lag`), which needs
+    // more stages than warps: the next one's stage must not be waiting for this
+    // plane.
+    const int hx = lane % TC_HX, hr = lane / TC_HX;
+    const int nl = min(4, P.hs);
+    const bool lag = P.hs > nl;
+    int u = 0, pending = -1;
+    auto hand_over = [&]() {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc_arrive(su32(&hfull[pending]));
+    };
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      const Tile T = tile_at(t);
+      int gx = T.x0 - 1 + hx;
+      gx = gx < 0 ? gx + dm.w : (gx >= dm.w ? gx - dm.w : gx);
+      for (int g = 0; g < ngroups && ok; g++) {
+        const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
+        const bf16* xg = x + (long long)gx * ldx + c0;
+        for (int q = 0; q < zt + 2; q++, u++) {
+          if (u % nl != warp) continue;
+          const int st = u % P.hs;
+          if (!(ok = tc_wait_warp(su32(&hempty[st]), ((u / P.hs) & 1) ^ 1))) break;
+          const int gz = T.z0 - 1 + q;
+          const bool in = gz >= 0 && gz < dm.d;
+          if (hr < 3)
+            for (int row = hr; row < TC_HY; row += 3) {
+              int gy = T.y0 - 1 + row;
+              gy = gy < 0 ? gy + dm.h : (gy >= dm.h ? gy - dm.h : gy);
+              const bf16* src = xg + voxel_at(dm, T.n, in ? gz : 0, gy, 0) * ldx;
+              const uint32_t dst = halo0 + st * plane_bytes + 16 * (row * TC_HX + hx);
+              for (int j = 0; j < nch; j++) cp16(dst + j * TC_PLANE, src + 8 * j, in);
+            }
+          asm volatile("cp.async.commit_group;" ::: "memory");
+          if (lag) {
+            if (pending >= 0) {
+              asm volatile("cp.async.wait_group 1;" ::: "memory");
+              hand_over();
+            }
+            pending = st;
+          } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            pending = st;
+            hand_over();
+            pending = -1;
+          }
+        }
+      }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (pending >= 0) hand_over();
+  } else if (warp < 8) {
+    // results: TMEM lane = output row (a warp reads the lanes of its quarter)
+    const int r = (warp - 4) * 32 + lane;
+    int it = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
+      const Tile T = tile_at(t);
+      const int st = it % P.as;
+      // (the warp stays together: TMEM loads are warp-wide)
+      if (!(ok = tc_wait_warp(su32(&afull[st]), (it / P.as) & 1))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc_store(tmem + ((uint32_t)((warp - 4) * 32) << 16) + (uint32_t)(st * zt * cout),
+               voxel_at(dm, T.n, T.z0, T.y0 + r / 8, T.x0 + (r % 8)), (long long)dm.h * dm.w, zt, sbias, cout, y, ldy,
+               relu, mask, ldm);
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      tc_arrive(su32(&aempty[st]));
+    }
+  } else if (warp == 8) {
+    if (tc_elect()) {
+      int hst = 0, hph = 0, as = 0, aph = 0;
+      const uint64_t a_desc = tc_desc(halo0, TC_PLANE, TC_HX * 16);
+      const uint32_t a_lo0 = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32);
+      const uint32_t idesc1 = tc_idesc(128, cout), istep = tc_idesc(0, cout) - tc_idesc(0, 0);
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        if (!(ok = tc_wait(su32(&aempty[as]), aph ^ 1))) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d_tile = tmem + (uint32_t)(as * zt * cout);
+        for (int g = 0; g < ngroups && ok; g++) {
+          if (!(ok = tc_wait(su32(&wfull[g]), 0))) break;
+          const int nk = min(TC_CG, cin - g * TC_CG) / 16;
+          const uint64_t b_desc = tc_desc(w0 + g * (27u * TC_CG * 2) * cout, 128, nk * 256);
+          const uint32_t b_hi = (uint32_t)(b_desc >> 32), b_grp = (uint32_t)b_desc;
+          const uint32_t blk16 = (uint32_t)(cout * nk * 2), tap16 = 3 * blk16;  // weights of a z tap, of a (y, x) tap
+          for (int q = 0; q < zt + 2; q++) {
+            if (!(ok = tc_wait(su32(&hfull[hst]), hph))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a_lo = a_lo0 + hst * (plane_bytes >> 4);
+            // output planes lo .. hi; plane p through z tap q - p, stacked from tap 2 down
+            const int lo = max(0, q - 2), np = min(zt - 1, q) - lo + 1;
+            const uint32_t d = d_tile + (uint32_t)(lo * cout), b_lo = b_grp + (q < 2 ? (2 - q) * blk16 : 0u);
+            const uint32_t idesc = idesc1 + (np - 1) * istep, idesc0 = np > 1 ? idesc - istep : 0u;
+            const bool fresh = g == 0 && q < zt;
+            const uint32_t d1 = (uint32_t)((np - 1) * cout), b1 = (uint32_t)(np - 1) * blk16;
+            switch (nk) {
+              case 1: tz_plane<1>(d, a_lo, a_hi, b_lo, b_hi, tap16, idesc, fresh, idesc0, idesc1, d1, b1); break;
+              case 2: tz_plane<2>(d, a_lo, a_hi, b_lo, b_hi, tap16, idesc, fresh, idesc0, idesc1, d1, b1); break;
+              case 3: tz_plane<3>(d, a_lo, a_hi, b_lo, b_hi, tap16, idesc, fresh, idesc0, idesc1, d1, b1); break;
+              default: tz_plane<4>(d, a_lo, a_hi, b_lo, b_hi, tap16, idesc, fresh, idesc0, idesc1, d1, b1);
+            }
+            tc_commit(su32(&hempty[hst]));
+            if (++hst == P.hs) hst = 0, hph ^= 1;
+          }
+        }
+        tc_commit(su32(&afull[as]));
+        if (++as == P.as) as = 0, aph ^= 1;
+      }
+      // the block may not end with MMAs in flight: the store warps have awaited
+      // the last tiles' results; after a time-out they may have left
+      if (!ok || sfail) {
+        tc_commit(su32(&drain));
+        tc_wait(su32(&drain), 0);
+      }
+    }
+  } else if (lane == 0) {
+    // weights, a group at a time
+    for (int g = 0; g < ngroups; g++) {
+      const uint32_t off = g * (27u * TC_CG * 2) * cout;
+      tc_bulk(w0 + off, reinterpret_cast<const uint8_t*>(wimg) + off, 27u * 2 * cout * min(TC_CG, cin - g * TC_CG),
+              su32(&wfull[g]));
+    }
+    for (int g = 0; g < ngroups; g++)
+      if (!tc_wait(su32(&wfull[g]), 0)) ok = false;
   }
   if (!ok) {
     sfail = 1;
@@ -1127,12 +1399,14 @@ __global__ void k_pack_weights(const float* __restrict__ w, int cout, int cin, b
   }
 }
 
-// wt [t][cout][cin] (BF16) -> the weights of k_conv3_tc exactly as its shared
-// memory holds them, so that a block loads them, or a tap of them, with one
-// bulk copy: for group g (64 channels), tap t, output o and
-// 8-channel chunk j, 16 bytes at g 27 S + t S + (o/8)(nch 128) + (o%8) 16 +
-// j 128, with S = 2 cout min(cin, 64) bytes a tap and nch the group's chunks
-__global__ void k_pack_image(const bf16* __restrict__ wt, int cin, int cout, bf16* __restrict__ img) {
+// wt [t][cout][cin] (BF16) -> the weights of the tcgen05 convolutions exactly as
+// their shared memory holds them, so that a block loads them with bulk copies:
+// 8-channel chunk j of output o, 16 bytes, at (o/8)(nch 128) + (o%8) 16 + j 128
+// of its tap (nch: chunks of the group of 64 channels).  k_conv3_tc: group g,
+// tap t at (27 g + t) S, S = 2 cout min(cin, 64).  k_conv3_tz (`stacked`): groups
+// at 27 x 64 x 2 cout g; a (y, x) tap holds its three z taps, 2 to 0, as 3 cout
+// outputs.
+__global__ void k_pack_image(const bf16* __restrict__ wt, int cin, int cout, int stacked, bf16* __restrict__ img) {
   const int cg = cin < TC_CG ? cin : TC_CG, ngroups = (cin + TC_CG - 1) / TC_CG;
   const long long S = 2LL * cout * cg;
   const long long total = (long long)ngroups * 27 * cout * (cg / 8);
@@ -1145,7 +1419,9 @@ __global__ void k_pack_image(const bf16* __restrict__ wt, int cin, int cout, bf1
     const int g = (int)(r / 27);
     const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
     if (j >= nch) continue;
-    const long long off = g * 27 * S + t * S + (o / 8) * (nch * 128) + (o % 8) * 16 + j * 128;
+    const int row = stacked ? (2 - t / 9) * cout + o : o;
+    const long long tap = stacked ? 54LL * cout * TC_CG * g + (t % 9) * (48LL * cout * nch) : (27LL * g + t) * S;
+    const long long off = tap + (row / 8) * (nch * 128) + (row % 8) * 16 + j * 128;
     *reinterpret_cast<uint4*>(reinterpret_cast<char*>(img) + off) =
         *reinterpret_cast<const uint4*>(wt + ((long long)t * cout + o) * cin + c0 + 8 * j);
   }
@@ -1248,7 +1524,7 @@ struct Layer {
   int cin, cout, taps;
   long long woff, boff;  // offsets of W and b in the flat parameter vector
   bf16 *wt = nullptr, *wtt = nullptr;
-  // wt and wtt in the shared-memory order of k_conv3_tc
+  // wt and wtt in the shared-memory order of the tcgen05 convolutions
   bf16 *img = nullptr, *timg = nullptr;
 };
 
@@ -1318,23 +1594,61 @@ int ualloc(stp_unet* n, T** p, size_t count) {
 int cu_width(int l) { return kCh[l + 1] + kCh[l]; }
 
 constexpr size_t kTcSmemMax = 200 * 1024;  // of the mma.sync convolution
-constexpr size_t kTcSmemSm = 226 * 1024;   // of an SM's blocks of k_conv3_tc
+constexpr size_t kTcSmemSm = 225 * 1024;   // of an SM's blocks of a tcgen05 convolution
 
 // weights image of k_conv3_tc, elements
 size_t tc_image_elems(int cin, int cout) {
   return (size_t)((cin + TC_CG - 1) / TC_CG) * 27 * cout * std::min(cin, TC_CG);
 }
 
-// How k_conv3_tc runs a layer; false if it does not take it.  Weights resident
-// up to 64 KB, else a ring of 64 KB.  Two halo stages and two accumulator
-// stages where shared memory (half an SM's, or a whole one's) and 512 columns
-// take them; planes a tile 4, 2 or 1, the most that leave two tiles an SM
-// (planes share halo planes: 6 loaded for 4 computed).  A forced count
+// Weights beside two halo planes in an SM's shared memory: k_conv3_tz.
+bool tz_takes(int cin, int cout) {
+  return cin % 16 == 0 && cout % 16 == 0 && cout <= 256 && cin <= TC_CG * TZ_GROUPS &&
+         (size_t)54 * cin * cout + 2 * (size_t)(std::min(cin, TC_CG) / 8) * TC_PLANE <= kTcSmemSm;
+}
+
+// How k_conv3_tz runs a layer it takes: planes a tile (8, 4, 2 or 1; an MMA's N
+// = 3 cout, or fewer planes', at most 256) and blocks an SM (2 or 1), the pair
+// with the fewest plane loads on the busiest SM, a lone block's counted at 6/5
+// (one thread issues MMAs at 58 clocks, two blocks' at 49 together).  Two
+// accumulator stages where the columns allow.  A forced count of planes
 // (STP_UNET_TC_PLANES: 1, 2 or 4) is halved until it fits.
+TzPlan tz_plan(const stp_unet* n, const Dims& dm, int cin, int cout) {
+  const size_t plane = (size_t)(std::min(cin, TC_CG) / 8) * TC_PLANE, w = (size_t)54 * cin * cout;
+  const long long tiles = dm.vox() / (TC_TX * TC_TY);
+  const bool forced = n->tc_planes == 1 || n->tc_planes == 2 || n->tc_planes == 4;
+  TzPlan best{};
+  long long cost = 0;
+  for (int zt = forced ? n->tc_planes : 8; zt >= 1; zt /= 2) {
+    if (dm.d % zt || std::min(zt, 3) * cout > 256) continue;
+    for (int per_sm = 2; per_sm >= 1; per_sm--) {
+      const size_t room = per_sm == 2 ? kTcSmemSm / 2 - 2048 : kTcSmemSm;
+      TzPlan p;
+      p.zt = zt;
+      p.per_sm = per_sm;
+      if (w + 2 * plane > room || zt * cout > 512 / per_sm) continue;
+      p.hs = (int)std::min<size_t>(TZ_HALO, (room - w) / plane);
+      p.as = 2 * zt * cout <= 512 / per_sm ? 2 : 1;
+      p.cols = 32;
+      while (p.cols < p.as * zt * cout) p.cols *= 2;
+      p.smem = w + p.hs * plane;
+      const long long blocks = 152LL * per_sm, rounds = (tiles / zt + blocks - 1) / blocks;
+      const long long c = rounds * (zt + 2 + (p.as == 1 && per_sm == 1 ? zt : 0)) * (per_sm == 2 ? 10 : 6);
+      if (best.zt == 0 || c < cost) best = p, cost = c;
+    }
+    if (forced && best.zt) break;
+  }
+  return best;
+}
+
+// How k_conv3_tc runs a layer; false if it does not take it.  A ring of 64 KB of
+// weights.  Two halo stages and two accumulator stages where shared memory
+// (half an SM's, or a whole one's) and 512 columns take them; planes a tile 4, 2
+// or 1, the most that leave two tiles an SM (planes share halo planes: 6 loaded
+// for 4 computed).  A forced count as above.
 bool tc_plan(const stp_unet* n, const Dims& dm, int cin, int cout, TcPlan* out) {
   const int cg = std::min(cin, TC_CG);
   const size_t tap = (size_t)2 * cout * cg;
-  const size_t res = (size_t)((cin + TC_CG - 1) / TC_CG) * 27 * tap;
   const long long tiles = dm.vox() / (TC_TX * TC_TY);
   const bool forced = n->tc_planes == 1 || n->tc_planes == 2 || n->tc_planes == 4;
   for (int q = 0; q < 6; q++) {
@@ -1345,12 +1659,12 @@ bool tc_plan(const stp_unet* n, const Dims& dm, int cin, int cout, TcPlan* out) 
     if (forced && zt > n->tc_planes) continue;
     if (dm.d % zt || zt * cout > 256) continue;
     if (!forced && zt > 1 && tiles / zt < 2 * 152) continue;
-    p.ring = res <= 64 * 1024 ? 0 : (int)std::min<size_t>(TC_RING, std::max<size_t>(2, 64 * 1024 / tap));
+    p.ring = (int)std::min<size_t>(TC_RING, std::max<size_t>(2, 64 * 1024 / tap));
     p.as = 2 * zt * cout <= 256 ? 2 : 1;
     p.cols = 32;
     while (p.cols < p.as * zt * cout) p.cols *= 2;
-    const size_t halo = (size_t)(cg / 8) * TC_PLANE * (zt + 2), w = p.ring ? p.ring * tap : res;
-    p.smem = p.hs * halo + w;
+    const size_t halo = (size_t)(cg / 8) * TC_PLANE * (zt + 2);
+    p.smem = p.hs * halo + p.ring * tap;
     if (p.smem > kTcSmemSm) continue;
     p.per_sm = p.smem <= kTcSmemSm / 2 - 2048 && 2 * p.cols <= 512 ? 2 : 1;
     *out = p;
@@ -1359,9 +1673,9 @@ bool tc_plan(const stp_unet* n, const Dims& dm, int cin, int cout, TcPlan* out) 
   return false;
 }
 
-bool conv3_tc_ok(const stp_unet* n, const Dims& dm, int ldx, int cin, int cout, int ldy, TcPlan* p) {
+bool conv3_tc_ok(const stp_unet* n, const Dims& dm, int ldx, int cin, int cout, int ldy, int ldm, TcPlan* p) {
   return n->use_tc && dm.w % TC_TX == 0 && dm.h % TC_TY == 0 && cin % 16 == 0 && cout % 16 == 0 && cout <= 256 &&
-         ldx % 8 == 0 && ldy % 16 == 0 && tc_plan(n, dm, cin, cout, p);
+         ldx % 8 == 0 && ldy % 16 == 0 && ldm % 8 == 0 && (tz_takes(cin, cout) || tc_plan(n, dm, cin, cout, p));
 }
 
 // launch a 3x3x3 convolution (forward form): tcgen05 where the shapes allow, else mma.sync
@@ -1369,7 +1683,17 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
           const float* bias, int cout, bf16* y, int ldy, int relu, const bf16* mask, int ldm) {
   const long long V = dm.vox();
   TcPlan p;
-  if (conv3_tc_ok(n, dm, ldx, cin, cout, ldy, &p)) {
+  if (conv3_tc_ok(n, dm, ldx, cin, cout, ldy, ldm, &p)) {
+    if (tz_takes(cin, cout)) {
+      static std::atomic<unsigned> donez{0u};
+      UTRY(n, smem_limit_once(k_conv3_tz, (int)kTcSmemSm, donez));
+      const TzPlan z = tz_plan(n, dm, cin, cout);
+      const unsigned tiles = (unsigned)(V / (TC_TX * TC_TY * z.zt));
+      k_conv3_tz<<<std::min(tiles, 152u * z.per_sm), TZ_THREADS, z.smem, n->st>>>(dm, x, ldx, cin, wimg, bias, cout, y, ldy,
+                                                                                 relu, mask, ldm, z, n->d_err);
+      UTRY(n, cudaGetLastError());
+      return STP_OK;
+    }
     const unsigned tiles = (unsigned)(V / (TC_TX * TC_TY * p.zt));
     auto go = [&](auto kern, std::atomic<unsigned>& done) -> cudaError_t {
       if (cudaError_t e = smem_limit_once(kern, (int)kTcSmemSm, done)) return e;
@@ -1460,8 +1784,8 @@ int pack_all(stp_unet* n) {
     const long long tot = (long long)ly.cout * ly.cin * 27;
     k_pack_weights<<<blocks_for(tot), 256, 0, n->st>>>(n->theta + ly.woff, ly.cout, ly.cin, ly.wt, ly.wtt);
     UTRY(n, cudaGetLastError());
-    k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wt, ly.cin, ly.cout, ly.img);
-    k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wtt, ly.cout, ly.cin, ly.timg);
+    k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wt, ly.cin, ly.cout, tz_takes(ly.cin, ly.cout), ly.img);
+    k_pack_image<<<blocks_for(tot / 8), 256, 0, n->st>>>(ly.wtt, ly.cout, ly.cin, tz_takes(ly.cout, ly.cin), ly.timg);
     UTRY(n, cudaGetLastError());
   }
   return STP_OK;
