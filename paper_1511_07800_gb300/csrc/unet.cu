@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
 // (16 bytes apart), the next 8 rows are the next y (SBO = 16 HX bytes), the
 // next 8 channels the next chunk (LBO = one chunk of the halo).  So the 27
 // taps need no data movement.  The weights come as bulk copies of an image
-// kept in shared-memory order, a tap at a time through a ring: this kernel takes
+// kept in shared-memory order, three taps at a time through a ring: this kernel takes
 // the layers whose weights do not fit an SM (64 -> 64, 192 -> 64 and back).
 //
 // What bounds it: an MMA of M = 128, K = 16 takes 68 clocks whatever the layout
@@ -294,6 +294,7 @@ constexpr int TC_TX = 8, TC_TY = 16, TC_HX = 10, TC_HY = 18;
 constexpr int TC_PLANE = TC_HX * TC_HY * 16;  // bytes of one halo plane of one 8-channel chunk
 constexpr int TC_CG = 64;                     // channels per halo group
 constexpr int TC_RING = 8;                    // most weight stages
+constexpr int TC_STAPS = 3;                   // taps a weight stage
 constexpr int TC_THREADS = 352;               // 4 loader warps, 4 store warps, 2 MMA warps, weights
 
 // shared-memory matrix descriptor: no swizzle, K-major core matrices
@@ -589,11 +590,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
           const uint32_t b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32), stage16 = stage_bytes >> 4;
           auto group = [&](auto nkc) {
             constexpr int NK = decltype(nkc)::value;
-#pragma unroll 9
-            for (int tap = 0; tap < 27; tap++) {
+#pragma unroll 3
+            for (int row = 0; row < 27 / TC_STAPS; row++) {
               if (!(ok = ok && tc_wait(su32(&wfull[ws]), wph))) continue;
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              tc_tap<NK, NP, ZT>(tap, d, a_lo, a_hi, b_lo + ws * stage16, b_hi, idesc, g == 0 && tap == 0);
+#pragma unroll
+              for (int i = 0; i < TC_STAPS; i++)
+                tc_tap<NK, NP, ZT>(row * TC_STAPS + i, d, a_lo, a_hi, b_lo + (ws * TC_STAPS + i) * stage16, b_hi, idesc,
+                                   g == 0 && row == 0 && i == 0);
               tc_commit(su32(&wempty[ws]));
               if (++ws == P.ring) ws = 0, wph ^= 1;
             }
@@ -620,12 +624,12 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
   } else if (warp == 10 && lane == 0) {
     // weights
     int wuse = 0;
+    const uint32_t bytes = TC_STAPS * stage_bytes;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
-      for (int q = 0; q < ngroups * 27; q++, wuse++) {
+      for (int q = 0; q < ngroups * 27 / TC_STAPS; q++, wuse++) {
         const int ws = wuse % P.ring;
         if (!(ok = tc_wait(su32(&wempty[ws]), ((wuse / P.ring) & 1) ^ 1))) break;
-        tc_bulk(w0 + ws * stage_bytes, reinterpret_cast<const uint8_t*>(wimg) + (size_t)q * stage_bytes, stage_bytes,
-                su32(&wfull[ws]));
+        tc_bulk(w0 + ws * bytes, reinterpret_cast<const uint8_t*>(wimg) + (size_t)q * bytes, bytes, su32(&wfull[ws]));
       }
     // copies still in flight land before the block ends
     for (int r = 0; r < P.ring && r < wuse; r++) {
@@ -1641,14 +1645,14 @@ TzPlan tz_plan(const stp_unet* n, const Dims& dm, int cin, int cout) {
   return best;
 }
 
-// How k_conv3_tc runs a layer; false if it does not take it.  A ring of 64 KB of
-// weights.  Two halo stages and two accumulator stages where shared memory
+// How k_conv3_tc runs a layer; false if it does not take it.  A ring of 96 KB of
+// weights, at least two stages of three taps.  Two halo stages and two accumulator stages where shared memory
 // (half an SM's, or a whole one's) and 512 columns take them; planes a tile 4, 2
 // or 1, the most that leave two tiles an SM (planes share halo planes: 6 loaded
 // for 4 computed).  A forced count as above.
 bool tc_plan(const stp_unet* n, const Dims& dm, int cin, int cout, TcPlan* out) {
   const int cg = std::min(cin, TC_CG);
-  const size_t tap = (size_t)2 * cout * cg;
+  const size_t stage = (size_t)2 * TC_STAPS * cout * cg;
   const long long tiles = dm.vox() / (TC_TX * TC_TY);
   const bool forced = n->tc_planes == 1 || n->tc_planes == 2 || n->tc_planes == 4;
   for (int q = 0; q < 6; q++) {
@@ -1659,12 +1663,12 @@ bool tc_plan(const stp_unet* n, const Dims& dm, int cin, int cout, TcPlan* out) 
     if (forced && zt > n->tc_planes) continue;
     if (dm.d % zt || zt * cout > 256) continue;
     if (!forced && zt > 1 && tiles / zt < 2 * 152) continue;
-    p.ring = (int)std::min<size_t>(TC_RING, std::max<size_t>(2, 64 * 1024 / tap));
+    p.ring = (int)std::min<size_t>(TC_RING, std::max<size_t>(2, 96 * 1024 / stage));
     p.as = 2 * zt * cout <= 256 ? 2 : 1;
     p.cols = 32;
     while (p.cols < p.as * zt * cout) p.cols *= 2;
     const size_t halo = (size_t)(cg / 8) * TC_PLANE * (zt + 2);
-    p.smem = p.hs * halo + p.ring * tap;
+    p.smem = p.hs * halo + p.ring * stage;
     if (p.smem > kTcSmemSm) continue;
     p.per_sm = p.smem <= kTcSmemSm / 2 - 2048 && 2 * p.cols <= 512 ? 2 : 1;
     *out = p;

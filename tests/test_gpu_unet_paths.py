@@ -59,3 +59,30 @@ def test_tiny_and_ragged_levels(stp_lib, orc, shape):
     rel = np.linalg.norm(gg - g_o) / np.linalg.norm(g_o)
     assert rel < 5e-2, rel
     net.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 8, 128, 64), (2, 16, 128, 64)])
+def test_streamed_weights_of_the_deepest_level(stp_lib, orc, monkeypatch, shape):
+    """A network whose 128-channel level runs on tcgen05 too (16 rows): weights
+    of 64 to 128 and 128 to 128 channels through the ring, two groups of
+    channels, one and two planes a level.  Against the mma.sync kernels within
+    the bounds of the smaller shapes."""
+    torch = pytest.importorskip("torch")
+    unet, theta, x, t = _setup(8, shape)
+    n, d, h, w = x.shape
+    tx = torch.from_numpy(x.astype(np.float32)).cuda()
+    tt = torch.from_numpy(t.astype(np.float32)).cuda()
+    out = []
+    for tc in ("0", "1"):
+        monkeypatch.setenv("STP_UNET_TC", tc)
+        net = stp_lib.UNet(n, d, h, w)
+        net.set_params(theta.astype(np.float32))
+        ty = torch.zeros_like(tx)
+        net.forward(tx, ty)
+        g = torch.zeros(stp_lib.UNet.param_count(), dtype=torch.float32, device="cuda")
+        net.gradient(tx, tt, g)
+        out.append((ty.cpu().numpy().astype(np.float64), g.cpu().numpy().astype(np.float64)))
+        net.close()
+    (y0, g0), (y1, g1) = out
+    assert np.abs(y1 - y0).max() < 2e-2 * np.abs(y0).max()
+    assert np.linalg.norm(g1 - g0) < 5e-2 * np.linalg.norm(g0)
