@@ -43,7 +43,10 @@ LINE_NAMES = {1: "k_line_sweep_chunk<32,6> (z-line SRJ sweep: residual, column r
 TILE_NAMES = {0: "k_sweep_f32_z<1,8>", 1: "k_sweep_f32_z<2,8>", 2: "k_sweep_f32_z<4,8>", 3: "k_sweep_f32_z<2,4>",
               4: "k_sweep_f32_z<4,4>", 5: "k_sweep_f32_z<8,4>", 6: "k_sweep_f32_flat<2>", 7: "k_sweep_f32_flat<4>",
               8: "k_sweep_f32_flat<8>", 9: "k_sweep_f32_pair<8,4>", 10: "k_sweep_f32_pair<4,4>",
-              11: "k_sweep_f32_pair<4,8>"}
+              11: "k_sweep_f32_pair<4,8>", 12: "k_cluster_cycle (16 blocks, z slabs)",
+              13: "k_cluster_cycle (16 blocks, y slabs)", 14: "k_cluster_cycle (8 blocks, z slabs)",
+              15: "k_cluster_cycle (8 blocks, y slabs)"}
+LINE_F64 = "k_line_f64 (z-line SRJ sweep, column recurrences in level chunks)"
 
 
 def parse():
@@ -566,12 +569,35 @@ def timed_steps(ch, steps, stream, flush):
     return dict(ms=ms, sweeps=sweeps, passes=passes, launches=launches, solve_ms=solve_ms, converged=conv)
 
 
-def sweep_roofline(word, cells, r, kernel, peak, traffic_key):
+def two_colour(cfg, precision):
+    """Whether a channel's FP32 inner solve runs two-colour sweeps (one colour
+    a sweep): even rows and row counts, at least 2^21 cells, z lines of at
+    most 192 levels, and none of the environment's other choices."""
+    return (precision == "fp32" and cfg["nx"] % 2 == 0 and cfg["ny"] % 2 == 0 and
+            cfg["nx"] * cfg["ny"] * cfg["nz"] >= 1 << 21 and (not cfg.get("zline") or cfg["nz"] <= 192) and
+            not os.environ.get("STP_SRJ_COLOURS", "").startswith("0") and "STP_SWEEP_VARIANT" not in os.environ and
+            not os.environ.get("STP_LINE_VARIANT", "").startswith("0"))
+
+
+def sweep_kernel(cfg, precision, ch):
+    """Name of the sweep kernel a channel runs."""
+    if two_colour(cfg, precision):
+        return ("k_col_line" if cfg.get("zline") else "k_col_point") + " (two-colour SRJ sweep, one colour a sweep)"
+    if cfg.get("zline"):
+        return LINE_NAMES[ch.line_kernel()] if precision == "fp32" else LINE_F64
+    variant, _ = ch.sweep_tile()
+    if precision == "fp32":
+        return TILE_NAMES.get(variant, "k_sweep_f32") + " (SRJ sweep, autotuned tile variant %d)" % variant
+    return "k_sweep_f64 (SRJ sweep)"
+
+
+def sweep_roofline(words, word, cells, r, kernel, peak, traffic_key):
     """HBM roofline of the SRJ sweep: 3 words a cell (read p and b, write
-    p'), over the mean time per sweep of the solve graphs (GPU events around
-    each solve, charged with its once-per-cycle checks and refinement
-    kernels: a lower bound on the sweep's own rate)."""
-    bytes_per_sweep = 3 * word * cells
+    p') or, a colour at a time, 2 (half of p relaxed in place, the other half
+    and half of b read), over the mean time per sweep of the solve graphs
+    (GPU events around each solve, charged with its once-per-cycle checks and
+    refinement kernels: a lower bound on the sweep's own rate)."""
+    bytes_per_sweep = words * word * cells
     t = r["solve_ms"] / max(1, r["sweeps"]) / 1e3
     ach = bytes_per_sweep / t / 1e9 if r["sweeps"] else None
     tr = traffic_for(traffic_key)
@@ -581,8 +607,8 @@ def sweep_roofline(word, cells, r, kernel, peak, traffic_key):
     return {"bound": "hbm", "kernel": kernel, "achieved": ach, "peak": peak, "unit": "GB/s",
             "frac": ach / peak if ach else None, "traffic": traffic, "bytes_per_launch": bytes_per_sweep,
             "mean_launch_us": t * 1e6,
-            "note": "achieved = algorithmic bytes (3 words a cell) / (solve-graph GPU time / sweeps), the "
-                    "once-per-cycle residual checks and refinement kernels charged to the sweeps"}
+            "note": "achieved = algorithmic bytes (%d words a cell) / (solve-graph GPU time / sweeps), the "
+                    "once-per-cycle residual checks and refinement kernels charged to the sweeps" % words}
 
 
 def side_steps(stp, cfg, precision, fields, steps, warmup, stream, flush, peak, traffic_key):
@@ -594,18 +620,13 @@ def side_steps(stp, cfg, precision, fields, steps, warmup, stream, flush, peak, 
         for _ in range(max(3, warmup)):
             ch.step(1)
         r = timed_steps(ch, steps, stream, flush)
-        variant, _ = ch.sweep_tile()
-        lk = ch.line_kernel()
-    if cfg.get("zline"):
-        kern = LINE_NAMES[lk] if precision == "fp32" else "k_line_sweep_vec<double> (z-line)"
-    else:
-        kern = (TILE_NAMES.get(variant, "k_sweep_f32") + " (autotuned tile variant %d)" % variant
-                if precision == "fp32" else "k_sweep_f64_v2")
+        kern = sweep_kernel(cfg, precision, ch)
+    words = 2 if two_colour(cfg, precision) else 3
     out = {"value": cells * steps / (r["ms"] / 1e3) / 1e6, "unit": "Mcell*steps/s", "ms_per_step": r["ms"] / steps,
            "steps": steps, "warmup": max(3, warmup), "sweeps_per_step": r["sweeps"] / steps,
            "solve_ms_per_step": r["solve_ms"] / steps, "converged": r["converged"],
            "gpu_launches_per_step": r["launches"] / steps,
-           "roofline": sweep_roofline(word, cells, r, kern, peak, traffic_key)}
+           "roofline": sweep_roofline(words, word, cells, r, kern, peak, traffic_key)}
     if precision == "fp64":
         out["roofline"]["note"] += ("; in FP64 the sweep is bound by GB300's FP64 pipe, not by HBM "
                                     "(profiles/srj_sweep_f64_os_instability.md)")
@@ -639,18 +660,16 @@ def sweeps_above_l2(stp, peak):
                 ch.poisson_solve(b, p, tol=0.0, maxit=M)  # warm-up (and the FP32 tile autotuner)
                 p.zero_()
                 st = ch.poisson_solve(b, p, tol=0.0, maxit=2 * M)
-                variant, _ = ch.sweep_tile()
-                lk = ch.line_kernel()
+                colours = two_colour(dict(cfg, zline=zl), prec)
+                kern = sweep_kernel(dict(cfg, zline=zl), prec, ch)
             t = st["solve_ms"] / max(1, st["sweeps"]) / 1e3
-            ach = 3 * word * cells / t / 1e9
+            ach = (2 if colours else 3) * word * cells / t / 1e9
             res[solver] = {"sweeps": st["sweeps"], "us_per_sweep": t * 1e6, "achieved_GBs": ach,
                            "frac": ach / peak,
-                           "kernel": (LINE_NAMES[lk].split(" ")[0] if zl and prec == "fp32" else
-                                      "k_line_sweep_vec<double,RB>" if zl else
-                                      (TILE_NAMES.get(variant, "k_sweep_f32") if prec == "fp32" else "k_sweep_f64_v2"))}
+                           "kernel": kern.split(" ")[0]}
         out[name] = res
     out["note"] = ("time per sweep of a solve graph held to 2 cycles (its two residual checks and, in FP32, the "
-                   "refinement kernels charged to the sweeps); achieved = 3 words a cell / that time")
+                   "refinement kernels charged to the sweeps); achieved = 3 words a cell (a two-colour sweep: 2) / that time")
     return out
 
 
@@ -713,16 +732,12 @@ def run_ours(args):
     peaks = measured_peaks()
     peak = peaks.get("hbm_gbs", 6800.0)
     word = 4 if args.precision == "fp32" else 8
-    variant, _ = ch.sweep_tile()
-    if cfg.get("zline"):
-        kern = (LINE_NAMES[ch.line_kernel()] if args.precision == "fp32"
-                else "k_line_sweep_vec<double,RB> (z-line SRJ sweep)")
-        tkey = "zline_sweep_%s_%s" % (args.precision, args.workload)
-    else:
-        kern = (TILE_NAMES.get(variant, "k_sweep_f32") + " (SRJ sweep, autotuned tile variant %d)" % variant
-                if args.precision == "fp32" else "k_sweep_f64_v2 (SRJ sweep)")
-        tkey = "point_sweep_%s_%s" % (args.precision, args.workload)
-    roof = sweep_roofline(word, cells, r, kern, peak, tkey)
+    kern = sweep_kernel(cfg, args.precision, ch)
+    words = 2 if two_colour(cfg, args.precision) else 3
+    # (the recorded DRAM bytes are a Jacobi sweep's)
+    tkey = "%s_%s_%s" % ("two_colour" if words == 2 else "zline_sweep" if cfg.get("zline") else "point_sweep",
+                         args.precision, args.workload)
+    roof = sweep_roofline(words, word, cells, r, kern, peak, tkey)
     roof["peak_source"] = "MEASURED_PEAKS.json hbm_gbs (measured)" if "hbm_gbs" in peaks else "fallback"
     roof["l2_note"] = ("the FP32 inner solve's working set (d, d', r: 12 bytes a cell, %.0f MB) %s the 126 MB L2; "
                        "the sweeps' HBM rate on working sets above L2 is under srj_sweeps_above_l2"

@@ -23,7 +23,13 @@
  * returns; it owns all its device memory and frees it in stp_destroy.
  *
  * The pressure solve runs as one CUDA graph steered from the device (graph
- * conditional nodes), one kernel per SRJ sweep.  With STP_PERSISTENT=1 at
+ * conditional nodes), one kernel per SRJ sweep.  The FP32 inner solve of a
+ * channel of at least 2^21 cells with even nx and ny (z lines: nz <= 192) runs
+ * two-colour sweeps: a sweep relaxes one colour of cells (z lines: of columns)
+ * in place, with the Chebyshev factors of a two-coloured grid, so that a cycle
+ * of M sweeps gains what M Jacobi sweeps do.  STP_SRJ_COLOURS=0 at stp_init
+ * keeps Jacobi sweeps, as do schedules of the caller's own, a learned guess,
+ * STP_SWEEP_VARIANT, STP_LINE_VARIANT=0 and the persistent cycles.  With STP_PERSISTENT=1 at
  * stp_init an FP32 cycle instead runs as one persistent cooperative kernel
  * with bounded grid barriers between its sweeps (slower on GB300: kept as an
  * option); each barrier wait gives up after STP_BARRIER_WAIT SM clock cycles
@@ -40,12 +46,15 @@
  * (Sec. 3.4's line relaxation with the twisted elimination split into
  * chunked recurrences); elsewhere, or with STP_LINE_VARIANT=0 at stp_init,
  * a block stages its columns in shared memory and solves them in lock
- * step.  The two round differently (a few units in the last place).  The FP32 sweep kernel's tile shape (z levels per thread, rows
- * per block) is picked on first use by timing the variants on the grid
- * (STP_SWEEP_VARIANT=<0..11> forces one; variants 6..8 pack warps along the
+ * step.  The two round differently (a few units in the last place).  FP64
+ * z-line sweeps solve their columns in level chunks too, up to 384 levels.
+ * The FP32 sweep kernel's tile shape (z levels per thread, rows per block) is
+ * picked on first use by timing the variants on the grid
+ * (STP_SWEEP_VARIANT=<0..15> forces one; variants 6..8 pack warps along the
  * plane for rows shorter than 128 cells, 9..11 run two sweeps per launch on
- * a shared-memory tile; STP_TUNE_LOG=1 prints the timings to stderr).  With STP_HOST_SOLVE=1 at
- * stp_init the same kernels are driven from the host instead, one host
+ * a shared-memory tile, 12..15 a whole cycle on one cluster of 16 or 8 blocks,
+ * for channels that fit its shared memory; STP_TUNE_LOG=1 prints the timings
+ * to stderr).  With STP_HOST_SOLVE=1 at stp_init the same kernels are driven from the host instead, one host
  * round trip per SRJ cycle (for profilers that cannot see kernels inside
  * conditional graphs).
  *
@@ -230,15 +239,16 @@ int stp_stats_accumulate(stp_handle *h);
 int stp_stats_read(stp_handle *h, double *moments, double *corr, long long *nsamples, int *kc);
 
 /* The FP32 sweep tile variant the autotuner picked for this handle's grid
-   (0..8, see above; -1 before the first solve, 0 in FP64) and, when it was
-   timed, its time per sweep in microseconds (*us may be NULL). */
+   (0..15, see above; with two-colour sweeps the variant of their kernel; -1
+   before the first solve, 0 in FP64) and, when it was timed, its time per
+   sweep in microseconds (*us may be NULL). */
 int stp_sweep_tile(const stp_handle *h, float *us);
 
 /* The z-line sweep kernel of a handle with line relaxation (Sec. 3.4):
    1 for the register-chunked FP32 kernel (rows of a multiple of 32 cells,
-   columns of 2 to 192 levels), 0 for the shared-memory lock-step kernel
-   (FP64, other grids, or STP_LINE_VARIANT=0 at stp_init); -1 for point
-   sweeps or a NULL handle.  No GPU work. */
+   columns of 2 to 192 levels; two-colour solves keep this answer), 0 for the
+   shared-memory lock-step kernel (other FP32 grids, or STP_LINE_VARIANT=0 at
+   stp_init) and in FP64; -1 for point sweeps or a NULL handle.  No GPU work. */
 int stp_line_kernel(const stp_handle *h);
 
 /* Lock-step groups of the batch (built at the first stp_batch_step).
@@ -333,12 +343,12 @@ long long stp_unet_param_count(void);
    least 8) on the current device; stream NULL: its own stream.  Parameters
    start at zero: set them with stp_unet_set_params.  Its 3x3x3 convolutions
    run on tcgen05 where a level's shape allows (STP_UNET_TC=0 at create:
-   mma.sync everywhere), a block computing 1, 2 or 4 z planes chosen by the
-   layer's shape (STP_UNET_TC_PLANES=<1|2|4> forces a count where it is
-   valid; the forward output does not depend on it).  The mma.sync ones take
-   64, 32, 16 or 8 output channels a block by grid size (STP_UNET_MMA_NT=
-   <8|4|2|1> forces a width where the channels allow; results do not depend
-   on it either). */
+   mma.sync everywhere), a block computing 1, 2, 4 or 8 z planes at a time
+   chosen by the layer's shape (STP_UNET_TC_PLANES=<1|2|4> forces a count where
+   it is valid; the forward output does not depend on it).  The mma.sync ones
+   take 32, 16 or 8 output channels a block by grid size (STP_UNET_MMA_NT=
+   <8|4|2|1> forces a width where the channels allow, 8 as 4; results do not
+   depend on it either). */
 int stp_unet_create(int nmax, int nz, int ny, int nx, void *stream, stp_unet **out);
 void stp_unet_destroy(stp_unet *net);
 const char *stp_unet_last_error(const stp_unet *net);
