@@ -268,8 +268,8 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
 // (16 bytes apart), the next 8 rows are the next y (SBO = 16 HX bytes), the
 // next 8 channels the next chunk (LBO = one chunk of the halo).  So the 27
 // taps need no data movement.  The weights come as bulk copies of an image
-// kept in shared-memory order, three taps at a time through a ring: this kernel takes
-// the layers whose weights do not fit an SM (64 -> 64, 192 -> 64 and back).
+// kept in shared-memory order, three taps at a time through a ring: this kernel
+// takes the layers whose weights do not fit an SM (64 -> 64, 192 -> 64 and back).
 //
 // What bounds it: an MMA of M = 128, K = 16 takes 68 clocks whatever the layout
 // and N up to 128 when one thread issues them in a loop, 48 when an elected
@@ -277,13 +277,14 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
 // 27 cin/16 x 48 clocks a 128 voxels.  To keep the MMAs back to back, blocks
 // stay for many tiles and their warps take roles: four load halos (hs stages),
 // one thread copies weights, two threads issue MMAs, four warps store results
-// (as accumulator stages), each waiting on mbarriers for the others.  128 x 64 x 128 voxels, us, with blocks that load,
-// multiply and store one tile after another, several an SM / this: 16 -> 16 77 /
-// 49, 48 -> 16 190 / 113; 32 -> 32 at half that size 34 / 20, 96 -> 32 125 / 65;
-// all of a forward's layers 755 / 415, of a gradient's (4 x 64 x 32 x 64) 627 /
-// 430.  Without the MMAs 16 -> 16 takes 30 and 48 -> 16 85: the halo copies (16
-// bytes a lane and instruction) bound the widest level, the MMAs the others.
-// Eight loader warps (62, 124) or a pair of lanes a voxel (53, 130) are slower.
+// (as accumulator stages), each waiting on mbarriers for the others.  us, with
+// blocks that load, multiply and store one tile after another, several an SM /
+// this (both with resident weights where they fit): 16 -> 16 at 128 x 64 x 128 77
+// / 49, 48 -> 16 190 / 113, 32 -> 32 at half that size 34 / 20.  With a weight
+// stage a tap, handing it over (0.36 us) took as long as its copy: 64 -> 64 at 32
+// x 16 x 32 15.5 with one tap a stage, 12.5 with three; 192 -> 64 28.8 / 27.5,
+// bound by its weights (660 KB a tile) and three halos in sequence.  Eight
+// loader warps (16 -> 16 62) or a pair of lanes a voxel (53) are slower.
 //
 // Each accumulator sees the same MMAs in the same order (groups, taps,
 // 16-channel steps) whatever the plan.  Every wait is bounded; on a time-out
