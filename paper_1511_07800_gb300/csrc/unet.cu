@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
   r /= ty;
   const int z0 = (r % tz) * CS_TZ, nn = r / tz;
   const int cob = blockIdx.y * NT * 8;
+  cudaGridDependencySynchronize();
   for (int i = tid; i < CS_HVOX; i += 128) {
     const int hx = i % CS_HX, hy = (i / CS_HX) % CS_HY, hz = i / (CS_HX * CS_HY);
     const int vz = z0 - 1 + hz;
@@ -495,11 +496,12 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sfail = 0;
   }
-  for (int i = tid; i < cout; i += blockDim.x) sbias[i] = bias ? bias[i] : 0.f;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(P.cols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  cudaGridDependencySynchronize();
+  for (int i = tid; i < cout; i += blockDim.x) sbias[i] = bias ? bias[i] : 0.f;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -735,11 +737,12 @@ __global__ void __launch_bounds__(TZ_THREADS) k_conv3_tz(Dims dm, const bf16* __
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sfail = 0;
   }
-  for (int i = tid; i < cout; i += blockDim.x) sbias[i] = bias ? bias[i] : 0.f;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(P.cols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  cudaGridDependencySynchronize();
+  for (int i = tid; i < cout; i += blockDim.x) sbias[i] = bias ? bias[i] : 0.f;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -958,6 +961,7 @@ __global__ void __launch_bounds__(128) k_conv_in(Dims dm, const float* __restric
 // Output layer: 1x1x1, 16 channels -> 1, linear, FP32 output.
 __global__ void k_conv_out(long long V, const bf16* __restrict__ x, int ldx, const float* __restrict__ w,
                            const float* __restrict__ bias, float* __restrict__ y) {
+  cudaGridDependencySynchronize();
   float ws[16];
 #pragma unroll
   for (int c = 0; c < 16; c++) ws[c] = __bfloat162float(__float2bfloat16(w[c]));
@@ -977,6 +981,7 @@ __global__ void k_conv_out(long long V, const bf16* __restrict__ x, int ldx, con
 __global__ void k_conv_out_bwd(long long V, const float* __restrict__ gy, const bf16* __restrict__ d1, int ldx,
                                const float* __restrict__ w, bf16* __restrict__ gd, int ldg, float* __restrict__ gw,
                                float* __restrict__ gb) {
+  cudaGridDependencySynchronize();
   __shared__ float red[17][33];
   float ws[16], acc[17];
 #pragma unroll
@@ -1116,6 +1121,7 @@ __global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict_
       for (int ch = 0; ch < CT / 8; ch++) cp16(sx + st + 16 * (ch * WG_HVOX + v), src + 8 * ch, in);
     }
   };
+  cudaGridDependencySynchronize();
   if (t0 < t1) load(t0, 0);
   asm volatile("cp.async.commit_group;" ::: "memory");
   for (int tile = t0; tile < t1; tile++) {
@@ -1174,6 +1180,7 @@ __global__ void __launch_bounds__(288) k_wgrad3(Dims dm, const bf16* __restrict_
 // output walking up to 304 slices waited on memory: 15 us a layer)
 __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, int slices, int cin, int cout,
                                                    float* __restrict__ gw, float* __restrict__ gb) {
+  cudaGridDependencySynchronize();
   __shared__ float red[8][32];
   const int n = 27 * cout * cin, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
   const bool in = e < n + cout;
@@ -1201,6 +1208,7 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ par
 // [32][16] in scratch, one a block.
 __global__ void __launch_bounds__(256) k_wgrad_in(Dims dm, const float* __restrict__ x, const bf16* __restrict__ gz,
                                                   int ldg, float* __restrict__ part) {
+  cudaGridDependencySynchronize();
   __shared__ __align__(128) uint4 sgz[2 * WG_VOX];
   __shared__ unsigned short sxv[WG_HVOX];
   __shared__ float red[8][16][33];
@@ -1281,6 +1289,7 @@ __global__ void __launch_bounds__(256) k_wgrad_in(Dims dm, const float* __restri
 }
 __global__ void k_wgrad_in_sum(const float* __restrict__ part, int slices, float* __restrict__ gw,
                                float* __restrict__ gb) {
+  cudaGridDependencySynchronize();
   // a warp an output (28 x 16 of them): lanes stride the slices
   const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (e >= 28 * 16) return;
@@ -1302,6 +1311,7 @@ __global__ void k_wgrad_in_sum(const float* __restrict__ part, int slices, float
 // stores).
 // out (coarse) = mean of the 2x2x2 fine block (summed in block order); fine dims dm
 __global__ void k_pool(Dims dm, const bf16* __restrict__ x, int ldx, int c, bf16* __restrict__ y, int ldy) {
+  cudaGridDependencySynchronize();
   const Dims cd{dm.n, dm.d / 2, dm.h / 2, dm.w / 2};
   const unsigned V = (unsigned)cd.vox();
   if ((int)blockIdx.y * 8 >= c) return;
@@ -1327,6 +1337,7 @@ __global__ void k_pool(Dims dm, const bf16* __restrict__ x, int ldx, int c, bf16
 
 // fine = coarse value (nearest); coarse dims cd
 __global__ void k_upsample(Dims cd, const bf16* __restrict__ x, int ldx, int c, bf16* __restrict__ y, int ldy) {
+  cudaGridDependencySynchronize();
   const Dims fd{cd.n, cd.d * 2, cd.h * 2, cd.w * 2};
   const unsigned V = (unsigned)fd.vox();
   for (unsigned v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
@@ -1340,6 +1351,7 @@ __global__ void k_upsample(Dims cd, const bf16* __restrict__ x, int ldx, int c, 
 // order), times (act > 0)
 __global__ void k_upsample_bwd_mask(Dims cd, const bf16* __restrict__ gf, int ldg, int c, const bf16* __restrict__ act,
                                     int lda, bf16* __restrict__ out, int ldo) {
+  cudaGridDependencySynchronize();
   const Dims fd{cd.n, cd.d * 2, cd.h * 2, cd.w * 2};
   const unsigned V = (unsigned)cd.vox();
   if ((int)blockIdx.y * 8 >= c) return;
@@ -1369,6 +1381,7 @@ __global__ void k_upsample_bwd_mask(Dims cd, const bf16* __restrict__ gf, int ld
 __global__ void k_pool_bwd_add_mask(Dims fd, const bf16* __restrict__ gc, int ldc, const bf16* __restrict__ gskip,
                                     int lds, int c, const bf16* __restrict__ act, int lda, bf16* __restrict__ out,
                                     int ldo) {
+  cudaGridDependencySynchronize();
   const Dims cd{fd.n, fd.d / 2, fd.h / 2, fd.w / 2};
   const unsigned V = (unsigned)fd.vox();
   for (unsigned v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
@@ -1553,7 +1566,9 @@ struct stp_unet {
   bf16 *ha[4] = {}, *e4 = nullptr, *u[3] = {}, *q[3] = {}, *hd[3] = {}, *d[3] = {};
   // gradients of activations
   bf16 *ga[4] = {}, *gb[4] = {}, *gu[3] = {};
-  float *y = nullptr, *gy = nullptr, *loss = nullptr, *h_loss = nullptr;
+  float *y = nullptr, *gy = nullptr, *loss = nullptr;
+  float* h_loss = nullptr;  // pinned: loss, then h_err
+  int* h_err = nullptr;
   float* wpart = nullptr;                                  // slices of the weight gradients (kWgradScratch)
   float *xin = nullptr, *tin = nullptr, *snorm = nullptr;  // normalised pairs, per-sample norms
   int guess_kernels = 0;                                   // kernels launched by one guess
@@ -1568,6 +1583,28 @@ struct stp_unet {
 
 namespace {
 
+// Launch as a programmatic dependent of the stream's previous kernel: the grid
+// is set up while that one's last blocks finish, and the kernel waits with
+// cudaGridDependencySynchronize before it touches memory.  A forward has 21
+// launches, a gradient 57, with gaps of 2 to 3 us between plain ones: 527 us a
+// forward of 128 x 64 x 128 and 1516 a gradient of 4 x 64 x 32 x 64, 471 and
+// 1362 this way (some 10 us of each by reading the error flag with the results).
+template <typename... K, typename... A>
+cudaError_t launch_dep(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 int ufail(stp_unet* n, int code, const std::string& m) {
   if (n) n->err = m;
   return code;
@@ -1579,11 +1616,11 @@ int ufail(stp_unet* n, int code, const std::string& m) {
     if (e_ != cudaSuccess) return ufail(n, STP_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-// after a synchronisation: did a tensor-core convolution give up waiting?
+// synchronises; did a tensor-core convolution give up waiting?
 int check_tc_timeout(stp_unet* n) {
-  int e = 0;
-  UTRY(n, cudaMemcpy(&e, n->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (e) return ufail(n, STP_ETIMEOUT, "a tensor-core convolution timed out waiting for its MMAs");
+  UTRY(n, cudaMemcpyAsync(n->h_err, n->d_err, sizeof(int), cudaMemcpyDeviceToHost, n->st));
+  UTRY(n, cudaStreamSynchronize(n->st));
+  if (*n->h_err) return ufail(n, STP_ETIMEOUT, "a tensor-core convolution timed out waiting for its MMAs");
   return STP_OK;
 }
 
@@ -1694,17 +1731,15 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
       UTRY(n, smem_limit_once(k_conv3_tz, (int)kTcSmemSm, donez));
       const TzPlan z = tz_plan(n, dm, cin, cout);
       const unsigned tiles = (unsigned)(V / (TC_TX * TC_TY * z.zt));
-      k_conv3_tz<<<std::min(tiles, 152u * z.per_sm), TZ_THREADS, z.smem, n->st>>>(dm, x, ldx, cin, wimg, bias, cout, y, ldy,
-                                                                                 relu, mask, ldm, z, n->d_err);
-      UTRY(n, cudaGetLastError());
+      UTRY(n, launch_dep(k_conv3_tz, std::min(tiles, 152u * z.per_sm), TZ_THREADS, z.smem, n->st, dm, x, ldx, cin, wimg,
+                         bias, cout, y, ldy, relu, mask, ldm, z, n->d_err));
       return STP_OK;
     }
     const unsigned tiles = (unsigned)(V / (TC_TX * TC_TY * p.zt));
     auto go = [&](auto kern, std::atomic<unsigned>& done) -> cudaError_t {
       if (cudaError_t e = smem_limit_once(kern, (int)kTcSmemSm, done)) return e;
-      kern<<<std::min(tiles, 152u * p.per_sm), TC_THREADS, p.smem, n->st>>>(dm, x, ldx, cin, wimg, bias, cout, y, ldy, relu,
-                                                                           mask, ldm, p, n->d_err);
-      return cudaGetLastError();
+      return launch_dep(kern, std::min(tiles, 152u * p.per_sm), TC_THREADS, p.smem, n->st, dm, x, ldx, cin, wimg, bias,
+                        cout, y, ldy, relu, mask, ldm, p, n->d_err);
     };
     static std::atomic<unsigned> done1{0u}, done2{0u}, done4{0u};
     UTRY(n, p.zt == 4 ? go(k_conv3_tc<4>, done4) : p.zt == 2 ? go(k_conv3_tc<2>, done2) : go(k_conv3_tc<1>, done1));
@@ -1723,9 +1758,8 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
   const bool ring = !(conv3_smem(cin, nt, false) <= kTcSmemMax && (conv3_smem(cin, nt, false) <= 56 * 1024 || blocks <= 152));
   auto go = [&](auto kern, std::atomic<unsigned>& done) -> cudaError_t {
     if (cudaError_t e = smem_limit_once(kern, (int)kTcSmemMax, done)) return e;
-    kern<<<dim3((unsigned)tiles, (unsigned)(cout / (8 * nt))), 128, conv3_smem(cin, nt, ring), n->st>>>(
-        dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask, ldm);
-    return cudaGetLastError();
+    return launch_dep(kern, dim3((unsigned)tiles, (unsigned)(cout / (8 * nt))), 128, conv3_smem(cin, nt, ring), n->st,
+                      dm, x, ldx, cin, wt, bias, cout, y, ldy, relu, mask, ldm);
   };
   static std::atomic<unsigned> done[6];
   if (ring)
@@ -1754,9 +1788,8 @@ cudaError_t wgrad_launch(const Dims& dm, const bf16* x, int ldx, int cin, const 
                          int slices, cudaStream_t st) {
   static std::atomic<unsigned> done{0u};
   if (cudaError_t e = smem_limit_once(k_wgrad3<OT, CT>, wg_smem(OT, CT), done)) return e;
-  k_wgrad3<OT, CT><<<dim3((unsigned)((cin / CT) * (cout / OT)), (unsigned)slices), 288, wg_smem(OT, CT), st>>>(
-      dm, x, ldx, cin, gz, ldg, cout, part);
-  return cudaGetLastError();
+  return launch_dep(k_wgrad3<OT, CT>, dim3((unsigned)((cin / CT) * (cout / OT)), (unsigned)slices), 288,
+                    wg_smem(OT, CT), st, dm, x, ldx, cin, gz, ldg, cout, part);
 }
 
 // weight and bias gradient of a 3x3x3 layer, stored (not added) into n->grad
@@ -1769,16 +1802,15 @@ int wgrad3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const b
   else
     UTRY(n, (ct == 48 ? wgrad_launch<16, 48> : ct == 32 ? wgrad_launch<16, 32> : wgrad_launch<16, 16>)(dm, x, ldx, cin, gz, ldg, cout, n->wpart, slices, n->st));
   const int total = 27 * cin * cout + cout;
-  k_wgrad_sum<<<(total + 31) / 32, 256, 0, n->st>>>(n->wpart, slices, cin, cout, n->grad + ly.woff, n->grad + ly.boff);
-  UTRY(n, cudaGetLastError());
+  UTRY(n, launch_dep(k_wgrad_sum, (total + 31) / 32, 256, 0, n->st, n->wpart, slices, cin, cout, n->grad + ly.woff,
+                     n->grad + ly.boff));
   return STP_OK;
 }
 int wgrad_in(stp_unet* n, const Dims& dm, const float* x, const bf16* gz, int ldg, const Layer& ly) {
   const int slices = std::min(wg_tiles(dm).count(dm.n), 4 * 152);
-  k_wgrad_in<<<slices, 256, 0, n->st>>>(dm, x, gz, ldg, n->wpart);
-  UTRY(n, cudaGetLastError());
-  k_wgrad_in_sum<<<(28 * 16 * 32 + 127) / 128, 128, 0, n->st>>>(n->wpart, slices, n->grad + ly.woff, n->grad + ly.boff);
-  UTRY(n, cudaGetLastError());
+  UTRY(n, launch_dep(k_wgrad_in, slices, 256, 0, n->st, dm, x, gz, ldg, n->wpart));
+  UTRY(n, launch_dep(k_wgrad_in_sum, (28 * 16 * 32 + 127) / 128, 128, 0, n->st, n->wpart, slices, n->grad + ly.woff,
+                     n->grad + ly.boff));
   return STP_OK;
 }
 
@@ -1820,8 +1852,8 @@ int forward(stp_unet* n, const float* x, int nb) {
     const int lde = l < 3 ? cu_width(l) : c;
     if ((rc = conv3(n, dm[l], n->ha[l], c, c, lb.wt, lb.img, n->theta + lb.boff, c, e, lde, 1, nullptr, 0))) return rc;
     if (l < 3) {
-      k_pool<<<dim3(blocks_for(dm[l + 1].vox()), c / 8), 256, 0, n->st>>>(dm[l], e, lde, c, n->q[l], c);
-      UTRY(n, cudaGetLastError());
+      UTRY(n, launch_dep(k_pool, dim3(blocks_for(dm[l + 1].vox()), c / 8), 256, 0, n->st, dm[l], e, lde, c, n->q[l],
+                         c));
       in = n->q[l];
       ldin = c;
     }
@@ -1831,8 +1863,8 @@ int forward(stp_unet* n, const float* x, int nb) {
   int cdeep = kCh[3];
   for (int l = 2; l >= 0; l--) {
     const int c = kCh[l], cw = cu_width(l);
-    k_upsample<<<blocks_for(dm[l].vox()), 256, 0, n->st>>>(dm[l + 1], deeper, cdeep, cdeep, n->u[l], cw);
-    UTRY(n, cudaGetLastError());
+    UTRY(n, launch_dep(k_upsample, blocks_for(dm[l].vox()), 256, 0, n->st, dm[l + 1], deeper, cdeep, cdeep, n->u[l],
+                       cw));
     const Layer& la = P[8 + 2 * (2 - l)];
     const Layer& lb = P[9 + 2 * (2 - l)];
     if ((rc = conv3(n, dm[l], n->u[l], cw, cw, la.wt, la.img, n->theta + la.boff, c, n->hd[l], c, 1, nullptr, 0))) return rc;
@@ -1841,24 +1873,23 @@ int forward(stp_unet* n, const float* x, int nb) {
     cdeep = c;
   }
   const Layer& lo = P[14];
-  k_conv_out<<<blocks_for(dm[0].vox()), 256, 0, n->st>>>(dm[0].vox(), n->d[0], 16, n->theta + lo.woff,
-                                                          n->theta + lo.boff, n->y);
-  UTRY(n, cudaGetLastError());
+  UTRY(n, launch_dep(k_conv_out, blocks_for(dm[0].vox()), 256, 0, n->st, dm[0].vox(), n->d[0], 16, n->theta + lo.woff,
+                     n->theta + lo.boff, n->y));
   return STP_OK;
 }
 
-// backward from gy (FP32 [V0]) into n->grad (zeroed here)
+// backward from gy (FP32 [V0]) into n->grad: the 3x3x3 layers store theirs, the
+// output layer's, the last 17 values, is zeroed here and added into
 int backward(stp_unet* n, const float* x, int nb) {
   Dims dm[4];
   for (int l = 0; l < 4; l++) dm[l] = Dims{nb, n->dm[l].d, n->dm[l].h, n->dm[l].w};
   const Layer* P = n->L.data();
   int rc;
-  UTRY(n, cudaMemsetAsync(n->grad, 0, sizeof(float) * n->np, n->st));
   // output layer -> gradient of the pre-activation of d1 (ga[0])
   const Layer& lo = P[14];
-  k_conv_out_bwd<<<blocks_for(dm[0].vox()), 256, 0, n->st>>>(dm[0].vox(), n->gy, n->d[0], 16, n->theta + lo.woff,
-                                                              n->ga[0], 16, n->grad + lo.woff, n->grad + lo.boff);
-  UTRY(n, cudaGetLastError());
+  UTRY(n, cudaMemsetAsync(n->grad + lo.woff, 0, sizeof(float) * (n->np - lo.woff), n->st));
+  UTRY(n, launch_dep(k_conv_out_bwd, blocks_for(dm[0].vox()), 256, 0, n->st, dm[0].vox(), n->gy, n->d[0], 16,
+                     n->theta + lo.woff, n->ga[0], 16, n->grad + lo.woff, n->grad + lo.boff));
   // decoder, level 0 up to 2; ga[l] holds the gradient of d_l's pre-activation
   for (int l = 0; l <= 2; l++) {
     const int c = kCh[l], cw = cu_width(l);
@@ -1874,9 +1905,8 @@ int backward(stp_unet* n, const float* x, int nb) {
     const int cd = kCh[l + 1];
     const bf16* act = l < 2 ? n->d[l + 1] : n->e4;
     bf16* out = l < 2 ? n->ga[l + 1] : n->ga[3];
-    k_upsample_bwd_mask<<<dim3(blocks_for(dm[l + 1].vox()), cd / 8), 256, 0, n->st>>>(dm[l + 1], n->gu[l], cw, cd, act, cd, out,
-                                                                              cd);
-    UTRY(n, cudaGetLastError());
+    UTRY(n, launch_dep(k_upsample_bwd_mask, dim3(blocks_for(dm[l + 1].vox()), cd / 8), 256, 0, n->st, dm[l + 1],
+                       n->gu[l], cw, cd, act, cd, out, cd));
   }
   // encoder, level 3 down to 0.  Buffers at level l: gz (gradient of e_l's
   // pre-activation), gha (of ha_l's), gq (of q_{l-1}, handed to level l-1).
@@ -1892,9 +1922,8 @@ int backward(stp_unet* n, const float* x, int nb) {
     if (l < 3) {
       // gz = (pool backward of the gradient of q_l + skip gradient) * (e_l > 0)
       const bf16* e = n->u[l] + kCh[l + 1];
-      k_pool_bwd_add_mask<<<blocks_for(dm[l].vox()), 256, 0, n->st>>>(dm[l], gq_in, c, n->gu[l] + kCh[l + 1],
-                                                                            cu_width(l), c, e, cu_width(l), gz, c);
-      UTRY(n, cudaGetLastError());
+      UTRY(n, launch_dep(k_pool_bwd_add_mask, blocks_for(dm[l].vox()), 256, 0, n->st, dm[l], gq_in, c,
+                         n->gu[l] + kCh[l + 1], cu_width(l), c, e, cu_width(l), gz, c));
     }
     // conv b: input ha[l]
     if ((rc = wgrad3(n, dm[l], n->ha[l], c, c, gz, c, c, lb))) return rc;
@@ -2048,7 +2077,8 @@ int stp_unet_create(int nmax, int nz, int ny, int nx, void* stream, stp_unet** o
   if (const char* e = std::getenv("STP_UNET_TC")) n->use_tc = std::atoi(e) != 0;
   if (const char* e = std::getenv("STP_UNET_TC_PLANES")) n->tc_planes = std::atoi(e);
   if (const char* e = std::getenv("STP_UNET_MMA_NT")) n->mma_nt = std::atoi(e);
-  if (rc == STP_OK && cudaMallocHost((void**)&n->h_loss, sizeof(float)) != cudaSuccess) rc = STP_ENOMEM;
+  if (rc == STP_OK && cudaMallocHost((void**)&n->h_loss, sizeof(float) + sizeof(int)) != cudaSuccess) rc = STP_ENOMEM;
+  if (rc == STP_OK) n->h_err = reinterpret_cast<int*>(n->h_loss + 1);
   if (rc == STP_OK) {
     cudaMemsetAsync(n->theta, 0, sizeof(float) * n->np, n->st);
     cudaMemsetAsync(n->m, 0, sizeof(float) * n->np, n->st);
@@ -2102,7 +2132,6 @@ int stp_unet_forward(stp_unet* n, const float* x, float* y, int nb) {
   int rc = forward(n, x, nb);
   if (rc) return rc;
   UTRY(n, cudaMemcpyAsync(y, n->y, sizeof(float) * n->dm[0].vox() / n->nmax * nb, cudaMemcpyDeviceToDevice, n->st));
-  UTRY(n, cudaStreamSynchronize(n->st));
   return check_tc_timeout(n);
 }
 
@@ -2118,9 +2147,9 @@ int stp_unet_gradient(stp_unet* n, const float* x, const float* target, int nb, 
   if ((rc = backward(n, x, nb))) return rc;
   if (grad) UTRY(n, cudaMemcpyAsync(grad, n->grad, sizeof(float) * n->np, cudaMemcpyDeviceToDevice, n->st));
   UTRY(n, cudaMemcpyAsync(n->h_loss, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->st));
-  UTRY(n, cudaStreamSynchronize(n->st));
-  if (loss) *loss = *n->h_loss;
-  return check_tc_timeout(n);
+  rc = check_tc_timeout(n);
+  if (loss && (rc == STP_OK || rc == STP_ETIMEOUT)) *loss = *n->h_loss;
+  return rc;
 }
 
 int stp_unet_train_step(stp_unet* n, const float* x, const float* target, int nb, float lr, float* loss) {
@@ -2232,9 +2261,9 @@ int stp_unet_eval_pairs(stp_unet* n, const float* r, const float* dp, int nb, fl
   k_mse<<<std::min(blocks_for(Vs * nb), 4 * 152), 256, 0, n->st>>>(Vs * nb, n->y, n->tin, n->gy, n->loss);
   UTRY(n, cudaGetLastError());
   UTRY(n, cudaMemcpyAsync(n->h_loss, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->st));
-  UTRY(n, cudaStreamSynchronize(n->st));
-  if (loss) *loss = *n->h_loss;
-  return check_tc_timeout(n);
+  rc = check_tc_timeout(n);
+  if (loss && (rc == STP_OK || rc == STP_ETIMEOUT)) *loss = *n->h_loss;
+  return rc;
 }
 
 }  // extern "C"
