@@ -734,7 +734,6 @@ def run_ours(args):
     word = 4 if args.precision == "fp32" else 8
     kern = sweep_kernel(cfg, args.precision, ch)
     words = 2 if two_colour(cfg, args.precision) else 3
-    # (the recorded DRAM bytes are a Jacobi sweep's)
     tkey = "%s_%s_%s" % ("two_colour" if words == 2 else "zline_sweep" if cfg.get("zline") else "point_sweep",
                          args.precision, args.workload)
     roof = sweep_roofline(words, word, cells, r, kern, peak, tkey)
