@@ -668,9 +668,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
 // us at 128 x 64 x 128, a tap at a time (k_conv3_tc with resident weights) /
 // this: 16 -> 16 49 / 38, 48 -> 16 113 / 70; half that size 16 -> 32 20 / 16, 32
 // -> 32 21 / 19, 96 -> 32 65 / 46; a quarter 32 -> 64 17 / 9.5.  16 -> 16 takes
-// 26 without MMAs and stores, 16 with no loads either: what bounds it is what a
-// plane costs its MMA thread (wait, descriptors, commit: some 0.2 us) and the
-// first loads and last stores of a block.  Three blocks an SM (64 registers) 39.
+// 26 without MMAs and stores, 16 with no loads either, 29 without loads alone:
+// the latencies of a block's chain of planes add up.  Not faster: two planes a
+// halo stage 40, 16 planes a tile (one accumulator stage) 44, 4 planes 41, three
+// blocks an SM (64 registers) 39.
 struct TzPlan {
   int zt;      // planes a tile
   int hs;      // halo stages (planes)
