@@ -423,6 +423,8 @@ Geom<T> geom_from(const stp_handle* h, T* pack) {
   g.tlb = pack + 15 * L;
   g.pf = pack + 16 * L;
   g.pe = pack + 17 * L;
+  g.lf = pack + 18 * L;
+  g.lb = pack + 19 * L;
   // the packed level coefficients follow the kMetricArrays arrays (offset
   // 80 L bytes: 16-byte aligned)
   if constexpr (sizeof(T) == sizeof(float)) g.lz4 = reinterpret_cast<const float4*>(pack + kMetricArrays * L);
@@ -494,16 +496,21 @@ std::vector<double> metric_pack(const stp_config& c) {
       }
     }
   }
-  // products of the elimination's and the substitution's coefficients inside
-  // the FP64 z-line chunks
+  // the twisted factorisation on undivided values (Geom::lf, lb), and the
+  // products of its coefficients inside the FP64 z-line chunks
+  for (int k = 0; k < nz; k++) {
+    const double dn = k > 0 ? cdn[k] * m[13 * L + k - 1] : 0.0, up = k < nz - 1 ? cup[k] * m[13 * L + k + 1] : 0.0;
+    m[18 * L + k] = k <= nz / 2 ? dn : up;
+    m[19 * L + k] = k <= nz / 2 ? up : dn;
+  }
   if (const int nch = line_f64_chunks(c.nx, c.ny, nz)) {
     for (int ch = 0; ch < nch; ch++) {
       const int k0 = line_chunk_start(ch, nch, nz), k1 = line_chunk_start(ch + 1, nch, nz);
       const bool lower = ch < nch / 2;
       const int f0 = ch == nch / 2 ? k0 + 1 : k0;  // the twist level stays out
       double up = 1.0, dn = 1.0;
-      for (int k = f0; k < k1; k++) m[(lower ? 16 : 17) * L + k] = up *= m[(lower ? 14 : 15) * L + k];
-      for (int k = k1 - 1; k >= f0; k--) m[(lower ? 17 : 16) * L + k] = dn *= m[(lower ? 15 : 14) * L + k];
+      for (int k = f0; k < k1; k++) m[(lower ? 16 : 17) * L + k] = up *= m[(lower ? 18 : 19) * L + k];
+      for (int k = k1 - 1; k >= f0; k--) m[(lower ? 17 : 16) * L + k] = dn *= m[(lower ? 19 : 18) * L + k];
     }
   }
   for (int k = 0; k <= nz; k++) {

@@ -70,142 +70,158 @@ __global__ void __launch_bounds__(128) k_sweep_f64(Geom<double> g, const double*
   out[q] = fma(om1, pc, t);
 }
 
-// One z-line Jacobi-SOR sweep, p' = p + omega (p^L - p), the columns solved in
-// registers in level chunks as in k_line_sweep_chunk (kernels_poisson.cu).  A
-// block takes CW columns of a row x NCH chunks of at most LMAX levels.  The right-hand side is that of the line value itself,
-//   A p^L = (p_{i+1} + p_{i-1})/dx^2 + (p_{j+1} + p_{j-1})/dy^2 - b,
-// six FP64 operations a cell with the pivot (thirteen for A^-1 (b - L p)), and
-// the running products of the chunk's coefficients come from tables (pf, pe),
-// so that a cell costs twelve FP64 operations in all.  Every chunk a carry
-// passes is another multiply-add, so the chunks are long (line_f64_chunks);
-// LMAX is the least even bound of their levels, because a predicated
-// operation past the chunk's end takes its slot on the FP64 pipe all the same.
+// One z-line Jacobi-SOR sweep, p' = p - omega A^-1 (b - L p), the columns solved
+// in registers in level chunks as in k_line_sweep_chunk (kernels_poisson.cu).  A
+// block takes CW columns of a row x NCH chunks of at most LMAX levels.
+//
+// The right-hand side is the residual, in differences of neighbours: solved for
+// the line value itself (A p^L = sum of the x and y neighbours - b: six
+// operations a cell) it would round with the size of S p, and solves of smooth
+// fields stall 1.7 to 2.5 times higher (64 x 32 x 192, stretch 2: 1.0e-11 of ||b||
+// against 4.2e-12).  A difference serves both its cells where it costs less than
+// it saves: along the chunk in registers, along x by shuffle, the difference
+// into the block's first column being taken for all levels at once, a lane a
+// level.  The elimination runs on undivided values (Geom::lf, lb), so that the
+// pivot joins omega in one coefficient a level: fifteen operations a cell.  us a
+// sweep, line values with every thread walking its own carries (twelve
+// operations) / this: 32 x 16 x 32 6.3 / 5.5, 96 x 48 x 64 11.1 / 11.4, 64 x 30 x
+// 100 13.9 / 11.4, 64 x 32 x 192 18.1 / 16.9, and where the FP64 pipe alone
+// bounds it 112 x 56 x 112 22.4 / 25.1, 128 x 64 x 128 31.6 / 38.2 (of which 512
+// blocks on 152 SMs leave a fifth idle); the lock-step kernel took 41.2 at 96 x 48
+// x 64.
+//
+// A thread counts its levels from the wall's side of the chunk to the twist
+// level's, so both sides run the same code.  What enters a chunk is walked chunk
+// by chunk by one warp, a lane a column and side (by every thread for itself it
+// took as many operations as the columns' own recurrences).  Chunks stay long
+// (line_f64_chunks): each is a step of that walk.  LMAX is the most levels a
+// chunk has, no more, because an operation past the chunk's end takes its slot
+// on the FP64 pipe all the same.
 template <int CW, int NCH, int LMAX>
 __global__ void __launch_bounds__(CW * NCH) k_line_f64(Geom<double> g, const double* __restrict__ p,
                                                        const double* __restrict__ b, double omega,
                                                        double* __restrict__ out) {
   constexpr int H = NCH / 2;
-  __shared__ double ZB[NCH][CW], WB[NCH][CW], XT[CW];
+  static_assert(CW == 16 && LMAX <= CW && H % 2 == 0, "a warp holds two chunks of one side, a lane a level");
+  extern __shared__ double wt[];  // [nz] omega / pivot
+  __shared__ double EB[NCH][CW], CB[NCH][CW], YL[CW], XT[CW], PF[NCH], PE[NCH];
   const int nx = g.nx, ny = g.ny, nz = g.nz, t = nz >> 1;
-  const int u = threadIdx.x % CW, c = threadIdx.x / CW;
-  const int nxb = (nx + CW - 1) / CW, j = blockIdx.x / nxb, i0 = (blockIdx.x % nxb) * CW + u;
-  const bool act = i0 < nx;
-  const int i = act ? i0 : nx - 1;
-  const unsigned plane = (unsigned)nx * ny, rc = (unsigned)j * nx + i;
-  const unsigned xe = (unsigned)j * nx + (i + 1 == nx ? 0 : i + 1), xw = (unsigned)j * nx + (i == 0 ? nx - 1 : i - 1);
+  const int u = threadIdx.x % CW, c = threadIdx.x / CW, half = threadIdx.x & CW;
+  const int nxb = (nx + CW - 1) / CW, j = blockIdx.x / nxb, ib = (blockIdx.x % nxb) * CW;
+  const bool act = ib + u < nx;
+  const int i = act ? ib + u : nx - 1;
+  const unsigned plane = (unsigned)nx * ny, row = (unsigned)j * nx, rc = row + i;
+  const unsigned xe = row + (i + 1 == nx ? 0 : i + 1), x0 = row + ib, xw = row + (ib == 0 ? nx - 1 : ib - 1);
   const unsigned yn = (unsigned)(j + 1 == ny ? 0 : j + 1) * nx + i, ys = (unsigned)(j == 0 ? ny - 1 : j - 1) * nx + i;
   const bool lower = c < H;
   const int k0 = line_chunk_start(c, NCH, nz), k1 = line_chunk_start(c + 1, NCH, nz), L = k1 - k0;
-  const bool twist = c == H;
-  // the first level that the elimination and the substitution run over
-  const int q0 = twist ? 1 : 0;
-  double G[LMAX];
+  const bool twist = c == H;  // holds the twist level t = k0, its last; it has LMAX levels
+  const int Le = twist ? LMAX - 1 : L;  // levels the elimination runs over
+  // level q of the chunk, within the column
+  auto level = [&](int q) { return min(max(lower ? k0 + q : k1 - 1 - q, 0), nz - 1); };
+  auto lev = [&](int q) { return (unsigned)level(q) * plane; };
+  for (int k = threadIdx.x; k < nz; k += CW * NCH) wt[k] = omega * __ldg(g.tli + k);
+  if (u == 0) {
+    PF[c] = L > 0 ? __ldg(g.pf + level(L - 1)) : 1.0;
+    PE[c] = L > 0 ? __ldg(g.pe + level(0)) : 1.0;
+  }
+  const double* cin = lower ? g.cup : g.cdn;   // coupling to level q + 1
+  const double* cout = lower ? g.cdn : g.cup;  // to level q - 1 (zero at the wall)
+  double C[LMAX + 1], D[LMAX], G[LMAX];
   const double idx2 = g.idx2, idy2 = g.idy2;
   cudaGridDependencySynchronize();
 #pragma unroll
-  for (int q = 0; q < LMAX; q++)
+  for (int q = 0; q <= LMAX; q++) C[q] = __ldg(p + lev(q) + rc);
+#pragma unroll
+  for (int q = 0; q < LMAX; q++) D[q] = __ldg(p + lev(q) + xe) - C[q];
+  const unsigned le = lev(u < LMAX ? u : 0);
+  const double edge = __ldg(p + le + x0) - __ldg(p + le + xw);
+  double dz = C[0] - __ldg(p + lev(-1) + rc);
+#pragma unroll
+  for (int q = 0; q < LMAX; q++) {
+    const double first = __shfl_sync(0xffffffffu, edge, half + q);
+    double dw = __shfl_up_sync(0xffffffffu, D[q], 1);
+    dw = u == 0 ? first : dw;
     if (q < L) {
-      const unsigned lev = (unsigned)(k0 + q) * plane;
-      double r = idx2 * (__ldg(p + lev + xe) + __ldg(p + lev + xw));
-      r = fma(idy2, __ldg(p + lev + yn) + __ldg(p + lev + ys), r) - __ldg(b + lev + rc);
-      G[q] = r * __ldg(g.tli + k0 + q);
+      const unsigned l = lev(q);
+      const int k = level(q);
+      double r = fma(-idx2, D[q] - dw, __ldg(b + l + rc));
+      r = fma(-idy2, (__ldg(p + l + yn) - C[q]) + (__ldg(p + l + ys) - C[q]), r);
+      r = fma(__ldg(cout + k), dz, r);
+      dz = C[q + 1] - C[q];
+      G[q] = fma(-__ldg(cin + k), dz, r);
     }
-  // elimination inside the chunk: upward below t, downward above it
-  if (lower) {
-    double z = 0.0;
+  }
+  // elimination inside the chunk
+  {
+    double z = 0 < Le ? G[0] : 0.0;
+#pragma unroll
+    for (int q = 1; q < LMAX; q++)
+      if (q < Le) G[q] = z = fma(__ldg(g.lf + level(q)), z, G[q]);
+    EB[c][u] = z;
+  }
+  __syncthreads();
+  // the values entering the chunks, from the walls; the last one from below
+  // enters the twist level
+  if (threadIdx.x < 32) {
+    double carry = 0.0;
+#pragma unroll
+    for (int s = 0; s < H; s++) {
+      const int cc = half ? NCH - 1 - s : s;
+      CB[cc][u] = carry;
+      carry = fma(PF[cc], carry, EB[cc][u]);
+    }
+    if (!half) YL[u] = carry;
+  }
+  __syncthreads();
+  {
+    const double carry = CB[c][u];
 #pragma unroll
     for (int q = 0; q < LMAX; q++)
-      if (q < L) G[q] = z = fma(__ldg(g.tlf + k0 + q), z, G[q]);
-    ZB[c][u] = z;
-  } else {
-    double z = 0.0;
+      if (q < Le) G[q] = fma(__ldg(g.pf + level(q)), carry, G[q]);
+    if (twist) {
+      // lf: from y_{t-1}; lb: from y_{t+1} (zero if t is the top level)
+      const double yup = LMAX > 1 ? G[LMAX > 1 ? LMAX - 2 : 0] : carry;
+      G[LMAX - 1] = fma(__ldg(g.lb + t), yup, fma(__ldg(g.lf + t), YL[u], G[LMAX - 1]));
+      XT[u] = G[LMAX - 1];
+    }
+  }
+  // substitution inside the chunk (the twist chunk starts from X_t itself)
+  {
+    double w = 0.0;
 #pragma unroll
     for (int q = LMAX - 1; q >= 0; q--)
-      if (q < L && q >= q0) G[q] = z = fma(__ldg(g.tlf + k0 + q), z, G[q]);
-    ZB[c][u] = z;
+      if (q < L) G[q] = w = q == LMAX - 1 ? G[q] : fma(__ldg(g.lb + level(q)), w, G[q]);
+    EB[c][u] = w;
   }
   __syncthreads();
-  // the value entering the chunk, from the walls
-  {
-    double carry = 0.0;
-    if (lower) {
-      for (int cc = 0; cc < c; cc++) {
-        const int e = line_chunk_start(cc + 1, NCH, nz);
-        if (e > line_chunk_start(cc, NCH, nz)) carry = fma(__ldg(g.pf + e - 1), carry, ZB[cc][u]);
-      }
-    } else {
-      for (int cc = NCH - 1; cc > c; cc--) {
-        const int e = line_chunk_start(cc, NCH, nz);
-        if (e < line_chunk_start(cc + 1, NCH, nz)) carry = fma(__ldg(g.pf + e), carry, ZB[cc][u]);
-      }
-    }
+  // the values entering the chunks, from the twist level (above it from the
+  // top of the twist chunk, which is complete)
+  if (threadIdx.x < 32) {
+    double carry = half ? 0.0 : XT[u];
 #pragma unroll
-    for (int q = 0; q < LMAX; q++)
-      if (q < L && q >= q0) G[q] = fma(__ldg(g.pf + k0 + q), carry, G[q]);
-    if (twist) {
-      double ylow = 0.0;  // y_{t-1}
-      for (int cc = 0; cc < H; cc++) {
-        const int e = line_chunk_start(cc + 1, NCH, nz);
-        if (e > line_chunk_start(cc, NCH, nz)) ylow = fma(__ldg(g.pf + e - 1), ylow, ZB[cc][u]);
-      }
-      const double yup = L >= 2 ? G[1] : carry;  // y_{t+1}
-      const double ft = t > 0 ? __ldg(g.tlf + t) : 0.0, et = t < nz - 1 ? __ldg(g.tlb + t) : 0.0;
-      G[0] = fma(et, yup, fma(ft, ylow, G[0]));
-      XT[u] = G[0];
+    for (int s = 0; s < H; s++) {
+      const int cc = half ? H + s : H - 1 - s;
+      CB[cc][u] = carry;
+      carry = fma(PE[cc], carry, EB[cc][u]);
     }
-  }
-  // substitution inside the chunk: downward below t, upward above it (the
-  // twist chunk starts from x_t itself)
-  {
-    double w = twist ? G[0] : 0.0;
-    if (lower) {
-#pragma unroll
-      for (int q = LMAX - 1; q >= 0; q--)
-        if (q < L) G[q] = w = fma(__ldg(g.tlb + k0 + q), w, G[q]);
-    } else {
-#pragma unroll
-      for (int q = 0; q < LMAX; q++)
-        if (q < L && q >= q0) G[q] = w = fma(__ldg(g.tlb + k0 + q), w, G[q]);
-    }
-    WB[c][u] = w;
   }
   __syncthreads();
-  {
-    double carry = XT[u];
-    if (lower) {
-      for (int cc = H - 1; cc > c; cc--) {
-        const int e = line_chunk_start(cc, NCH, nz);
-        if (e < line_chunk_start(cc + 1, NCH, nz)) carry = fma(__ldg(g.pe + e), carry, WB[cc][u]);
-      }
-    } else if (!twist) {
-      carry = WB[H][u];
-      for (int cc = H + 1; cc < c; cc++) {
-        const int e = line_chunk_start(cc + 1, NCH, nz);
-        if (e > line_chunk_start(cc, NCH, nz)) carry = fma(__ldg(g.pe + e - 1), carry, WB[cc][u]);
-      }
-    }
-    if (!twist) {
+  const double carry = CB[c][u];
 #pragma unroll
-      for (int q = 0; q < LMAX; q++)
-        if (q < L) G[q] = fma(__ldg(g.pe + k0 + q), carry, G[q]);
+  for (int q = 0; q < LMAX; q++)
+    if (q < L) {
+      if (!twist) G[q] = fma(__ldg(g.pe + level(q)), carry, G[q]);
+      if (act) out[lev(q) + rc] = fma(-wt[level(q)], G[q], C[q]);
     }
-    if (act) {
-#pragma unroll
-      for (int q = 0; q < LMAX; q++)
-        if (q < L) {
-          const unsigned a = (unsigned)(k0 + q) * plane + rc;
-          const double pv = __ldg(p + a);
-          out[a] = fma(omega, G[q] - pv, pv);
-        }
-    }
-  }
 }
 
 template <typename... P, typename... A>
-cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t s, A... a) {
+cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -227,29 +243,28 @@ cudaError_t launch_sweep_f64(const Geom<double>& g, const double* p, const doubl
                              double* out, cudaStream_t s) {
   const unsigned n = (unsigned)g.nx * g.ny * g.nz;
   const double om1 = 1.0 - omega;
-  return launch_dep(tab ? k_sweep_f64<true> : k_sweep_f64<false>, dim3((n + 127) / 128), dim3(128), s, g, p, b, omega,
+  return launch_dep(tab ? k_sweep_f64<true> : k_sweep_f64<false>, dim3((n + 127) / 128), dim3(128), 0, s, g, p, b, omega,
                     om1, tab, out);
 }
 
 namespace {
-// Columns a block.  us a sweep at 32 / 16 / 8: 96 x 48 x 64 10.9 / 11.1 / 11.5,
-// 64 x 30 x 100 18.8 / 13.8 / 14.1, 112 x 56 x 112 28.6 / 22.5 / 23.5, 32 x 16
-// x 32 7.3 / 6.5 / 6.4 (the lock-step shared-memory kernel: 41.2, 35.2, 39.1,
-// 21.7): 32 leave SMs without a block or a last wave nearly empty.
+// Columns a block.  us a sweep at 32 / 16 / 8 (line values): 96 x 48 x 64 10.9 /
+// 11.1 / 11.5, 64 x 30 x 100 18.8 / 13.8 / 14.1, 112 x 56 x 112 28.6 / 22.5 / 23.5,
+// 32 x 16 x 32 7.3 / 6.5 / 6.4: 32 leave SMs without a block or a last wave nearly
+// empty.
 constexpr int kLineCols = 16;
 
 template <int NCH>
 cudaError_t line_nch(const Geom<double>& g, const double* p, const double* b, double omega, double* out, cudaStream_t s) {
   const dim3 blocks((unsigned)(((g.nx + kLineCols - 1) / kLineCols) * g.ny)), threads(kLineCols * NCH);
-  switch ((line_f64_levels(g.nz, NCH) + 1) / 2) {
-    case 1: return launch_dep(k_line_f64<kLineCols, NCH, 2>, blocks, threads, s, g, p, b, omega, out);
-    case 2: return launch_dep(k_line_f64<kLineCols, NCH, 4>, blocks, threads, s, g, p, b, omega, out);
-    case 3: return launch_dep(k_line_f64<kLineCols, NCH, 6>, blocks, threads, s, g, p, b, omega, out);
-    case 4: return launch_dep(k_line_f64<kLineCols, NCH, 8>, blocks, threads, s, g, p, b, omega, out);
-    case 5: return launch_dep(k_line_f64<kLineCols, NCH, 10>, blocks, threads, s, g, p, b, omega, out);
-    case 6: return launch_dep(k_line_f64<kLineCols, NCH, 12>, blocks, threads, s, g, p, b, omega, out);
+#define LEVELS(L) \
+  case L: return launch_dep(k_line_f64<kLineCols, NCH, L>, blocks, threads, sizeof(double) * g.nz, s, g, p, b, omega, out);
+  switch (line_f64_levels(g.nz, NCH)) {
+    LEVELS(1) LEVELS(2) LEVELS(3) LEVELS(4) LEVELS(5) LEVELS(6)
+    LEVELS(7) LEVELS(8) LEVELS(9) LEVELS(10) LEVELS(11) LEVELS(12)
     default: return cudaErrorInvalidValue;
   }
+#undef LEVELS
 }
 }  // namespace
 

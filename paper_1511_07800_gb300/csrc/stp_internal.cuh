@@ -48,9 +48,13 @@ struct Geom {
   const T* tli;    // [nz]    1/m_k (k < t), 1/gamma_t (k = t), 1/m'_k (k > t)
   const T* tlf;    // [nz]    elimination: cdn_k/m_k (k < t), cdn_t/gamma_t, cup_k/m'_k (k > t)
   const T* tlb;    // [nz]    substitution: cup_k/m_k (k < t), cup_t/gamma_t, cdn_k/m'_k (k > t)
-  // FP64 z-line chunks (line_chunk_start): products of the elimination's
-  // (pf) and the substitution's (pe) coefficients from the level where the
-  // recurrence enters the chunk through level k (the twist level left out)
+  // FP64 z-line chunks (line_chunk_start), the same factorisation on values
+  // not yet divided by their pivot: elimination y_k = r_k + lf_k y_{k-+1},
+  // substitution X_k = y_k + lb_k X_{k+-1}, x_k = tli_k X_k
+  const T* lf;     // [nz]    cdn_k tli_{k-1} (k <= t), cup_k tli_{k+1} (k > t)
+  const T* lb;     // [nz]    cup_k tli_{k+1} (k <= t), cdn_k tli_{k-1} (k > t)
+  // products of lf (pf) and of lb (pe) from the level where the recurrence
+  // enters the chunk through level k (the twist level left out)
   const T* pf;     // [nz]
   const T* pe;     // [nz]
   // FP32 only (null in FP64): {cup_k, cdn_k, tli_k, tlf_k} packed per level,
