@@ -603,7 +603,7 @@ cudaError_t launch_cluster(stp_handle* h, float* d, const float* r, int M, cudaS
 
 // sweep m of a cycle of point Jacobi-SOR sweeps
 cudaError_t launch_jacobi(stp_handle* h, const double* p, const double* b, int m, double* out, cudaStream_t s) {
-  return launch_sweep_f64(h->g64, p, b, h->omega[m], h->sweep_tab ? h->sweep_tab + (size_t)5 * h->nz * m : nullptr, out, s);
+  return launch_sweep_f64(h->g64, p, b, h->omega[m], h->sweep_tab ? h->sweep_tab + (size_t)6 * h->nz * m : nullptr, out, s);
 }
 cudaError_t launch_jacobi(stp_handle* h, const float* p, const float* b, int m, float* out, cudaStream_t s) {
   return launch_sweep_f32(h->g32, p, b, (float)h->omega[m], out, s);
@@ -1436,9 +1436,9 @@ int stp_init(const stp_config* cfg, stp_handle** out) {
   };
   const int L = h->nz + 1;
   // the metrics and, behind them, the level coefficients of the FP64 point
-  // sweeps (up to 64 MB; beyond it the sweeps form them) and the schedule
-  size_t tab_words = (size_t)5 * h->nz * h->omega.size();
-  if (h->prec != STP_FP64 || cfg->zline || tab_words > (size_t)8 << 20) tab_words = 0;
+  // sweeps (up to 80 MB; beyond it the sweeps form them) and the schedule
+  size_t tab_words = (size_t)6 * h->nz * h->omega.size();
+  if (h->prec != STP_FP64 || cfg->zline || tab_words > (size_t)10 << 20) tab_words = 0;
   A((void**)&h->m64, sizeof(double) * ((size_t)kMetricArrays * L + tab_words + (tab_words ? h->omega.size() : 0)));
   if (tab_words && h->m64) h->sweep_tab = h->m64 + (size_t)kMetricArrays * L;
   A((void**)&h->m32, sizeof(float) * (kMetricArrays + 4) * L);

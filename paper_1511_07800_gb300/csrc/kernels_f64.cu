@@ -12,28 +12,43 @@
 namespace stp {
 namespace {
 
-// tab[(m nz + k) 5 ..]: omega_m/S_k times 1/dx^2, 1/dy^2, cup_k, cdn_k, 1
+// tab[(m nz + k) 6 ..]: omega_m/S_k times 1/dx^2, 1/dy^2, cup_k, cdn_k, 1, and
+// 1 - omega_m as 1 less the six neighbours' coefficients as rounded, so that a
+// sweep keeps a constant
 __global__ void k_sweep_table(Geom<double> g, const double* __restrict__ omega, int M, double* __restrict__ tab) {
   const long long n = (long long)M * g.nz;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
     const int m = (int)(q / g.nz), k = (int)(q - (long long)m * g.nz);
     const double w = omega[m] * g.iS[k];
-    double* t = tab + 5 * q;
+    double* t = tab + 6 * q;
     t[0] = w * g.idx2;
     t[1] = w * g.idy2;
     t[2] = w * g.cup[k];
     t[3] = w * g.cdn[k];
     t[4] = w;
+    double hi = 1.0, lo = 0.0;
+    for (int i = 0; i < 4; i++) {
+      const double a = i < 2 ? -2.0 * t[i] : -t[i], s = hi + a, z = s - hi;
+      lo += (hi - (s - z)) + (a - z);
+      hi = s;
+    }
+    t[5] = hi + lo;
   }
 }
 
 // One Jacobi-SOR sweep: p + omega (p^J - p) with p^J = (sum_nb c p_nb - b)/S,
 // as (1 - omega) p + sum_nb (omega c/S) p_nb - (omega/S) b: eight FP64
-// operations a cell (ten with the coefficients applied one by one).  om1 =
-// 1 - omega.  Without a table (TAB false) a thread forms the coefficients; both
-// in one kernel would cost their predicated multiplications either way.
+// operations a cell (ten with the coefficients applied one by one).  The
+// right-hand side comes first and the z couplings, largest next to stretched
+// walls, last: every rounding is of a partial sum, and these stay small the
+// longest.  The table's coefficient of p makes the coefficients of p and its
+// neighbours sum to one as they are rounded.  Without both, solves stall 1.15
+// times higher than with ten operations (1.3 to 1.5 at stretch 3), with them no
+// higher.  Without a table (TAB false) a thread forms the coefficients, that of p
+// as om1 = 1 - omega; both in one kernel would cost their predicated
+// multiplications either way.
 // us a sweep, ten operations on double2 units / this: 128 x 64 x 128 19.2 /
-// 16.5 (505 Gop/s of the 500-545 the FP64 pipe gives), 112 x 56 x 112 15.4 /
+// 16.3 (505 Gop/s of the 500-545 the FP64 pipe gives), 112 x 56 x 112 15.4 /
 // 11.5, 64^3 6.5 / 5.2, 32 x 16 x 32 2.78 / 1.76 (its rows left half a warp of
 // double2 units idle).  Two cells a thread at eight operations: 16.6, 13.2,
 // 5.5, 2.25.
@@ -46,11 +61,11 @@ __global__ void __launch_bounds__(128) k_sweep_f64(Geom<double> g, const double*
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned row = q / nx, i = q - row * nx, k = row / ny, j = row - k * ny;
   const bool act = k < nz;
-  double ax = 0, ay = 0, au = 0, ad = 0, ab = 0;
+  double ax = 0, ay = 0, au = 0, ad = 0, ab = 0, ac = om1;
   if (act) {
     if constexpr (TAB) {
-      ax = __ldg(tab + 5 * k), ay = __ldg(tab + 5 * k + 1), au = __ldg(tab + 5 * k + 2);
-      ad = __ldg(tab + 5 * k + 3), ab = __ldg(tab + 5 * k + 4);
+      ax = __ldg(tab + 6 * k), ay = __ldg(tab + 6 * k + 1), au = __ldg(tab + 6 * k + 2);
+      ad = __ldg(tab + 6 * k + 3), ab = __ldg(tab + 6 * k + 4), ac = __ldg(tab + 6 * k + 5);
     } else {
       ab = omega * __ldg(g.iS + k);
       ax = ab * g.idx2, ay = ab * g.idy2, au = ab * __ldg(g.cup + k), ad = ab * __ldg(g.cdn + k);
@@ -62,12 +77,12 @@ __global__ void __launch_bounds__(128) k_sweep_f64(Geom<double> g, const double*
   const double e = __ldg(p + (i + 1 == nx ? q + 1 - nx : q + 1)), w = __ldg(p + (i == 0 ? q + nx - 1 : q - 1));
   const double n = __ldg(p + (j + 1 == ny ? q + nx - plane : q + nx)), s = __ldg(p + (j == 0 ? q + plane - nx : q - nx));
   const double u = k + 1 < nz ? __ldg(p + q + plane) : pc, d = k > 0 ? __ldg(p + q - plane) : pc;  // coefficient 0 there
-  double t = ax * (e + w);
+  double t = -ab * __ldg(b + q);
+  t = fma(ax, e + w, t);
   t = fma(ay, n + s, t);
   t = fma(au, u, t);
   t = fma(ad, d, t);
-  t = fma(-ab, __ldg(b + q), t);
-  out[q] = fma(om1, pc, t);
+  out[q] = fma(ac, pc, t);
 }
 
 // One z-line Jacobi-SOR sweep, p' = p - omega A^-1 (b - L p), the columns solved

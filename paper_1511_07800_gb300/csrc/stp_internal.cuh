@@ -231,7 +231,7 @@ cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* 
                              cudaStream_t s);
 
 // FP64 sweeps (kernels_f64.cu).  tab: the level coefficients of this sweep's
-// factor (5 nz doubles of launch_sweep_table's M), null: formed in the kernel.
+// factor (6 nz doubles of launch_sweep_table's M), null: formed in the kernel.
 cudaError_t launch_sweep_table(const Geom<double>& g, const double* omega, int M, double* tab, cudaStream_t s);
 cudaError_t launch_sweep_f64(const Geom<double>& g, const double* p, const double* b, double omega, const double* tab,
                              double* out, cudaStream_t s);
