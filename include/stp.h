@@ -27,7 +27,9 @@
  * channel of at least 2^21 cells with even nx and ny (z lines: nz <= 192) runs
  * two-colour sweeps: a sweep relaxes one colour of cells (z lines: of columns)
  * in place, with the Chebyshev factors of a two-coloured grid, so that a cycle
- * of M sweeps gains what M Jacobi sweeps do.  STP_SRJ_COLOURS=0 at stp_init
+ * of M sweeps gains what M Jacobi sweeps do; its tile shape is picked by timing
+ * as below (STP_COLOUR_VARIANT=<0..2> forces one), and results do not depend on
+ * it.  STP_SRJ_COLOURS=0 at stp_init
  * keeps Jacobi sweeps, as do schedules of the caller's own, a learned guess,
  * STP_SWEEP_VARIANT, STP_LINE_VARIANT=0 and the persistent cycles.  With STP_PERSISTENT=1 at
  * stp_init an FP32 cycle instead runs as one persistent cooperative kernel

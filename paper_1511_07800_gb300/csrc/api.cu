@@ -764,10 +764,19 @@ int pick_variant(const std::vector<std::pair<int, float>>& timed, float* us) {
   return 0;
 }
 
-// Autotuner of the two-colour sweep: the levels a thread relaxes, timed as
-// tune_sweep times its tiles; cached per device, grid and kind.
+// Autotuner of the two-colour sweep: the levels (z lines: the columns) a thread
+// relaxes, timed as tune_sweep times its tiles; cached per device, grid and
+// kind.  STP_COLOUR_VARIANT=<v> forces a variant.  All compute the same values.
 int tune_colour(stp_handle* h) {
   const bool line = h->cfg.zline != 0;
+  if (const char* env = std::getenv("STP_COLOUR_VARIANT")) {
+    const int v = std::atoi(env);
+    h->sweep_us = 0.f;
+    h->sweep_variant = 0;
+    while (!colour_variant_ok(h->sweep_variant, h->nx, h->nz, line)) h->sweep_variant++;
+    if (colour_variant_ok(v, h->nx, h->nz, line)) h->sweep_variant = v;
+    return STP_OK;
+  }
   static std::mutex mu;
   static std::map<std::tuple<int, int, int, int, bool>, std::pair<int, float>> cache;
   const auto key = std::make_tuple(h->dev, h->nx, h->ny, h->nz, line);

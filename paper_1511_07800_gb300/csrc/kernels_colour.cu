@@ -199,11 +199,12 @@ __global__ void __launch_bounds__(8 * NCH, MINB) k_col_line(Geom<float> g, float
         for (int e = 0; e < W; e++) {
           const float pc = cc.v[e];
           const float prev = e == 0 ? ex : oc.v[e - 1], next = e == W - 1 ? ex : oc.v[e + 1];
-          float lap = idx2 * ((oc.v[e] - pc) + ((odd ? next : prev) - pc)) +
-                      idy2 * ((yn.v[e] - pc) + (ys.v[e] - pc));
-          lap += cf.x * (zu.v[e] - pc);
-          lap += cf.y * (zd.v[e] - pc);
-          G[q].v[e] = (bq.v[e] - lap) * cf.z;
+          // (a fixed sequence of roundings: the widths give the same bits)
+          float lap = __fmul_rn(idy2, __fadd_rn(__fsub_rn(yn.v[e], pc), __fsub_rn(ys.v[e], pc)));
+          lap = __fmaf_rn(idx2, __fadd_rn(__fsub_rn(oc.v[e], pc), __fsub_rn(odd ? next : prev, pc)), lap);
+          lap = __fmaf_rn(cf.x, __fsub_rn(zu.v[e], pc), lap);
+          lap = __fmaf_rn(cf.y, __fsub_rn(zd.v[e], pc), lap);
+          G[q].v[e] = __fmul_rn(__fsub_rn(bq.v[e], lap), cf.z);
         }
         zd = cc;
         cc = zu;
@@ -456,12 +457,13 @@ cudaError_t point_w(const Geom<float>& g, float* own, const float* oth, const fl
   return launch_dep(k_col_point<W, KZ>, (unsigned)((units + 255) / 256), 256, s, g, own, oth, r, om, c);
 }
 
-// z-line variants: columns a thread and level chunks a block
-struct LineVariant {
-  int w, nch;
-};
-constexpr LineVariant kLineVariants[] = {{4, 32}, {2, 32}, {1, 32}, {4, 16}, {2, 16}, {1, 16}};
+// z-line variants: columns a thread.  The chunks a column are no variant, since
+// they round differently and a solve has to repeat bitwise wherever it is timed:
+// 16 where their six levels each are enough, else 32 (us a sweep at 16 / 32: 512 x
+// 64 x 64 5.8 / 7.0, 256 x 128 x 96 7.3 / 8.1).
+constexpr int kLineWidths[] = {4, 2, 1};
 constexpr int kLineLevels = 6;  // levels a chunk at most
+int line_chunks(int nz) { return nz <= 16 * kLineLevels ? 16 : 32; }
 
 template <int W, int NCH, int MINB>
 cudaError_t line_w(const Geom<float>& g, float* own, const float* oth, const float* r, float om, int c,
@@ -485,13 +487,13 @@ bool colour_ok(int nx, int ny, int nz, bool line) {
   return nx % 2 == 0 && ny % 2 == 0 && (!line || nz <= 192) && (long long)nx * ny * nz >= kColourCells;
 }
 
-int colour_variants(bool line) { return line ? (int)(sizeof(kLineVariants) / sizeof(LineVariant)) : 3; }
+int colour_variants(bool line) { return line ? (int)(sizeof(kLineWidths) / sizeof(int)) : 3; }
 
-// point sweeps: 1, 2 or 4 levels a thread; z-line sweeps: kLineVariants
+// point sweeps: 1, 2 or 4 levels a thread; z-line sweeps: kLineWidths
 bool colour_variant_ok(int v, int nx, int nz, bool line) {
   if (v < 0 || v >= colour_variants(line)) return false;
   if (!line) return nz >= (1 << v);
-  return nx / 2 % kLineVariants[v].w == 0 && nz <= kLineVariants[v].nch * kLineLevels;
+  return nx / 2 % kLineWidths[v] == 0;
 }
 
 cudaError_t launch_colour_sweep(const Geom<float>& g, float* d, const float* r, float om, int c, int line, int variant,
@@ -500,13 +502,11 @@ cudaError_t launch_colour_sweep(const Geom<float>& g, float* d, const float* r, 
   float* own = d + (c ? half : 0);
   const float *oth = d + (c ? 0 : half), *rc = r + (c ? half : 0);
   if (line) {
+    const bool few = line_chunks(g.nz) == 16;
     switch (variant) {
-      case 0: return line_w<4, 32, 4>(g, own, oth, rc, om, c, s);
-      case 1: return line_w<2, 32, 5>(g, own, oth, rc, om, c, s);
-      case 2: return line_w<1, 32, 6>(g, own, oth, rc, om, c, s);
-      case 3: return line_w<4, 16, 8>(g, own, oth, rc, om, c, s);
-      case 4: return line_w<2, 16, 10>(g, own, oth, rc, om, c, s);
-      case 5: return line_w<1, 16, 12>(g, own, oth, rc, om, c, s);
+      case 0: return few ? line_w<4, 16, 8>(g, own, oth, rc, om, c, s) : line_w<4, 32, 4>(g, own, oth, rc, om, c, s);
+      case 1: return few ? line_w<2, 16, 10>(g, own, oth, rc, om, c, s) : line_w<2, 32, 5>(g, own, oth, rc, om, c, s);
+      case 2: return few ? line_w<1, 16, 12>(g, own, oth, rc, om, c, s) : line_w<1, 32, 6>(g, own, oth, rc, om, c, s);
       default: return cudaErrorInvalidValue;
     }
   }

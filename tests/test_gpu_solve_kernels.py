@@ -1,0 +1,35 @@
+"""Which kernels a pressure solve runs, and what must not depend on that choice."""
+import numpy as np
+import pytest
+
+from .test_gpu_parity import case
+from .test_gpu_zline import mean_free_rhs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape,zline", [((128, 128, 130), 0), ((132, 128, 126), 0), ((134, 126, 126), 0),
+                                         ((256, 128, 65), 1), ((256, 92, 96), 1), ((252, 90, 97), 1),
+                                         ((134, 170, 96), 1), ((128, 128, 192), 1)])
+def test_colour_variants_bitwise(stp_lib, monkeypatch, shape, zline):
+    """The tile shapes among which a two-colour sweep is picked by timing give the
+    same bits (two cycles from zero), so that a resumed run does not depend on
+    the clock: half rows of whole float4, float2 and single entries, z lines in
+    16 and in 32 level chunks, full and partial."""
+    nx, ny, nz = shape
+    cfg = case(nx=nx, ny=ny, nz=nz, stretch=1.0, zline=zline)
+    b, _ = mean_free_rhs(cfg, 5)
+    M = len(stp_lib.srj_schedule(cfg)[0])
+    ran = {}
+    for v in (0, 1, 2):
+        monkeypatch.setenv("STP_COLOUR_VARIANT", str(v))
+        with stp_lib.Channel(cfg, precision="fp32") as ch:
+            p = np.zeros_like(b)
+            ch.poisson_solve(b, p, tol=0.0, maxit=2 * M)
+            ran[ch.sweep_tile()[0]] = p
+    # rows that hold no whole vectors of a width leave it out
+    widths = [w for w in (4, 2, 1) if nx // 2 % w == 0]
+    assert sorted(ran) == ([0, 1, 2][-len(widths):] if zline else [0, 1, 2])
+    first = ran[min(ran)]
+    for v, p in ran.items():
+        assert np.array_equal(p, first), v
