@@ -29,9 +29,9 @@
  * in place, with the Chebyshev factors of a two-coloured grid, so that a cycle
  * of M sweeps gains what M Jacobi sweeps do; its tile shape is picked by timing
  * as below (STP_COLOUR_VARIANT=<0..2> forces one), and results do not depend on
- * it.  STP_SRJ_COLOURS=0 at stp_init
- * keeps Jacobi sweeps, as do schedules of the caller's own, a learned guess,
- * STP_SWEEP_VARIANT, STP_LINE_VARIANT=0 and the persistent cycles.  With STP_PERSISTENT=1 at
+ * it.  STP_SRJ_COLOURS=0 at stp_init keeps Jacobi sweeps, as do schedules of
+ * the caller's own, a learned guess, STP_SWEEP_VARIANT, the persistent cycles
+ * and, on z lines, STP_LINE_VARIANT=0.  With STP_PERSISTENT=1 at
  * stp_init an FP32 cycle instead runs as one persistent cooperative kernel
  * with bounded grid barriers between its sweeps (slower on GB300: kept as an
  * option); each barrier wait gives up after STP_BARRIER_WAIT SM clock cycles

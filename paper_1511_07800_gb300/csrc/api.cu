@@ -1503,11 +1503,13 @@ int stp_init(const stp_config* cfg, stp_handle** out) {
     if (allow && h->prec == STP_FP32_REFINE && h->nx % 4 == 0 && !cfg->zline)
       h->cycle_blocks = cycle_grid_f32(h->dev);
   }
-  if (h->prec == STP_FP32_REFINE && cfg->zline && line_chunk_ok(h->nx, h->nz)) {
-    // FP32 z-line sweeps solve their columns in registers where the grid
-    // allows it; STP_LINE_VARIANT=0 keeps the shared-memory lock-step kernel
+  // FP32 z-line sweeps solve their columns in registers where the grid allows
+  // it; STP_LINE_VARIANT=0 keeps the shared-memory lock-step kernel on any grid
+  bool lock_step = false;
+  if (h->prec == STP_FP32_REFINE && cfg->zline) {
     const char* env = std::getenv("STP_LINE_VARIANT");
-    h->line_variant = (env && env[0] == '0') ? 0 : 1;
+    lock_step = env && env[0] == '0';
+    h->line_variant = !lock_step && line_chunk_ok(h->nx, h->nz) ? 1 : 0;
   }
   {
     // persistent z-line cycles (STP_LINE_PERSISTENT=1): one cooperative
@@ -1523,8 +1525,7 @@ int stp_init(const stp_config* cfg, stp_handle** out) {
         h->line_rb = rb;
     }
   }
-  if (h->prec == STP_FP32_REFINE && !cfg->srj_omega && h->cycle_blocks == 0 && h->line_rb == 0 &&
-      (!cfg->zline || h->line_variant == 1 || !line_chunk_ok(h->nx, h->nz)) &&
+  if (h->prec == STP_FP32_REFINE && !cfg->srj_omega && h->cycle_blocks == 0 && h->line_rb == 0 && !lock_step &&
       colour_ok(h->nx, h->ny, h->nz, cfg->zline != 0)) {
     const char* env = std::getenv("STP_SRJ_COLOURS");
     h->colour = !(env && env[0] == '0') && !std::getenv("STP_SWEEP_VARIANT");

@@ -33,3 +33,24 @@ def test_colour_variants_bitwise(stp_lib, monkeypatch, shape, zline):
     first = ran[min(ran)]
     for v, p in ran.items():
         assert np.array_equal(p, first), v
+
+
+@pytest.mark.parametrize("shape,zline,jacobi", [((134, 170, 96), 1, True), ((128, 128, 130), 1, True),
+                                                ((128, 128, 130), 0, False)])
+def test_line_variant_0_keeps_jacobi_sweeps(stp_lib, monkeypatch, shape, zline, jacobi):
+    """STP_LINE_VARIANT=0 keeps Jacobi sweeps on every z-line grid, also one whose
+    rows are no multiple of 32 cells: bitwise those of STP_SRJ_COLOURS=0.  It says
+    nothing about point sweeps."""
+    nx, ny, nz = shape
+    cfg = case(nx=nx, ny=ny, nz=nz, stretch=1.0, zline=zline)
+    b, _ = mean_free_rhs(cfg, 5)
+    M = len(stp_lib.srj_schedule(cfg)[0])
+    monkeypatch.setenv("STP_LINE_VARIANT", "0")
+    got = []
+    for colours in ("1", "0"):
+        monkeypatch.setenv("STP_SRJ_COLOURS", colours)
+        with stp_lib.Channel(cfg, precision="fp32") as ch:
+            p = np.zeros_like(b)
+            ch.poisson_solve(b, p, tol=0.0, maxit=M)
+        got.append(p)
+    assert np.array_equal(*got) == jacobi
