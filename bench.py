@@ -36,17 +36,6 @@ WORKLOAD_DESC = ("les_channel 256x128x192, Lx 4pi Ly 2pi Lz 2, tanh walls gamma 
                  "Smagorinsky Cs 0.1 + van Driest A 25, constant flux U_b 1, dt 1e-3, laminar + 10% noise (seed 1); "
                  "FP32 stencils and sweeps, FP64 reductions and refinement, z-line SRJ, Poisson to 1e-8")
 METRIC = "Mcell*steps/s (projection step, Poisson to 1e-8 rel. residual)"
-LINE_NAMES = {1: "k_line_sweep_chunk<32,6> (z-line SRJ sweep: residual, column recurrences in registers by level "
-                 "chunks, update)",
-              0: "k_line_sweep_vec<float,RB> (z-line SRJ sweep: residual, twisted column solve in shared memory, "
-                 "update)"}
-TILE_NAMES = {0: "k_sweep_f32_z<1,8>", 1: "k_sweep_f32_z<2,8>", 2: "k_sweep_f32_z<4,8>", 3: "k_sweep_f32_z<2,4>",
-              4: "k_sweep_f32_z<4,4>", 5: "k_sweep_f32_z<8,4>", 6: "k_sweep_f32_flat<2>", 7: "k_sweep_f32_flat<4>",
-              8: "k_sweep_f32_flat<8>", 9: "k_sweep_f32_pair<8,4>", 10: "k_sweep_f32_pair<4,4>",
-              11: "k_sweep_f32_pair<4,8>", 12: "k_cluster_cycle (16 blocks, z slabs)",
-              13: "k_cluster_cycle (16 blocks, y slabs)", 14: "k_cluster_cycle (8 blocks, z slabs)",
-              15: "k_cluster_cycle (8 blocks, y slabs)"}
-LINE_F64 = "k_line_f64 (z-line SRJ sweep, column recurrences in level chunks)"
 
 
 def parse():
@@ -569,26 +558,17 @@ def timed_steps(ch, steps, stream, flush):
     return dict(ms=ms, sweeps=sweeps, passes=passes, launches=launches, solve_ms=solve_ms, converged=conv)
 
 
-def two_colour(cfg, precision):
-    """Whether a channel's FP32 inner solve runs two-colour sweeps (one colour
-    a sweep): even rows and row counts, at least 2^21 cells, z lines of at
-    most 192 levels, and none of the environment's other choices."""
-    return (precision == "fp32" and cfg["nx"] % 2 == 0 and cfg["ny"] % 2 == 0 and
-            cfg["nx"] * cfg["ny"] * cfg["nz"] >= 1 << 21 and (not cfg.get("zline") or cfg["nz"] <= 192) and
-            not os.environ.get("STP_SRJ_COLOURS", "").startswith("0") and "STP_SWEEP_VARIANT" not in os.environ and
-            not os.environ.get("STP_LINE_VARIANT", "").startswith("0"))
-
-
-def sweep_kernel(cfg, precision, ch):
-    """Name of the sweep kernel a channel runs."""
-    if two_colour(cfg, precision):
-        return ("k_col_line" if cfg.get("zline") else "k_col_point") + " (two-colour SRJ sweep, one colour a sweep)"
-    if cfg.get("zline"):
-        return LINE_NAMES[ch.line_kernel()] if precision == "fp32" else LINE_F64
-    variant, _ = ch.sweep_tile()
-    if precision == "fp32":
-        return TILE_NAMES.get(variant, "k_sweep_f32") + " (SRJ sweep, autotuned tile variant %d)" % variant
-    return "k_sweep_f64 (SRJ sweep)"
+def sweep_kernel(ch):
+    """(name, words a cell that a sweep moves) of the sweep kernel a channel runs:
+    3 words (read p and b, write p') or, a colour at a time, 2."""
+    name = ch.sweep_kernel()
+    if name.startswith("k_col_"):
+        return name + " (two-colour SRJ sweep, one colour a sweep)", 2
+    if "line" in name:
+        return name + " (z-line SRJ sweep)", 3
+    if name.startswith("k_sweep_f32"):
+        return name + " (SRJ sweep, autotuned tile variant %d)" % ch.sweep_tile()[0], 3
+    return name + " (SRJ sweep)", 3
 
 
 def sweep_roofline(words, word, cells, r, kernel, peak, traffic_key):
@@ -620,8 +600,7 @@ def side_steps(stp, cfg, precision, fields, steps, warmup, stream, flush, peak, 
         for _ in range(max(3, warmup)):
             ch.step(1)
         r = timed_steps(ch, steps, stream, flush)
-        kern = sweep_kernel(cfg, precision, ch)
-    words = 2 if two_colour(cfg, precision) else 3
+        kern, words = sweep_kernel(ch)
     out = {"value": cells * steps / (r["ms"] / 1e3) / 1e6, "unit": "Mcell*steps/s", "ms_per_step": r["ms"] / steps,
            "steps": steps, "warmup": max(3, warmup), "sweeps_per_step": r["sweeps"] / steps,
            "solve_ms_per_step": r["solve_ms"] / steps, "converged": r["converged"],
@@ -660,10 +639,9 @@ def sweeps_above_l2(stp, peak):
                 ch.poisson_solve(b, p, tol=0.0, maxit=M)  # warm-up (and the FP32 tile autotuner)
                 p.zero_()
                 st = ch.poisson_solve(b, p, tol=0.0, maxit=2 * M)
-                colours = two_colour(dict(cfg, zline=zl), prec)
-                kern = sweep_kernel(dict(cfg, zline=zl), prec, ch)
+                kern, words = sweep_kernel(ch)
             t = st["solve_ms"] / max(1, st["sweeps"]) / 1e3
-            ach = (2 if colours else 3) * word * cells / t / 1e9
+            ach = words * word * cells / t / 1e9
             res[solver] = {"sweeps": st["sweeps"], "us_per_sweep": t * 1e6, "achieved_GBs": ach,
                            "frac": ach / peak,
                            "kernel": kern.split(" ")[0]}
@@ -732,8 +710,7 @@ def run_ours(args):
     peaks = measured_peaks()
     peak = peaks.get("hbm_gbs", 6800.0)
     word = 4 if args.precision == "fp32" else 8
-    kern = sweep_kernel(cfg, args.precision, ch)
-    words = 2 if two_colour(cfg, args.precision) else 3
+    kern, words = sweep_kernel(ch)
     tkey = "%s_%s_%s" % ("two_colour" if words == 2 else "zline_sweep" if cfg.get("zline") else "point_sweep",
                          args.precision, args.workload)
     roof = sweep_roofline(words, word, cells, r, kern, peak, tkey)

@@ -253,6 +253,15 @@ int stp_sweep_tile(const stp_handle *h, float *us);
    stp_init) and in FP64; -1 for point sweeps or a NULL handle.  No GPU work. */
 int stp_line_kernel(const stp_handle *h);
 
+/* Name of the kernel that runs the sweeps of this handle's pressure solves: in
+   FP32 k_col_point and k_col_line (two-colour sweeps), k_cluster_cycle (cycles on
+   one cluster), k_cycle_f32 and k_line_cycle_f32 (persistent cycles),
+   k_sweep_f32... (Jacobi tiles), k_line_sweep... (Jacobi z lines); in FP64
+   k_sweep_f64, k_line_f64 and k_line_sweep<double>.  "" for a NULL handle and, where
+   the choice is timed, before the first solve.  A static string; no GPU work.
+   (A batch may solve its small channels in groups: stp_batch_groups.) */
+const char *stp_sweep_kernel(const stp_handle *h);
+
 /* Lock-step groups of the batch (built at the first stp_batch_step).
    Channels of at most 2^17 cells in FP32 with refinement that share the SRJ
    cycle length M (at least two of them, rows a multiple of 4 cells, no

@@ -2443,6 +2443,21 @@ int stp_line_kernel(const stp_handle* h) {
   return h->line_variant;
 }
 
+// (the order of build_cycle)
+const char* stp_sweep_kernel(const stp_handle* h) {
+  if (!h) return "";
+  const bool line = h->cfg.zline != 0;
+  if (h->prec == STP_FP64) return line ? line_sweep_name(true, h->nx, h->ny, h->nz, 0) : "k_sweep_f64";
+  if (use_colour(h)) return line ? "k_col_line" : "k_col_point";
+  if (h->cycle_blocks > 0) return "k_cycle_f32";
+  if (h->line_rb > 0) return "k_line_cycle_f32";
+  if (line) return line_sweep_name(false, h->nx, h->ny, h->nz, h->line_variant);
+  if (h->sweep_variant < 0 || h->tuned_colour) return "";
+  if (uses_cluster(h)) return "k_cluster_cycle";
+  const bool pair = sweep_variant_is_pair(h->sweep_variant);
+  return sweep_f32_name(pair && !uses_pairs(h) ? 0 : h->sweep_variant, h->nx, h->ny, h->nz);
+}
+
 int stp_batch_groups(const stp_batch* b, int max_groups, stp_batch_group* out) {
   if (!b) return STP_EINVAL;
   const int n = (int)b->groups.size();

@@ -1130,6 +1130,16 @@ cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* 
   return launch_sweep_cfg(w == 2 ? (const void*)k_sweep_f32<2> : (const void*)k_sweep_f32<1>, grid, block, s, args);
 }
 
+const char* sweep_f32_name(int variant, int nx, int ny, int nz) {
+  static const char* const tiles[] = {"k_sweep_f32_z<1,8>",    "k_sweep_f32_z<2,8>",    "k_sweep_f32_z<4,8>",
+                                      "k_sweep_f32_z<2,4>",    "k_sweep_f32_z<4,4>",    "k_sweep_f32_z<8,4>",
+                                      "k_sweep_f32_flat<2>",   "k_sweep_f32_flat<4>",   "k_sweep_f32_flat<8>",
+                                      "k_sweep_f32_pair<8,4>", "k_sweep_f32_pair<4,4>", "k_sweep_f32_pair<4,8>"};
+  static_assert(sizeof(tiles) / sizeof(tiles[0]) == kSweepVariants, "a name a variant");
+  if (nx % 4) return nx % 2 ? "k_sweep_f32<1>" : "k_sweep_f32<2>";
+  return tiles[sweep_variant_ok(variant, nx, ny, nz) ? variant : 0];
+}
+
 // rows per block of the shared-memory line sweep: 4, 2 or 1 (so that the
 // 32 rb columns divide the 512 threads), the most whose columns x nz values
 // fit in 96 KB (two blocks an SM); 0 when one row does not fit
@@ -1208,6 +1218,12 @@ cudaError_t launch_line_sweep(const Geom<T>& g, const T* p, const T* b, T omega,
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, k_line_sweep<T>, g, p, b, omega, out);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+const char* line_sweep_name(bool f64, int nx, int ny, int nz, int variant) {
+  if (f64) return line_f64_chunks(nx, ny, nz) ? "k_line_f64" : "k_line_sweep<double>";
+  if (variant == 1 && line_chunk_ok(nx, nz)) return "k_line_sweep_chunk";
+  if (!line_rows(nz, sizeof(float))) return "k_line_sweep<float>";
+  return nx % VecOf<float>::W == 0 ? "k_line_sweep_vec" : "k_line_sweep_smem";
 }
 template cudaError_t launch_line_sweep<float>(const Geom<float>&, const float*, const float*, float, float*,
                                               cudaStream_t, int);

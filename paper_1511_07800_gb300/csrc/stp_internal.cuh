@@ -225,6 +225,9 @@ cudaError_t launch_line_sweep(const Geom<T>& g, const T* p, const T* b, T omega,
                               int variant);
 // whether the register-chunked FP32 line sweep (variant 1) takes the grid
 bool line_chunk_ok(int nx, int nz);
+// name of the kernel that launch_line_sweep, or launch_sweep_f32 with a variant set, runs
+const char* line_sweep_name(bool f64, int nx, int ny, int nz, int variant);
+const char* sweep_f32_name(int variant, int nx, int ny, int nz);
 
 // One Jacobi-SOR sweep of L p = b with factor omega: out = p - omega (b - Lp)/S.
 cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* b, float omega, float* out,

@@ -86,7 +86,7 @@ EXPORTS = ("stp_config_defaults", "stp_init", "stp_destroy", "stp_last_error", "
            "stp_get_state", "stp_set_state", "stp_batch_create", "stp_batch_destroy", "stp_batch_last_error",
            "stp_batch_step", "stp_batch_groups", "stp_sweep_tile", "stp_stats_reset",
            "stp_stats_accumulate", "stp_stats_read", "stp_unet_layer", "stp_set_learned_mode",
-           "stp_line_kernel")
+           "stp_line_kernel", "stp_sweep_kernel")
 
 _lib = None
 
@@ -142,6 +142,8 @@ def lib():
     L.stp_batch_groups.argtypes = [vp, ctypes.c_int, ctypes.POINTER(BatchGroup)]
     L.stp_sweep_tile.argtypes = [vp, ctypes.POINTER(ctypes.c_float)]
     L.stp_line_kernel.argtypes = [vp]
+    L.stp_sweep_kernel.argtypes = [vp]
+    L.stp_sweep_kernel.restype = ctypes.c_char_p
     L.stp_stats_reset.argtypes = [vp, ctypes.c_int]
     L.stp_stats_accumulate.argtypes = [vp]
     L.stp_stats_read.argtypes = [vp, dp, dp, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_int)]
@@ -355,6 +357,11 @@ class Channel:
         """z-line sweep kernel: 1 register-chunked (FP32), 0 shared-memory
         lock step, -1 point sweeps."""
         return lib().stp_line_kernel(self._h)
+
+    def sweep_kernel(self):
+        """Name of the kernel that runs the sweeps of this channel's pressure
+        solves ("" where it is picked by the first solve)."""
+        return lib().stp_sweep_kernel(self._h).decode()
 
     def close(self):
         if getattr(self, "_h", None) is not None and _lib is not None:

@@ -54,3 +54,33 @@ def test_line_variant_0_keeps_jacobi_sweeps(stp_lib, monkeypatch, shape, zline, 
             ch.poisson_solve(b, p, tol=0.0, maxit=M)
         got.append(p)
     assert np.array_equal(*got) == jacobi
+
+
+@pytest.mark.parametrize("shape,zline,precision,env,want", [
+    ((128, 128, 130), 0, "fp32", {}, "k_col_point"),
+    ((134, 170, 96), 1, "fp32", {}, "k_col_line"),
+    ((134, 170, 96), 1, "fp32", {"STP_LINE_VARIANT": "0"}, "k_line_sweep_smem"),
+    ((128, 128, 130), 1, "fp32", {"STP_LINE_VARIANT": "0"}, "k_line_sweep_vec"),
+    ((128, 128, 130), 0, "fp32", {"STP_LINE_VARIANT": "0"}, "k_col_point"),
+    ((128, 128, 130), 1, "fp32", {"STP_SRJ_COLOURS": "0"}, "k_line_sweep_chunk"),
+    ((8, 5, 800), 1, "fp32", {}, "k_line_sweep<float>"),
+    ((64, 24, 32), 1, "fp32", {"STP_LINE_PERSISTENT": "1"}, "k_line_cycle_f32"),
+    ((64, 24, 32), 0, "fp32", {"STP_PERSISTENT": "1"}, "k_cycle_f32"),
+    ((32, 32, 32), 0, "fp32", {"STP_SWEEP_VARIANT": "12"}, "k_cluster_cycle"),
+    ((64, 24, 32), 0, "fp32", {"STP_SWEEP_VARIANT": "4"}, "k_sweep_f32_z<4,4>"),
+    ((64, 24, 32), 0, "fp32", {"STP_SWEEP_VARIANT": "10"}, "k_sweep_f32_pair<4,4>"),
+    ((37, 24, 32), 0, "fp32", {}, "k_sweep_f32<1>"),
+    ((64, 24, 32), 0, "fp64", {}, "k_sweep_f64"),
+    ((64, 24, 32), 1, "fp64", {}, "k_line_f64"),
+    ((8, 5, 400), 1, "fp64", {}, "k_line_sweep<double>"),
+])
+def test_sweep_kernel_names_what_runs(stp_lib, monkeypatch, shape, zline, precision, env, want):
+    """stp_sweep_kernel follows the dispatch of the solve."""
+    nx, ny, nz = shape
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    cfg = case(nx=nx, ny=ny, nz=nz, stretch=1.0, zline=zline)
+    b, _ = mean_free_rhs(cfg, 5)
+    with stp_lib.Channel(cfg, precision=precision) as ch:
+        ch.poisson_solve(b, np.zeros_like(b), tol=0.0, maxit=32)
+        assert ch.sweep_kernel() == want
