@@ -815,8 +815,10 @@ int tune_colour(stp_handle* h) {
 
 // Autotuner of the FP32 sweep kernel: times every variant valid for this
 // grid (time_sweeps, on the handle's own scratch buffers) and keeps the
-// choice of pick_variant; cached per (device, nx, ny, nz).
-// STP_SWEEP_VARIANT=<v> forces a variant.  All variants compute the same values.
+// choice of pick_variant; cached per device, grid and what else the candidates
+// and their times depend on: the cycle's length (a cluster loads and stores its
+// channel once a cycle, pairs need a multiple of 4 sweeps) and whether cycles run
+// persistent.  STP_SWEEP_VARIANT=<v> forces a variant.  All variants compute the same values.
 int tune_sweep(stp_handle* h) {
   const bool colour = use_colour(h);
   if (h->sweep_variant >= 0 && h->tuned_colour == colour) return STP_OK;
@@ -833,8 +835,9 @@ int tune_sweep(stp_handle* h) {
     return STP_OK;
   }
   static std::mutex mu;
-  static std::map<std::tuple<int, int, int, int>, std::pair<int, float>> cache;
-  const auto key = std::make_tuple(h->dev, h->nx, h->ny, h->nz);
+  static std::map<std::tuple<int, int, int, int, int, bool, bool>, std::pair<int, float>> cache;
+  const int M = (int)h->omega.size();
+  const auto key = std::make_tuple(h->dev, h->nx, h->ny, h->nz, std::min(256, M), M % 4 == 0, can_cluster);
   {
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(key);

@@ -84,3 +84,33 @@ def test_sweep_kernel_names_what_runs(stp_lib, monkeypatch, shape, zline, precis
     with stp_lib.Channel(cfg, precision=precision) as ch:
         ch.poisson_solve(b, np.zeros_like(b), tol=0.0, maxit=32)
         assert ch.sweep_kernel() == want
+
+
+@pytest.mark.parametrize("order", ["short first", "long first", "persistent first"])
+def test_tile_choice_is_per_cycle_length(stp_lib, monkeypatch, order):
+    """What the autotuner picks for one handle says nothing about a handle of
+    another cycle length, or without persistent cycles, on the same grid: a cluster
+    loads and stores its channel once a cycle, far too often for cycles of two
+    sweeps and well worth it for long ones (32 x 32 x 32: 0.7 of the best
+    launched sweep)."""
+    # grids of their own: choices are kept for the process
+    cfg = case(nx=32, ny=32, nz={"short first": 33, "long first": 34, "persistent first": 36}[order], stretch=0.0)
+    b, _ = mean_free_rhs(cfg, 5)
+
+    def kernel(omega=None):
+        with stp_lib.Channel(cfg, precision="fp32", omega=omega) as ch:
+            ch.poisson_solve(b, np.zeros_like(b), tol=0.0, maxit=2)
+            return ch.sweep_kernel()
+
+    short = [1.0, 1.0]
+    if order == "long first":
+        assert kernel() == "k_cluster_cycle"
+        assert kernel(short).startswith("k_sweep_f32")
+        return
+    if order == "short first":
+        assert kernel(short).startswith("k_sweep_f32")
+    else:
+        monkeypatch.setenv("STP_PERSISTENT", "1")
+        assert kernel() == "k_cycle_f32"
+        monkeypatch.delenv("STP_PERSISTENT")
+    assert kernel() == "k_cluster_cycle"
