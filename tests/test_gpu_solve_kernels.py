@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from .test_gpu_parity import case
+from .test_gpu_parity import case, schedule
 from .test_gpu_zline import mean_free_rhs
 
 pytestmark = pytest.mark.gpu
@@ -114,3 +114,41 @@ def test_tile_choice_is_per_cycle_length(stp_lib, monkeypatch, order):
         assert kernel() == "k_cycle_f32"
         monkeypatch.delenv("STP_PERSISTENT")
     assert kernel() == "k_cluster_cycle"
+
+
+CLUSTER_COLUMNS = [
+    # shape, variants it fits, those among them of two columns a thread
+    ((76, 57, 32), {12, 13}, {12}),              # 4-cell vectors, slabs of 2 levels; 1083 columns
+    ((76, 32, 57), {12, 13}, {13}),              # the same across y
+    ((76, 27, 48), {12, 13, 14, 15}, {14}),      # slabs of up to 6 on 8 blocks, 513 columns of 512 threads
+    ((76, 48, 27), {12, 13, 14, 15}, {15}),
+    ((76, 40, 96), {12}, {12}),                  # slabs of 6 on 16 blocks, 760 columns
+    ((76, 96, 27), {13}, {13}),
+    ((66, 33, 32), {12, 13, 14}, {12, 13, 14}),  # 2-cell vectors, slabs of 2 and of 4, odd column counts
+    ((66, 32, 33), {12, 13, 15}, {12, 13, 15}),
+    ((76, 57, 16), {12, 13, 14, 15}, {12, 14}),  # slabs of one level
+]
+
+
+@pytest.mark.parametrize("shape,fits,two", CLUSTER_COLUMNS)
+def test_cluster_two_columns_a_thread_bitwise(stp_lib, monkeypatch, shape, fits, two):
+    """Cluster-resident cycles whose blocks have more columns than threads, so that
+    a thread takes two: bitwise the launched sweeps, and every variant that fits
+    did run."""
+    nx, ny, nz = shape
+    assert two <= fits
+    cfg = case(nx=nx, ny=ny, nz=nz, stretch=2.0)
+    om = schedule(cfg, 32)
+    b, _ = mean_free_rhs(cfg, 3)
+    ref, ran = None, set()
+    for v in (0, 12, 13, 14, 15):
+        monkeypatch.setenv("STP_SWEEP_VARIANT", str(v))
+        with stp_lib.Channel(cfg, precision="fp32", omega=om) as ch:
+            p = np.zeros_like(b)
+            st = ch.poisson_solve(b, p, tol=1e-8, maxit=96)
+            if ch.sweep_kernel() == "k_cluster_cycle":
+                ran.add(ch.sweep_tile()[0])
+        if ref is None:
+            ref = (p, st["sweeps"])
+        assert st["sweeps"] == ref[1] and np.array_equal(p, ref[0]), v
+    assert ran == fits
