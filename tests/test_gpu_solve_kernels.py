@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 
+from .conftest import gauge, rel_err
 from .test_gpu_parity import case, schedule
 from .test_gpu_zline import mean_free_rhs
 
@@ -152,3 +153,20 @@ def test_cluster_two_columns_a_thread_bitwise(stp_lib, monkeypatch, shape, fits,
             ref = (p, st["sweeps"])
         assert st["sweeps"] == ref[1] and np.array_equal(p, ref[0]), v
     assert ran == fits
+
+
+def test_sweeps_without_a_table(stp_lib, orc):
+    """FP64 point sweeps whose level coefficients would exceed the table's 80 MB (4096
+    sweeps a cycle, 430 levels: 85 MB) form them in the kernel: a cycle of
+    contracting factors against the oracle to 1e-10."""
+    cfg = case(nx=6, ny=5, nz=430, stretch=2.0)
+    om = [0.6, 0.9, 0.7, 1.0] * 1024
+    cfg["omega"] = om
+    b, rng = mean_free_rhs(cfg, 11)
+    p0 = rng.standard_normal(b.shape) * 0.1
+    p_o, it_o, _, _ = orc.Oracle(cfg).poisson(b, p0, tol=0.0, maxit=4096)
+    with stp_lib.Channel(cfg, omega=om) as ch:
+        p_g = p0.copy()
+        st = ch.poisson_solve(b, p_g, tol=0.0, maxit=4096)
+    assert st["sweeps"] == it_o == 4096
+    assert rel_err(p_g, gauge(p_o, cfg)) < 1e-10
