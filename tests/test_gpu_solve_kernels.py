@@ -170,3 +170,43 @@ def test_sweeps_without_a_table(stp_lib, orc):
         st = ch.poisson_solve(b, p_g, tol=0.0, maxit=4096)
     assert st["sweeps"] == it_o == 4096
     assert rel_err(p_g, gauge(p_o, cfg)) < 1e-10
+
+
+@pytest.mark.parametrize("zline,host", [(0, "0"), (1, "0"), (0, "1")])
+def test_network_on_and_off_a_two_colour_channel(stp_lib, orc, monkeypatch, zline, host):
+    """A learned guess takes a large channel from two-colour to Jacobi sweeps and
+    back: layout of the residual and the correction, tile choice and solve graph
+    all change.  With the network (as the guess and as the preconditioner) solves
+    reach 1e-8 measured with the oracle's operator; without it again they end
+    bitwise where they did before."""
+    unet = pytest.importorskip("oracle.unet")
+    monkeypatch.setenv("STP_HOST_SOLVE", host)
+    n = 128
+    cfg = case(nx=n, ny=n, nz=n, stretch=0.0, zline=zline)
+    b, _ = mean_free_rhs(cfg, 5)
+    oracle = orc.Oracle(dict(cfg, omega=[1.0]))
+    colour = "k_col_line" if zline else "k_col_point"
+    net = stp_lib.UNet(1, n, n, n)
+    net.set_params(unet.init_params(11).astype(np.float32))
+    net.set_output_scale(1e3)  # an untrained network: small corrections
+    with stp_lib.Channel(cfg, precision="fp32") as ch:
+
+        def solve():
+            p = np.zeros_like(b)
+            st = ch.poisson_solve(b, p, tol=1e-8)
+            r = b - oracle.laplacian(p)
+            assert st["converged"] and np.sqrt(np.sum(r * r) / np.sum(b * b)) <= 1e-8 * 1.0001
+            return p
+
+        first = solve()
+        assert ch.sweep_kernel() == colour
+        for mode in (0, 1):
+            ch.set_learned_mode(mode)
+            ch.set_learned_guess(net)
+            solve()
+            assert ch.sweep_kernel() not in ("", colour)
+        ch.set_learned_guess(None)
+        again = solve()
+        assert ch.sweep_kernel() == colour
+        assert np.array_equal(again, first)
+    net.close()
