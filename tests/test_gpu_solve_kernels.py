@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from .conftest import gauge, rel_err
-from .test_gpu_parity import case, schedule
+from .test_gpu_parity import case, schedule, turbulent_like
 from .test_gpu_zline import mean_free_rhs
 
 pytestmark = pytest.mark.gpu
@@ -210,3 +210,34 @@ def test_network_on_and_off_a_two_colour_channel(stp_lib, orc, monkeypatch, zlin
         assert ch.sweep_kernel() == colour
         assert np.array_equal(again, first)
     net.close()
+
+
+def test_two_colour_channel_in_a_batch(stp_lib):
+    """Channels of two-colour sweeps, point and z line, beside channels that are
+    solved in a group: each ends bitwise where it ends when stepped alone."""
+    specs = [case(nx=128, ny=128, nz=128, nu=1 / 500.0),
+             case(nx=32, ny=16, nz=32, nu=1 / 500.0),
+             case(nx=160, ny=116, nz=114, nu=1 / 500.0, stretch=1.0, zline=1),
+             case(nx=32, ny=16, nz=32, nu=1 / 800.0)]
+    alone, kernels = [], []
+    for i, cfg in enumerate(specs):
+        with stp_lib.Channel(cfg, precision="fp32") as ch:
+            ch.set_fields(*turbulent_like(cfg, 30 + i))
+            ch.step(2)
+            alone.append(ch.get_fields())
+            kernels.append(ch.sweep_kernel())
+    assert kernels[0] == "k_col_point" and kernels[2] == "k_col_line"
+    chans = [stp_lib.Channel(cfg, precision="fp32") for cfg in specs]
+    for i, ch in enumerate(chans):
+        ch.set_fields(*turbulent_like(specs[i], 30 + i))
+    batch = stp_lib.Batch(chans)
+    st = batch.step(2)
+    assert st["converged"]
+    assert [g["channels"] for g in batch.groups()] == [2]
+    for i, ch in enumerate(chans):
+        got = ch.get_fields()
+        for k in ("u", "v", "w", "p"):
+            assert np.array_equal(got[k], alone[i][k]), (i, k)
+    batch.close()
+    for ch in chans:
+        ch.close()
