@@ -19,7 +19,6 @@
 #include <cmath>
 #include <cstdlib>
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include "device_util.cuh"
@@ -255,12 +254,14 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
 // ---------------------------------------------------------------------------
 // The same convolution on the fifth-generation tensor cores (tcgen05, TMEM
 // accumulator), for layers whose level has w % 8 == 0 and h % 16 == 0 and
-// channel counts that are multiples of 16.
+// channel counts that are multiples of 16 (k_conv3_tz below) or whose weights do
+// not fit an SM (this kernel: 64 -> 64, 64 -> 128, 128 -> 128, 192 -> 64 and back;
+// input channels a multiple of 64).
 //
 // A tile is zt planes of 128 voxels, 8 (x) x 16 (y) at zt consecutive z, for
 // all cout channels: per plane M = 128, N = cout, K = 27 taps x cin, the zt
 // accumulators side by side in tensor memory.  The input is staged by groups
-// of up to 64 channels as a halo of 10 x 18 x (zt + 2) voxels (periodic in x
+// of 64 channels as a halo of 10 x 18 x (zt + 2) voxels (periodic in x
 // and y, zeros outside the walls) in the K-major core-matrix layout without
 // swizzle: 8-channel chunk j of halo voxel (hx, hy, hz) is 16 bytes at
 // j CHUNK + ((hz HY + hy) HX + hx) 16, CHUNK = 16 HX HY (zt + 2).  The A operand
@@ -269,23 +270,24 @@ __global__ void __launch_bounds__(128) k_conv3(Dims dm, const bf16* __restrict__
 // (16 bytes apart), the next 8 rows are the next y (SBO = 16 HX bytes), the
 // next 8 channels the next chunk (LBO = one chunk of the halo).  So the 27
 // taps need no data movement.  The weights come as bulk copies of an image
-// kept in shared-memory order, three taps at a time through a ring: this kernel
-// takes the layers whose weights do not fit an SM (64 -> 64, 192 -> 64 and back).
+// kept in shared-memory order, three taps at a time through a ring.
 //
 // What bounds it: an MMA of M = 128, K = 16 takes 68 clocks whatever the layout
 // and N up to 128 when one thread issues them in a loop, 48 when an elected
 // thread issues unrolled taps, so a layer cannot take less than
 // 27 cin/16 x 48 clocks a 128 voxels.  To keep the MMAs back to back, blocks
-// stay for many tiles and their warps take roles: four load halos (hs stages),
-// one thread copies weights, two threads issue MMAs, four warps store results
-// (as accumulator stages), each waiting on mbarriers for the others.  us, with
+// stay for many tiles and their warps take roles: four load halos, one thread
+// copies weights, up to two threads issue MMAs, four warps store results (as
+// accumulator stages), each waiting on mbarriers for the others.  us, with
 // blocks that load, multiply and store one tile after another, several an SM /
 // this (both with resident weights where they fit): 16 -> 16 at 128 x 64 x 128 77
 // / 49, 48 -> 16 190 / 113, 32 -> 32 at half that size 34 / 20.  With a weight
 // stage a tap, handing it over (0.36 us) took as long as its copy: 64 -> 64 at 32
 // x 16 x 32 15.5 with one tap a stage, 12.5 with three; 192 -> 64 28.8 / 27.5,
-// bound by its weights (660 KB a tile) and three halos in sequence.  Eight
-// loader warps (16 -> 16 62) or a pair of lanes a voxel (53) are slower.
+// bound by its weights (660 KB a tile) and three halos in sequence: beside the
+// ring there is room for one halo, so a group is loaded when the one before it
+// has been multiplied.  Eight loader warps (16 -> 16 62) or a pair of lanes a
+// voxel (53) are slower.
 //
 // Each accumulator sees the same MMAs in the same order (groups, taps,
 // 16-channel steps) whatever the plan.  Every wait is bounded; on a time-out
@@ -445,14 +447,12 @@ __device__ __forceinline__ void tc_store(uint32_t acc, long long v, long long vz
   }
 }
 
-// how k_conv3_tc runs a layer
+// how k_conv3_tc runs a layer, one block an SM
 struct TcPlan {
-  int zt;      // planes a tile
-  int hs;      // halo stages
-  int ring;    // weight stages
-  int as;      // accumulator stages
-  int cols;    // tensor-memory columns
-  int per_sm;  // blocks an SM
+  int zt;    // planes a tile
+  int ring;  // weight stages
+  int as;    // accumulator stages
+  int cols;  // tensor-memory columns
   size_t smem;
 };
 
@@ -464,27 +464,24 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
   extern __shared__ __align__(1024) uint8_t tsm[];
   // mbarriers: halo full and empty, weight full and empty, accumulator full and
   // empty
-  __shared__ __align__(8) uint64_t hfull[2], hempty[2], wfull[TC_RING], wempty[TC_RING], afull[2], aempty[2],
-      drain[2];
+  __shared__ __align__(8) uint64_t hfull, hempty, wfull[TC_RING], wempty[TC_RING], afull[2], aempty[2], drain[2];
   __shared__ uint32_t tslot;
   __shared__ volatile int sfail;
   __shared__ __align__(16) float sbias[256];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int zt = ZT, hz_n = zt + 2;
   constexpr int NI = ZT > 1 ? 2 : 1, NP = ZT / NI;  // issuing threads, planes each
-  const int cgmax = cin < TC_CG ? cin : TC_CG;            // channels of the widest group
-  const uint32_t stage_bytes = (uint32_t)cout * cgmax * 2;  // one tap's weights of one group
+  const uint32_t stage_bytes = (uint32_t)cout * TC_CG * 2;  // one tap's weights of one group
   constexpr uint32_t chunk = TC_PLANE * hz_n;             // bytes of one 8-channel chunk of the halo
-  const uint32_t halo_bytes = (cgmax / 8) * chunk;
-  const uint32_t halo0 = su32(tsm), w0 = halo0 + P.hs * halo_bytes;
-  const int ngroups = (cin + TC_CG - 1) / TC_CG;
+  const uint32_t halo0 = su32(tsm), w0 = halo0 + (TC_CG / 8) * chunk;
+  const int ngroups = cin / TC_CG;
   const int nxt = dm.w / TC_TX, nyt = dm.h / TC_TY, nzt = dm.d / zt;
   const int ntiles = nxt * nyt * nzt * dm.n;
   if (tid == 0) {
     auto init = [](uint64_t* m, int count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(m)), "r"(count)); };
+    init(&hfull, 128);
+    init(&hempty, NI);
     for (int i = 0; i < 2; i++) {
-      init(&hfull[i], 128);
-      init(&hempty[i], NI);
       init(&afull[i], NI);
       init(&aempty[i], 128);
     }
@@ -530,11 +527,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
       int gx = T.x0 - 1 + hx;
       gx = gx < 0 ? gx + dm.w : (gx >= dm.w ? gx - dm.w : gx);
       for (int g = 0; g < ngroups; g++, use++) {
-        const int st = use % P.hs;
-        if (!(ok = tc_wait_warp(su32(&hempty[st]), ((use / P.hs) & 1) ^ 1))) break;
-        const int c0 = g * TC_CG, nch = min(TC_CG, cin - c0) / 8;
-        const uint32_t base = halo0 + st * halo_bytes + 16 * hx;
-        const bf16* xg = x + (long long)gx * ldx + c0;
+        if (!(ok = tc_wait_warp(su32(&hempty), (use & 1) ^ 1))) break;
+        const uint32_t base = halo0 + 16 * hx;
+        const bf16* xg = x + (long long)gx * ldx + g * TC_CG;
         for (int row = warp * 3 + hr; row < rows; row += 12) {
           if (hr == 3) break;
           const int hz = row / TC_HY, hy = row - hz * TC_HY;
@@ -544,11 +539,11 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
           const bool in = gz >= 0 && gz < dm.d;
           const bf16* src = xg + voxel_at(dm, T.n, in ? gz : 0, gy, 0) * ldx;
           const uint32_t dst = base + row * (16 * TC_HX);  // chunk 0; chunk j is `chunk` further
-          for (int j = 0; j < nch; j++) cp16(dst + j * chunk, src + 8 * j, in);
+          for (int j = 0; j < TC_CG / 8; j++) cp16(dst + j * chunk, src + 8 * j, in);
         }
         asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_arrive(su32(&hfull[st]));
+        tc_arrive(su32(&hfull));
       }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -576,7 +571,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
     if (tc_elect()) {
       const int mw = warp - 8;
       const uint32_t idesc = tc_idesc(128, cout);
-      int hst = 0, hph = 0, ws = 0, wph = 0, as = 0, aph = 0;
+      int hph = 0, ws = 0, wph = 0, as = 0, aph = 0;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         if (!(ok = tc_wait(su32(&aempty[as]), aph ^ 1))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -584,35 +579,26 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv3_tc(Dims dm, const bf16* __
 #pragma unroll
         for (int pl = 0; pl < NP; pl++) d[pl] = tmem + (uint32_t)((as * ZT + mw * NP + pl) * cout);
         for (int g = 0; g < ngroups && ok; g++) {
-          if (!(ok = tc_wait(su32(&hfull[hst]), hph))) break;
+          if (!(ok = tc_wait(su32(&hfull), hph))) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const int nk = min(TC_CG, cin - g * TC_CG) / 16;
-          const uint64_t a_desc = tc_desc(halo0 + hst * halo_bytes + mw * NP * TC_PLANE, chunk, TC_HX * 16);
-          const uint64_t b_desc = tc_desc(w0, 128, nk * 256);
+          constexpr int NK = TC_CG / 16;
+          const uint64_t a_desc = tc_desc(halo0 + mw * NP * TC_PLANE, chunk, TC_HX * 16);
+          const uint64_t b_desc = tc_desc(w0, 128, NK * 256);
           const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32);
           const uint32_t b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32), stage16 = stage_bytes >> 4;
-          auto group = [&](auto nkc) {
-            constexpr int NK = decltype(nkc)::value;
 #pragma unroll 3
-            for (int row = 0; row < 27 / TC_STAPS; row++) {
-              if (!(ok = ok && tc_wait(su32(&wfull[ws]), wph))) continue;
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          for (int row = 0; row < 27 / TC_STAPS; row++) {
+            if (!(ok = ok && tc_wait(su32(&wfull[ws]), wph))) continue;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-              for (int i = 0; i < TC_STAPS; i++)
-                tc_tap<NK, NP, ZT>(row * TC_STAPS + i, d, a_lo, a_hi, b_lo + (ws * TC_STAPS + i) * stage16, b_hi, idesc,
-                                   g == 0 && row == 0 && i == 0);
-              tc_commit(su32(&wempty[ws]));
-              if (++ws == P.ring) ws = 0, wph ^= 1;
-            }
-          };
-          switch (nk) {
-            case 1: group(std::integral_constant<int, 1>{}); break;
-            case 2: group(std::integral_constant<int, 2>{}); break;
-            case 3: group(std::integral_constant<int, 3>{}); break;
-            default: group(std::integral_constant<int, 4>{});
+            for (int i = 0; i < TC_STAPS; i++)
+              tc_tap<NK, NP, ZT>(row * TC_STAPS + i, d, a_lo, a_hi, b_lo + (ws * TC_STAPS + i) * stage16, b_hi, idesc,
+                                 g == 0 && row == 0 && i == 0);
+            tc_commit(su32(&wempty[ws]));
+            if (++ws == P.ring) ws = 0, wph ^= 1;
           }
-          tc_commit(su32(&hempty[hst]));
-          if (++hst == P.hs) hst = 0, hph ^= 1;
+          tc_commit(su32(&hempty));
+          hph ^= 1;
         }
         tc_commit(su32(&afull[as]));
         if (++as == P.as) as = 0, aph ^= 1;
@@ -1685,31 +1671,27 @@ TzPlan tz_plan(const stp_unet* n, const Dims& dm, int cin, int cout) {
 }
 
 // How k_conv3_tc runs a layer; false if it does not take it.  A ring of 96 KB of
-// weights, at least two stages of three taps.  Two halo stages and two accumulator stages where shared memory
-// (half an SM's, or a whole one's) and 512 columns take them; planes a tile 4, 2
-// or 1, the most that leave two tiles an SM (planes share halo planes: 6 loaded
-// for 4 computed).  A forced count as above.
+// weights, at least two stages of three taps, and one halo stage (a second does
+// not fit beside it).  Planes a tile 2 or 1, two if they leave two tiles an SM
+// (planes share halo planes: 4 loaded for 2 computed) and the accumulators'
+// columns allow; two accumulator stages in 256 columns, else one.  A forced count
+// as above.
 bool tc_plan(const stp_unet* n, const Dims& dm, int cin, int cout, TcPlan* out) {
-  const int cg = std::min(cin, TC_CG);
-  const size_t stage = (size_t)2 * TC_STAPS * cout * cg;
+  if (cin % TC_CG) return false;
+  const size_t stage = (size_t)2 * TC_STAPS * cout * TC_CG;
   const long long tiles = dm.vox() / (TC_TX * TC_TY);
   const bool forced = n->tc_planes == 1 || n->tc_planes == 2 || n->tc_planes == 4;
-  for (int q = 0; q < 6; q++) {
-    // two halo stages with the most planes, else one
-    TcPlan p;
-    p.hs = q < 3 ? 2 : 1;
-    const int zt = p.zt = 4 >> (q % 3);
-    if (forced && zt > n->tc_planes) continue;
+  for (int zt = 2; zt >= 1; zt--) {
+    if (forced ? zt > n->tc_planes : zt > 1 && tiles / zt < 2 * 152) continue;
     if (dm.d % zt || zt * cout > 256) continue;
-    if (!forced && zt > 1 && tiles / zt < 2 * 152) continue;
+    TcPlan p;
+    p.zt = zt;
     p.ring = (int)std::min<size_t>(TC_RING, std::max<size_t>(2, 96 * 1024 / stage));
     p.as = 2 * zt * cout <= 256 ? 2 : 1;
     p.cols = 32;
     while (p.cols < p.as * zt * cout) p.cols *= 2;
-    const size_t halo = (size_t)(cg / 8) * TC_PLANE * (zt + 2);
-    p.smem = p.hs * halo + p.ring * stage;
+    p.smem = (size_t)(TC_CG / 8) * TC_PLANE * (zt + 2) + p.ring * stage;
     if (p.smem > kTcSmemSm) continue;
-    p.per_sm = p.smem <= kTcSmemSm / 2 - 2048 && 2 * p.cols <= 512 ? 2 : 1;
     *out = p;
     return true;
   }
@@ -1739,11 +1721,11 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
     const unsigned tiles = (unsigned)(V / (TC_TX * TC_TY * p.zt));
     auto go = [&](auto kern, std::atomic<unsigned>& done) -> cudaError_t {
       if (cudaError_t e = smem_limit_once(kern, (int)kTcSmemSm, done)) return e;
-      return launch_dep(kern, std::min(tiles, 152u * p.per_sm), TC_THREADS, p.smem, n->st, dm, x, ldx, cin, wimg, bias,
+      return launch_dep(kern, std::min(tiles, 152u), TC_THREADS, p.smem, n->st, dm, x, ldx, cin, wimg, bias,
                         cout, y, ldy, relu, mask, ldm, p, n->d_err);
     };
-    static std::atomic<unsigned> done1{0u}, done2{0u}, done4{0u};
-    UTRY(n, p.zt == 4 ? go(k_conv3_tc<4>, done4) : p.zt == 2 ? go(k_conv3_tc<2>, done2) : go(k_conv3_tc<1>, done1));
+    static std::atomic<unsigned> done1{0u}, done2{0u};
+    UTRY(n, p.zt == 2 ? go(k_conv3_tc<2>, done2) : go(k_conv3_tc<1>, done1));
     return STP_OK;
   }
   // output channels a block: 32, 16 or 8, the widest that still gives 100
