@@ -20,7 +20,9 @@
  *
  * Pointers: `where` = STP_HOST for host memory, STP_DEVICE for memory on the
  * handle's device.  The library never keeps a caller pointer after a call
- * returns; it owns all its device memory and frees it in stp_destroy.
+ * returns; it owns all its device memory and frees it in stp_destroy.  (Among
+ * it, for FP64 point sweeps, the coefficients of every sweep of a cycle: 48
+ * bytes a level and sweep, up to 80 MB; longer schedules form them as they go.)
  *
  * The pressure solve runs as one CUDA graph steered from the device (graph
  * conditional nodes), one kernel per SRJ sweep.  The FP32 inner solve of a
@@ -359,7 +361,9 @@ long long stp_unet_param_count(void);
    it is valid; the forward output does not depend on it).  The mma.sync ones
    take 32, 16 or 8 output channels a block by grid size (STP_UNET_MMA_NT=
    <8|4|2|1> forces a width where the channels allow, 8 as 4; results do not
-   depend on it either). */
+   depend on it either).  A network holds what its training needs from the
+   start: optimiser state, activation gradients, and the partial sums of its
+   largest weight gradient (at most 24 MB, by its levels' sizes). */
 int stp_unet_create(int nmax, int nz, int ny, int nx, void *stream, stp_unet **out);
 void stp_unet_destroy(stp_unet *net);
 const char *stp_unet_last_error(const stp_unet *net);

@@ -1556,7 +1556,7 @@ struct stp_unet {
   float *y = nullptr, *gy = nullptr, *loss = nullptr;
   float* h_loss = nullptr;  // pinned: loss, then h_err
   int* h_err = nullptr;
-  float* wpart = nullptr;                                  // slices of the weight gradients (kWgradScratch)
+  float* wpart = nullptr;                                  // slices of the weight gradients (wgrad_scratch)
   float *xin = nullptr, *tin = nullptr, *snorm = nullptr;  // normalised pairs, per-sample norms
   int guess_kernels = 0;                                   // kernels launched by one guess
   float out_scale = 1.f;                                   // the network predicts out_scale * dp / s
@@ -1757,13 +1757,26 @@ int conv3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const bf
 int wgrad_tile(int c) { return c % 32 == 0 ? 32 : 16; }
 // input channels a block: with 16 outputs all of 48 (gz is then read once)
 int wgrad_ctile(int cin, int cout) { return cin == 48 && wgrad_tile(cout) == 16 ? 48 : wgrad_tile(cin); }
-constexpr size_t kWgradScratch = (size_t)6 << 20;  // floats
+constexpr size_t kWgradScratch = (size_t)6 << 20;  // floats at most
 int wgrad_slices(const Dims& dm, int cin, int cout) {
   const long long pairs = (long long)(cin / wgrad_ctile(cin, cout)) * (cout / wgrad_tile(cout));
   const long long tiles = wg_tiles(dm).count(dm.n);
   long long s = std::max<long long>(1, (2 * 152 + pairs - 1) / pairs);
   s = std::min(s, (long long)(kWgradScratch / ((size_t)WG_SLOTS * cin * cout)));
   return (int)std::max<long long>(1, std::min(s, tiles));
+}
+
+int wgrad_in_slices(const Dims& dm) { return std::min(wg_tiles(dm).count(dm.n), 4 * 152); }
+// floats of the slices of the largest weight gradient of a network (smaller
+// batches have no more tiles, so no more slices)
+size_t wgrad_scratch(const stp_unet* n) {
+  size_t need = (size_t)512 * wgrad_in_slices(n->dm[0]);
+  for (int i = 1; i < 14; i++) {
+    const Layer& ly = n->L[i];
+    const Dims& dm = n->dm[i < 8 ? i / 2 : 2 - (i - 8) / 2];
+    need = std::max(need, (size_t)WG_SLOTS * ly.cin * ly.cout * wgrad_slices(dm, ly.cin, ly.cout));
+  }
+  return need;
 }
 
 template <int OT, int CT>
@@ -1790,7 +1803,7 @@ int wgrad3(stp_unet* n, const Dims& dm, const bf16* x, int ldx, int cin, const b
   return STP_OK;
 }
 int wgrad_in(stp_unet* n, const Dims& dm, const float* x, const bf16* gz, int ldg, const Layer& ly) {
-  const int slices = std::min(wg_tiles(dm).count(dm.n), 4 * 152);
+  const int slices = wgrad_in_slices(dm);
   UTRY(n, launch_dep(k_wgrad_in, slices, 256, 0, n->st, dm, x, gz, ldg, n->wpart));
   UTRY(n, launch_dep(k_wgrad_in_sum, (28 * 16 * 32 + 127) / 128, 128, 0, n->st, n->wpart, slices, n->grad + ly.woff,
                      n->grad + ly.boff));
@@ -2055,7 +2068,7 @@ int stp_unet_create(int nmax, int nz, int ny, int nx, void* stream, stp_unet** o
   A(&n->snorm, (size_t)nmax);
   A(&n->gy, (size_t)V[0]);
   A(&n->loss, 1);
-  A(&n->wpart, kWgradScratch);
+  A(&n->wpart, wgrad_scratch(n));
   A(&n->d_err, 1);
   if (const char* e = std::getenv("STP_UNET_TC")) n->use_tc = std::atoi(e) != 0;
   if (const char* e = std::getenv("STP_UNET_TC_PLANES")) n->tc_planes = std::atoi(e);
