@@ -168,11 +168,9 @@ __global__ void __launch_bounds__(8 * NCH, MINB) k_col_line(Geom<float> g, float
   const unsigned rs = (unsigned)(j == 0 ? ny - 1 : j - 1) * hx + x;
   const bool odd = (j + c0l) & 1;
   const unsigned xe = (unsigned)j * hx + (odd ? (x + W == hx ? 0 : x + W) : (x == 0 ? hx - 1 : x - 1));
-  // level range of chunk c: [0, t) cut evenly, [t, nz) cut with the first
-  // piece (holding the twist level t) never empty
   const bool lower = c < H;
-  const int k0 = lower ? c * t / H : t + ((c - H) * (nz - t) + H - 1) / H;
-  const int k1 = lower ? (c + 1) * t / H : (c + 1 == NCH ? nz : t + ((c - H + 1) * (nz - t) + H - 1) / H);
+  int k0, k1;
+  line_chunk_levels<NCH>(c, nz, k0, k1);
   const int L = k1 - k0;
   const bool twist = c == H;
   const float idx2 = g.idx2, idy2 = g.idy2;
@@ -435,26 +433,11 @@ __global__ void __launch_bounds__(256) k_col_addcorr(double* __restrict__ p, con
   }
 }
 
-template <typename... P, typename... A>
-cudaError_t launch_dep(void (*kern)(P...), unsigned grid, unsigned block, cudaStream_t s, A... a) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a...);
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 template <int W, int KZ>
 cudaError_t point_w(const Geom<float>& g, float* own, const float* oth, const float* r, float om, int c,
                     cudaStream_t s) {
   const long long units = (long long)(g.nx / 2 / W) * g.ny * ((g.nz + KZ - 1) / KZ);
-  return launch_dep(k_col_point<W, KZ>, (unsigned)((units + 255) / 256), 256, s, g, own, oth, r, om, c);
+  return launch_dep(k_col_point<W, KZ>, (unsigned)((units + 255) / 256), 256, 0, s, g, own, oth, r, om, c);
 }
 
 // z-line variants: columns a thread.  The chunks a column are no variant, since
@@ -469,14 +452,19 @@ template <int W, int NCH, int MINB>
 cudaError_t line_w(const Geom<float>& g, float* own, const float* oth, const float* r, float om, int c,
                    cudaStream_t s) {
   const unsigned blocks = (unsigned)((g.nx / 2 / W + 7) / 8 * g.ny);
-  return launch_dep(k_col_line<W, NCH, kLineLevels, MINB>, blocks, 8 * NCH, s, g, own, oth, r, om, c);
+  return launch_dep(k_col_line<W, NCH, kLineLevels, MINB>, blocks, 8 * NCH, 0, s, g, own, oth, r, om, c);
 }
 
-// Channels of at least this many cells.  Below it a sweep is bound by its launch
-// rather than by its cells (us a Jacobi / colour sweep: 32^3 1.68 / 1.62,
-// 64 x 48 x 40 1.73 / 1.58, 128 x 64 x 128 2.83 / 2.33; 240 x 140 x 120 6.7 /
-// 5.2, 256 x 128 x 192 z lines 17.7 / 11.5), and such channels have other ways
-// to save launches (kernels_cluster.cu).
+// Channels of at least this many cells: the size from which two colours lose on
+// no grid measured.  ms a solve to 1e-8, Jacobi / two colours, point sweeps: 64^3
+// 1.8 / 1.6, 128 x 64 x 64 2.7 / 1.9, 128 x 64 x 128 5.6 / 4.7, 160 x 96 x 128 11.2 /
+// 6.3; above the line 192 x 96 x 128 12.4 / 6.5, 240 x 140 x 120 20.6 / 13.2.  z
+// lines: 128 x 64 x 64 4.7 / 4.3, 96 x 80 x 128 6.1 / 6.8, 128 x 64 x 128 6.1 / 6.5,
+// 128 x 96 x 128 9.0 / 7.8; above it 192 x 96 x 128 11.1 / 10.3, 256 x 128 x 192 36.2 /
+// 29.6.  So z lines cross over near 1.5 x 2^20 cells, while point sweeps gain
+// down to 2^18 and lose to the cluster below (32^3, three steps: 2.5 / 3.2).
+// The two end equally far from the exact solution on every grid (steps of
+// 32^3 to 256 x 128 x 192: errors within 2 % of one another).
 constexpr long long kColourCells = 1 << 21;
 
 int col_width(int nx) { return nx % 8 == 0 ? 4 : nx % 4 == 0 ? 2 : 1; }

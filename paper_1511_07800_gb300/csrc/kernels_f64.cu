@@ -129,7 +129,9 @@ __global__ void __launch_bounds__(CW * NCH) k_line_f64(Geom<double> g, const dou
   const unsigned xe = row + (i + 1 == nx ? 0 : i + 1), x0 = row + ib, xw = row + (ib == 0 ? nx - 1 : ib - 1);
   const unsigned yn = (unsigned)(j + 1 == ny ? 0 : j + 1) * nx + i, ys = (unsigned)(j == 0 ? ny - 1 : j - 1) * nx + i;
   const bool lower = c < H;
-  const int k0 = line_chunk_start(c, NCH, nz), k1 = line_chunk_start(c + 1, NCH, nz), L = k1 - k0;
+  int k0, k1;
+  line_chunk_levels<NCH>(c, nz, k0, k1);
+  const int L = k1 - k0;
   const bool twist = c == H;  // holds the twist level t = k0, its last; it has LMAX levels
   const int Le = twist ? LMAX - 1 : L;  // levels the elimination runs over
   // level q of the chunk, within the column
@@ -229,22 +231,6 @@ __global__ void __launch_bounds__(CW * NCH) k_line_f64(Geom<double> g, const dou
       if (!twist) G[q] = fma(__ldg(g.pe + level(q)), carry, G[q]);
       if (act) out[lev(q) + rc] = fma(-wt[level(q)], G[q], C[q]);
     }
-}
-
-template <typename... P, typename... A>
-cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a...);
-  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace

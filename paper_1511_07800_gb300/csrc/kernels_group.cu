@@ -220,32 +220,12 @@ __global__ void __launch_bounds__(kBX* kBY) kg_addcorr(Group G) {
 
 template <int KZ, int BY>
 cudaError_t launch_gs(const Group& G, int m, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)G.vtiles);
-  cfg.blockDim = dim3(kBX, BY, 1);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kg_sweep<KZ, BY>, G, m);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_dep(kg_sweep<KZ, BY>, dim3((unsigned)G.vtiles), dim3(kBX, BY, 1), 0, s, G, m);
 }
 
 template <int KZ>
 cudaError_t launch_gf(const Group& G, int m, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)G.vtiles);
-  cfg.blockDim = dim3(kBX, kBY, 1);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kg_sweep_flat<KZ>, G, m);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_dep(kg_sweep_flat<KZ>, dim3((unsigned)G.vtiles), dim3(kBX, kBY, 1), 0, s, G, m);
 }
 
 }  // namespace

@@ -618,11 +618,9 @@ __global__ void __launch_bounds__(8 * NCH, 4) k_line_sweep_chunk(Geom<float> g, 
   const unsigned c0 = (unsigned)j * nx + i;
   const unsigned yp = (unsigned)(j == ny - 1 ? 0 : j + 1) * nx + i, ym = (unsigned)(j == 0 ? ny - 1 : j - 1) * nx + i;
   const unsigned xl = (unsigned)j * nx + (i == 0 ? nx - 1 : i - 1), xr = (unsigned)j * nx + (i + 4 == nx ? 0 : i + 4);
-  // level range [k0, k1) of chunk c: [0, t) cut evenly from below, [t, nz)
-  // cut with the first piece (holding t) never empty
   const bool lower = c < H;
-  const int k0 = lower ? c * t / H : t + ((c - H) * (nz - t) + H - 1) / H;
-  const int k1 = lower ? (c + 1) * t / H : (c + 1 == NCH ? nz : t + ((c - H + 1) * (nz - t) + H - 1) / H);
+  int k0, k1;
+  line_chunk_levels<NCH>(c, nz, k0, k1);
   const int L = k1 - k0;
   const bool twist = c == H;
   const float idx2 = g.idx2, idy2 = g.idy2;
@@ -1040,19 +1038,7 @@ static cudaError_t launch_pair(const Geom<float>& g, const float* p, const float
     e = smem_limit_once(k_sweep_f32_pair<TY, TZ>, optin, done);
     if (e != cudaSuccess) return e;
   }
-  const dim3 grid(g.ny / TY, g.nz / TZ), block(256);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep_f32_pair<TY, TZ>, g, p, b, om_a, om_b, out);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_dep(k_sweep_f32_pair<TY, TZ>, dim3(g.ny / TY, g.nz / TZ), 256, smem, s, g, p, b, om_a, om_b, out);
 }
 
 cudaError_t launch_sweep_pair(const Geom<float>& g, const float* p, const float* b, float om_a, float om_b,
@@ -1066,45 +1052,19 @@ cudaError_t launch_sweep_pair(const Geom<float>& g, const float* p, const float*
   }
 }
 
-static cudaError_t launch_sweep_cfg(const void* kern, dim3 grid, dim3 block, cudaStream_t s, void** args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelExC(&cfg, kern, args);
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 template <int KZ>
 static cudaError_t launch_flat(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
                                cudaStream_t s) {
   const long long units = (long long)(g.nz / KZ) * (g.nx / 4) * g.ny;
   const dim3 grid((unsigned)((units + kBX * kBY - 1) / (kBX * kBY))), block(kBX, kBY, 1);
-  Geom<float> gg = g;
-  void* args[] = {&gg, &p, &b, &omega, &out};
-  return launch_sweep_cfg((const void*)k_sweep_f32_flat<KZ>, grid, block, s, args);
+  return launch_dep(k_sweep_f32_flat<KZ>, grid, block, 0, s, g, p, b, omega, out);
 }
 
 template <int KZ, int BY>
 static cudaError_t launch_z(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
                             cudaStream_t s) {
   const dim3 grid((g.nx / 4 + kBX - 1) / kBX, (g.ny + BY - 1) / BY, g.nz / KZ), block(kBX, BY, 1);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep_f32_z<KZ, BY>, g, p, b, omega, out);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_dep(k_sweep_f32_z<KZ, BY>, grid, block, 0, s, g, p, b, omega, out);
 }
 
 cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
@@ -1125,9 +1085,7 @@ cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* 
   }
   const int w = g.nx % 2 == 0 ? 2 : 1;
   const dim3 grid((unsigned)(((long long)(g.nx / w) * g.ny * g.nz + kBX * kBY - 1) / (kBX * kBY))), block(kBX * kBY);
-  Geom<float> gg = g;
-  void* args[] = {&gg, &p, &b, &omega, &out};
-  return launch_sweep_cfg(w == 2 ? (const void*)k_sweep_f32<2> : (const void*)k_sweep_f32<1>, grid, block, s, args);
+  return launch_dep(w == 2 ? k_sweep_f32<2> : k_sweep_f32<1>, grid, block, 0, s, g, p, b, omega, out);
 }
 
 const char* sweep_f32_name(int variant, int nx, int ny, int nz) {
@@ -1152,23 +1110,16 @@ static int line_rows(int nz, size_t es) {
 
 // the shared-memory line sweeps at RB rows per block (the vector kernel when
 // rows hold whole vectors); raises their shared-memory limit once a device
-template <typename T, int RB>
-static cudaError_t launch_line_rows(const Geom<T>& g, const T* p, const T* b, T omega, T* out, cudaStream_t s,
-                                    cudaLaunchAttribute* attr) {
+template <int RB>
+static cudaError_t launch_line_rows(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
+                                    cudaStream_t s) {
   static std::atomic<unsigned> done_smem{0u}, done_vec{0u};
-  cudaError_t e0 = smem_limit_once(k_line_sweep_smem<T, RB>, 96 * 1024, done_smem);
-  if (e0 == cudaSuccess) e0 = smem_limit_once(k_line_sweep_vec<T, RB>, 96 * 1024, done_vec);
-  if (e0 != cudaSuccess) return e0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(((g.nx + 31) / 32) * ((g.ny + RB - 1) / RB)));
-  cfg.blockDim = dim3(512);
-  cfg.dynamicSmemBytes = (size_t)32 * RB * g.nz * sizeof(T);
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = g.nx % VecOf<T>::W == 0 ? cudaLaunchKernelEx(&cfg, k_line_sweep_vec<T, RB>, g, p, b, omega, out)
-                                          : cudaLaunchKernelEx(&cfg, k_line_sweep_smem<T, RB>, g, p, b, omega, out);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  cudaError_t e = smem_limit_once(k_line_sweep_smem<float, RB>, 96 * 1024, done_smem);
+  if (e == cudaSuccess) e = smem_limit_once(k_line_sweep_vec<float, RB>, 96 * 1024, done_vec);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)(((g.nx + 31) / 32) * ((g.ny + RB - 1) / RB)));
+  return launch_dep(g.nx % VecOf<float>::W == 0 ? k_line_sweep_vec<float, RB> : k_line_sweep_smem<float, RB>, grid, 512,
+                    (size_t)32 * RB * g.nz * sizeof(float), s, g, p, b, omega, out);
 }
 
 // levels a chunk of the register-chunked line sweep holds at most, and the
@@ -1182,53 +1133,32 @@ bool line_chunk_ok(int nx, int nz) {
          (nz - t + H - 1) / H <= kLineChunkLevels;
 }
 
-template <typename T>
-cudaError_t launch_line_sweep(const Geom<T>& g, const T* p, const T* b, T omega, T* out, cudaStream_t s,
-                              int variant) {
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  if constexpr (sizeof(T) == 4) {
-    if (variant == 1 && line_chunk_ok(g.nx, g.nz)) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)((g.nx / 32) * g.ny));
-      cfg.blockDim = dim3(8 * kLineChunks);
-      cfg.stream = s;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      cudaError_t e = cudaLaunchKernelEx(&cfg, k_line_sweep_chunk<kLineChunks, kLineChunkLevels>, g, p, b, omega, out);
-      return e != cudaSuccess ? e : cudaGetLastError();
-    }
-  }
-  if constexpr (sizeof(T) == 8) {
-    if (line_f64_chunks(g.nx, g.ny, g.nz) > 0) return launch_line_f64(g, p, b, omega, out, s);
-  } else
-  switch (line_rows(g.nz, sizeof(T))) {
-    case 4: return launch_line_rows<T, 4>(g, p, b, omega, out, s, attr);
-    case 2: return launch_line_rows<T, 2>(g, p, b, omega, out, s, attr);
-    case 1: return launch_line_rows<T, 1>(g, p, b, omega, out, s, attr);
-    default: break;
-  }
-  const dim3 grid((g.nx + 127) / 128, g.ny), block(128);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_line_sweep<T>, g, p, b, omega, out);
-  return e != cudaSuccess ? e : cudaGetLastError();
+template <>
+cudaError_t launch_line_sweep<double>(const Geom<double>& g, const double* p, const double* b, double omega, double* out,
+                                      cudaStream_t s, int) {
+  if (line_f64_chunks(g.nx, g.ny, g.nz) > 0) return launch_line_f64(g, p, b, omega, out, s);
+  return launch_dep(k_line_sweep<double>, dim3((g.nx + 127) / 128, g.ny), 128, 0, s, g, p, b, omega, out);
 }
+template <>
+cudaError_t launch_line_sweep<float>(const Geom<float>& g, const float* p, const float* b, float omega, float* out,
+                                     cudaStream_t s, int variant) {
+  if (variant == 1 && line_chunk_ok(g.nx, g.nz))
+    return launch_dep(k_line_sweep_chunk<kLineChunks, kLineChunkLevels>, dim3((unsigned)((g.nx / 32) * g.ny)),
+                      8 * kLineChunks, 0, s, g, p, b, omega, out);
+  switch (line_rows(g.nz, sizeof(float))) {
+    case 4: return launch_line_rows<4>(g, p, b, omega, out, s);
+    case 2: return launch_line_rows<2>(g, p, b, omega, out, s);
+    case 1: return launch_line_rows<1>(g, p, b, omega, out, s);
+    default: return launch_dep(k_line_sweep<float>, dim3((g.nx + 127) / 128, g.ny), 128, 0, s, g, p, b, omega, out);
+  }
+}
+
 const char* line_sweep_name(bool f64, int nx, int ny, int nz, int variant) {
   if (f64) return line_f64_chunks(nx, ny, nz) ? "k_line_f64" : "k_line_sweep<double>";
   if (variant == 1 && line_chunk_ok(nx, nz)) return "k_line_sweep_chunk";
   if (!line_rows(nz, sizeof(float))) return "k_line_sweep<float>";
   return nx % VecOf<float>::W == 0 ? "k_line_sweep_vec" : "k_line_sweep_smem";
 }
-template cudaError_t launch_line_sweep<float>(const Geom<float>&, const float*, const float*, float, float*,
-                                              cudaStream_t, int);
-template cudaError_t launch_line_sweep<double>(const Geom<double>&, const double*, const double*, double, double*,
-                                               cudaStream_t, int);
 
 // Persistent z-line cycles (FP32, vector kernel): the rows per tile of the
 // line sweep, and 0 when the grid does not take them (rows not a multiple

@@ -223,6 +223,11 @@ cudaError_t launch_diffusion_only(const Geom<T>& g, bool les, const T* u, const 
 template <typename T>
 cudaError_t launch_line_sweep(const Geom<T>& g, const T* p, const T* b, T omega, T* out, cudaStream_t s,
                               int variant);
+template <>
+cudaError_t launch_line_sweep<float>(const Geom<float>&, const float*, const float*, float, float*, cudaStream_t, int);
+template <>
+cudaError_t launch_line_sweep<double>(const Geom<double>&, const double*, const double*, double, double*, cudaStream_t,
+                                      int);
 // whether the register-chunked FP32 line sweep (variant 1) takes the grid
 bool line_chunk_ok(int nx, int nz);
 // name of the kernel that launch_line_sweep, or launch_sweep_f32 with a variant set, runs
@@ -419,6 +424,25 @@ inline cudaError_t smem_limit_once(K kern, int bytes, std::atomic<unsigned>& don
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_acq_rel);
   return e;
+}
+
+// Launch as a programmatic dependent of the stream's previous kernel: the grid
+// is set up while that one's last blocks finish, and the kernel waits with
+// cudaGridDependencySynchronize before it touches what that one wrote.
+template <typename... K, typename... A>
+cudaError_t launch_dep(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace stp

@@ -1570,27 +1570,11 @@ struct stp_unet {
 
 namespace {
 
-// Launch as a programmatic dependent of the stream's previous kernel: the grid
-// is set up while that one's last blocks finish, and the kernel waits with
-// cudaGridDependencySynchronize before it touches memory.  A forward has 21
-// launches, a gradient 57, with gaps of 2 to 3 us between plain ones: 527 us a
-// forward of 128 x 64 x 128 and 1516 a gradient of 4 x 64 x 32 x 64, 471 and
-// 1362 this way (some 10 us of each by reading the error flag with the results).
-template <typename... K, typename... A>
-cudaError_t launch_dep(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
+// The network's kernels are launched as programmatic dependents (launch_dep): a
+// forward has 21 launches, a gradient 57, with gaps of 2 to 3 us between plain
+// ones: 527 us a forward of 128 x 64 x 128 and 1516 a gradient of 4 x 64 x 32 x
+// 64, 471 and 1362 this way (some 10 us of each by reading the error flag with the
+// results).
 
 int ufail(stp_unet* n, int code, const std::string& m) {
   if (n) n->err = m;
