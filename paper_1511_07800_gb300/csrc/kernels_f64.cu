@@ -64,8 +64,9 @@ __global__ void __launch_bounds__(128) k_sweep_f64(Geom<double> g, const double*
   double ax = 0, ay = 0, au = 0, ad = 0, ab = 0, ac = om1;
   if (act) {
     if constexpr (TAB) {
-      ax = __ldg(tab + 6 * k), ay = __ldg(tab + 6 * k + 1), au = __ldg(tab + 6 * k + 2);
-      ad = __ldg(tab + 6 * k + 3), ab = __ldg(tab + 6 * k + 4), ac = __ldg(tab + 6 * k + 5);
+      const double2* c = reinterpret_cast<const double2*>(tab) + 3 * k;
+      const double2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
+      ax = c0.x, ay = c0.y, au = c1.x, ad = c1.y, ab = c2.x, ac = c2.y;
     } else {
       ab = omega * __ldg(g.iS + k);
       ax = ab * g.idx2, ay = ab * g.idy2, au = ab * __ldg(g.cup + k), ad = ab * __ldg(g.cdn + k);
