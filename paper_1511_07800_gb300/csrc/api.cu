@@ -628,6 +628,20 @@ int launch_colour_cycle(stp_handle* h, cudaStream_t s) {
     CUDA_TRY(h, launch_colour_sweep(h->g32, h->d1, h->r32, h->col_omega[m], m & 1, h->cfg.zline, h->sweep_variant, s));
   return STP_OK;
 }
+// FP64 z-line cycles run on corrections (k_line_f64)
+bool uses_line_f64(const stp_handle* h) {
+  return h->prec == STP_FP64 && h->cfg.zline && line_f64_chunks(h->nx, h->ny, h->nz) > 0;
+}
+// one of them, in place in p.  Residual and correction take the Crank-Nicolson
+// right-hand sides' arrays, which are free outside the velocity half step.
+int launch_line_f64_cycle(stp_handle* h, cudaStream_t s) {
+  const int M = (int)h->omega.size();
+  double *r = (double*)h->ru, *d[2] = {h->p2, (double*)h->rv};
+  CUDA_TRY(h, launch_residual_f64(h->g64, h->p, h->b, r, s));
+  for (int m = 0; m < M; m++)
+    CUDA_TRY(h, launch_line_f64(h->g64, m ? d[(m - 1) & 1] : nullptr, r, h->omega[m], d[m & 1], m == M - 1 ? h->p : nullptr, s));
+  return STP_OK;
+}
 cudaError_t launch_cycle_check(stp_handle* h, const Geom<double>& g, const double* A, const double* rhs, int mode, int graph,
                                cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_body, cudaStream_t s) {
   return launch_check<double>(g, A, rhs, mode, h->ctl, h->red, graph, h_loop, h_body, s);
@@ -676,6 +690,10 @@ int build_cycle(stp_handle* h, const Geom<T>& g, cudaGraph_t wb, cudaGraphCondit
     if (sizeof(T) == sizeof(float) && h->line_rb > 0) {
       CUDA_TRY(h, launch_line_cycle_f32(h->g32, h->line_rb, (float*)A, (float*)B, (const float*)rhs, h->d_omega32, M,
                                         h->line_flags, h->ctl, h->cap));
+      return end_capture(h, ib);
+    }
+    if (sizeof(T) == sizeof(double) && uses_line_f64(h)) {
+      if ((rc = launch_line_f64_cycle(h, h->cap))) return rc;
       return end_capture(h, ib);
     }
     for (int m = 0; m < M; m++)
@@ -995,7 +1013,7 @@ int arm_solves(stp_handle* h, double tol, int maxit) {
   c.max_sweeps = maxit;
   c.max_passes = 64;
   c.M = (int)h->omega.size();
-  c.kpc = use_colour(h) ? c.M : (uses_cluster(h) || h->cycle_blocks > 0 || h->line_rb > 0) ? 1 : uses_pairs(h) ? c.M / 2 : c.M;
+  c.kpc = use_colour(h) ? c.M : (uses_cluster(h) || h->cycle_blocks > 0 || h->line_rb > 0) ? 1 : uses_pairs(h) ? c.M / 2 : uses_line_f64(h) ? c.M + 1 : c.M;
   c.bar_wait = 2000000000LL;
   if (const char* e = std::getenv("STP_BARRIER_WAIT")) {
     const long long w = std::atoll(e);
@@ -1050,6 +1068,10 @@ int host_cycles(stp_handle* h, const Geom<T>& g, T* A, T* B, const T* rhs, int m
       if (sizeof(T) == sizeof(float) && h->line_rb > 0) {
         CUDA_TRY(h, launch_line_cycle_f32(h->g32, h->line_rb, (float*)A, (float*)B, (const float*)rhs, h->d_omega32,
                                           M, h->line_flags, h->ctl, h->st));
+        continue;
+      }
+      if (sizeof(T) == sizeof(double) && uses_line_f64(h)) {
+        if ((rc = launch_line_f64_cycle(h, h->st))) return rc;
         continue;
       }
       for (int m = 0; m < M; m++)

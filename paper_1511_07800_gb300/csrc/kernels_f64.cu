@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "device_util.cuh"
+#include "poisson_common.cuh"
 #include "stp_internal.cuh"
 
 namespace stp {
@@ -86,48 +87,60 @@ __global__ void __launch_bounds__(128) k_sweep_f64(Geom<double> g, const double*
   out[q] = fma(ac, pc, t);
 }
 
-// One z-line Jacobi-SOR sweep, p' = p - omega A^-1 (b - L p), the columns solved
-// in registers in level chunks as in k_line_sweep_chunk (kernels_poisson.cu).  A
-// block takes CW columns of a row x NCH chunks of at most LMAX levels.
+// r = b - L p in differences of neighbours
+__global__ void __launch_bounds__(kBX* kBY) k_residual_f64(Geom<double> g, const double* __restrict__ p,
+                                                            const double* __restrict__ b, double* __restrict__ r) {
+  const int i = blockIdx.x * kBX + threadIdx.x, j = blockIdx.y * kBY + threadIdx.y, k = blockIdx.z;
+  if (i >= g.nx || j >= g.ny) return;
+  double pc;
+  r[at(g.nx, g.ny, i, j, k)] = point_residual(g, p, b, i, j, k, &pc);
+}
+
+// One z-line Jacobi-SOR sweep d' = d + omega (d^L - d) of L d = r, the columns
+// solved in registers in level chunks as in k_line_sweep_chunk
+// (kernels_poisson.cu).  A block takes CW columns of a row x NCH chunks of at most
+// LMAX levels.
 //
-// The right-hand side is the residual, in differences of neighbours: solved for
-// the line value itself (A p^L = sum of the x and y neighbours - b: six
-// operations a cell) it would round with the size of S p, and solves of smooth
-// fields stall 1.7 to 2.5 times higher (64 x 32 x 192, stretch 2: 1.0e-11 of ||b||
-// against 4.2e-12).  A difference serves both its cells where it costs less than
-// it saves: along the chunk in registers, along x by shuffle, the difference
-// into the block's first column being taken for all levels at once, a lane a
-// level.  The elimination runs on undivided values (Geom::lf, lb), so that the
-// pivot joins omega in one coefficient a level: fifteen operations a cell.  us a
-// sweep, line values with every thread walking its own carries (twelve
-// operations) / this: 32 x 16 x 32 6.3 / 5.5, 96 x 48 x 64 11.1 / 11.4, 64 x 30 x
-// 100 13.9 / 11.4, 64 x 32 x 192 18.1 / 16.9, and where the FP64 pipe alone
-// bounds it 112 x 56 x 112 22.4 / 25.1, 128 x 64 x 128 31.6 / 38.2 (of which 512
-// blocks on 152 SMs leave a fifth idle); the lock-step kernel took 41.2 at 96 x 48
-// x 64.
+// The sweeps of a cycle run on the correction d to the pressure the cycle starts
+// from, r being its residual: the line value's own equation A d^L = (sum of the
+// x and y neighbours) - r takes four operations a cell where A^-1 (r - L d)
+// takes ten, and what it rounds is of the size of S d, which vanishes as the solve
+// converges: a solve of a smooth field on 64 x 32 x 192 at stretch 2 stalls at
+// 4.0e-13 of ||b||; with the same sweeps on the pressure itself, which round with
+// S p, at 1.0e-11, in residual form at 4.3e-12.  The cycle's
+// first sweep has d = 0 (d null) and its last adds d to the pressure (base:
+// written in place of out).
 //
-// A thread counts its levels from the wall's side of the chunk to the twist
-// level's, so both sides run the same code.  What enters a chunk is walked chunk
-// by chunk by one warp, a lane a column and side (by every thread for itself it
-// took as many operations as the columns' own recurrences).  Chunks stay long
+// The elimination runs on undivided values (Geom::lf, lb), so that the pivot
+// joins omega in one coefficient a level: ten operations a cell (twelve on the
+// pressure, fifteen in residual form).  us a sweep, on the pressure with every
+// thread walking its own carries / in residual form / this: 32 x 16 x 32 6.3 /
+// 5.5 / 4.4, 96 x 48 x 64 11.1 / 11.4 / 8.6, 64 x 30 x 100 13.9 / 11.4 / 9.0, 64 x 32
+// x 192 18.1 / 16.9 / 12.5, 112 x 56 x 112 22.4 / 25.1 / 17.7, 128 x 64 x 128 31.6 /
+// 38.2 / 27.7 (of which 512 blocks on 152 SMs leave a fifth idle); the lock-step
+// kernel took 41.2 at 96 x 48 x 64.  A thread
+// counts its levels from the wall's side of the chunk to the twist level's, so
+// both sides run the same code.  What enters a chunk is walked chunk by chunk by
+// one warp, a lane a column and side (by every thread for itself it took as many
+// operations as the columns' own recurrences).  Chunks stay long
 // (line_f64_chunks): each is a step of that walk.  LMAX is the most levels a
 // chunk has, no more, because an operation past the chunk's end takes its slot
 // on the FP64 pipe all the same.
 template <int CW, int NCH, int LMAX>
-__global__ void __launch_bounds__(CW * NCH) k_line_f64(Geom<double> g, const double* __restrict__ p,
-                                                       const double* __restrict__ b, double omega,
-                                                       double* __restrict__ out) {
+__global__ void __launch_bounds__(CW * NCH) k_line_f64(Geom<double> g, const double* __restrict__ d,
+                                                       const double* __restrict__ r, double omega, double om1,
+                                                       double* __restrict__ out, double* __restrict__ base) {
   constexpr int H = NCH / 2;
-  static_assert(CW == 16 && LMAX <= CW && H % 2 == 0, "a warp holds two chunks of one side, a lane a level");
+  static_assert(CW == 16 && H % 2 == 0, "a warp holds two chunks of one side");
   extern __shared__ double wt[];  // [nz] omega / pivot
   __shared__ double EB[NCH][CW], CB[NCH][CW], YL[CW], XT[CW], PF[NCH], PE[NCH];
   const int nx = g.nx, ny = g.ny, nz = g.nz, t = nz >> 1;
   const int u = threadIdx.x % CW, c = threadIdx.x / CW, half = threadIdx.x & CW;
-  const int nxb = (nx + CW - 1) / CW, j = blockIdx.x / nxb, ib = (blockIdx.x % nxb) * CW;
-  const bool act = ib + u < nx;
-  const int i = act ? ib + u : nx - 1;
+  const int nxb = (nx + CW - 1) / CW, j = blockIdx.x / nxb, i0 = (blockIdx.x % nxb) * CW + u;
+  const bool act = i0 < nx;
+  const int i = act ? i0 : nx - 1;
   const unsigned plane = (unsigned)nx * ny, row = (unsigned)j * nx, rc = row + i;
-  const unsigned xe = row + (i + 1 == nx ? 0 : i + 1), x0 = row + ib, xw = row + (ib == 0 ? nx - 1 : ib - 1);
+  const unsigned xe = row + (i + 1 == nx ? 0 : i + 1), xw = row + (i == 0 ? nx - 1 : i - 1);
   const unsigned yn = (unsigned)(j + 1 == ny ? 0 : j + 1) * nx + i, ys = (unsigned)(j == 0 ? ny - 1 : j - 1) * nx + i;
   const bool lower = c < H;
   int k0, k1;
@@ -135,40 +148,31 @@ __global__ void __launch_bounds__(CW * NCH) k_line_f64(Geom<double> g, const dou
   const int L = k1 - k0;
   const bool twist = c == H;  // holds the twist level t = k0, its last; it has LMAX levels
   const int Le = twist ? LMAX - 1 : L;  // levels the elimination runs over
-  // level q of the chunk, within the column
-  auto level = [&](int q) { return min(max(lower ? k0 + q : k1 - 1 - q, 0), nz - 1); };
-  auto lev = [&](int q) { return (unsigned)level(q) * plane; };
+  auto level = [&](int q) { return lower ? k0 + q : k1 - 1 - q; };
   for (int k = threadIdx.x; k < nz; k += CW * NCH) wt[k] = omega * __ldg(g.tli + k);
   if (u == 0) {
     PF[c] = L > 0 ? __ldg(g.pf + level(L - 1)) : 1.0;
     PE[c] = L > 0 ? __ldg(g.pe + level(0)) : 1.0;
   }
-  const double* cin = lower ? g.cup : g.cdn;   // coupling to level q + 1
-  const double* cout = lower ? g.cdn : g.cup;  // to level q - 1 (zero at the wall)
-  double C[LMAX + 1], D[LMAX], G[LMAX];
+  double C[LMAX], G[LMAX];
   const double idx2 = g.idx2, idy2 = g.idy2;
   cudaGridDependencySynchronize();
+  if (d) {
 #pragma unroll
-  for (int q = 0; q <= LMAX; q++) C[q] = __ldg(p + lev(q) + rc);
+    for (int q = 0; q < LMAX; q++)
+      if (q < L) {
+        const unsigned l = (unsigned)level(q) * plane;
+        C[q] = __ldg(d + l + rc);
+        double v = fma(idx2, __ldg(d + l + xe) + __ldg(d + l + xw), -__ldg(r + l + rc));
+        G[q] = fma(idy2, __ldg(d + l + yn) + __ldg(d + l + ys), v);
+      }
+  } else {
 #pragma unroll
-  for (int q = 0; q < LMAX; q++) D[q] = __ldg(p + lev(q) + xe) - C[q];
-  const unsigned le = lev(u < LMAX ? u : 0);
-  const double edge = __ldg(p + le + x0) - __ldg(p + le + xw);
-  double dz = C[0] - __ldg(p + lev(-1) + rc);
-#pragma unroll
-  for (int q = 0; q < LMAX; q++) {
-    const double first = __shfl_sync(0xffffffffu, edge, half + q);
-    double dw = __shfl_up_sync(0xffffffffu, D[q], 1);
-    dw = u == 0 ? first : dw;
-    if (q < L) {
-      const unsigned l = lev(q);
-      const int k = level(q);
-      double r = fma(-idx2, D[q] - dw, __ldg(b + l + rc));
-      r = fma(-idy2, (__ldg(p + l + yn) - C[q]) + (__ldg(p + l + ys) - C[q]), r);
-      r = fma(__ldg(cout + k), dz, r);
-      dz = C[q + 1] - C[q];
-      G[q] = fma(-__ldg(cin + k), dz, r);
-    }
+    for (int q = 0; q < LMAX; q++)
+      if (q < L) {
+        C[q] = 0.0;
+        G[q] = -__ldg(r + (unsigned)level(q) * plane + rc);
+      }
   }
   // elimination inside the chunk
   {
@@ -230,8 +234,18 @@ __global__ void __launch_bounds__(CW * NCH) k_line_f64(Geom<double> g, const dou
   for (int q = 0; q < LMAX; q++)
     if (q < L) {
       if (!twist) G[q] = fma(__ldg(g.pe + level(q)), carry, G[q]);
-      if (act) out[lev(q) + rc] = fma(-wt[level(q)], G[q], C[q]);
+      G[q] = fma(wt[level(q)], G[q], om1 * C[q]);
     }
+  if (!act) return;
+  if (base) {
+#pragma unroll
+    for (int q = 0; q < LMAX; q++)
+      if (q < L) base[(unsigned)level(q) * plane + rc] += G[q];
+  } else {
+#pragma unroll
+    for (int q = 0; q < LMAX; q++)
+      if (q < L) out[(unsigned)level(q) * plane + rc] = G[q];
+  }
 }
 
 }  // namespace
@@ -250,17 +264,20 @@ cudaError_t launch_sweep_f64(const Geom<double>& g, const double* p, const doubl
 }
 
 namespace {
-// Columns a block.  us a sweep at 32 / 16 / 8 (line values): 96 x 48 x 64 10.9 /
+// Columns a block.  us a sweep at 32 / 16 / 8 (on the pressure): 96 x 48 x 64 10.9 /
 // 11.1 / 11.5, 64 x 30 x 100 18.8 / 13.8 / 14.1, 112 x 56 x 112 28.6 / 22.5 / 23.5,
 // 32 x 16 x 32 7.3 / 6.5 / 6.4: 32 leave SMs without a block or a last wave nearly
 // empty.
 constexpr int kLineCols = 16;
 
 template <int NCH>
-cudaError_t line_nch(const Geom<double>& g, const double* p, const double* b, double omega, double* out, cudaStream_t s) {
+cudaError_t line_nch(const Geom<double>& g, const double* d, const double* r, double omega, double* out, double* base,
+                     cudaStream_t s) {
   const dim3 blocks((unsigned)(((g.nx + kLineCols - 1) / kLineCols) * g.ny)), threads(kLineCols * NCH);
 #define LEVELS(L) \
-  case L: return launch_dep(k_line_f64<kLineCols, NCH, L>, blocks, threads, sizeof(double) * g.nz, s, g, p, b, omega, out);
+  case L:                                                                                                      \
+    return launch_dep(k_line_f64<kLineCols, NCH, L>, blocks, threads, sizeof(double) * g.nz, s, g, d, r, omega, \
+                      1.0 - omega, out, base);
   switch (line_f64_levels(g.nz, NCH)) {
     LEVELS(1) LEVELS(2) LEVELS(3) LEVELS(4) LEVELS(5) LEVELS(6)
     LEVELS(7) LEVELS(8) LEVELS(9) LEVELS(10) LEVELS(11) LEVELS(12)
@@ -270,15 +287,21 @@ cudaError_t line_nch(const Geom<double>& g, const double* p, const double* b, do
 }
 }  // namespace
 
-cudaError_t launch_line_f64(const Geom<double>& g, const double* p, const double* b, double omega, double* out,
-                            cudaStream_t s) {
+cudaError_t launch_line_f64(const Geom<double>& g, const double* d, const double* r, double omega, double* out,
+                            double* base, cudaStream_t s) {
   switch (line_f64_chunks(g.nx, g.ny, g.nz)) {
-    case 4: return line_nch<4>(g, p, b, omega, out, s);
-    case 8: return line_nch<8>(g, p, b, omega, out, s);
-    case 16: return line_nch<16>(g, p, b, omega, out, s);
-    case 32: return line_nch<32>(g, p, b, omega, out, s);
+    case 4: return line_nch<4>(g, d, r, omega, out, base, s);
+    case 8: return line_nch<8>(g, d, r, omega, out, base, s);
+    case 16: return line_nch<16>(g, d, r, omega, out, base, s);
+    case 32: return line_nch<32>(g, d, r, omega, out, base, s);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_residual_f64(const Geom<double>& g, const double* p, const double* b, double* r, cudaStream_t s) {
+  const Launch l = plane_launch(g.nx, g.ny, g.nz);
+  k_residual_f64<<<l.grid, l.block, 0, s>>>(g, p, b, r);
+  return cudaGetLastError();
 }
 
 }  // namespace stp

@@ -1136,7 +1136,6 @@ bool line_chunk_ok(int nx, int nz) {
 template <>
 cudaError_t launch_line_sweep<double>(const Geom<double>& g, const double* p, const double* b, double omega, double* out,
                                       cudaStream_t s, int) {
-  if (line_f64_chunks(g.nx, g.ny, g.nz) > 0) return launch_line_f64(g, p, b, omega, out, s);
   return launch_dep(k_line_sweep<double>, dim3((g.nx + 127) / 128, g.ny), 128, 0, s, g, p, b, omega, out);
 }
 template <>

@@ -219,7 +219,8 @@ cudaError_t launch_diffusion_only(const Geom<T>& g, bool les, const T* u, const 
                                   T nu0, T* Du, T* Dv, T* Dw, cudaStream_t s);
 
 // One z-line Jacobi-SOR sweep: out = p - omega A^-1 (b - L p), A the z
-// column operator -L_z + (2/dx^2 + 2/dy^2) I (Thomas with the pivots li, lu).
+// column operator -L_z + (2/dx^2 + 2/dy^2) I (Thomas with the pivots li, lu).  In
+// FP64 for columns that launch_line_f64 does not take.
 template <typename T>
 cudaError_t launch_line_sweep(const Geom<T>& g, const T* p, const T* b, T omega, T* out, cudaStream_t s,
                               int variant);
@@ -243,8 +244,12 @@ cudaError_t launch_sweep_f32(const Geom<float>& g, const float* p, const float* 
 cudaError_t launch_sweep_table(const Geom<double>& g, const double* omega, int M, double* tab, cudaStream_t s);
 cudaError_t launch_sweep_f64(const Geom<double>& g, const double* p, const double* b, double omega, const double* tab,
                              double* out, cudaStream_t s);
-cudaError_t launch_line_f64(const Geom<double>& g, const double* p, const double* b, double omega, double* out,
-                            cudaStream_t s);
+// z lines of up to 384 levels: a cycle's sweeps on the correction d to its
+// pressure, L d = r, r = b - L p.  d null: d = 0; base not null: base += the
+// sweep's d, out not written.
+cudaError_t launch_residual_f64(const Geom<double>& g, const double* p, const double* b, double* r, cudaStream_t s);
+cudaError_t launch_line_f64(const Geom<double>& g, const double* d, const double* r, double omega, double* out,
+                            double* base, cudaStream_t s);
 
 // FP32 sweep variant used by launch_sweep_f32 on this host thread
 // (chosen by the autotuner in api.cu).

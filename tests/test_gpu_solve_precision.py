@@ -32,14 +32,14 @@ def offset_pressure(cfg):
 @pytest.mark.parametrize("nx,ny,nz,stretch", [(32, 16, 32, 0.0), (48, 24, 48, 2.0), (37, 21, 66, 2.0), (64, 32, 97, 2.0),
                                               (16, 8, 200, 2.0)])
 def test_line_sweeps_round_with_the_differences(stp_lib, nx, ny, nz, stretch):
-    """An FP64 z-line sweep forms b - L p in differences of neighbours, which drop
+    """An FP64 z-line cycle takes b - L p in differences of neighbours, which drop
     the pressure's level, so a solution stays where it is even under a large factor:
     two sweeps (20, then 0.5) from the solution itself move no cell by more than two
-    units in its last place.  Half a unit is each sweep's rounding of p (the
-    second sweep amplifies none of the first's: |1 - mu/2| <= 1) and half each the
-    rounding of the mean and of the returned p - mean; 20 A^-1 times the rounding of
-    the differences is some 1e-15, a hundredth of a unit.  Sweeps that form the
-    line value itself round with S p: 37 units at least."""
+    units in its last place.  Half a unit each are the rounding of p once or
+    twice (the second sweep amplifies nothing of the first's: |1 - mu/2| <= 1), of
+    the mean and of the returned p - mean; 20 A^-1 times the rounding of the
+    differences is some 1e-15, a hundredth of a unit.  Sweeps that form the line
+    value of the pressure itself round with S p: 37 units at least."""
     cfg = inputs.preset("os_instability", nx=nx, ny=ny, nz=nz, stretch=stretch, zline=1)
     p0, b = offset_pressure(cfg)
     with stp_lib.Channel(cfg, precision="fp64", omega=[20.0, 0.5]) as ch:
@@ -47,6 +47,19 @@ def test_line_sweeps_round_with_the_differences(stp_lib, nx, ny, nz, stretch):
         st = ch.poisson_solve(b, p, tol=0.0, maxit=2)
     assert st["sweeps"] == 2
     assert np.abs(p - gauge(p0, cfg)).max() <= 2 * 2.0 ** -43
+
+
+def test_line_solve_to_a_tight_tolerance(stp_lib):
+    """A strongly stretched channel (48 x 24 x 96, stretch 3) solved to 5e-12 of ||b||
+    with z lines: the sweeps of a cycle run on a correction that keeps shrinking,
+    and only its last addition rounds the pressure.  (Sweeps on the pressure stall
+    at 8.7e-12 in residual form and at 1.5e-11 on line values.)"""
+    cfg = inputs.preset("os_instability", nx=48, ny=24, nz=96, stretch=3.0, zline=1)
+    p0, b = offset_pressure(cfg)
+    with stp_lib.Channel(cfg, precision="fp64") as ch:
+        p = np.zeros_like(p0)
+        st = ch.poisson_solve(b, p, tol=5e-12, maxit=2048)
+    assert st["converged"], st["rel_res"]
 
 
 def fma(a, b, c):
