@@ -51,7 +51,8 @@
  * chunked recurrences); elsewhere, or with STP_LINE_VARIANT=0 at stp_init,
  * a block stages its columns in shared memory and solves them in lock
  * step.  The two round differently (a few units in the last place).  FP64
- * z-line sweeps solve their columns in level chunks too, up to 384 levels.
+ * z-line sweeps solve their columns in level chunks too, up to 384 levels, a
+ * cycle's sweeps on the correction to the pressure it starts from.
  * The FP32 sweep kernel's tile shape (z levels per thread, rows per block) is
  * picked on first use by timing the variants on the grid
  * (STP_SWEEP_VARIANT=<0..15> forces one; variants 6..8 pack warps along the
