@@ -241,3 +241,33 @@ def test_two_colour_channel_in_a_batch(stp_lib):
     batch.close()
     for ch in chans:
         ch.close()
+
+
+def test_line_f64_cycles_wherever_they_run(stp_lib, monkeypatch):
+    """FP64 z-line cycles borrow arrays of the velocity half step for the residual
+    and the correction: whole steps by the solve graph, driven from the host, and in
+    a batch beside a second channel end bitwise alike."""
+    specs = [case(nx=37, ny=12, nz=50, stretch=2.0, zline=1, les=1, nu=1 / 500.0),
+             case(nx=32, ny=16, nz=20, nu=1 / 500.0, zline=1, cn_zline=1)]
+    alone = []
+    for host in ("0", "1"):
+        monkeypatch.setenv("STP_HOST_SOLVE", host)
+        for i, cfg in enumerate(specs):
+            with stp_lib.Channel(cfg, precision="fp64") as ch:
+                ch.set_fields(*turbulent_like(cfg, 40 + i))
+                assert ch.step(4)["converged"]
+                assert ch.sweep_kernel() == "k_line_f64"
+                alone.append(ch.get_fields())
+    monkeypatch.delenv("STP_HOST_SOLVE")
+    chans = [stp_lib.Channel(cfg, precision="fp64") for cfg in specs]
+    for i, ch in enumerate(chans):
+        ch.set_fields(*turbulent_like(specs[i], 40 + i))
+    batch = stp_lib.Batch(chans)
+    assert batch.step(4)["converged"]
+    for i, ch in enumerate(chans):
+        got = ch.get_fields()
+        for k in ("u", "v", "w", "p"):
+            assert np.array_equal(got[k], alone[i][k]) and np.array_equal(alone[2 + i][k], alone[i][k]), (i, k)
+    batch.close()
+    for ch in chans:
+        ch.close()
